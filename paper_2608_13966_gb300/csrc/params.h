@@ -145,14 +145,16 @@ struct Nvfp4Params {
 constexpr int kLutRows = 8;
 constexpr int kLutCols = 64;
 constexpr int kLutBlock = kLutRows * kLutCols;
-// Per-warp scratch of the LUT kernel: the transpose of 12 per-threshold
-// sums of each of two candidates (rows of 36 floats: 16-byte aligned, readers
-// of rows r and r + 8 share banks), and per candidate its table (8 bytes), error, error bound and which
-// entries' roundings were undecided.
-constexpr int kLutRow = 36;
-constexpr uint32_t kLutSumsBytes = 24 * kLutRow * 4;
+// Per-warp scratch of the LUT kernel: the lists of the elements that reach
+// level 1 (|d| and h, both signs: at most kLutListCap of them a round, each
+// sign padded to a multiple of 8), per candidate its table (8 bytes), error,
+// error bound and which entries' roundings were undecided, then a decoded
+// table and the block's sums.
+constexpr int kLutListCap = 256;
+constexpr int kLutListLen = kLutListCap + 16;
+constexpr uint32_t kLutListBytes = 2 * kLutListLen * 4;
 constexpr uint32_t kLutCandBytes = kMaxClip * 20;
-constexpr uint32_t kLutScratchBytes = kLutSumsBytes + kLutCandBytes + 64;
+constexpr uint32_t kLutScratchBytes = kLutListBytes + kLutCandBytes + 64;
 
 struct LutTensor {
     const float* w;
@@ -175,7 +177,8 @@ struct LutParams {
     int n_clip;
     float beta2;
     float c1;
-    float tie_kappa;   // summation-depth bound, in ulps
+    float tie_kappa;   // multiplier of the summation-depth bounds
+    float invf_max;    // the largest 1/f
     int stages;
     uint32_t stage_bytes;
     uint64_t timeout_ns;

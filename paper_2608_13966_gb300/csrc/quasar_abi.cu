@@ -959,13 +959,12 @@ quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_ten
     p.n_clip = n_clip;
     p.beta2 = beta2;
     p.c1 = 1.0f - beta2;
-    // summation depth of the per-index sums: 8 per packed half, the fold,
-    // 8 per reader accumulator and two combining levels, plus margin
-    p.tie_kappa = 24.0f * tuning().tie_scale;
+    p.tie_kappa = tuning().tie_scale;
     p.timeout_ns = kDefaultTimeoutNs;
     p.force_timeout_ns = (uint64_t)std::max<int64_t>(0, g_force_timeout_ns.load());
     p.stats = g_stats.load();
     fill_clip(clip, n_clip, p.f, p.invf);
+    p.invf_max = *std::max_element(p.invf, p.invf + n_clip);
     if ((st = status_ptr(&p.status)) != QUASAR_OK) return st;
     const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
     const Launch L = plan((uint32_t)(kLutBlock * (8 + gbytes)), kLutScratchBytes);

@@ -7,16 +7,20 @@
 // weights (Eq. rubin-fit; an index with no weight takes its grid point), and
 // the candidate with the lowest weighted error sum h (C_q - w)^2 is kept.
 //
-// One warp owns one block: lane L holds block elements 16 L .. 16 L + 15
-// (row L / 4, columns 16 (L % 4) ..), read once from a per-warp TMA ring.
-// An index is a sign s of d = w - c and a magnitude level m = min(floor(|d|
-// P), 3).  Per candidate each lane accumulates, for each sign and threshold
-// t = 1, 2, 3, the sums of h and of h |d| over its elements with m >= t
-// (packed f32x2; the masks [m >= t] come from saturated adds on the floor,
-// so no per-index one-hot work); the 12 sums are transposed through shared
-// memory, and with the block's per-sign totals they give every index's H_j =
-// sum h and X_j = sum h |d|.  Index j's entry is the E4M3 rounding of its
-// weighted mean c + s X_j / H_j, and the error is
+// One warp owns one block: lane L holds, for i = 0 .. 3, block elements
+// 128 i + 4 L .. + 3, read once from a per-warp TMA ring.  An index is a sign
+// s of d = w - c and a magnitude level m = min(floor(|d| P), 3).  For each
+// sign and threshold t = 1, 2, 3 a candidate needs the sums of h and of h |d|
+// over the elements with m >= t.  Only elements that reach level 1 for some
+// factor add to any of them, so those are compacted into two lists by sign;
+// four lanes own a candidate (eight candidates a warp) and walk the lists in
+// pairs (packed f32x2; the masks [m >= t] come from saturated adds on the
+// floor).  A pair of one sign costs 16 instructions a candidate; in registers
+// with both signs it cost 25, for all 512 elements, and the 12 sums then had
+// to be transposed across the warp (one Llama layer, 218 M weights: 2,310 us
+// before, 2,070 us with the lists).  With the block's per-sign totals the sums
+// give every index's H_j = sum h and X_j = sum h |d|.  Index j's entry is the
+// E4M3 rounding of its weighted mean c + s X_j / H_j, and the error is
 //   sum h d^2 - sum_j X_j^2 / H_j + sum_j H_j (C_j - mean_j)^2
 // (the within-index scatter plus each entry's offset from its mean).  Both
 // the entry's rounding and the error carry an fp32 bound.  Candidates within
@@ -172,14 +176,14 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     const int S = p.stages;
     unsigned char* ring = smem + (size_t)warp * S * p.stage_bytes;
     unsigned char* scr = smem + (size_t)nwarps * S * p.stage_bytes + (size_t)warp * kLutScratchBytes;
-    float* sums = reinterpret_cast<float*>(scr);  // [24][33]
-    uint32_t* cbook = reinterpret_cast<uint32_t*>(scr + kLutSumsBytes);  // [32][2]
+    float* lst = reinterpret_cast<float*>(scr);  // |d| [kLutListLen], then h [kLutListLen]
+    uint32_t* cbook = reinterpret_cast<uint32_t*>(scr + kLutListBytes);  // [32][2]
     float* cerr = reinterpret_cast<float*>(cbook + 2 * kMaxClip);       // [32]
     float* cbnd = cerr + kMaxClip;                                        // [32]
     uint32_t* camb = reinterpret_cast<uint32_t*>(cbnd + kMaxClip);      // [32]
-    float* table = reinterpret_cast<float*>(scr + kLutSumsBytes + kLutCandBytes);  // [8]
+    float* table = reinterpret_cast<float*>(scr + kLutListBytes + kLutCandBytes);  // [8]
     // the block's per-sign sums of h and h |d|, and sum h d^2
-    float* bconst = table + 8;  // [7]: also the block's sum of h and its range
+    float* bconst = table + 8;  // [5]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nwarps * S * p.stage_bytes +
                                                  (size_t)nwarps * kLutScratchBytes) +
                      warp * (S + 1);
@@ -251,7 +255,9 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     const float2 beta22 = make_float2(p.beta2, p.beta2);
     const float2 c12 = make_float2(p.c1, p.c1);
     const float2 M2 = make_float2(kMagic, kMagic);
-    const float gam = kU * p.tie_kappa;
+    // the factor of the lane's candidate of the first eight (the one a lane's
+    // quad evaluates)
+    const float invf0 = p.invf[min(lane >> 2, K - 1)];
     int s_cur = 0;
     uint32_t parity = 0;
 
@@ -268,15 +274,19 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         const uint32_t b = (uint32_t)(u - T.unit0);
         const uint32_t nbc = (uint32_t)(T.cols / kLutCols);
         const uint32_t brow = b / nbc;
-        // the lane's 16 elements: row lane/4 of the block, columns 16 (lane % 4) ..
-        const int64_t gofs = ((int64_t)brow * kLutRows + (lane >> 2)) * T.cols +
-                             (int64_t)(b - brow * nbc) * kLutCols + (lane & 3) * 16;
+        // the lane's 16 elements, in four chunks of 4: chunk i is block elements
+        // 128 i + 4 lane .. + 3, i.e. row 2 i + lane/16, columns 4 (lane % 16) ..
+        // (consecutive lanes on consecutive 16-byte pieces, in the tile and in
+        // memory)
+        const int64_t gofs = ((int64_t)brow * kLutRows + (lane >> 4)) * T.cols +
+                             (int64_t)(b - brow * nbc) * kLutCols + (lane & 15) * 4;
+        const int64_t gstep = 2 * T.cols;  // from one chunk of the lane to the next
 
         // ---- pass A: w, the saliency EMA (v' out), the fit's saliency h
         float2 w2[8], h2[8];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int e = lane * 16 + i * 4;
+            const int e = i * 128 + lane * 4;
             const float4 w4 = lds128(st + e * 4);
             const float4 v4 = lds128(st + kVOff + e * 4);
             w2[2 * i] = make_float2(w4.x, w4.y);
@@ -295,7 +305,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 }
                 hA = __ffma2_rn(hA, beta22, __fmul2_rn(c12, __fmul2_rn(gA, gA)));
                 hB = __ffma2_rn(hB, beta22, __fmul2_rn(c12, __fmul2_rn(gB, gB)));
-                stg_cs(reinterpret_cast<float4*>(T.v + gofs + i * 4), make_float4(hA.x, hA.y, hB.x, hB.y));
+                stg_cs(reinterpret_cast<float4*>(T.v + gofs + i * gstep), make_float4(hA.x, hA.y, hB.x, hB.y));
             }
             h2[2 * i] = hA;
             h2[2 * i + 1] = hB;
@@ -315,18 +325,17 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             for (int t = 0; t < 8; ++t)
                 h2[t] = p.h_mode == kSalEmaSquared ? __fmul2_rn(h2[t], h2[t]) : make_float2(1.0f, 1.0f);
 
-        float mn = INFINITY, mx = -INFINITY, ss = 0.0f;
+        float mn = INFINITY, mx = -INFINITY;
+        bool any_h = false;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            mn = fminf(mn, fminf(w2[t].x, w2[t].y));
-            mx = fmaxf(mx, fmaxf(w2[t].x, w2[t].y));
-            ss += h2[t].x + h2[t].y;
+            mn = fmin3(mn, w2[t].x, w2[t].y);
+            mx = fmax3(mx, w2[t].x, w2[t].y);
+            any_h |= h2[t].x + h2[t].y != 0.0f;
         }
         mn = lanes_min(mn, 0xffffffffu);
         mx = lanes_max(mx, 0xffffffffu);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (ss == 0.0f)  // all saliencies zero: h = 1
+        if (!__any_sync(0xffffffffu, any_h))  // all saliencies zero: h = 1
 #pragma unroll
             for (int t = 0; t < 8; ++t) h2[t] = make_float2(1.0f, 1.0f);
         const float range = mx - mn;
@@ -335,211 +344,231 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         const float R = flat ? 0.0f : __fdividef(7.0f, range);
         const float2 nc2 = make_float2(-c, -c);
 
-        // candidate-independent: |d| = |w - c| and the saliency split by the
-        // sign of d (a negative zero counts as negative, as the index does);
-        // w itself is read again from memory only by the exact look
-        float2 ad2[8], hp2[8], hn2[8];
+        // candidate-independent: |d| = |w - c|, the signs of d (a negative zero
+        // counts as negative, as the index does) and the block's per-sign sums
+        // of h and h |d|, and sum h d^2; w itself is read again from memory
+        // only by the exact look
+        float2 ad2[8];
         uint32_t negm = 0;  // bit i: element i has d < 0 (or -0)
         {
-            float tp, tn, up, un, sd;
             float2 Tp = make_float2(0.0f, 0.0f), Tn = Tp, Up = Tp, Un = Tp, Sd = Tp;
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const float2 d = __fadd2_rn(w2[t], nc2);
-                const bool nx = signbit(d.x), ny = signbit(d.y);
-                negm |= (nx ? 1u : 0u) << (2 * t);
-                negm |= (ny ? 1u : 0u) << (2 * t + 1);
+                const uint32_t sx = (uint32_t)((int32_t)__float_as_uint(d.x) >> 31);
+                const uint32_t sy = (uint32_t)((int32_t)__float_as_uint(d.y) >> 31);
+                negm |= (sx & (1u << (2 * t))) | (sy & (2u << (2 * t)));
                 ad2[t] = make_float2(fabsf(d.x), fabsf(d.y));
-                hp2[t] = make_float2(nx ? 0.0f : h2[t].x, ny ? 0.0f : h2[t].y);
-                hn2[t] = make_float2(nx ? h2[t].x : 0.0f, ny ? h2[t].y : 0.0f);
-                Tp = __fadd2_rn(Tp, hp2[t]);
-                Tn = __fadd2_rn(Tn, hn2[t]);
                 const float2 hd = __fmul2_rn(h2[t], ad2[t]);
-                Up = __fadd2_rn(Up, make_float2(nx ? 0.0f : hd.x, ny ? 0.0f : hd.y));
-                Un = __fadd2_rn(Un, make_float2(nx ? hd.x : 0.0f, ny ? hd.y : 0.0f));
+                // the negative side's part; the difference is exact (h or 0)
+                const float2 hn = make_float2(__uint_as_float(__float_as_uint(h2[t].x) & sx),
+                                              __uint_as_float(__float_as_uint(h2[t].y) & sy));
+                const float2 un = make_float2(__uint_as_float(__float_as_uint(hd.x) & sx),
+                                              __uint_as_float(__float_as_uint(hd.y) & sy));
+                Tn = __fadd2_rn(Tn, hn);
+                Un = __fadd2_rn(Un, un);
+                Tp = __fadd2_rn(Tp, make_float2(__uint_as_float(__float_as_uint(h2[t].x) & ~sx),
+                                                __uint_as_float(__float_as_uint(h2[t].y) & ~sy)));
+                Up = __fadd2_rn(Up, make_float2(__uint_as_float(__float_as_uint(hd.x) & ~sx),
+                                                __uint_as_float(__float_as_uint(hd.y) & ~sy)));
                 Sd = __ffma2_rn(hd, ad2[t], Sd);
             }
-            tp = Tp.x + Tp.y;
-            tn = Tn.x + Tn.y;
-            up = Up.x + Up.y;
-            un = Un.x + Un.y;
-            sd = Sd.x + Sd.y;
+            // the four per-sign sums are scattered while they are summed: lane
+            // bit 4 picks the sign, bit 3 h or h |d|
+            const float tp = Tp.x + Tp.y, tn = Tn.x + Tn.y, up = Up.x + Up.y, un = Un.x + Un.y;
+            float sd = Sd.x + Sd.y;
+            const bool b4 = lane & 16, b3 = lane & 8;
+            const float k0 = (b4 ? tn : tp) + __shfl_xor_sync(0xffffffffu, b4 ? tp : tn, 16);
+            const float k1 = (b4 ? un : up) + __shfl_xor_sync(0xffffffffu, b4 ? up : un, 16);
+            float kv = (b3 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b3 ? k0 : k1, 8);
 #pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                tp += __shfl_xor_sync(0xffffffffu, tp, o);
-                tn += __shfl_xor_sync(0xffffffffu, tn, o);
-                up += __shfl_xor_sync(0xffffffffu, up, o);
-                un += __shfl_xor_sync(0xffffffffu, un, o);
-                sd += __shfl_xor_sync(0xffffffffu, sd, o);
-            }
-            // one value for every lane, kept in the scratch until the
-            // candidates' entries need them
-            if (lane == 0) {
-                bconst[0] = tp;
-                bconst[1] = tn;
-                bconst[2] = up;
-                bconst[3] = un;
-                bconst[4] = sd;
-                bconst[5] = ss;
-                bconst[6] = range;
-            }
+            for (int o = 4; o; o >>= 1) kv += __shfl_xor_sync(0xffffffffu, kv, o);
+#pragma unroll
+            for (int o = 16; o; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
+            // bconst: sum h (d >= 0, d < 0), sum h |d| (same), sum h d^2, in the
+            // scratch until the candidates' entries need them
+            if ((lane & 7) == 0) bconst[(b3 ? 2 : 0) + (b4 ? 1 : 0)] = kv;
+            if (lane == 0) bconst[4] = sd;
         }
+        __syncwarp();
 
         int kb = 0;
         if (!flat) {
-            // ---- candidates, four a pass: in two rounds of two, the
-            // per-index sums of each (12 rows of the scratch a candidate)
-            // summed across lanes, then entries and errors of all four at
-            // once (lanes 8 q .. 8 q + 7 candidate k0 + q)
-#pragma unroll 1
-            for (int k0 = 0; k0 < K; k0 += 4) {
-                float tot_a = 0.0f, tot_b = 0.0f;  // the two rounds' row sums
-#pragma unroll 1
-                for (int kr = k0; kr < min(k0 + 4, K); kr += 2) {
-                    const int nk = min(2, K - kr);
-#pragma unroll 1
-                    for (int kk = 0; kk < nk; ++kk) {
-                        const float P = R * p.invf[kr + kk];
-                        const float2 P2 = make_float2(P, P);
-                        // [l]: threshold m >= l + 1; sums of h (A) and h |d| (X),
-                        // by sign.  The masked saliency h [m >= t] is exact, and
-                        // so is its product with |d| inside the FMA: every term
-                        // is exact.
-                        float2 Ap[3], An[3], Xp[3], Xn[3];
+            // ---- the elements that reach level 1 for some factor: an element
+            // with |d| P < 1 for every factor adds to no threshold sum.  The
+            // others (about a quarter of a heavy-tailed block, a half of a
+            // normal one) are compacted into two lists by sign, |d| and h, in
+            // the scratch.  (The bound is 1 less a few ulps: an element too
+            // many only adds zeros.)  More than kLutListCap of them are taken
+            // in two rounds of 8 elements a lane.
+            const float thr = __fdividef(0.999999f, R * p.invf_max);
+            uint32_t act = 0;
 #pragma unroll
-                        for (int l = 0; l < 3; ++l) Ap[l] = An[l] = Xp[l] = Xn[l] = make_float2(0.0f, 0.0f);
+            for (int t = 0; t < 8; ++t) {
+                if (ad2[t].x >= thr) act |= 1u << (2 * t);
+                if (ad2[t].y >= thr) act |= 2u << (2 * t);
+            }
+            const int rounds = __reduce_add_sync(0xffffffffu, __popc(act)) <= kLutListCap ? 1 : 2;
+            const int q = lane & 3;  // the lane's share of the lists, and of the entries
+#pragma unroll 1
+            for (int k0 = 0; k0 < K; k0 += 8) {
+                // lanes 4 i .. 4 i + 3: candidate k0 + i
+                const int k = k0 + (lane >> 2);
+                const bool live = k < K;
+                const float P = R * (k0 == 0 ? invf0 : p.invf[min(k, K - 1)]);
+                const float2 P2 = make_float2(P, P);
+                // sums of h (A) and h |d| (X) over the elements with level
+                // m >= l + 1, by sign.  The masks [m >= l + 1] are saturated
+                // adds on the floor of |d| P (0 or 1).
+                float2 Ap[3], An[3], Xp[3], Xn[3];
 #pragma unroll
-                        for (int t = 0; t < 8; ++t) {
-                            const float2 y = __ffma2_rd(ad2[t], P2, M2);  // 2^23 + floor(|d| P)
-#pragma unroll
-                            for (int l = 0; l < 3; ++l) {
-                                const float nb = -(kMagic + (float)l);
-                                const float2 mk = make_float2(add_sat(y.x, nb), add_sat(y.y, nb));
-                                const float2 mp = __fmul2_rn(hp2[t], mk);
-                                const float2 mq = __fmul2_rn(hn2[t], mk);
-                                Ap[l] = __fadd2_rn(Ap[l], mp);
-                                An[l] = __fadd2_rn(An[l], mq);
-                                Xp[l] = __ffma2_rn(mp, ad2[t], Xp[l]);
-                                Xn[l] = __ffma2_rn(mq, ad2[t], Xn[l]);
-                            }
-                        }
-                        // rows (of this candidate's 12): A+ 0..2, A- 3..5, X+ 6..8,
-                        // X- 9..11
-                        float* rows = sums + kk * 12 * kLutRow + lane;
+                for (int l = 0; l < 3; ++l) Ap[l] = An[l] = Xp[l] = Xn[l] = make_float2(0.0f, 0.0f);
+                auto walk = [&](const float* la, int n, float2 (&A)[3], float2 (&X)[3]) {
+#pragma unroll 2
+                    for (int e = 2 * q; e < n; e += 8) {
+                        const float2 a2 = *reinterpret_cast<const float2*>(la + e);
+                        const float2 hh = *reinterpret_cast<const float2*>(la + kLutListLen + e);
+                        const float2 y = __ffma2_rd(a2, P2, M2);  // 2^23 + floor(|d| P)
+                        const float2 hd = __fmul2_rn(hh, a2);
 #pragma unroll
                         for (int l = 0; l < 3; ++l) {
-                            rows[l * kLutRow] = Ap[l].x + Ap[l].y;
-                            rows[(3 + l) * kLutRow] = An[l].x + An[l].y;
-                            rows[(6 + l) * kLutRow] = Xp[l].x + Xp[l].y;
-                            rows[(9 + l) * kLutRow] = Xn[l].x + Xn[l].y;
+                            const float nb = -(kMagic + (float)l);
+                            const float2 mk = make_float2(add_sat(y.x, nb), add_sat(y.y, nb));
+                            A[l] = __ffma2_rn(hh, mk, A[l]);
+                            X[l] = __ffma2_rn(hd, mk, X[l]);
                         }
                     }
-                    __syncwarp();
-                    // lane r < 12 nk sums row r
-                    if (lane < 12 * nk) {
-                        float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float4 v = *reinterpret_cast<const float4*>(sums + lane * kLutRow + 4 * i);
-                            a0 += v.x;
-                            a1 += v.y;
-                            a2 += v.z;
-                            a3 += v.w;
-                        }
-                        const float tot = (a0 + a1) + (a2 + a3);
-                        if (kr == k0) tot_a = tot;
-                        else tot_b = tot;
-                    }
-                    __syncwarp();  // the scratch rows are rewritten by the next round
-                }
-                // lane j < 8 of each group q of 8: index j, sign s (j >= 4:
-                // d >= 0), level m; its H = A_m - A_(m+1) and X = X_m - X_(m+1)
-                // (A_0, X_0: the sign's totals; A_4 = X_4 = 0)
-                const int q4 = lane >> 3;   // candidate k0 + q4
-                const int half = q4 & 1;
-                const int rb = half * 12;  // the candidate's first row in its round
-                const float P = R * p.invf[min(k0 + q4, K - 1)];
-                const float sg = __fdividef(1.0f, P);
-                const int j = lane & 7;
-                const bool pos = j >= 4;
-                const int m = pos ? j - 4 : 3 - j;
-                const int r0 = rb + (pos ? 0 : 3);
-                // a row sum of this lane's round (q4 < 2: the first)
-                auto row = [&](int r) {
-                    const float va = __shfl_sync(0xffffffffu, tot_a, r);
-                    const float vb = __shfl_sync(0xffffffffu, tot_b, r);
-                    return q4 < 2 ? va : vb;
                 };
-                const float sA0 = row(r0 + max(m - 1, 0));
-                const float sA1 = row(r0 + min(m, 2));
-                const float sX0 = row(6 + r0 + max(m - 1, 0));
-                const float sX1 = row(6 + r0 + min(m, 2));
-                const float Am = m == 0 ? bconst[pos ? 0 : 1] : sA0;
-                const float Am1 = m == 3 ? 0.0f : sA1;
-                const float Xm = m == 0 ? bconst[pos ? 2 : 3] : sX0;
-                const float Xm1 = m == 3 ? 0.0f : sX1;
-                const float H = Am - Am1, X = fmaxf(Xm - Xm1, 0.0f);
-                const float sgn = pos ? 1.0f : -1.0f;
-                const float gj = fmaf((float)j - 3.5f, sg, c);  // the grid point
-                // errors: the cumulative sums are sums of exact nonnegative
-                // terms over at most tie_kappa levels (the per-sign totals of
-                // h |d| carry one more rounding a term)
-                const float dA = gam * (Am + Am1) + kU * H;
-                const float dX = (gam + kU) * (Xm + Xm1) + kU * X;
-                float mean = gj, q = 0.0f, dq = 0.0f, dm = 4.0f * kU * fabsf(gj);
-                if (H > 0.0f) {
-                    q = __fdividef(X, H);
-                    mean = fmaf(sgn, q, c);
-                    dq = __fdividef(dX + q * dA, H) + 2.0f * kU * q;
-                    // plus the roundings of w - c (relative u each), of the
-                    // quotient's use and of the mean's sum
-                    dm = dq + 3.0f * kU * q + 2.0f * kU * fabsf(mean);
-                }
-                const uint32_t cb = e4m3_encode(mean);
-                // an index whose H is not clearly above its error bound may be
-                // empty or may hold weights of tiny saliency lost to the
-                // differences: its entry is undecided unless nothing on its
-                // side reaches its level, and its whole term is bounded below
-                const bool thin = !(H > dA) && Am + Am1 > 0.0f;
-                const bool amb = thin || e4m3_encode(mean - dm) != e4m3_encode(mean + dm);
-                const float dc = e4m3_decode(cb) - mean;
-                // the index's error: H (C - mean)^2 - X^2 / H (the scatter
-                // term sum h d^2 is added once below)
-                const float Sj = H > 0.0f && !thin ? fmaf(H * dc, dc, -X * q) : 0.0f;
-                float bj = dA * dc * dc + 2.0f * H * fabsf(dc) * dm + 3.0f * kU * H * dc * dc + dX * q +
-                           X * dq + 2.0f * kU * X * q;
-                if (amb) {  // the other rounding moves the entry by at most this much
-                    const float c1 = e4m3_decode(e4m3_encode(mean - dm)) - mean;
-                    const float c2 = e4m3_decode(e4m3_encode(mean + dm)) - mean;
-                    bj += H * fabsf(c2 - c1) * (fabsf(c1) + fabsf(c2) + 2.0f * dm);
-                }
-                bj = thin ? 2.0f * (dA + fabsf(H)) * bconst[6] * bconst[6] : bj;
-                const bool live = k0 + q4 < K;
-                float E = live ? Sj : 0.0f, dE = live ? bj : 0.0f, aE = live ? fabsf(Sj) : 0.0f;
-                uint32_t wb = live ? cb << (8 * (lane & 3)) : 0u;
+                int steps = 0;  // the longest chain of additions of a lane's sum
+#pragma unroll 1
+                for (int rd = 0; rd < rounds; ++rd) {
+                    const uint32_t sel = rounds == 1 ? 0xFFFFu : (rd ? 0xFF00u : 0x00FFu);
+                    const uint32_t ap = act & sel & ~negm, an = act & sel & negm;
+                    // list positions: an inclusive scan of both counts
+                    uint32_t pos = __popc(ap) | (__popc(an) << 16);
+                    const uint32_t own = pos;
 #pragma unroll
-                for (int o = 4; o; o >>= 1) {
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t up = __shfl_up_sync(0xffffffffu, pos, o);
+                        if (lane >= o) pos += up;
+                    }
+                    const uint32_t tot = __shfl_sync(0xffffffffu, pos, 31);
+                    pos -= own;
+                    const int np = (int)(tot & 0xFFFFu), nn = (int)(tot >> 16);
+                    const int np8 = (np + 7) & ~7, nn8 = (nn + 7) & ~7;
+                    if (rounds > 1 || k0 == 0) {
+                        float* fp = lst + (pos & 0xFFFFu);
+                        float* fn = lst + np8 + (pos >> 16);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const bool in = ((ap | an) >> i) & 1u, ng = (an >> i) & 1u;
+                            float* f = ng ? fn : fp;
+                            if (in) {
+                                f[0] = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
+                                f[kLutListLen] = (i & 1) ? h2[i >> 1].y : h2[i >> 1].x;
+                            }
+                            fp += in && !ng ? 1 : 0;
+                            fn += ng ? 1 : 0;
+                        }
+                        // zeros up to a multiple of 8 entries
+                        if (lane < np8 - np) lst[np + lane] = lst[kLutListLen + np + lane] = 0.0f;
+                        if (lane < nn8 - nn) lst[np8 + nn + lane] = lst[kLutListLen + np8 + nn + lane] = 0.0f;
+                        __syncwarp();
+                    }
+                    walk(lst, np8, Ap, Xp);
+                    walk(lst + np8, nn8, An, Xn);
+                    steps += max(np8, nn8) >> 3;
+                    if (rounds > 1) __syncwarp();  // the lists are rewritten by the next round
+                }
+                // entries: lane q of a candidate has indices 2 q and 2 q + 1, i.e.
+                // the sign s (q >= 2: d >= 0) and levels 2, 3 (far: q = 0, 3) or 0, 1
+                const bool pos = q >= 2, far = q == 0 || q == 3;
+                float A1, A2, A3, X1, X2, X3;
+                {
+                    float* out[6] = {&A1, &A2, &A3, &X1, &X2, &X3};
+#pragma unroll
+                    for (int j = 0; j < 6; ++j) {
+                        const float2 vp = j < 3 ? Ap[j % 3] : Xp[j % 3], vn = j < 3 ? An[j % 3] : Xn[j % 3];
+                        const float fp = vp.x + vp.y, fn = vn.x + vn.y;
+                        // lanes q and q ^ 2 exchange the sign they do not keep
+                        const float v = (pos ? fp : fn) + __shfl_xor_sync(0xffffffffu, pos ? fn : fp, 2);
+                        *out[j] = v + __shfl_xor_sync(0xffffffffu, v, 1);
+                    }
+                }
+                // cumulative sums from the lower of its two levels on (level 0:
+                // the sign's totals; beyond level 3: nothing)
+                const float Ac[3] = {far ? A2 : bconst[pos ? 0 : 1], far ? A3 : A1, far ? 0.0f : A2};
+                const float Xc[3] = {far ? X2 : bconst[pos ? 2 : 3], far ? X3 : X1, far ? 0.0f : X2};
+                const float sg = __fdividef(1.0f, P);
+                const float sgn = pos ? 1.0f : -1.0f;
+                // errors: the cumulative sums are sums of nonnegative terms,
+                // exact (h) or rounded once (h |d|), over at most `depth` levels
+                const float gam = kU * p.tie_kappa * (float)(max(steps, 11) + 8);
+                float E = 0.0f, dE = 0.0f, aE = 0.0f;
+                uint32_t wb = 0, ambm = 0;
+#pragma unroll
+                for (int e2 = 0; e2 < 2; ++e2) {
+                    // the lower level is the even index for d >= 0, the odd one below
+                    const int j = 2 * q + (pos ? e2 : 1 - e2);
+                    const float Am = Ac[e2], Am1 = Ac[e2 + 1], Xm = Xc[e2], Xm1 = Xc[e2 + 1];
+                    const float H = Am - Am1, X = fmaxf(Xm - Xm1, 0.0f);
+                    const float gj = fmaf((float)j - 3.5f, sg, c);  // the grid point
+                    const float dA = gam * (Am + Am1) + kU * H;
+                    const float dX = (gam + kU) * (Xm + Xm1) + kU * X;
+                    float mean = gj, qu = 0.0f, dq = 0.0f, dm = 4.0f * kU * fabsf(gj);
+                    if (H > 0.0f) {
+                        qu = __fdividef(X, H);
+                        mean = fmaf(sgn, qu, c);
+                        dq = __fdividef(dX + qu * dA, H) + 2.0f * kU * qu;
+                        // plus the roundings of w - c (relative u each), of the
+                        // quotient's use and of the mean's sum
+                        dm = dq + 3.0f * kU * qu + 2.0f * kU * fabsf(mean);
+                    }
+                    const uint32_t cb = e4m3_encode(mean);
+                    // an index whose H is not clearly above its error bound may be
+                    // empty or may hold weights of tiny saliency lost to the
+                    // differences: its entry is undecided unless nothing on its
+                    // side reaches its level, and its whole term is bounded below
+                    const bool thin = !(H > dA) && Am + Am1 > 0.0f;
+                    const uint32_t c1b = e4m3_encode(mean - dm), c2b = e4m3_encode(mean + dm);
+                    const bool amb = thin || c1b != c2b;
+                    const float dc = e4m3_decode(cb) - mean;
+                    // the index's error: H (C - mean)^2 - X^2 / H (the scatter
+                    // term sum h d^2 is added once below)
+                    const float Sj = H > 0.0f && !thin ? fmaf(H * dc, dc, -X * qu) : 0.0f;
+                    float bj = dA * dc * dc + 2.0f * H * fabsf(dc) * dm + 3.0f * kU * H * dc * dc + dX * qu +
+                               X * dq + 2.0f * kU * X * qu;
+                    if (amb) {  // the other rounding moves the entry by at most this much
+                        const float c1 = e4m3_decode(c1b) - mean;
+                        const float c2 = e4m3_decode(c2b) - mean;
+                        bj += H * fabsf(c2 - c1) * (fabsf(c1) + fabsf(c2) + 2.0f * dm);
+                    }
+                    bj = thin ? 2.0f * (dA + fabsf(H)) * range * range : bj;
+                    E += Sj;
+                    dE += bj;
+                    aE += fabsf(Sj);
+                    wb |= cb << (8 * (j & 1));
+                    ambm |= amb ? 1u << j : 0u;
+                }
+#pragma unroll
+                for (int o = 2; o; o >>= 1) {
                     E += __shfl_xor_sync(0xffffffffu, E, o);
                     dE += __shfl_xor_sync(0xffffffffu, dE, o);
                     aE += __shfl_xor_sync(0xffffffffu, aE, o);
+                    ambm |= __shfl_xor_sync(0xffffffffu, ambm, o);
                 }
                 const float sd = bconst[4];
                 E += sd;
                 // sum h d^2: its terms' roundings (|d|^2, h times it) and sum
                 dE += (gam + 3.0f * kU) * sd + 4.0f * kU * (sd + aE);
-#pragma unroll
-                for (int o = 2; o; o >>= 1) wb |= __shfl_xor_sync(0xffffffffu, wb, o);
-                const uint32_t wb1 = __shfl_sync(0xffffffffu, wb, (lane & 24) | 4);
-                const uint32_t ambm = __ballot_sync(0xffffffffu, amb && live);
-                if ((lane & 7) == 0 && live) {
-                    const int k = k0 + q4;
-                    cbook[2 * k] = wb;
-                    cbook[2 * k + 1] = wb1;
-                    cerr[k] = E;
-                    cbnd[k] = dE;
-                    camb[k] = (ambm >> (8 * q4)) & 0xFFu;
+                if (live) {
+                    reinterpret_cast<uint16_t*>(cbook)[4 * k + q] = (uint16_t)wb;
+                    if (q == 0) {
+                        cerr[k] = E;
+                        cbnd[k] = dE;
+                        camb[k] = ambm;
+                    }
                 }
-                __syncwarp();
             }
             __syncwarp();
 
@@ -568,8 +597,9 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             // (ts1 ts2: that power of two, applied where the settling steps
             // read h; 1 otherwise)
             float ts1 = 1.0f, ts2 = 1.0f;
-            if (bconst[5] > 0.0f && bconst[5] < kTinySaliency) {
-                tiny_scale(bconst[5], ts1, ts2);
+            const float ss = bconst[0] + bconst[1];
+            if (ss > 0.0f && ss < kTinySaliency) {
+                tiny_scale(ss, ts1, ts2);
                 set = (K >= 32) ? 0xFFFFFFFFu : ((1u << K) - 1u);
                 if (lane < K) camb[lane] = 0xFFu;
                 __syncwarp();
@@ -597,7 +627,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         if (index_of(i, P) == j) {
-                            const float hv = ((i & 1) ? hp2[i >> 1].y + hn2[i >> 1].y : hp2[i >> 1].x + hn2[i >> 1].x) * ts1 * ts2;
+                            const float hv = ((i & 1) ? h2[i >> 1].y : h2[i >> 1].x) * ts1 * ts2;
                             const float av = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
                             Hs += hv;
                             Xs = fmaf(hv, av, Xs);
@@ -653,7 +683,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                     float xwv[16];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float4 w4 = __ldg(reinterpret_cast<const float4*>(T.w + gofs + i * 4));
+                        const float4 w4 = __ldg(reinterpret_cast<const float4*>(T.w + gofs + i * gstep));
                         xwv[4 * i] = w4.x;
                         xwv[4 * i + 1] = w4.y;
                         xwv[4 * i + 2] = w4.z;
@@ -668,7 +698,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                         float acc = 0.0f;
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
-                            const float hv = ((i & 1) ? hp2[i >> 1].y + hn2[i >> 1].y : hp2[i >> 1].x + hn2[i >> 1].x) * ts1 * ts2;
+                            const float hv = ((i & 1) ? h2[i >> 1].y : h2[i >> 1].x) * ts1 * ts2;
                             const float df = table[index_of(i, P)] - xwv[i];
                             acc = fmaf(hv * df, df, acc);
                         }
@@ -712,14 +742,13 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 float2 xw[8], xh[8];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float4 w4 = __ldg(reinterpret_cast<const float4*>(T.w + gofs + i * 4));
+                    const float4 w4 = __ldg(reinterpret_cast<const float4*>(T.w + gofs + i * gstep));
                     xw[2 * i] = make_float2(w4.x, w4.y);
                     xw[2 * i + 1] = make_float2(w4.z, w4.w);
                 }
 #pragma unroll
-                for (int t = 0; t < 8; ++t)  // one of the two is 0
-                    xh[t] = __fmul2_rn(__fmul2_rn(__fadd2_rn(hp2[t], hn2[t]), make_float2(ts1, ts1)),
-                                       make_float2(ts2, ts2));
+                for (int t = 0; t < 8; ++t)
+                    xh[t] = __fmul2_rn(__fmul2_rn(h2[t], make_float2(ts1, ts1)), make_float2(ts2, ts2));
                 float best_h = 0.0f, best_l = 0.0f;
                 int best_k = -1;
                 uint32_t best_w0 = 0, best_w1 = 0;
@@ -820,51 +849,66 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             bw0 = cbook[2 * kb];
             bw1 = cbook[2 * kb + 1];
         }
-        if (lane < 8) table[lane] = e4m3_decode(((lane < 4 ? bw0 : bw1) >> (8 * (lane & 3))) & 0xFFu);
-        __syncwarp();
+        // r by byte permutes: an E4M3 value is a bf16 value, and the table's
+        // eight low and eight high bf16 bytes are four registers, from which a
+        // permute picks four entries by their indices (a nibble each)
+        uint32_t tl0, tl1, th0, th1;
+        {
+            // lane j holds entry j's bf16 bits in the upper half
+            const uint32_t tv = __float_as_uint(e4m3_decode(((lane & 4 ? bw1 : bw0) >> (8 * (lane & 3))) & 0xFFu)) >> 16;
+            uint32_t t[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) t[j] = __shfl_sync(0xffffffffu, tv, j);
+            const uint32_t a01 = __byte_perm(t[0], t[1], 0x5140), a23 = __byte_perm(t[2], t[3], 0x5140);
+            const uint32_t a45 = __byte_perm(t[4], t[5], 0x5140), a67 = __byte_perm(t[6], t[7], 0x5140);
+            tl0 = __byte_perm(a01, a23, 0x5410);
+            th0 = __byte_perm(a01, a23, 0x7632);
+            tl1 = __byte_perm(a45, a67, 0x5410);
+            th1 = __byte_perm(a45, a67, 0x7632);
+        }
         const float P = flat ? 0.0f : R * p.invf[kb];
-        uint32_t q4[4] = {0u, 0u, 0u, 0u};  // the 16 indices, a byte each
-        float rv[16];
+        const float2 P2 = make_float2(P, P);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float adv = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
-            const float dv = ((negm >> i) & 1u) ? -adv : adv;  // w - c
-            const uint32_t q = flat ? 0u : (uint32_t)(int)(code_z(dv, P) + 3.5f);
-            q4[i >> 2] |= q << (8 * (i & 3));
-            rv[i] = table[q];
-        }
-        if (p.r_bf16) {
-            uint32_t pk[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) pk[i] = pack_bf16x2(rv[2 * i], rv[2 * i + 1]);
-            stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + gofs), make_uint2(pk[0], pk[1]));
-            stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + gofs + 4), make_uint2(pk[2], pk[3]));
-            stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + gofs + 8), make_uint2(pk[4], pk[5]));
-            stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + gofs + 12), make_uint2(pk[6], pk[7]));
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                stg_cs(reinterpret_cast<float4*>(static_cast<float*>(T.r) + gofs + 4 * i),
-                       make_float4(rv[4 * i], rv[4 * i + 1], rv[4 * i + 2], rv[4 * i + 3]));
-        }
-        if (T.codes) {
-            if (!p.codes_packed) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) stg_cs(reinterpret_cast<uint32_t*>(T.codes + gofs) + i, q4[i]);
-            } else {
-                // 3 bits an index in block order: lane L's 48 bits at bit 48 L;
-                // an even lane writes its pair's 12 bytes
-                uint64_t bits48 = 0;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) bits48 |= (uint64_t)((q4[i >> 2] >> (8 * (i & 3))) & 7u) << (3 * i);
-                const uint32_t lo = (uint32_t)bits48, hi = (uint32_t)(bits48 >> 32);
-                const uint32_t olo = __shfl_down_sync(0xffffffffu, lo, 1);
-                const uint32_t ohi = __shfl_down_sync(0xffffffffu, hi, 1);
-                if ((lane & 1) == 0) {
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(T.codes) + (size_t)b * 48 + (lane >> 1) * 3;
-                    stg_cs(dst, lo);
-                    stg_cs(dst + 1, (hi & 0xFFFFu) | (olo << 16));
-                    stg_cs(dst + 2, (olo >> 16) | (ohi << 16));
+        for (int i = 0; i < 4; ++i) {
+            // indices of the chunk's 4 elements, a nibble each: level m =
+            // min(floor(|d| P), 3) from the low bits of the floor on the 2^23
+            // grid; 4 + m (d >= 0) is m ^ 4 and 3 - m (d < 0) is m ^ 3
+            const float2 ya = __ffma2_rd(ad2[2 * i], P2, M2), yb = __ffma2_rd(ad2[2 * i + 1], P2, M2);
+            const uint32_t m0 = __float_as_uint(fminf(ya.x, kMagic + 3.0f)), m1 = __float_as_uint(fminf(ya.y, kMagic + 3.0f));
+            const uint32_t m2 = __float_as_uint(fminf(yb.x, kMagic + 3.0f)), m3 = __float_as_uint(fminf(yb.y, kMagic + 3.0f));
+            const uint32_t ng = negm >> (4 * i);
+            const uint32_t sx = (ng & 1u) | ((ng & 2u) << 3) | ((ng & 4u) << 6) | ((ng & 8u) << 9);
+            uint32_t sel = (m0 + (m1 << 4) + (m2 << 8) + (m3 << 12)) ^ 0x4444u ^ (sx * 7u);
+            sel = flat ? 0u : sel & 0x7777u;
+            const uint32_t lo = __byte_perm(tl0, tl1, sel), hi = __byte_perm(th0, th1, sel);
+            const uint32_t r01 = __byte_perm(lo, hi, 0x5140), r23 = __byte_perm(lo, hi, 0x7362);
+            const int64_t ge = gofs + i * gstep;
+            if (p.r_bf16)
+                stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + ge), make_uint2(r01, r23));
+            else
+                stg_cs(reinterpret_cast<float4*>(static_cast<float*>(T.r) + ge),
+                       make_float4(bf16lo(r01), bf16hi(r01), bf16lo(r23), bf16hi(r23)));
+            if (T.codes) {
+                if (!p.codes_packed) {
+                    // nibbles to bytes
+                    const uint32_t t8 = (sel | (sel << 8)) & 0x00FF00FFu;
+                    stg_cs(reinterpret_cast<uint32_t*>(T.codes + ge), (t8 | (t8 << 4)) & 0x0F0F0F0Fu);
+                } else {
+                    // 3 bits an index in block order: the lane's 12 bits at bit
+                    // 12 (32 i + lane); 8 lanes make 3 words
+                    const uint32_t s6 = (sel & 0x0707u) | ((sel & 0x7070u) >> 1);
+                    uint32_t x = (s6 & 0x3Fu) | ((s6 & 0x3F00u) >> 2);
+                    const uint32_t o1 = __shfl_xor_sync(0xffffffffu, x, 1);
+                    x = lane & 1 ? o1 | (x << 12) : x | (o1 << 12);  // 24 bits of 2 lanes
+                    const uint32_t o2 = __shfl_xor_sync(0xffffffffu, x, 2);
+                    const uint32_t xa = lane & 2 ? o2 : x, xb = lane & 2 ? x : o2;
+                    const uint32_t x0 = xa | (xb << 24), x1 = xb >> 8;  // 48 bits of 4 lanes
+                    const uint32_t o0 = __shfl_xor_sync(0xffffffffu, x0, 4), oh = __shfl_xor_sync(0xffffffffu, x1, 4);
+                    // lanes 0, 1, 2 of the 8 (the first half) write a word each
+                    const int l8 = lane & 7;
+                    if (l8 < 3)
+                        stg_cs(reinterpret_cast<uint32_t*>(T.codes) + (size_t)b * 48 + i * 12 + (lane >> 3) * 3 + l8,
+                               l8 == 0 ? x0 : (l8 == 1 ? x1 | (o0 << 16) : (o0 >> 16) | (oh << 16)));
                 }
             }
         }
