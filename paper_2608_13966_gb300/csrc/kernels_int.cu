@@ -1,7 +1,7 @@
-// Instantiations of the integer-code kernel for one candidate-chunk count
-// (QUASAR_NCH = 1, 2 or 4 chunks of 8 candidates) and one clamp-set size
-// (QUASAR_SS = 4, 2 or 1 candidates; with a single chunk also 8, or 3 for
-// the sets 3-3-2); compiled once per pair, in parallel.
+// Instantiations of the integer-code kernel for one chunk of 8 candidates
+// (QUASAR_NCH = 1) or up to four (2), and one clamp-set size (QUASAR_SS = 4, 2
+// or 1 candidates; with a single chunk also 8, or 3 for the sets 3-3-2);
+// compiled once per pair, in parallel.
 #include "recon_int.cuh"
 
 #if !defined(QUASAR_NCH) || !defined(QUASAR_SS)

@@ -17,12 +17,12 @@ constexpr int kGroupsPerUnit = 4;
 constexpr int kMaxClip = 32;
 
 // The asymmetric integer kernel: 4 lanes a group, 8 groups a unit, and a
-// ring of unit tiles shared by the warps of a CTA.  The candidate sums of a
-// quad of candidates are transposed through the tile's gradient region once
-// the gradient is consumed: at least 2 KB (32 lanes x 4 x 16 bytes).
+// ring of unit tiles shared by the warps of a CTA.  Once the gradient is
+// consumed, the tile's gradient region holds the candidates' table: 16 bytes
+// for each of a chunk's 8 candidates and the unit's 8 groups.
 constexpr int kIntLanes = 4;
 constexpr int kIntGroups = 8;
-constexpr uint32_t kIntXposeBytes = 2048;
+constexpr uint32_t kIntTableBytes = 8 * kIntGroups * 16;
 
 // One tensor of an integer-code launch: its buffers, group count, and the
 // index of its first unit in the launch's sequence of units.
@@ -78,9 +78,8 @@ struct IntParams {
     // kernel)
     float cap[kMaxClip];
     int set_size;
-    // 1/f is non-decreasing in k over the real candidates (the factors come
-    // in decreasing order, as the paper's grids do): codes then move
-    // monotonically with k, element by element
+    // the factors come in order, decreasing or increasing (as the paper's
+    // grid does): codes then move monotonically with k, element by element
     int monotone;
     // centre of each 8-candidate chunk's moments: the mean of 1/f over the
     // chunk's factors

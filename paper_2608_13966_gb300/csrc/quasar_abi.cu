@@ -15,12 +15,12 @@
 #include "quasar.h"
 
 namespace quasar {
-// integer-code kernels: one entry per (8-candidate chunks, clamp-set size)
+// integer-code kernels: one entry per (one chunk of 8 candidates, or more;
+// clamp-set size)
 #define QUASAR_INT_ENTRY(n, s) const void* int_kernel_nch##n##_ss##s(int epl, bool batch, bool adam, bool var);
 QUASAR_INT_ENTRY(1, 8) QUASAR_INT_ENTRY(1, 4) QUASAR_INT_ENTRY(1, 3) QUASAR_INT_ENTRY(1, 2)
 QUASAR_INT_ENTRY(1, 1)
 QUASAR_INT_ENTRY(2, 4) QUASAR_INT_ENTRY(2, 2) QUASAR_INT_ENTRY(2, 1)
-QUASAR_INT_ENTRY(4, 4) QUASAR_INT_ENTRY(4, 2) QUASAR_INT_ENTRY(4, 1)
 #undef QUASAR_INT_ENTRY
 const void* nvfp4_kernel(int nch, bool batch);
 const void* amax_kernel(bool batch);
@@ -425,14 +425,14 @@ uint32_t int_unit_bytes(int group_size, int g_kind, bool adam)
 
 // Shared memory of the asymmetric integer kernel's CTA ring: S slots of one
 // unit tile each (w, v, m for the fused AdamW step, then the gradient
-// region, which is also the transpose scratch and so at least
-// kIntXposeBytes), S + 1 mbarriers and S sequence words.  S is one slot a
+// region, which is also the candidate table and so at least kIntTableBytes
+// for each 8 candidates), S + 1 mbarriers and S sequence words.  S is one slot a
 // warp plus `extra` slots in flight (QUASAR_STAGES, default 2).
-Launch plan_ring(int group_size, int g_kind, bool adam, int warps)
+Launch plan_ring(int group_size, int g_kind, bool adam, int warps, int n_clip)
 {
     const uint32_t gbytes = g_kind == 2 ? 2u : (g_kind == 1 ? 4u : 0u);
     const uint32_t unit = (uint32_t)(kIntGroups * group_size);
-    const uint32_t tile = unit * (adam ? 12u : 8u) + std::max(unit * gbytes, kIntXposeBytes);
+    const uint32_t tile = unit * (adam ? 12u : 8u) + std::max(unit * gbytes, (uint32_t)((n_clip + 7) / 8) * kIntTableBytes);
     Launch L;
     L.stage_bytes = (tile + 127u) & ~127u;
     auto total = [&](int s) {
@@ -482,8 +482,12 @@ quasar_status int_params(quasar_dtype g_dtype, bool has_g, float beta2, int bits
     p->stats = g_stats.load();
     fill_clip(clip, n_clip, p->f, p->invf);
     fill_caps(p, 4);
-    p->monotone = 1;
-    for (int k = 1; k < n_clip; ++k) p->monotone &= p->invf[k] >= p->invf[k - 1] ? 1 : 0;
+    bool up = true, down = true;
+    for (int k = 1; k < n_clip; ++k) {
+        up &= p->invf[k] >= p->invf[k - 1];
+        down &= p->invf[k] <= p->invf[k - 1];
+    }
+    p->monotone = up || down;
     quasar_status st;
     if ((st = status_ptr(&p->status)) != QUASAR_OK) return st;
     if (adam) {
@@ -517,11 +521,11 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
     if (units == 0) return QUASAR_OK;
     const int warps = adam ? kAdamWarps : kWarps;
     const Launch L = symmetric ? plan(int_unit_bytes(group_size, Lp.p.g_kind, adam), kIntScratchBytes, warps)
-                               : plan_ring(group_size, Lp.p.g_kind, adam, warps);
+                               : plan_ring(group_size, Lp.p.g_kind, adam, warps, n_clip);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
     const int epl = group_size / (symmetric ? kLanesPerGroup : kIntLanes);
-    const int nch = nch_for(n_clip);
+    const bool one_chunk = n_clip <= 8;
     const bool batch = MAXT > 1;
     const bool var = Lp.p.h_mode != kSalEma || Lp.p.codes_packed;
     // clamp sets: as large as the factors allow, unless switched off (sets of
@@ -529,14 +533,13 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
     // step with sets of four or one
     const int hoist_on = g_hoist.load() < 0 ? tuning().hoist : g_hoist.load();
     // (sets of 8 or 3-3-2 with a single chunk, not for the fused AdamW step)
-    fill_caps(&Lp.p, (!hoist_on || var) ? 1 : 4, nch == 1 && !adam);
+    fill_caps(&Lp.p, (!hoist_on || var) ? 1 : 4, one_chunk && !adam);
     if (adam && Lp.p.set_size == 2) fill_caps(&Lp.p, 1);
     using Entry = const void* (*)(int, bool, bool, bool);
-    static const Entry table[3][5] = {
+    static const Entry table[2][5] = {
         {int_kernel_nch1_ss8, int_kernel_nch1_ss4, int_kernel_nch1_ss3, int_kernel_nch1_ss2, int_kernel_nch1_ss1},
-        {nullptr, int_kernel_nch2_ss4, nullptr, int_kernel_nch2_ss2, int_kernel_nch2_ss1},
-        {nullptr, int_kernel_nch4_ss4, nullptr, int_kernel_nch4_ss2, int_kernel_nch4_ss1}};
-    const int ci = nch == 1 ? 0 : (nch == 2 ? 1 : 2);
+        {nullptr, int_kernel_nch2_ss4, nullptr, int_kernel_nch2_ss2, int_kernel_nch2_ss1}};
+    const int ci = one_chunk ? 0 : 1;
     const int ss = Lp.p.set_size;
     const int si = ss == 8 ? 0 : (ss == 4 ? 1 : (ss == 3 ? 2 : (ss == 2 ? 3 : 4)));
     if (!table[ci][si]) return QUASAR_ERR_UNSUPPORTED;

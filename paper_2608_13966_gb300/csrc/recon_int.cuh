@@ -13,8 +13,8 @@
 // and, done with a tile, issues the copy of the unit that many slots ahead
 // into the same slot.  w, g and v are read from HBM exactly once, and the
 // loads of later units overlap the arithmetic of the current ones.  After
-// pass A the tile's gradient region is the warp's transpose scratch.  The
-// grid is persistent.
+// pass A the tile's gradient region holds the candidates' table.  The grid
+// is persistent.
 //
 // Codes.  With d = (w - min) - rho (the offset from the group's centre,
 // formed without rounding the centre itself: w - min and the half range are
@@ -33,14 +33,14 @@
 // Per group (fp32):
 //   pass A  v' = beta2*v + (1-beta2)*g^2 (written back; kept in the tile as
 //           the saliency h), min/max -> range, sum h, sum h w -> mu;
-//   pass B  for the 8 candidates of a single chunk at once (4 at a time with
-//           more chunks), the codes and the moments about a
-//           centre zeta0 shared by the candidates of an 8-candidate chunk
-//           (the code of the weighted mean, from mu): S1 = sum h (zeta -
-//           zeta0), S2 = sum h (zeta - zeta0)^2, S3 = sum h (zeta - zeta0) e,
-//           e = w - mu (plus the candidate-independent sum h e, sum h e^2);
-//   reduce  the 4 lanes' partial sums are transposed through the scratch so
-//           that lane sl owns candidate sl of each 4-candidate quad;
+//   pass B  for a chunk of 8 candidates at once, the codes and the moments
+//           about a centre zeta0 shared by the chunk (the code of the weighted
+//           mean, from mu): S1 = sum h (zeta - zeta0), S2 = sum h (zeta -
+//           zeta0)^2, S3 = sum h (zeta - zeta0) e, e = w - mu (plus the
+//           candidate-independent sum h e, sum h e^2);
+//   reduce  the 4 lanes scatter their partial sums while adding them: lane
+//           sl keeps candidates sl and 4 + sl of the chunk and writes them to
+//           the group's table;
 //   select  D = S2 - S1^2/Ss, N = S3 - S1*Se/Ss: the weighted error of
 //           candidate k is C - N^2/D with C common, so argmin error =
 //           argmax E = N^2/D; the winner's fit is a = N/D with the offset
@@ -122,10 +122,17 @@ __device__ __forceinline__ void ff_norm(float& hi, float& lo)
 }
 
 // Sum of a float pair over the 32 lanes of the warp, renormalised.
+// ROLL (here and in the group helpers below): loops stay rolled.  The careful
+// paths are cold code.  With more than 8 candidates a quarter of the units
+// enters them, and what counts is how much of the instruction cache they
+// take: rolled, one Qwen3 layer at INT2, 16 factors took 1,907 us, unrolled
+// 1,953.  With up to 8 it is a tenth, and latency counts: 806 against 822 us
+// on a Llama layer at INT3.
+template <bool ROLL>
 __device__ __forceinline__ void ff_reduce32(float& hi, float& lo)
 {
     ff_norm(hi, lo);
-#pragma unroll
+#pragma unroll (ROLL ? 1 : 5)
     for (int o = 16; o; o >>= 1) {
         const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
         const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
@@ -198,7 +205,7 @@ __device__ bool coop_same_codes(const float* ws, const GroupGeom& gq, float Pa, 
 // with w - A exact: the grid then follows the group's range rather than its
 // magnitude, and the rounded fit stays a tiny fraction of a level from the
 // given one (the error's excess is second order in that distance).
-template <int G>
+template <int G, bool ROLL>
 __device__ void coop_error(const float* ws, const float* hs, const GroupGeom& gq, float P,
                            float Jp1, float cref, float a, float bc, float* err_hi, float* err_lo)
 {
@@ -229,29 +236,26 @@ __device__ void coop_error(const float* ws, const float* hs, const GroupGeom& gq
 #pragma unroll
         for (int m = 0; m + s < M; m += 2 * s) t[m] += t[m + s];
     float eh = t[0], el = 0.0f;
-    ff_reduce32(eh, el);
+    ff_reduce32<ROLL>(eh, el);
     *err_hi = eh;
     *err_lo = el;
 }
 
-// Exact evaluation of one candidate: codes q, exact degenerate test (all
-// weighted elements on one code), two-pass centred fit, and the direct error
-// sum h (a q + B - w)^2 with (a, B) rounded to a common power-of-two grid U
-// so that a*q + B is exact and only "- w" rounds; lanes combine as a float
-// pair (coop_error).  dbar is the weighted mean of w - cref.  Returns the fit
-// as (a, Bz) with r = a zeta + Bz (offset at zeta = 0, i.e. q = J + 1), and a
-// condition estimate kap of the slope (see the tier-2 trigger in the kernel).
-template <int G>
+// Exact fit of one candidate: codes q, exact degenerate test (all weighted
+// elements on one code), two-pass centred fit.  dbar is the weighted mean of
+// w - cref.  Returns the fit as (a, bc) with bc the offset at q = 0 of w -
+// cref, and a condition estimate kap of the slope (see the tier-2 trigger in
+// the kernel).
+template <int G, bool ROLL>
 __device__ void coop_exact(const float* ws, const float* hs, const GroupGeom& gq, float P,
-                           float Jp1, float Ss, float dbar, float step, float cref, float* err_hi,
-                           float* err_lo, float* a_out, float* Bz_out, float* kap_out,
-                           bool* degenerate)
+                           float Ss, float dbar, float step, float cref, float* a_out,
+                           float* bc_out, float* kap_out, bool* degenerate)
 {
     constexpr int M = G / 32;
     const int lane = threadIdx.x & 31;
     float s1 = 0.0f;
     int qlo = 1 << 30, qhi = -1;
-#pragma unroll
+#pragma unroll (ROLL ? 1 : M)
     for (int m = 0; m < M; ++m) {
         const int e = lane + 32 * m;
         const float h = hs[e];
@@ -276,7 +280,7 @@ __device__ void coop_exact(const float* ws, const float* hs, const GroupGeom& gq
         bc = dbar - step * (float)qlo;
     } else {
         float dd = 0.0f, nn = 0.0f, ww = 0.0f;
-#pragma unroll
+#pragma unroll (ROLL ? 1 : M)
         for (int m = 0; m < M; ++m) {
             const int e = lane + 32 * m;
             const float h = hs[e];
@@ -295,9 +299,8 @@ __device__ void coop_exact(const float* ws, const float* hs, const GroupGeom& gq
         bc = dbar - a * qbar;
         kap = sqrtf(dd * ww) / fabsf(nn) + 1.0f;
     }
-    coop_error<G>(ws, hs, gq, P, Jp1, cref, a, bc, err_hi, err_lo);
     *a_out = a;
-    *Bz_out = fmaf(a, Jp1, bc + cref);
+    *bc_out = bc;
     *kap_out = kap;
 }
 
@@ -311,7 +314,7 @@ __device__ void coop_exact(const float* ws, const float* hs, const GroupGeom& gq
 // this part is a small fraction of fp32's); the offset is
 // mu - s*mq + mean_h(w - mu - s (q - mq)).  Returns the fit as float pairs,
 // with the offset Bz at the code origin zeta = 0 (q = J + 1, r = a zeta + Bz).
-template <int G>
+template <int G, bool ROLL>
 __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& gq, float P,
                              float Jp1, float Ss, float mu, float* a_hi, float* a_lo,
                              float* Bz_hi, float* Bz_lo)
@@ -319,7 +322,7 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
     constexpr int M = G / 32;
     const int lane = threadIdx.x & 31;
     float s1 = 0.0f;
-#pragma unroll
+#pragma unroll (ROLL ? 1 : M)
     for (int m = 0; m < M; ++m) {
         const int e = lane + 32 * m;
         s1 = fmaf(hs[e], int_code_q(centred(ws[e], gq.nmn, gq.nrho), P, gq.ylo, gq.yhi), s1);
@@ -327,7 +330,7 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
     const float mq = rintf(wsum32(s1) / Ss * 16.0f) * 0.0625f;
 
     float Dh = 0.0f, Dl = 0.0f, Nh = 0.0f, Nl = 0.0f, A = 0.0f, B = 0.0f;
-#pragma unroll
+#pragma unroll (ROLL ? 1 : M)
     for (int m = 0; m < M; ++m) {
         const int e = lane + 32 * m;
         const float h = hs[e];
@@ -345,8 +348,8 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
         A = __fadd_rn(A, xh);
         B = fmaf(h, wh, B);
     }
-    ff_reduce32(Dh, Dl);
-    ff_reduce32(Nh, Nl);
+    ff_reduce32<ROLL>(Dh, Dl);
+    ff_reduce32<ROLL>(Nh, Nl);
     A = wsum32(A);
     B = wsum32(B);
     {
@@ -364,7 +367,7 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
     const float shi = Nh / Dh;
     const float slo = __fadd_rn(fmaf(-shi, Dh, Nh), fmaf(-shi, Dl, Nl)) / Dh;
     float Rs = 0.0f;
-#pragma unroll
+#pragma unroll (ROLL ? 1 : M)
     for (int m = 0; m < M; ++m) {
         const int e = lane + 32 * m;
         const float h = hs[e];
@@ -415,19 +418,18 @@ __device__ __forceinline__ bool warp_wait_seq(const volatile int* seq, int t, ui
 // SS: candidates per clamp set (4, 2 or 1; with a single chunk also 8, or 3:
 // the sets 0-2, 3-5 and 6-7): the host picks the largest size whose sets all
 // admit a cap (see the header comment); every size gives the same codes.
+// NCH: 1 for up to 8 candidates (one chunk), 2 for up to 32 (p.n_clip / 8
+// chunks, rounded up).
 template <int EPL, int NCH, int MAXT, bool ADAM, bool VAR, int SS>
 __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
     k_recon_int(const __grid_constant__ IntLaunch<MAXT> Lp)
 {
     static_assert(SS == 1 || SS == 2 || SS == 4 || ((SS == 3 || SS == 8) && NCH == 1),
                   "clamp sets of 1, 2 or 4 candidates, or of 8 or 3-3-2 in a single chunk");
-    // candidates a sweep of pass B over the tile: all 8 of the chunk with
-    // one chunk (the loads, offsets and loop shared by 8), a quad with more
-    // (whose other live state leaves no room for 8 sets of sums)
-    constexpr int QW = NCH == 1 ? 8 : 4;
-    // clamp sets a sweep, and the set of the sweep's candidate kk (its first
-    // slot is kq + set * SS)
-    constexpr int NSETS = SS == 3 ? 3 : QW / SS;
+    static_assert(NCH == 1 || NCH == 2, "one chunk of 8 candidates, or more");
+    // clamp sets a sweep of 8 candidates, and the set of the sweep's candidate
+    // kk (its first slot is kq + set * SS)
+    constexpr int NSETS = SS == 3 ? 3 : 8 / SS;
     auto set_of = [](int kk) { return SS == 3 ? (kk < 3 ? 0 : (kk < 6 ? 1 : 2)) : kk / SS; };
     const IntParams& p = Lp.p;
     constexpr int G = EPL * kIntLanes;
@@ -454,8 +456,9 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * p.stage_bytes);
     volatile int* seq = reinterpret_cast<volatile int*>(bars + S + 1);
 
+    const int nch = (p.n_clip + 7) >> 3;  // chunks of 8 candidates
     const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
-    // stage: w | v | m (fused AdamW only) | g, then the transpose scratch
+    // stage: w | v | m (fused AdamW only) | g, then the candidates' table
     constexpr uint32_t kVOff = UNIT * 4;
     constexpr uint32_t kMOff = UNIT * 8;
     constexpr uint32_t kGOff = UNIT * (ADAM ? 12 : 8);
@@ -553,7 +556,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
         float* ws = reinterpret_cast<float*>(st);
         float* hs = reinterpret_cast<float*>(st + kVOff);
         const unsigned char* gsm = st + kGOff;
-        // transpose scratch (the gradient region, free once pass A is done)
+        // candidates' table (the gradient region, free once pass A is done)
         float* red = reinterpret_cast<float*>(st + kGOff);
 
         tensor_of(u, ti);
@@ -730,7 +733,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 sw = sw2;
             }
         }
-        // the gradient region becomes the transpose scratch: every lane is
+        // the gradient region becomes the candidates' table: every lane is
         // past pass A, and the h rewrites above are visible to all lanes
         __syncwarp();
         const float range = mx - mn;
@@ -754,117 +757,124 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
         const float2 nmu2 = make_float2(-mu, -mu);
         // the weighted mean's offset from the centre, for the chunks' centres
         const float dmu = centred(mu, -mn, -rho);
+        auto chunk_y0 = [&](int ch) {
+            return fminf(fmaxf(__fmaf_rd(dmu, R * p.invfc[ch], kGridMagic), ylo), yhi);
+        };
 
-        // ---- pass B + reduction + candidate errors, 8 candidates a chunk,
-        // QW a sweep over the tile.  Codes from d = (w - mn) - rho; moments
-        // about the chunk's centre code zeta0 and, for S3, e = w - mu.  Lane
-        // sl owns candidates 8 ch + 4 qd + sl.
-        float Ek[NCH][2], dEk[NCH][2], T1k[NCH][2], T2k[NCH][2], T3k[NCH][2], Y0k[NCH];
-        bool suspk[NCH][2];
-        float se = 0.0f, see = 0.0f;
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
+        // ---- pass B + reduction + candidate errors, a chunk of 8 candidates a
+        // sweep over the tile.  Codes from d = (w - mn) - rho; moments about the
+        // chunk's centre code zeta0 and, for S3, e = w - mu.  Lane sl owns
+        // candidates 8 ch + sl and 8 ch + 4 + sl; their sums and the upper end
+        // of E's error interval go to the group's table in the scratch (row k:
+        // T1, T2, T3, E + dE), from which every later step reads them, so that
+        // nothing per candidate stays in registers and the chunk loop can stay
+        // rolled: unrolled, two chunks' code (98 KB of it) left the instruction
+        // cache (2.6 no_instruction stalls an issue on the 16-factor INT2 step).
+        float4* tab = reinterpret_cast<float4*>(red) + gs;  // row k at tab[8 k]
+        float se = 0.0f, see = 0.0f, ebar = 0.0f;
+        float Eb = -INFINITY, dEb = 0.0f;  // this lane's best candidate
+        int kb = 0x7fff;
+        unsigned suspm = 0;  // this lane's candidates left to the exact comparison
+        // E (-1: out of the running) and dE of this lane's two candidates of the
+        // last chunk
+        float Ek[2], dEk[2];
+#pragma unroll 1
+        for (int ch = 0; ch < (NCH == 1 ? 1 : nch); ++ch) {
             // centre: the code of the weighted mean for the chunk's mean 1/f
-            const float y0 = fminf(fmaxf(__fmaf_rd(dmu, R * p.invfc[ch], kGridMagic), ylo), yhi);
+            const float y0 = chunk_y0(ch);
             const float2 nY02 = make_float2(-y0, -y0);
-            Y0k[ch] = y0;
-            float2 SE = make_float2(0.0f, 0.0f), SEE = make_float2(0.0f, 0.0f);
-            float4 xq[2];
+            const int kq = ch * 8;
+            float2 A1[8], A2[8], A3[8];
+            {
+                float2 P2[8];
 #pragma unroll
-            for (int sw = 0; sw < 8 / QW; ++sw) {
-                const int kq = ch * 8 + sw * QW;
-                float2 A1[QW], A2[QW], A3[QW];
+                for (int kk = 0; kk < 8; ++kk) {
+                    const float P = R * p.invf[kq + kk];
+                    P2[kk] = make_float2(P, P);
+                    A1[kk] = A2[kk] = A3[kk] = make_float2(0.0f, 0.0f);
+                }
+                float cp[NSETS];
 #pragma unroll
-                for (int kk = 0; kk < QW; ++kk) A1[kk] = A2[kk] = A3[kk] = make_float2(0.0f, 0.0f);
-                if ((ch == 0 && sw == 0) || kq < p.n_clip) {
-                    float2 P2[QW];
-#pragma unroll
-                    for (int kk = 0; kk < QW; ++kk) {
-                        const float P = R * p.invf[kq + kk];
-                        P2[kk] = make_float2(P, P);
-                    }
-                    float cp[NSETS];
-#pragma unroll
-                    for (int s = 0; s < NSETS; ++s) cp[s] = p.cap[kq + s * SS] * range;
+                for (int s = 0; s < NSETS; ++s) cp[s] = p.cap[kq + s * SS] * range;
+                float2 SE = make_float2(0.0f, 0.0f), SEE = make_float2(0.0f, 0.0f);
 // rolled: a compact unit loop keeps the careful paths' code from evicting it
 // from the instruction cache when they run
 #pragma unroll 1
-                    for (int i = 0; i < NCHK; ++i) {
-                        const int e = eoff(i);
-                        const float4 w4 = lds128(gws + e);
-                        const float4 h4 = lds128(ghs + e);
+                for (int i = 0; i < NCHK; ++i) {
+                    const int e = eoff(i);
+                    const float4 w4 = lds128(gws + e);
+                    const float4 h4 = lds128(ghs + e);
 #pragma unroll
-                        for (int pr = 0; pr < 2; ++pr) {
-                            const float2 wv = pr ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
-                            const float2 h = pr ? make_float2(h4.z, h4.w) : make_float2(h4.x, h4.y);
-                            const float2 d = __fadd2_rn(__fadd2_rn(wv, nmn2), nrho2);
-                            const float2 ev = __fadd2_rn(wv, nmu2);
-                            if (ch == 0 && sw == 0) {
-                                const float2 he = __fmul2_rn(h, ev);
-                                SE = __fadd2_rn(SE, he);
-                                SEE = __ffma2_rn(he, ev, SEE);
-                            }
-                            float2 dc[NSETS];
+                    for (int pr = 0; pr < 2; ++pr) {
+                        const float2 wv = pr ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
+                        const float2 h = pr ? make_float2(h4.z, h4.w) : make_float2(h4.x, h4.y);
+                        const float2 d = __fadd2_rn(__fadd2_rn(wv, nmn2), nrho2);
+                        const float2 ev = __fadd2_rn(wv, nmu2);
+                        if (NCH == 1 || ch == 0) {
+                            const float2 he = __fmul2_rn(h, ev);
+                            SE = __fadd2_rn(SE, he);
+                            SEE = __ffma2_rn(he, ev, SEE);
+                        }
+                        float2 dc[NSETS];
 #pragma unroll
-                            for (int s = 0; s < NSETS; ++s)
-                                dc[s] = make_float2(fminf(fmaxf(d.x, -cp[s]), cp[s]),
-                                                    fminf(fmaxf(d.y, -cp[s]), cp[s]));
+                        for (int s = 0; s < NSETS; ++s)
+                            dc[s] = make_float2(fminf(fmaxf(d.x, -cp[s]), cp[s]),
+                                                fminf(fmaxf(d.y, -cp[s]), cp[s]));
 #pragma unroll
-                            for (int kk = 0; kk < QW; ++kk) {
-                                const float2 y = __ffma2_rd(dc[set_of(kk)], P2[kk], Mg2);
-                                const float2 zc = __fadd2_rn(y, nY02);  // zeta - zeta0, exact
-                                const float2 t2 = __fmul2_rn(h, zc);
-                                A1[kk] = __ffma2_rn(h, zc, A1[kk]);
-                                A2[kk] = __ffma2_rn(t2, zc, A2[kk]);
-                                A3[kk] = __ffma2_rn(t2, ev, A3[kk]);
-                            }
+                        for (int kk = 0; kk < 8; ++kk) {
+                            const float2 y = __ffma2_rd(dc[set_of(kk)], P2[kk], Mg2);
+                            const float2 zc = __fadd2_rn(y, nY02);  // zeta - zeta0, exact
+                            const float2 t2 = __fmul2_rn(h, zc);
+                            A1[kk] = __ffma2_rn(h, zc, A1[kk]);
+                            A2[kk] = __ffma2_rn(t2, zc, A2[kk]);
+                            A3[kk] = __ffma2_rn(t2, ev, A3[kk]);
                         }
                     }
                 }
-                // transpose each quad through the scratch: lane L writes row L
-                // (its sums of candidate kk in 16-byte column kk ^ ((L >> 1) &
-                // 3)), and lane (gs, sl) sums column sl of its group's 4 rows
-                // (each group starting at another row, so that an access
-                // phase's two groups read rows of both parities: no bank
-                // conflicts)
+                if (ch == 0) {
+                    se = SE.x + SE.y;
+                    see = SEE.x + SEE.y;
 #pragma unroll
-                for (int q4 = 0; q4 < QW / 4; ++q4) {
-                    __syncwarp();
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const int c = q4 * 4 + kk;
-                        *reinterpret_cast<float4*>(red + lane * 16 + ((kk ^ ((lane >> 1) & 3)) << 2)) =
-                            make_float4(A1[c].x + A1[c].y, A2[c].x + A2[c].y, A3[c].x + A3[c].y, 0.0f);
+                    for (int o = 2; o; o >>= 1) {
+                        se += shx(se, o);
+                        see += shx(see, o);
                     }
-                    __syncwarp();
-                    float4 x[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int row = gs * 4 + ((j + gs) & 3);
-                        x[j] = *reinterpret_cast<const float4*>(red + row * 16 + ((sl ^ ((row >> 1) & 3)) << 2));
-                    }
-                    xq[sw * (QW / 4) + q4] = make_float4((x[0].x + x[1].x) + (x[2].x + x[3].x),
-                                                         (x[0].y + x[1].y) + (x[2].y + x[3].y),
-                                                         (x[0].z + x[1].z) + (x[2].z + x[3].z), 0.0f);
+                    ebar = se * inv_ss;
                 }
             }
-            if (ch == 0) {
-                se = SE.x + SE.y;
-                see = SEE.x + SEE.y;
+            // the group's 4 lanes scatter the sums while they add them: lane sl
+            // keeps candidates kq + sl and kq + 4 + sl (a step exchanges the
+            // candidates the two lanes do not keep)
+            float T[2][3];
+            const int mate = lane ^ (gs & 1 ? 3 : 1);
 #pragma unroll
-                for (int o = 2; o; o >>= 1) {
-                    se += shx(se, o);
-                    see += shx(see, o);
+            for (int c = 0; c < 3; ++c) {
+                float x[8], y[4];
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    const float2 a = c == 0 ? A1[kk] : (c == 1 ? A2[kk] : A3[kk]);
+                    x[kk] = a.x + a.y;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {  // the pair 2 j, 2 j + 1: bit 0 of sl picks
+                    const float keep = sl & 1 ? x[2 * j + 1] : x[2 * j], give = sl & 1 ? x[2 * j] : x[2 * j + 1];
+                    y[j] = keep + __shfl_sync(0xffffffffu, give, mate);
+                }
+#pragma unroll
+                for (int qd = 0; qd < 2; ++qd) {
+                    const float keep = sl & 2 ? y[2 * qd + 1] : y[2 * qd];
+                    const float give = sl & 2 ? y[2 * qd] : y[2 * qd + 1];
+                    T[qd][c] = keep + shx(give, 2);
                 }
             }
-            // candidates 8 ch + 4 qd + sl: E = N^2/D and a bound dE on its fp32
-            // error.  The sums are accumulated over tie_kappa levels at most,
-            // so each is within tie_kappa ulps of the sum of its terms'
-            // magnitudes: sum h zc^2 = S2, sum |h zc e| <= sqrt(S2 * sum h e^2).
-            const float ebar = se * inv_ss;
+            // E = N^2/D and a bound dE on its fp32 error.  The sums are
+            // accumulated over tie_kappa levels at most, so each is within
+            // tie_kappa ulps of the sum of its terms' magnitudes: sum h zc^2 =
+            // S2, sum |h zc e| <= sqrt(S2 * sum h e^2).
 #pragma unroll
             for (int qd = 0; qd < 2; ++qd) {
-                const float T1 = xq[qd].x, T2 = xq[qd].y, T3 = xq[qd].z;
+                const int k = kq + qd * 4 + sl;
+                const float T1 = T[qd][0], T2 = T[qd][1], T3 = T[qd][2];
                 const float zbar = T1 * inv_ss;
                 const float D = T2 - T1 * zbar;
                 const float N = T3 - T1 * ebar;
@@ -872,62 +882,55 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 // a near-degenerate code variance, or a non-finite E (sums
                 // near the denormal range): left to the exact comparison
                 const bool susp = !(D > 1e-3f * T2) || !(N * a < INFINITY);
-                const float E = susp ? 0.0f : N * a;
+                const float E = N * a;
                 const float s2e = fmaxf(T2 * see, 1e-37f);
                 const float dN = ulp * (s2e * rsqrtf(s2e) * 1.001f + fabsf(T1 * ebar));
                 const float dD = ulp * (T2 + fabsf(T1 * zbar));
-                const bool real = ch * 8 + qd * 4 + sl < p.n_clip;
-                Ek[ch][qd] = real && !susp ? E : -INFINITY;
-                dEk[ch][qd] = 2.0f * fabsf(a) * dN + a * a * dD;
-                suspk[ch][qd] = real && susp;
-                T1k[ch][qd] = T1;
-                T2k[ch][qd] = T2;
-                T3k[ch][qd] = T3;
+                const float dE = 2.0f * fabsf(a) * dN + a * a * dD;
+                const bool real = k < p.n_clip;
+                if (real && susp) suspm |= 1u << k;
+                const bool run = real && !susp;
+                if (NCH != 1 && run && E > Eb) {  // strict: keeps the lower k of this lane
+                    Eb = E;
+                    dEb = dE;
+                    kb = k;
+                }
+                Ek[qd] = run ? E : -1.0f;
+                dEk[qd] = dE;
+                tab[8 * k] = make_float4(T1, T2, T3, run ? E + dE : -INFINITY);
             }
         }
-        const float ebar = se * inv_ss;
+        __syncwarp();
 
-        // ---- argmax of E over the group (ties: lowest index)
-        float Eb = -INFINITY, dEb = 0.0f;
-        int kb = 0x7fff;
+        // ---- argmax of E over the group's 4 lanes (ties: lowest index)
         if constexpr (NCH == 1) {
             // the max of integer keys, E's bits (E >= 0 orders like them) with
-            // the low 3 replaced by 7 - k; a candidate out of the running
-            // (E = -inf) has key 0.  Two candidates within 7 ulps of each other
-            // are both within the tie bound below (dE is at least 2 tie_kappa
-            // ulps of E, since sqrt(S2 sum h e^2) >= |N|, and the host's
-            // tie_kappa is at least 12), so whichever the key picks, the exact
-            // comparison settles them.
+            // the low 3 replaced by 7 - k; 0 for a candidate out of the running.
+            // (Every candidate takes part with its key, not each lane's best:
+            // the winner is then the lowest of its twins.)  Two candidates
+            // within 7 ulps of each other are both within the tie bound below
+            // (dE is at least 2 tie_kappa ulps of E, since sqrt(S2 sum h e^2) >=
+            // |N|, and the host's tie_kappa is at least 12), so whichever the
+            // key picks, the exact comparison settles them.
             uint32_t key = 0;
 #pragma unroll
             for (int qd = 0; qd < 2; ++qd) {
-                const uint32_t k = (uint32_t)(qd * 4 + sl);
-                const uint32_t kq = Ek[0][qd] >= 0.0f ? ((__float_as_uint(Ek[0][qd]) & ~7u) | (7u - k)) : 0u;
-                key = max(key, kq);
+                const uint32_t kq = (__float_as_uint(Ek[qd]) & ~7u) | (7u - (uint32_t)(qd * 4 + sl));
+                key = max(key, Ek[qd] >= 0.0f ? kq : 0u);
             }
 #pragma unroll
             for (int o = 2; o; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
             const int kk = 7 - (int)(key & 7u);
-            const int owner = (gs * 4) | (kk & 3);
-            const float Eo0 = __shfl_sync(0xffffffffu, Ek[0][0], owner);
-            const float Eo1 = __shfl_sync(0xffffffffu, Ek[0][1], owner);
-            const float dEo0 = __shfl_sync(0xffffffffu, dEk[0][0], owner);
-            const float dEo1 = __shfl_sync(0xffffffffu, dEk[0][1], owner);
+            const float Eo = __shfl_sync(0xffffffffu, kk & 4 ? Ek[1] : Ek[0], (gs * 4) | (kk & 3));
+            const float dEo = __shfl_sync(0xffffffffu, kk & 4 ? dEk[1] : dEk[0], (gs * 4) | (kk & 3));
+            Eb = -INFINITY;
+            kb = 0x7fff;
             if (key != 0u) {
-                Eb = kk & 4 ? Eo1 : Eo0;
-                dEb = kk & 4 ? dEo1 : dEo0;
+                Eb = Eo;
+                dEb = dEo;
                 kb = kk;
             }
         } else {
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                for (int qd = 0; qd < 2; ++qd)
-                    if (Ek[ch][qd] > Eb) {  // strict: keeps the lower k of this lane
-                        Eb = Ek[ch][qd];
-                        dEb = dEk[ch][qd];
-                        kb = ch * 8 + qd * 4 + sl;
-                    }
 #pragma unroll
             for (int o = 2; o; o >>= 1) {
                 const float Eo = shx(Eb, o);
@@ -942,118 +945,79 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
         }
         if (kb > 0x7ff) kb = 0;  // every candidate suspicious: the exact path picks
 
-        // the sums of candidate k, from its owner lane (every lane of a group
-        // names the same k)
-        auto sums_of = [&](int k, float& t1, float& t2, float& t3) {
-            const int owner = (gs * 4) | (k & 3);
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                for (int qd = 0; qd < 2; ++qd) {
-                    const float a1 = __shfl_sync(0xffffffffu, T1k[ch][qd], owner);
-                    const float a2 = __shfl_sync(0xffffffffu, T2k[ch][qd], owner);
-                    const float a3 = __shfl_sync(0xffffffffu, T3k[ch][qd], owner);
-                    if ((k >> 2) == ch * 2 + qd) {
-                        t1 = a1;
-                        t2 = a2;
-                        t3 = a3;
-                    }
-                }
-        };
-        float T1b = 0.0f, T2b = 0.0f, T3b = 0.0f;
-        sums_of(kb, T1b, T2b, T3b);
         // Candidates needing an exact comparison: within the fp32 error bound
-        // of the winner.  Those whose sums, about the winner's centre code
-        // (their chunk's or another chunk's with the same centre), equal the
-        // winner's bit for bit ("twins") almost always have the winner's
-        // codes -- equal codes give equal errors, and the lower index is
-        // kept, as Algorithm 1's argmin does -- but an element of tiny
-        // saliency can differ without moving the sums, so twins are first
-        // checked code by code (cheaply, deferred) -- unless every saliency
-        // of the group is too large for that.  Between two factors every
-        // element's code moves away from the centre or stays, and a moving
-        // element has |d| >= range f / q_max (f the smaller factor), so a
+        // of the winner (their E + dE reaches its E - dE).  Those whose sums,
+        // about the winner's centre code (their chunk's or another chunk's with
+        // the same centre), equal the winner's bit for bit ("twins") almost
+        // always have the winner's codes -- equal codes give equal errors, and
+        // the lower index is kept, as Algorithm 1's argmin does -- but an
+        // element of tiny saliency can differ without moving the sums, so twins
+        // are first checked code by code (cheaply, deferred) -- unless every
+        // saliency of the group is too large for that.  Between two factors
+        // every element's code moves away from the centre or stays, and a
+        // moving element has |d| >= range f / q_max (f the smaller factor), so a
         // code difference moves T3 - (c - mu) T1 by at least h_min range f /
         // q_max, less the roundings of e, d and c (every term has the sign of
         // the move: e - (c - mu) is d up to those roundings).  Bitwise-equal
         // sums bound that change by twice their fp32 errors, ulp sqrt(T2 see)
         // and |c - mu| ulp sqrt(Ss T2); a larger bound leaves the codes
         // equal (up to elements of zero saliency, which move no error).
-        float y0w = Y0k[0];
+        unsigned set = suspm, twins = 0;
+        {
+            unsigned cont = 0;
+            if constexpr (NCH == 1) {
 #pragma unroll
-        for (int ch = 1; ch < NCH; ++ch)
-            if ((kb >> 3) == ch) y0w = Y0k[ch];
-        bool twinf[NCH][2];
-        bool anytwin = false;
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-            for (int qd = 0; qd < 2; ++qd) {
-                const int k = ch * 8 + qd * 4 + sl;
-                twinf[ch][qd] = k != kb && Y0k[ch] == y0w && T1k[ch][qd] == T1b &&
-                                T2k[ch][qd] == T2b && T3k[ch][qd] == T3b;
-                anytwin |= twinf[ch][qd];
-            }
-        // the bound (only where a warp has twins): the group's smallest
-        // saliency, from the tile (the fit's h, 1 for all-zero groups).
-        // Built for 16 or more candidates, where twins are common (with 8
-        // they are rare and the code costs more than it saves).
-        constexpr bool kCertify = NCH >= 2 && !ADAM;
-        float twin_q = INFINITY, twin_h = 0.0f, twin_e = 0.0f;
-        if (kCertify && __any_sync(0xffffffffu, anytwin)) {
-            float hmn = INFINITY;
+                for (int qd = 0; qd < 2; ++qd)
+                    if (qd * 4 + sl != kb && Ek[qd] >= 0.0f && Eb - Ek[qd] <= dEb + dEk[qd])
+                        cont |= 1u << (qd * 4 + sl);
+            } else {
+                const float lo = Eb - dEb;
 #pragma unroll 1
-            for (int i = 0; i < NCHK; ++i) {
-                const float4 h4 = lds128(ghs + eoff(i));
-                hmn = fmin3(fmin3(hmn, h4.x, h4.y), h4.z, h4.w);
-            }
-#pragma unroll
-            for (int o = 2; o; o >>= 1) hmn = fminf(hmn, shx(hmn, o));
-            const float t2s = fmaxf(T2b * see, 0.0f), t2w = fmaxf(ss * T2b, 0.0f);
-            twin_q = 2.0f * ulp * (sqrtf(t2s) + fabsf(cref - mu) * sqrtf(t2w)) * qmaxf;
-            twin_h = hmn * range;
-            twin_e = hmn * qmaxf * (8.0f * 5.9604645e-8f) * (range + fabsf(cref));
-        }
-        unsigned set = 0, twins = 0;
-        if constexpr (!kCertify) {
-            // contenders first; the twins among them only where a warp has any
-            bool cont[NCH][2];
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                for (int qd = 0; qd < 2; ++qd) {
-                    const int k = ch * 8 + qd * 4 + sl;
-                    cont[ch][qd] = k != kb && Ek[ch][qd] > -INFINITY &&
-                                   Eb - Ek[ch][qd] <= dEb + dEk[ch][qd];
-                    const unsigned bal = __ballot_sync(0xffffffffu, cont[ch][qd] || suspk[ch][qd]);
-                    set |= ((bal >> (gs * 4)) & 0xFu) << (ch * 8 + qd * 4);
+                for (int k = sl; k < p.n_clip; k += 4) {
+                    const float up = tab[8 * k].w;
+                    if (k != kb && up >= lo && up > -INFINITY) cont |= 1u << k;
                 }
-            if (__any_sync(0xffffffffu, set != 0u)) {
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                    for (int qd = 0; qd < 2; ++qd) {
-                        const unsigned balt =
-                            __ballot_sync(0xffffffffu, cont[ch][qd] && twinf[ch][qd] && !suspk[ch][qd]);
-                        twins |= ((balt >> (gs * 4)) & 0xFu) << (ch * 8 + qd * 4);
+            }
+            if (__any_sync(0xffffffffu, cont != 0u)) {
+                const float4 tb = tab[8 * kb];
+                const float y0w = chunk_y0(NCH == 1 ? 0 : kb >> 3);
+                // the bound (where twins are common): the group's smallest
+                // saliency, from the tile (the fit's h, 1 for all-zero groups)
+                constexpr bool kCertify = NCH >= 2 && !ADAM;
+                float twin_q = INFINITY, twin_h = 0.0f, twin_e = 0.0f;
+                if (kCertify) {
+                    float hmn = INFINITY;
+#pragma unroll 1
+                    for (int i = 0; i < NCHK; ++i) {
+                        const float4 h4 = lds128(ghs + eoff(i));
+                        hmn = fmin3(fmin3(hmn, h4.x, h4.y), h4.z, h4.w);
                     }
-            }
-        } else {
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                for (int qd = 0; qd < 2; ++qd) {
-                    const int k = ch * 8 + qd * 4 + sl;
-                    const bool twin = twinf[ch][qd];
-                    // a twin whose codes are certainly the winner's: as the winner
-                    const bool sure = twin && twin_h * fminf(p.f[k], p.f[kb]) - twin_e > twin_q;
-                    const bool contender = k != kb && !sure && Ek[ch][qd] > -INFINITY &&
-                                           Eb - Ek[ch][qd] <= dEb + dEk[ch][qd];
-                    const unsigned bal = __ballot_sync(0xffffffffu, contender || suspk[ch][qd]);
-                    set |= ((bal >> (gs * 4)) & 0xFu) << (ch * 8 + qd * 4);
-                    const unsigned balt = __ballot_sync(0xffffffffu, contender && twin && !suspk[ch][qd]);
-                    twins |= ((balt >> (gs * 4)) & 0xFu) << (ch * 8 + qd * 4);
+                    for (int o = 2; o; o >>= 1) hmn = fminf(hmn, shx(hmn, o));
+                    const float t2s = fmaxf(tb.y * see, 0.0f), t2w = fmaxf(ss * tb.y, 0.0f);
+                    twin_q = 2.0f * ulp * (sqrtf(t2s) + fabsf(cref - mu) * sqrtf(t2w)) * qmaxf;
+                    twin_h = hmn * range;
+                    twin_e = hmn * qmaxf * (8.0f * 5.9604645e-8f) * (range + fabsf(cref));
                 }
+                for (unsigned m = cont; m; m &= m - 1) {
+                    const int k = __ffs(m) - 1;
+                    const float4 tk = tab[8 * k];
+                    const bool twin = tk.x == tb.x && tk.y == tb.y && tk.z == tb.z &&
+                                      (NCH == 1 || chunk_y0(k >> 3) == y0w);
+                    // a twin whose codes are certainly the winner's: as the winner
+                    const bool sure =
+                        kCertify && twin && twin_h * fminf(p.f[k], p.f[kb]) - twin_e > twin_q;
+                    if (sure) cont &= ~(1u << k);
+                    else if (twin) twins |= 1u << k;
+                }
+                __syncwarp();
+            }
+            set |= cont;
+#pragma unroll
+            for (int o = 2; o; o >>= 1) {
+                set |= __shfl_xor_sync(0xffffffffu, set, o);
+                twins |= __shfl_xor_sync(0xffffffffu, twins, o);
+            }
         }
         if (Eb == -INFINITY) set = (p.n_clip >= 32) ? 0xFFFFFFFFu : ((1u << p.n_clip) - 1u);
         else if (set) set |= 1u << kb;
@@ -1086,71 +1050,60 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             int gw = __shfl_sync(0xffffffffu, kb, src);  // the winner
             const float* tws = ws + g * G;
             const float* ths = hs + g * G;
-            float gy0[NCH];
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) gy0[ch] = __shfl_sync(0xffffffffu, Y0k[ch], src);
-            if (p.stats && lane == 0) atomicAdd(&p.stats[2], 1u);
-            auto same_codes = [&](int k) {
-                if (p.stats && lane == 0) atomicAdd(&p.stats[6], 1u);
-                return coop_same_codes<G>(tws, ggq, gR * p.invf[k], gR * p.invf[gw]);
+            const float gdmu = __shfl_sync(0xffffffffu, dmu, src);
+            const float4* gtab = reinterpret_cast<const float4*>(red) + g;
+            // centre code of a chunk, as pass B took it
+            auto gy0 = [&](int ch) {
+                return fminf(fmaxf(__fmaf_rd(gdmu, gR * p.invfc[ch], kGridMagic), ylo), yhi);
             };
-            // Codes move monotonically with 1/f, element by element (the
-            // factors decrease with k), so two candidates with equal codes
-            // share them with every candidate between them: the highest twin
-            // settles all twins when its codes are the winner's.
+            if (p.stats && lane == 0) atomicAdd(&p.stats[2], 1u);
+            // Codes move monotonically with 1/f, element by element, so (with the
+            // factors in order) two candidates with equal codes share them with
+            // every candidate between them: the highest twin settles all twins
+            // when its codes are the winner's.
             const bool mono = p.monotone != 0;
-            unsigned tw = gtwins;
-            if (tw && mono) {
-                const int khi = 31 - __clz(tw);
-                tw &= ~(1u << khi);
-                if (same_codes(khi)) {
-                    gset &= ~((2u << khi) - (2u << gw));  // (gw, khi]
-                    tw = 0;
-                }
-            }
-            while (tw) {
-                const int k = __ffs(tw) - 1;
-                tw &= tw - 1;
-                if (same_codes(k)) gset &= ~(1u << k);
-            }
-            // Contenders about another centre code (their sums are not
-            // comparable with the winner's): first whether they share the
-            // winner's codes -- below the winner, lowest first, such a
-            // candidate becomes the winner; above it, highest first, it
-            // drops out (with monotone codes, so does everything between it
-            // and the winner).
             auto other_centres = [&]() {
-                float y0g = gy0[0];
-#pragma unroll
-                for (int ch = 1; ch < NCH; ++ch)
-                    if ((gw >> 3) == ch) y0g = gy0[ch];
+                const float y0g = gy0(gw >> 3);
                 unsigned m = 0;
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch)
-                    if (gy0[ch] != y0g) m |= 0xFFu << (8 * ch);
+#pragma unroll 1
+                for (int ch = 0; ch < nch; ++ch)
+                    if (gy0(ch) != y0g) m |= 0xFFu << (8 * ch);
                 return m;
             };
-            if (NCH > 1) {
-                const unsigned cmask = other_centres();
-                unsigned lo = gset & cmask & ((1u << gw) - 1u);
-                while (lo) {
-                    const int k = __ffs(lo) - 1;
-                    lo &= lo - 1;
-                    if (same_codes(k)) {
-                        gset &= ~(mono ? (2u << gw) - (2u << k) : 1u << gw);  // (k, gw]
-                        gw = k;
-                        break;
-                    }
+            // First the twins; then contenders about another centre code (their
+            // sums are not comparable with the winner's): whether they share the
+            // winner's codes -- below the winner, lowest first, such a candidate
+            // becomes the winner; above it, highest first, it drops out (with
+            // monotone codes, so does everything between it and the winner).
+            // One loop, so that the code check is built once.
+            enum { kTwins, kBelow, kAbove };
+            int phase = kTwins;
+            unsigned todo_k = gtwins;
+            bool top = mono;
+#pragma unroll 1
+            for (;;) {
+                if (todo_k == 0u) {
+                    if (NCH == 1 || phase == kAbove) break;
+                    ++phase;
+                    const unsigned below = (1u << gw) - 1u, above = ~((2u << gw) - 1u);
+                    todo_k = gset & other_centres() & (phase == kBelow ? below : above);
+                    continue;
                 }
-                unsigned hi = gset & cmask & ~((2u << gw) - 1u);
-                while (hi) {
-                    const int k = 31 - __clz(hi);
-                    hi &= ~(1u << k);
-                    if (same_codes(k)) {
-                        gset &= ~(mono ? (2u << k) - (2u << gw) : 1u << k);  // (gw, k]
-                        if (mono) break;
-                    }
+                const bool high = phase == kTwins ? top : phase == kAbove;
+                const int k = high ? 31 - __clz(todo_k) : __ffs(todo_k) - 1;
+                todo_k &= ~(1u << k);
+                if (p.stats && lane == 0) atomicAdd(&p.stats[6], 1u);
+                const bool same = coop_same_codes<G>(tws, ggq, gR * p.invf[k], gR * p.invf[gw]);
+                if (same && phase == kBelow) {
+                    gset &= ~(mono ? (2u << gw) - (2u << k) : 1u << gw);  // (k, gw]
+                    gw = k;
+                    todo_k = 0u;
+                } else if (same) {
+                    const bool span = phase == kTwins ? top : mono;
+                    gset &= ~(span ? (2u << k) - (2u << gw) : 1u << k);  // (gw, k]
+                    if (span) todo_k = 0u;
                 }
+                top = false;
             }
             if (gset == (1u << gw)) {  // only the winner left
                 if (gs == g) kb = gw;
@@ -1165,7 +1118,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             // have equal codes with unequal sums, and only the two-pass fit, a
             // function of the codes alone, then gives them bitwise-equal
             // errors, so that the lower index is kept
-            const bool one_chunk = (gset & other_centres()) == 0u;
+            const bool one_chunk = NCH == 1 || (gset & other_centres()) == 0u;
             const float gebar = __shfl_sync(0xffffffffu, ebar, src);
             const float gsee = __shfl_sync(0xffffffffu, see, src);
             while (gset) {
@@ -1177,24 +1130,8 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 // order: (rel. fit error)^2 times explained over residual
                 // variance): then one error pass settles it; otherwise (and
                 // for nearly degenerate code variance) the two-pass fit
-                float k1 = 0.0f, k2 = 0.0f, k3 = 0.0f, y0k = gy0[0];
-                {
-                    const int owner = src | (k & 3);
-#pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                        for (int qd = 0; qd < 2; ++qd) {
-                            const float a1 = __shfl_sync(0xffffffffu, T1k[ch][qd], owner);
-                            const float a2 = __shfl_sync(0xffffffffu, T2k[ch][qd], owner);
-                            const float a3 = __shfl_sync(0xffffffffu, T3k[ch][qd], owner);
-                            if ((k >> 2) == ch * 2 + qd) {
-                                k1 = a1;
-                                k2 = a2;
-                                k3 = a3;
-                                y0k = gy0[ch];
-                            }
-                        }
-                }
+                const float4 tk = gtab[8 * k];
+                const float k1 = tk.x, k2 = tk.y, k3 = tk.z, y0k = gy0(NCH == 1 ? 0 : k >> 3);
                 const float Dk = k2 - k1 * (k1 / gss), Nk = k3 - k1 * gebar;
                 const float ak = Nk / Dk, Exk = Nk * ak;
                 const float kapk = sqrtf(k2 * gsee) / fabsf(Nk) + k2 / Dk;
@@ -1204,14 +1141,15 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 float eh, el, a_k = 0.0f, B_k = 0.0f, kap_k = 0.0f;
                 bool deg_k = false;
                 if (p.stats && lane == 0) atomicAdd(&p.stats[quick ? 5 : 4], 1u);
-                if (quick) {
-                    // offset at q = 0 of w - cref: mean(w - cref) - a (mean zeta + J + 1)
-                    const float bck = gdbar - ak * ((y0k - kGridMagic) + k1 / gss + Jp1);
-                    coop_error<G>(tws, ths, ggq, gR * p.invf[k], Jp1, gcref, ak, bck, &eh, &el);
-                } else {
-                    coop_exact<G>(tws, ths, ggq, gR * p.invf[k], Jp1, gss, gdbar,
-                                  p.f[k] * grange / qmaxf, gcref, &eh, &el, &a_k, &B_k, &kap_k, &deg_k);
+                // (offset at q = 0 of w - cref: mean(w - cref) - a (mean zeta + J + 1))
+                float aq = ak, bq = gdbar - ak * ((y0k - kGridMagic) + k1 / gss + Jp1);
+                if (!quick) {
+                    coop_exact<G, NCH != 1>(tws, ths, ggq, gR * p.invf[k], gss, gdbar, p.f[k] * grange / qmaxf,
+                                  gcref, &aq, &bq, &kap_k, &deg_k);
+                    a_k = aq;
+                    B_k = fmaf(aq, Jp1, bq + gcref);
                 }
+                coop_error<G, NCH != 1>(tws, ths, ggq, gR * p.invf[k], Jp1, gcref, aq, bq, &eh, &el);
                 if (best_k < 0 || ff_less(eh, el, best_h, best_l)) {
                     best_h = eh;
                     best_l = el;
@@ -1233,11 +1171,9 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
 
         // ---- the fit (Eq. 4) from the kept candidate's centred sums: codes
         // about its chunk's centre zeta0, weights about mu
-        sums_of(kb, T1b, T2b, T3b);
-        float y0b = Y0k[0];
-#pragma unroll
-        for (int ch = 1; ch < NCH; ++ch)
-            if ((kb >> 3) == ch) y0b = Y0k[ch];
+        const float4 tbk = tab[8 * kb];
+        const float T1b = tbk.x, T2b = tbk.y, T3b = tbk.z;
+        const float y0b = chunk_y0(NCH == 1 ? 0 : kb >> 3);
         if (!deg_sel) {
             // T1 = sum h (zeta - zeta0) (small); sum h (w - mu) = Se
             const float Aq = T1b * inv_ss;
@@ -1324,7 +1260,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             const int gkb = __shfl_sync(0xffffffffu, kb, src);
             if (p.stats && lane == 0) atomicAdd(&p.stats[1], 1u);
             float ga, ga_lo, gB, gB_lo;
-            coop_precise<G>(ws + g * G, hs + g * G, ggq, gR * p.invf[gkb], Jp1, gss, gmu, &ga,
+            coop_precise<G, NCH != 1>(ws + g * G, hs + g * G, ggq, gR * p.invf[gkb], Jp1, gss, gmu, &ga,
                             &ga_lo, &gB, &gB_lo);
             if (gs == g) {
                 a_sel = ga;
