@@ -1,21 +1,13 @@
-// Instantiations of the NVFP4 kernel (1, 2 or 4 chunks of 8 candidates) and
-// of the tensor-absmax kernels.
+// Instantiations of the NVFP4 kernel and of the tensor-absmax kernels.
 #include "recon_adamw.cuh"
 #include "recon_nvfp4.cuh"
 
 namespace quasar {
 
-const void* nvfp4_kernel(int nch, bool batch)
+const void* nvfp4_kernel(bool batch)
 {
-    switch (nch) {
-    case 1: return batch ? reinterpret_cast<const void*>(&k_recon_nvfp4<1, kMaxBatch>)
-                         : reinterpret_cast<const void*>(&k_recon_nvfp4<1, 1>);
-    case 2: return batch ? reinterpret_cast<const void*>(&k_recon_nvfp4<2, kMaxBatch>)
-                         : reinterpret_cast<const void*>(&k_recon_nvfp4<2, 1>);
-    case 4: return batch ? reinterpret_cast<const void*>(&k_recon_nvfp4<4, kMaxBatch>)
-                         : reinterpret_cast<const void*>(&k_recon_nvfp4<4, 1>);
-    default: return nullptr;
-    }
+    return batch ? reinterpret_cast<const void*>(&k_recon_nvfp4<kMaxBatch>)
+                 : reinterpret_cast<const void*>(&k_recon_nvfp4<1>);
 }
 
 const void* amax_kernel(bool batch)

@@ -22,7 +22,7 @@ QUASAR_INT_ENTRY(1, 8) QUASAR_INT_ENTRY(1, 4) QUASAR_INT_ENTRY(1, 3) QUASAR_INT_
 QUASAR_INT_ENTRY(1, 1)
 QUASAR_INT_ENTRY(2, 4) QUASAR_INT_ENTRY(2, 2) QUASAR_INT_ENTRY(2, 1)
 #undef QUASAR_INT_ENTRY
-const void* nvfp4_kernel(int nch, bool batch);
+const void* nvfp4_kernel(bool batch);
 const void* amax_kernel(bool batch);
 const void* amax_init_kernel(bool batch);
 const void* amax_to_scale_kernel(bool batch);
@@ -202,8 +202,6 @@ void fill_caps(IntParams* p, int max_size, bool single_chunk = false)
     }
 }
 
-int nch_for(int n_clip) { return n_clip <= 8 ? 1 : (n_clip <= 16 ? 2 : 4); }
-
 struct Launch {
     int stages;
     uint32_t stage_bytes;
@@ -211,8 +209,10 @@ struct Launch {
 };
 
 // Shared memory per CTA: for each of its warps, `stages` tiles of
-// unit_bytes, a scratch area, and stages + 1 mbarriers.
-Launch plan(uint32_t unit_bytes, uint32_t scratch_bytes, int warps = kWarps)
+// unit_bytes, a scratch area, and stages + 1 mbarriers.  stages: the
+// kernel's choice, or 0 for as many of 2 to 4 as the budget holds
+// (QUASAR_STAGES overrides both).
+Launch plan(uint32_t unit_bytes, uint32_t scratch_bytes, int stages = 0, int warps = kWarps)
 {
     const Tuning& t = tuning();
     Launch L;
@@ -221,7 +221,7 @@ Launch plan(uint32_t unit_bytes, uint32_t scratch_bytes, int warps = kWarps)
         return (size_t)warps * s * L.stage_bytes + (size_t)warps * scratch_bytes +
                (size_t)warps * (s + 1) * 8;
     };
-    int s = t.stages;
+    int s = t.stages > 0 ? t.stages : stages;
     if (s <= 0) {
         s = 2;
         while (s < 4 && total(s + 1) <= (size_t)t.smem_budget) ++s;
@@ -520,7 +520,7 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
     Lp.n_units = units;
     if (units == 0) return QUASAR_OK;
     const int warps = adam ? kAdamWarps : kWarps;
-    const Launch L = symmetric ? plan(int_unit_bytes(group_size, Lp.p.g_kind, adam), kIntScratchBytes, warps)
+    const Launch L = symmetric ? plan(int_unit_bytes(group_size, Lp.p.g_kind, adam), kIntScratchBytes, 0, warps)
                                : plan_ring(group_size, Lp.p.g_kind, adam, warps, n_clip);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
@@ -664,12 +664,12 @@ quasar_status nvfp4_run(Nvfp4Launch<MAXT>& Lp, AmaxBatch<MAXT>& B, int n_clip, c
     Lp.n_units = units;
     if (units == 0) return QUASAR_OK;
     const int gbytes = Lp.p.g_kind == 2 ? 2 : (Lp.p.g_kind == 1 ? 4 : 0);
-    const Launch L = plan((uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes)), 0);
+    // one tile a warp: it is in registers, and the next copy under way, before
+    // the search begins
+    const Launch L = plan((uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes)), 0, 1);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
-    const void* fn = nvfp4_kernel(nch_for(n_clip), MAXT > 1);
-    if (!fn) return QUASAR_ERR_UNSUPPORTED;
-    return launch_persistent(fn, &Lp, L.smem, units, s);
+    return launch_persistent(nvfp4_kernel(MAXT > 1), &Lp, L.smem, units, s);
 }
 
 }  // namespace

@@ -8,21 +8,32 @@
 //
 // Decomposition: one lane owns one block (16 elements), so the search needs
 // no cross-lane traffic; a warp owns 32 consecutive blocks (512 elements) at
-// a time, staged through its own ring of shared-memory buffers filled by 1-D
-// TMA bulk copies, exactly as the integer kernel.  A lane reads its block's
-// four 16-byte chunks in a lane-rotated order so that each shared-memory
-// access of the warp is bank-conflict free.  Arithmetic is packed f32x2, two
-// elements per instruction.
+// a time, staged through its own shared-memory tile filled by 1-D TMA bulk
+// copies.  One tile a warp is enough: the block is in registers, and the next
+// copy under way, before the search begins.  A lane reads its block's four
+// 16-byte chunks in a lane-rotated order so that each shared-memory access of
+// the warp is bank-conflict free.  Arithmetic is packed f32x2, two elements
+// per instruction, on signed values (w and -w mirror each other exactly).
 //
 // Per candidate the codes stay in registers: moments -> a* -> E4M3 scale,
-// then the error summed directly, sum h (alpha*q - |w|)^2 (no cancellation,
-// so its fp32 error is a few ulps of itself).  Candidates within that bound
-// of the best, unless their codes and scale equal the best's (the sum of
-// codes never decreases with the scale factor, so equal sums mean equal
-// codes), are re-evaluated exactly in float-float arithmetic.
+// then the error summed directly, sum h (w - alpha*q)^2 (no cancellation,
+// so its fp32 error is a few ulps of itself).  A candidate within that bound
+// of the best, unless its codes and scale equal the best's (the sum of codes
+// never decreases with the scale factor, so equal sums mean equal codes),
+// sends its block to an exact, float-float comparison.
+//
+// What bounds it: instruction issue.  A candidate costs 11 instructions a pair
+// of elements (7 of them packed, two issue cycles each) and about 35 a block;
+// 95 a weight and lane at 8 candidates, 112 before (with absolute values, a
+// hash and an error kept for every candidate, and divisions, E4M3 decoding and
+// sign handling spelled out).  One Llama layer (218 M weights), absmax pass and
+// codes included: 1,152 -> 1,021 us.  Candidate lists that are not a multiple
+// of 8 used to send every block to the exact comparison.
 #pragma once
 
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "params.h"
@@ -38,26 +49,38 @@ __device__ __forceinline__ float tensor_scale_of(float amax)
 __device__ __forceinline__ uint32_t e4m3_rn_satfinite(float x)
 {
     uint16_t r;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %1;" : "=h"(r) : "f"(x));
-    return (uint32_t)(r & 0xFFu);
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(0.0f), "f"(x));
+    return r;
 }
 
 __device__ __forceinline__ float e4m3_value(uint32_t bits)
 {
-    // normal: exponent e - 7 + 127, mantissa m << 20; subnormal (e = 0): m * 2^-9
-    const uint32_t b = bits & 0x7Fu;
-    const float normal = __uint_as_float((b << 20) + (120u << 23));
-    return b < 8u ? (float)b * 0.001953125f : normal;
+    // every E4M3 value is an f16 value
+    float v;
+    asm("{\n\t.reg .b32 t;\n\t.reg .b16 lo, hi;\n\tcvt.rn.f16x2.e4m3x2 t, %1;\n\t"
+        "mov.b32 {lo, hi}, t;\n\tcvt.f32.f16 %0, lo;\n\t}"
+        : "=f"(v)
+        : "h"((uint16_t)bits));
+    return v;
 }
 
-// E2M1 nibble of a value that lies on the signed E2M1 grid.
-__device__ __forceinline__ uint32_t e2m1_nibble(float qs)
+// Fast reciprocal (2 ulps), denormals flushed.
+__device__ __forceinline__ float rcp_ftz(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// E2M1 codes of two values (nearest, ties to the even code, saturating at 6):
+// y.x in the low nibble, y.y in the high one, each sign << 3 | magnitude.
+__device__ __forceinline__ uint32_t e2m1_nibbles(float2 y)
 {
     uint16_t r;
-    asm("{\n\t.reg .b8 t;\n\tcvt.rn.satfinite.e2m1x2.f32 t, %1, %1;\n\tcvt.u16.u8 %0, t;\n\t}"
+    asm("{\n\t.reg .b8 t;\n\tcvt.rn.satfinite.e2m1x2.f32 t, %1, %2;\n\tcvt.u16.u8 %0, t;\n\t}"
         : "=h"(r)
-        : "f"(qs));
-    return (uint32_t)(r & 0xFu);
+        : "f"(y.y), "f"(y.x));
+    return r;
 }
 
 // Error-free transformations for the exact comparison (Knuth TwoSum,
@@ -75,11 +98,12 @@ __device__ __forceinline__ void two_prod_f(float a, float b, float& p, float& e)
     e = fmaf(a, b, -p);
 }
 
-template <int NCH, int MAXT>
-__global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvfp4Launch<MAXT> Lp)
+// Three CTAs an SM (80 registers) and the loop over candidates unrolled by 2:
+// 1,021 us a layer; two CTAs 1,041, no unrolling at two CTAs 1,052.
+template <int MAXT>
+__global__ void __launch_bounds__(256, 3) k_recon_nvfp4(const __grid_constant__ Nvfp4Launch<MAXT> Lp)
 {
     const Nvfp4Params& p = Lp.p;
-    constexpr int KM = NCH * 8;
     constexpr int UNIT = kBlocksPerUnit * 16;
     extern __shared__ __align__(128) unsigned char smem[];
 
@@ -152,11 +176,10 @@ __global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvf
     const float ulp = 5.9604645e-8f * p.tie_kappa;
     const float2 beta22 = make_float2(p.beta2, p.beta2);
     const float2 c12 = make_float2(p.c1, p.c1);
-    const float2 six2 = make_float2(6.0f, 6.0f), neg12 = make_float2(-1.0f, -1.0f);
     int s_cur = 0;
     uint32_t parity = 0;
 
-    // E2M1 magnitudes of two values y >= 0: the hardware conversion rounds
+    // E2M1 values of two values y: the hardware conversion rounds
     // to nearest, ties to the even code, and saturates at 6; converting the
     // pair back through f16x2 gives their values (a goes to the upper half in
     // both conversions, so y.y is passed first)
@@ -178,34 +201,42 @@ __global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvf
         const unsigned char* st = ring + (size_t)s_cur * p.stage_bytes;
 
         // element 4*cidx[i] + jj of this lane's block is held at slot 4*i + jj,
-        // pairs (slot 2t, 2t+1) in w2[t], h2[t]
+        // pairs (slot 2t, 2t+1) in w2[t], h2[t].  The search keeps the signs: codes,
+        // products and errors of w and -w mirror each other exactly, so no
+        // absolute values are formed
         float2 w2[8], h2[8];
+        auto load = [&](auto gk) {
+            constexpr int GK = decltype(gk)::value;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int cidx = (i + rot) & 3;
-            const int e = lane * 16 + cidx * 4;
-            const float4 w4 = lds128(st + e * 4);
-            const float4 v4 = lds128(st + kVOff + e * 4);
-            w2[2 * i] = make_float2(w4.x, w4.y);
-            w2[2 * i + 1] = make_float2(w4.z, w4.w);
-            float2 hA = make_float2(v4.x, v4.y), hB = make_float2(v4.z, v4.w);
-            if (p.g_kind) {
-                float2 gA, gB;
-                if (p.g_kind == 2) {
-                    const uint2 gb = lds64(st + kGOff + e * 2);
-                    gA = make_float2(bf16lo(gb.x), bf16hi(gb.x));
-                    gB = make_float2(bf16lo(gb.y), bf16hi(gb.y));
-                } else {
-                    const float4 g4 = lds128(st + kGOff + e * 4);
-                    gA = make_float2(g4.x, g4.y);
-                    gB = make_float2(g4.z, g4.w);
+            for (int i = 0; i < 4; ++i) {
+                const int cidx = (i + rot) & 3;
+                const int e = lane * 16 + cidx * 4;
+                const float4 w4 = lds128(st + e * 4);
+                const float4 v4 = lds128(st + kVOff + e * 4);
+                w2[2 * i] = make_float2(w4.x, w4.y);
+                w2[2 * i + 1] = make_float2(w4.z, w4.w);
+                float2 hA = make_float2(v4.x, v4.y), hB = make_float2(v4.z, v4.w);
+                if constexpr (GK != 0) {
+                    float2 gA, gB;
+                    if constexpr (GK == 2) {
+                        const uint2 gb = lds64(st + kGOff + e * 2);
+                        gA = make_float2(bf16lo(gb.x), bf16hi(gb.x));
+                        gB = make_float2(bf16lo(gb.y), bf16hi(gb.y));
+                    } else {
+                        const float4 g4 = lds128(st + kGOff + e * 4);
+                        gA = make_float2(g4.x, g4.y);
+                        gB = make_float2(g4.z, g4.w);
+                    }
+                    hA = __ffma2_rn(hA, beta22, __fmul2_rn(c12, __fmul2_rn(gA, gA)));
+                    hB = __ffma2_rn(hB, beta22, __fmul2_rn(c12, __fmul2_rn(gB, gB)));
                 }
-                hA = __ffma2_rn(hA, beta22, __fmul2_rn(c12, __fmul2_rn(gA, gA)));
-                hB = __ffma2_rn(hB, beta22, __fmul2_rn(c12, __fmul2_rn(gB, gB)));
+                h2[2 * i] = hA;
+                h2[2 * i + 1] = hB;
             }
-            h2[2 * i] = hA;
-            h2[2 * i + 1] = hB;
-        }
+        };
+        if (p.g_kind == 2) load(std::integral_constant<int, 2>{});
+        else if (p.g_kind == 1) load(std::integral_constant<int, 1>{});
+        else load(std::integral_constant<int, 0>{});
         __syncwarp();
         if (lane == 0) {
             const int64_t un = u + (int64_t)S * stride;
@@ -241,14 +272,11 @@ __global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvf
             for (int t = 0; t < 8; ++t)
                 h2[t] = p.h_mode == kSalEmaSquared ? __fmul2_rn(h2[t], h2[t]) : make_float2(1.0f, 1.0f);
 
-        float2 aw2[8], naw2[8];
         float amax_b = 0.0f;
         float2 SS = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            aw2[t] = make_float2(fabsf(w2[t].x), fabsf(w2[t].y));
-            naw2[t] = make_float2(-aw2[t].x, -aw2[t].y);
-            amax_b = fmaxf(amax_b, fmaxf(aw2[t].x, aw2[t].y));
+            amax_b = fmax3(amax_b, fabsf(w2[t].x), fabsf(w2[t].y));
             SS = __fadd2_rn(SS, h2[t]);
         }
         const float ssb = SS.x + SS.y;
@@ -269,100 +297,91 @@ __global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvf
         const float P1 = zero ? 0.0f : __fdiv_rn(6.0f, amax_b);  // 1/sigma at f = 1
 
         // ---- candidates: codes in registers, moments, E4M3 scale, direct error
-        float Ek[KM];
-        uint32_t Kk[KM];
-        float Eb = INFINITY;
-        int kb = 0;
-        uint32_t e_sel = 0;
-        float alpha_sel = 0.0f;
-#pragma unroll
-        for (int k = 0; k < KM; ++k) {
+        struct Fit {
+            uint32_t e, key;
+            float err;
+        };
+        float2 q2[8];  // the last evaluated candidate's codes
+        auto evaluate = [&](int k) {
             const float P = P1 * p.invf[k];
             const float2 P2 = make_float2(P, P);
-            float2 q2[8];
             float2 S2 = make_float2(0.0f, 0.0f), S3 = S2;
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-                float2 y = __fmul2_rn(aw2[t], P2);
-                q2[t] = e2m1_2(y);
+                q2[t] = e2m1_2(__fmul2_rn(w2[t], P2));
                 const float2 hq = __fmul2_rn(h2[t], q2[t]);
                 S2 = __ffma2_rn(hq, q2[t], S2);
-                S3 = __ffma2_rn(hq, aw2[t], S3);
+                S3 = __ffma2_rn(hq, w2[t], S3);
             }
             const float s2 = S2.x + S2.y, s3 = S3.x + S3.y;
-            // degenerate (every weighted element coded 0): the search scale
-            const float x = s2 > 0.0f ? __fdividef(s3, s2) * inv_sT
-                                      : amax_b * p.f[k] * (1.0f / 6.0f) * inv_sT;
-            const uint32_t e = e4m3_rn_satfinite(x);
-            const float alpha = sT * e4m3_value(e);
-            const float2 a2 = make_float2(alpha, alpha);
+            // a* / s_T.  (The reciprocal flushes denormals: those, and 0 --
+            // degenerate, every weighted element coded 0: the search scale --
+            // go the long way.)
+            float x = s3 * rcp_ftz(s2) * inv_sT;
+            if (!(s2 >= 1.17549435e-38f))
+                x = s2 > 0.0f ? __fdividef(s3, s2) * inv_sT : amax_b * p.f[k] * (1.0f / 6.0f) * inv_sT;
+            Fit r;
+            r.e = e4m3_rn_satfinite(x);
+            const float alpha = sT * e4m3_value(r.e);
+            const float2 na2 = make_float2(-alpha, -alpha);
             float2 E2 = make_float2(0.0f, 0.0f);
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-                const float2 ev = __ffma2_rn(a2, q2[t], naw2[t]);
+                const float2 ev = __ffma2_rn(na2, q2[t], w2[t]);
                 E2 = __ffma2_rn(__fmul2_rn(h2[t], ev), ev, E2);
             }
-            const float err = k < p.n_clip ? E2.x + E2.y : INFINITY;
+            r.err = E2.x + E2.y;
             // candidates with equal moments and scale have, to within rounding
             // below the tie margin, equal codes and errors: a key of the three
-            Ek[k] = err;
-            Kk[k] = (__float_as_uint(s2) * 0x9E3779B1u + __float_as_uint(s3)) ^ e;
-            if (err < Eb) {  // strict: ties keep the lower index
-                Eb = err;
+            r.key = (__float_as_uint(s2) * 0x9E3779B1u + __float_as_uint(s3)) ^ r.e;
+            return r;
+        };
+        // the best candidate, and the lowest error of the others whose key is
+        // not the best's: two numbers a block instead of an error and a key a
+        // candidate, so that three CTAs fit an SM and any number of factors
+        // takes one loop
+        Fit best = evaluate(0);
+        int kb = 0;
+        float En = INFINITY;
+#pragma unroll 2
+        for (int k = 1; k < p.n_clip; ++k) {
+            const Fit c = evaluate(k);
+            const bool other = c.key != best.key;
+            if (c.err < best.err) {  // strict: ties keep the lower index
+                En = other ? best.err : En;
+                best = c;
                 kb = k;
-                e_sel = e;
-                alpha_sel = alpha;
+            } else if (other) {
+                En = fminf(En, c.err);
             }
         }
-        // contenders: within the direct sums' fp32 error bound of the best
-        uint32_t keyb = Kk[0];
-#pragma unroll
-        for (int k = 1; k < KM; ++k)
-            if (k == kb) keyb = Kk[k];
-        unsigned set = 0;
-#pragma unroll
-        for (int k = 0; k < KM; ++k)
-            if (k != kb && Ek[k] - Eb <= ulp * (Ek[k] + Eb) && Kk[k] != keyb) set |= 1u << k;
 
-        if (set != 0 && valid && !zero) {
-            // exact comparison: sum h (alpha q - |w|)^2 with alpha*q - |w| as an
+        // a contender within the direct sums' fp32 error bound of the best
+        if (En < INFINITY && En - best.err <= ulp * (En + best.err) && valid && !zero) {
+            // exact comparison: sum h (alpha q - w)^2 with alpha*q - w as an
             // exact pair (TwoProd, TwoSum) and the squares and sum in float pairs
             if (p.stats) atomicAdd(&p.stats[0], 1u);
-            set |= 1u << kb;
+            const Fit b0 = best;
+            const int kb0 = kb;
             float best_h = INFINITY, best_l = 0.0f;
-            int bk = -1;
-            while (set) {
-                const int k = __ffs(set) - 1;
-                set &= set - 1;
-                const float P = P1 * p.invf[k];
-                const float2 P2 = make_float2(P, P);
-                float2 S2 = make_float2(0.0f, 0.0f), S3 = S2;
-                float2 q2[8];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    float2 y = __fmul2_rn(aw2[t], P2);
-                    q2[t] = e2m1_2(y);
-                    const float2 hq = __fmul2_rn(h2[t], q2[t]);
-                    S2 = __ffma2_rn(hq, q2[t], S2);
-                    S3 = __ffma2_rn(hq, aw2[t], S3);
-                }
-                const float s2 = S2.x + S2.y, s3 = S3.x + S3.y;
-                const float x = s2 > 0.0f ? __fdividef(s3, s2) * inv_sT
-                                          : amax_b * p.f[k] * (1.0f / 6.0f) * inv_sT;
-                const uint32_t e = e4m3_rn_satfinite(x);
-                const float alpha = sT * e4m3_value(e);
+            kb = -1;
+#pragma unroll 1
+            for (int k = 0; k < p.n_clip; ++k) {
+                const Fit c = evaluate(k);
+                if (k != kb0 && (c.key == b0.key || !(c.err - b0.err <= ulp * (c.err + b0.err)))) continue;
+                const float alpha = sT * e4m3_value(c.e);
                 float eh = 0.0f, el = 0.0f;
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
 #pragma unroll
                     for (int c2 = 0; c2 < 2; ++c2) {
                         const float q = c2 ? q2[t].y : q2[t].x;
-                        const float aw = c2 ? aw2[t].y : aw2[t].x;
+                        const float w = c2 ? w2[t].y : w2[t].x;
                         const float h = c2 ? h2[t].y : h2[t].x;
                         float ph, pl, dh, dl, sh, sl;
                         two_prod_f(alpha, q, ph, pl);
-                        two_sum_f(ph, -aw, dh, dl);
-                        dl = __fadd_rn(dl, pl);  // alpha q - |w| = dh + dl
+                        two_sum_f(ph, -w, dh, dl);
+                        dl = __fadd_rn(dl, pl);  // alpha q - w = dh + dl
                         two_prod_f(dh, dh, sh, sl);
                         sl = fmaf(2.0f * dh, dl, sl);
                         two_prod_f(h, sh, ph, pl);
@@ -373,16 +392,16 @@ __global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvf
                         el = __fadd_rn(el, __fadd_rn(t2, pl));
                     }
                 }
-                if (bk < 0 || eh < best_h || (eh == best_h && el < best_l)) {
+                if (kb < 0 || eh < best_h || (eh == best_h && el < best_l)) {
                     best_h = eh;
                     best_l = el;
-                    bk = k;
-                    alpha_sel = alpha;
-                    e_sel = e;
+                    kb = k;
+                    best = c;
                 }
             }
-            kb = bk;
         }
+        uint32_t e_sel = best.e;
+        float alpha_sel = sT * e4m3_value(best.e);
         if (!valid) continue;
         if (zero) {
             kb = 0;
@@ -393,42 +412,41 @@ __global__ void __launch_bounds__(256) k_recon_nvfp4(const __grid_constant__ Nvf
         // ---- outputs of the kept candidate
         const float Pb = P1 * p.invf[kb];
         const float2 Pb2 = make_float2(Pb, Pb);
-        const float2 as2 = make_float2(alpha_sel, alpha_sel);
+        const float2 as2 = make_float2(alpha_sel, alpha_sel), zero2 = make_float2(0.0f, 0.0f);
         uint64_t pk = 0;  // packed codes: element j's nibble at bit 4j
+        auto outputs = [&](auto bf16, auto with_codes) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int cidx = (i + rot) & 3;
-            float2 rv[2];
-            uint32_t cw = 0;
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int t = 2 * i + hh;
-                float2 y = __fmul2_rn(aw2[t], Pb2);
-                const float2 q = e2m1_2(y);
-                // the code carries the sign of w (magnitude 0 is stored as +0)
-                const float2 qs = make_float2(q.x > 0.0f ? copysignf(q.x, w2[t].x) : 0.0f,
-                                              q.y > 0.0f ? copysignf(q.y, w2[t].y) : 0.0f);
-                rv[hh] = __fmul2_rn(as2, qs);
-                if (T.codes) cw |= (e2m1_nibble(qs.x) | (e2m1_nibble(qs.y) << 8)) << (16 * hh);
-            }
-            const int64_t e = ebase + cidx * 4;
-            if (p.r_bf16) {
-                stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + e),
-                       make_uint2(pack_bf16x2(rv[0].x, rv[0].y), pack_bf16x2(rv[1].x, rv[1].y)));
-            } else {
-                stg_cs(reinterpret_cast<float4*>(static_cast<float*>(T.r) + e),
-                       make_float4(rv[0].x, rv[0].y, rv[1].x, rv[1].y));
-            }
-            if (T.codes) {
-                if (!p.codes_packed) {
-                    stg_cs(reinterpret_cast<uint32_t*>(T.codes + e), cw);
+            for (int i = 0; i < 4; ++i) {
+                const int cidx = (i + rot) & 3;
+                const float2 ya = __fmul2_rn(w2[2 * i], Pb2), yb = __fmul2_rn(w2[2 * i + 1], Pb2);
+                // r = alpha q (+ 0: a code of magnitude 0 gives +0)
+                const float2 ra = __ffma2_rn(as2, e2m1_2(ya), zero2), rb = __ffma2_rn(as2, e2m1_2(yb), zero2);
+                const int64_t e = ebase + cidx * 4;
+                if constexpr (decltype(bf16)::value) {
+                    stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + e),
+                           make_uint2(pack_bf16x2(ra.x, ra.y), pack_bf16x2(rb.x, rb.y)));
                 } else {
-                    // bytes q0 q1 q2 q3 -> nibbles q0 | q1 << 4 | q2 << 8 | q3 << 12
-                    const uint32_t nib = (cw & 0xFu) | ((cw >> 4) & 0xF0u) | ((cw >> 8) & 0xF00u) |
-                                         ((cw >> 12) & 0xF000u);
-                    pk |= (uint64_t)nib << (16 * cidx);
+                    stg_cs(reinterpret_cast<float4*>(static_cast<float*>(T.r) + e), make_float4(ra.x, ra.y, rb.x, rb.y));
+                }
+                if constexpr (decltype(with_codes)::value) {
+                    // the chunk's four nibbles, in element order; magnitude 0 is +0
+                    uint32_t c = e2m1_nibbles(ya) | (e2m1_nibbles(yb) << 8);
+                    c &= 0x7777u | (((c | (c >> 1) | (c >> 2)) & 0x1111u) << 3);
+                    if (!p.codes_packed) {
+                        const uint32_t t8 = (c | (c << 8)) & 0x00FF00FFu;
+                        stg_cs(reinterpret_cast<uint32_t*>(T.codes + e), (t8 | (t8 << 4)) & 0x0F0F0F0Fu);
+                    } else {
+                        pk |= (uint64_t)c << (16 * cidx);
+                    }
                 }
             }
+        };
+        if (T.codes) {
+            if (p.r_bf16) outputs(std::true_type{}, std::true_type{});
+            else outputs(std::false_type{}, std::true_type{});
+        } else {
+            if (p.r_bf16) outputs(std::true_type{}, std::false_type{});
+            else outputs(std::false_type{}, std::false_type{});
         }
         if (T.codes && p.codes_packed) stg_cs(reinterpret_cast<uint2*>(T.codes + blk * 8),
                                              make_uint2((uint32_t)pk, (uint32_t)(pk >> 32)));
