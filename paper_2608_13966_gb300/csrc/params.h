@@ -144,16 +144,14 @@ struct Nvfp4Params {
 constexpr int kLutRows = 8;
 constexpr int kLutCols = 64;
 constexpr int kLutBlock = kLutRows * kLutCols;
-// Per-warp scratch of the LUT kernel: the lists of the elements that reach
-// level 1 (|d| and h, both signs: at most kLutListCap of them a round, each
-// sign padded to a multiple of 8), per candidate its table (8 bytes), error,
-// error bound and which entries' roundings were undecided, then a decoded
-// table and the block's sums.
-constexpr int kLutListCap = 256;
-constexpr int kLutListLen = kLutListCap + 16;
+// The LUT kernel's lists of the elements that reach level 1 (|d| and h, each
+// sign padded to a multiple of 8 entries) take over the tile; per-warp scratch
+// beside it: per candidate its table (8 bytes), error, error bound and which
+// entries' roundings were undecided, then a decoded table and the block's sums.
+constexpr int kLutListLen = kLutBlock + 16;
 constexpr uint32_t kLutListBytes = 2 * kLutListLen * 4;
 constexpr uint32_t kLutCandBytes = kMaxClip * 20;
-constexpr uint32_t kLutScratchBytes = kLutListBytes + kLutCandBytes + 64;
+constexpr uint32_t kLutScratchBytes = kLutCandBytes + 64;
 
 struct LutTensor {
     const float* w;
@@ -178,9 +176,7 @@ struct LutParams {
     float c1;
     float tie_kappa;   // multiplier of the summation-depth bounds
     float invf_max;    // the largest 1/f
-    int stages;
-    uint32_t stage_bytes;
-    uint64_t timeout_ns;
+    uint32_t stage_bytes;  // a warp's tile: w, v, g, and large enough for the lists
     uint64_t force_timeout_ns;
     unsigned int* status;
     unsigned int* stats;  // optional: [0] blocks compared exactly, [1] candidates evaluated

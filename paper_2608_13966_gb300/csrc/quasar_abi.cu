@@ -963,16 +963,14 @@ quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_ten
     p.beta2 = beta2;
     p.c1 = 1.0f - beta2;
     p.tie_kappa = tuning().tie_scale;
-    p.timeout_ns = kDefaultTimeoutNs;
     p.force_timeout_ns = (uint64_t)std::max<int64_t>(0, g_force_timeout_ns.load());
     p.stats = g_stats.load();
     fill_clip(clip, n_clip, p.f, p.invf);
     p.invf_max = *std::max_element(p.invf, p.invf + n_clip);
     if ((st = status_ptr(&p.status)) != QUASAR_OK) return st;
-    const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
-    const Launch L = plan((uint32_t)(kLutBlock * (8 + gbytes)), kLutScratchBytes);
-    p.stages = L.stages;
-    p.stage_bytes = L.stage_bytes;
+    const uint32_t gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
+    p.stage_bytes = (std::max(kLutBlock * (8 + gbytes), kLutListBytes) + 127u) & ~127u;
+    const size_t smem = (size_t)kWarps * (p.stage_bytes + kLutScratchBytes);
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     for (int i0 = 0; i0 < n_tensors; i0 += kMaxBatch) {
         Lp.n_t = std::min(kMaxBatch, n_tensors - i0);
@@ -984,7 +982,7 @@ quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_ten
         }
         Lp.n_units = units;
         if (units == 0) continue;
-        if ((st = launch_persistent(lut_kernel(), &Lp, L.smem, units, s)) != QUASAR_OK) return st;
+        if ((st = launch_persistent(lut_kernel(), &Lp, smem, units, s)) != QUASAR_OK) return st;
     }
     return QUASAR_OK;
 }

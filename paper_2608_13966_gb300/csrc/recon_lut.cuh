@@ -8,18 +8,20 @@
 // the candidate with the lowest weighted error sum h (C_q - w)^2 is kept.
 //
 // One warp owns one block: lane L holds, for i = 0 .. 3, block elements
-// 128 i + 4 L .. + 3, read once from a per-warp TMA ring.  An index is a sign
-// s of d = w - c and a magnitude level m = min(floor(|d| P), 3).  For each
-// sign and threshold t = 1, 2, 3 a candidate needs the sums of h and of h |d|
-// over the elements with m >= t.  Only elements that reach level 1 for some
-// factor add to any of them, so those are compacted into two lists by sign;
-// four lanes own a candidate (eight candidates a warp) and walk the lists in
-// pairs (packed f32x2; the masks [m >= t] come from saturated adds on the
-// floor).  A pair of one sign costs 16 instructions a candidate; in registers
-// with both signs it cost 25, for all 512 elements, and the 12 sums then had
-// to be transposed across the warp (one Llama layer, 218 M weights: 2,310 us
-// before, 2,070 us with the lists).  With the block's per-sign totals the sums
-// give every index's H_j = sum h and X_j = sum h |d|.  Index j's entry is the
+// 128 i + 4 L .. + 3.  It copies those pieces itself (cp.async) into the warp's
+// tile, one block ahead, so that its own wait is all a read needs; as 24 bulk
+// copies of one row segment each, issuing a block took an eighth of the time.
+// An index is a sign s of d = w - c and a magnitude level m = min(floor(|d|
+// P), 3).  For each sign and threshold t = 1, 2, 3 a candidate needs the sums
+// of h and of h |d| over the elements with m >= t.  Only elements that reach
+// level 1 for some factor add to any of them, so those are compacted into two
+// lists by sign (in the tile, whose block is in registers by then); four lanes
+// own a candidate (eight candidates a warp) and walk the lists in pairs
+// (packed f32x2; the masks [m >= t] come from saturated adds on the floor).  A
+// pair of one sign costs 16 instructions a candidate; in registers with both
+// signs it cost 25, for all 512 elements, and the 12 sums then had to be
+// transposed across the warp.  With the block's per-sign totals the sums give
+// every index's H_j = sum h and X_j = sum h |d|.  Index j's entry is the
 // E4M3 rounding of its weighted mean c + s X_j / H_j, and the error is
 //   sum h d^2 - sum_j X_j^2 / H_j + sum_j H_j (C_j - mean_j)^2
 // (the within-index scatter plus each entry's offset from its mean).  Both
@@ -27,11 +29,19 @@
 // the bound of the best, and undecided roundings, are settled exactly
 // (float-float sums over the codes, whole warp), so indices, tables and the
 // kept candidate equal the exact computation's.
+//
+// What bounds it: instruction issue, 136 a weight and lane (263 with the sums
+// in registers).  One Llama layer (218 M weights, packed codes): 2,300 us with
+// the sums in registers, 2,070 with the lists, 1,576 with the pieces copied
+// and waited for by the lane that reads them, two-at-a-time E4M3 conversions,
+// redux for the minima and h re-read by the settling steps.
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "params.h"
@@ -58,6 +68,22 @@ __device__ __forceinline__ float e4m3_decode(uint32_t bits)
     // normal: exponent e - 7 + 127, mantissa m << 20; subnormal (e = 0): m * 2^-9
     const float mag = m < 8u ? (float)m * 0.001953125f : __uint_as_float((m << 20) + (120u << 23));
     return (bits & 0x80u) ? -mag : mag;
+}
+
+// Two E4M3 codes (a in the low byte) and their values; no -0 clean-up.
+__device__ __forceinline__ uint32_t e4m3_encode2(float a, float b)
+{
+    uint16_t r;
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(b), "f"(a));
+    return r;
+}
+
+__device__ __forceinline__ float2 e4m3_decode2(uint32_t bits)
+{
+    // every E4M3 value is an f16 value
+    uint32_t hh;
+    asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(hh) : "h"((uint16_t)bits));
+    return __half22float2(*reinterpret_cast<__half2*>(&hh));
 }
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
@@ -163,6 +189,9 @@ __device__ __forceinline__ uint32_t e4m3_round_ff(float xh, float xl)
 
 }  // namespace lut
 
+// Two CTAs an SM (128 registers): 1,639 us a layer where three (80 registers,
+// spilling) took 1,757; CTAs of 4 warps were slower at 96 registers (1,672
+// against 1,576) and at 128 (1,616).
 template <int MAXT>
 __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ LutLaunch<MAXT> Lp)
 {
@@ -173,22 +202,20 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
-    const int S = p.stages;
-    unsigned char* ring = smem + (size_t)warp * S * p.stage_bytes;
-    unsigned char* scr = smem + (size_t)nwarps * S * p.stage_bytes + (size_t)warp * kLutScratchBytes;
-    float* lst = reinterpret_cast<float*>(scr);  // |d| [kLutListLen], then h [kLutListLen]
-    uint32_t* cbook = reinterpret_cast<uint32_t*>(scr + kLutListBytes);  // [32][2]
+    // a warp's part: the tile, then the candidates' results.  Once the block is
+    // in registers, the tile holds the lists; once they are walked, the next
+    // block is copied into it.
+    unsigned char* st = smem + (size_t)warp * (p.stage_bytes + kLutScratchBytes);
+    unsigned char* scr = st + p.stage_bytes;
+    float* lst = reinterpret_cast<float*>(st);              // |d| [kLutListLen], then h [kLutListLen]
+    uint32_t* cbook = reinterpret_cast<uint32_t*>(scr);     // [32][2]
     float* cerr = reinterpret_cast<float*>(cbook + 2 * kMaxClip);       // [32]
     float* cbnd = cerr + kMaxClip;                                        // [32]
     uint32_t* camb = reinterpret_cast<uint32_t*>(cbnd + kMaxClip);      // [32]
-    float* table = reinterpret_cast<float*>(scr + kLutListBytes + kLutCandBytes);  // [8]
+    float* table = reinterpret_cast<float*>(scr + kLutCandBytes);  // [8]
     // the block's per-sign sums of h and h |d|, and sum h d^2
     float* bconst = table + 8;  // [5]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nwarps * S * p.stage_bytes +
-                                                 (size_t)nwarps * kLutScratchBytes) +
-                     warp * (S + 1);
 
-    const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
     constexpr uint32_t kVOff = kLutBlock * 4;
     constexpr uint32_t kGOff = kLutBlock * 8;
     const int K = p.n_clip;
@@ -201,55 +228,62 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     const int64_t first = (int64_t)blockIdx.x * nwarps + warp;
     const int64_t stride = (int64_t)gridDim.x * nwarps;
 
-    if (lane == 0) {
-        for (int s = 0; s <= S; ++s) mbar_init(&bars[s], 1);
-        mbar_init_fence();
-    }
-    __syncwarp();
-
-    // the 8 row segments of a block, each of w, v and g: lane 0 announces
-    // the bytes, lane r copies row r (every lane calls it)
-    auto issue = [&](int64_t u, int s) {
+    // the lane's 16 elements, in four chunks of 4: chunk i is block elements
+    // 128 i + 4 lane .. + 3, i.e. row 2 i + lane/16, columns 4 (lane % 16) ..
+    // (consecutive lanes on consecutive 16-byte pieces, in the tile and in
+    // memory); the offset of chunk 0 in the tensor
+    auto lane_offset = [&](const LutTensor& T, uint32_t b) {
+        // block row and column (a tensor holds fewer than 2^32 blocks)
+        const uint32_t nbc = (uint32_t)(T.cols / kLutCols);
+        const uint32_t brow = b / nbc;
+        return ((int64_t)brow * kLutRows + (lane >> 4)) * T.cols + (int64_t)(b - brow * nbc) * kLutCols +
+               (lane & 15) * 4;
+    };
+    // Copy a block into the tile: every lane copies the pieces that it will
+    // read itself, so its own wait is all that orders them.  (24 row segments
+    // a block as bulk copies took an eighth of the kernel to issue.)
+    auto issue = [&](int64_t u) {
         int tj = ti;
         tensor_of(u, tj);
         const LutTensor& T = Lp.t[tj];
-        // block row and column (a tensor holds fewer than 2^32 blocks)
-        const uint32_t b = (uint32_t)(u - T.unit0);
-        const uint32_t nbc = (uint32_t)(T.cols / kLutCols);
-        const uint32_t brow = b / nbc;
-        const int64_t base = (int64_t)brow * kLutRows * T.cols + (int64_t)(b - brow * nbc) * kLutCols;
-        unsigned char* st = ring + (size_t)s * p.stage_bytes;
-        if (lane == 0) mbar_arrive_expect_tx(&bars[s], (uint32_t)kLutBlock * (8u + (uint32_t)gbytes));
-        __syncwarp();
-        if (lane < kLutRows) {
-            const int r = lane;
-            const int64_t off = base + r * T.cols;
-            bulk_g2s(st + r * kLutCols * 4, T.w + off, kLutCols * 4, &bars[s]);
-            bulk_g2s(st + kVOff + r * kLutCols * 4, T.v + off, kLutCols * 4, &bars[s]);
-            if (gbytes)
-                bulk_g2s(st + kGOff + r * kLutCols * gbytes,
-                         static_cast<const unsigned char*>(T.g) + off * gbytes,
-                         (uint32_t)(kLutCols * gbytes), &bars[s]);
+        const int64_t off = lane_offset(T, (uint32_t)(u - T.unit0)), step = 2 * T.cols;
+        const uint32_t d = smem_u32(st) + lane * 16;
+        const float* w = T.w + off;
+        const float* v = T.v + off;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            cp_async16(d + i * 512, w + i * step);
+            cp_async16(d + kVOff + i * 512, v + i * step);
         }
-    };
-    auto fail = [&](int64_t it) {
-        if (lane == 0) record_timeout(p.status);
-        for (int j = 0; j < S; ++j) {
-            const int64_t u = first + (it + j) * stride;
-            if (u >= n_units) break;
-            mbar_wait_bounded(&bars[(it + j) % S], (uint32_t)(((it + j) / S) & 1), p.timeout_ns);
+        if (p.g_kind == 2) {
+            const uint32_t dg = smem_u32(st) + kGOff + lane * 8;
+            const __nv_bfloat16* g = static_cast<const __nv_bfloat16*>(T.g) + off;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async8(dg + i * 256, g + i * step);
+        } else if (p.g_kind == 1) {
+            const float* g = static_cast<const float*>(T.g) + off;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async16(d + kGOff + i * 512, g + i * step);
         }
     };
 
-    for (int s = 0; s < S; ++s) {
-        const int64_t u = first + s * stride;
-        if (u < n_units) issue(u, s);
-    }
+    if (first < n_units) issue(first);
     if (p.force_timeout_ns && blockIdx.x == 0 && warp == 0) {
-        if (!warp_wait_bounded(&bars[S], 0, p.force_timeout_ns)) {
-            fail(0);
+        // Failure-path hook: a barrier nothing ever arrives on.
+        // (in warp 0's candidate results, not in use yet)
+        uint64_t* bar = reinterpret_cast<uint64_t*>(scr);
+        if (lane == 0) {
+            mbar_init(bar, 1);
+            mbar_init_fence();
+        }
+        __syncwarp();
+        if (!warp_wait_bounded(bar, 0, p.force_timeout_ns)) {
+            if (lane == 0) record_timeout(p.status);
+            cp_async_wait_all();
             return;
         }
+        __syncwarp();
+        if (lane == 0) mbar_inval(bar);
     }
 
     const float2 beta22 = make_float2(p.beta2, p.beta2);
@@ -258,68 +292,50 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     // the factor of the lane's candidate of the first eight (the one a lane's
     // quad evaluates)
     const float invf0 = p.invf[min(lane >> 2, K - 1)];
-    int s_cur = 0;
-    uint32_t parity = 0;
 
-    for (int64_t it = 0;; ++it) {
-        const int64_t u = first + it * stride;
-        if (u >= n_units) break;
-        if (!warp_wait_bounded(&bars[s_cur], parity, p.timeout_ns)) {
-            fail(it);
-            return;
-        }
-        const unsigned char* st = ring + (size_t)s_cur * p.stage_bytes;
+    for (int64_t u = first; u < n_units; u += stride) {
+        cp_async_wait_all();
         tensor_of(u, ti);
         const LutTensor& T = Lp.t[ti];
         const uint32_t b = (uint32_t)(u - T.unit0);
-        const uint32_t nbc = (uint32_t)(T.cols / kLutCols);
-        const uint32_t brow = b / nbc;
-        // the lane's 16 elements, in four chunks of 4: chunk i is block elements
-        // 128 i + 4 lane .. + 3, i.e. row 2 i + lane/16, columns 4 (lane % 16) ..
-        // (consecutive lanes on consecutive 16-byte pieces, in the tile and in
-        // memory)
-        const int64_t gofs = ((int64_t)brow * kLutRows + (lane >> 4)) * T.cols +
-                             (int64_t)(b - brow * nbc) * kLutCols + (lane & 15) * 4;
+        const int64_t gofs = lane_offset(T, b);
         const int64_t gstep = 2 * T.cols;  // from one chunk of the lane to the next
 
         // ---- pass A: w, the saliency EMA (v' out), the fit's saliency h
         float2 w2[8], h2[8];
+        auto pass_a = [&](auto gk) {
+            constexpr int GK = decltype(gk)::value;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int e = i * 128 + lane * 4;
-            const float4 w4 = lds128(st + e * 4);
-            const float4 v4 = lds128(st + kVOff + e * 4);
-            w2[2 * i] = make_float2(w4.x, w4.y);
-            w2[2 * i + 1] = make_float2(w4.z, w4.w);
-            float2 hA = make_float2(v4.x, v4.y), hB = make_float2(v4.z, v4.w);
-            if (p.g_kind) {
-                float2 gA, gB;
-                if (p.g_kind == 2) {
-                    const uint2 gb = lds64(st + kGOff + e * 2);
-                    gA = make_float2(bf16lo(gb.x), bf16hi(gb.x));
-                    gB = make_float2(bf16lo(gb.y), bf16hi(gb.y));
-                } else {
-                    const float4 g4 = lds128(st + kGOff + e * 4);
-                    gA = make_float2(g4.x, g4.y);
-                    gB = make_float2(g4.z, g4.w);
+            for (int i = 0; i < 4; ++i) {
+                const int e = i * 128 + lane * 4;
+                const float4 w4 = lds128(st + e * 4);
+                const float4 v4 = lds128(st + kVOff + e * 4);
+                w2[2 * i] = make_float2(w4.x, w4.y);
+                w2[2 * i + 1] = make_float2(w4.z, w4.w);
+                float2 hA = make_float2(v4.x, v4.y), hB = make_float2(v4.z, v4.w);
+                if constexpr (GK != 0) {
+                    float2 gA, gB;
+                    if constexpr (GK == 2) {
+                        const uint2 gb = lds64(st + kGOff + e * 2);
+                        gA = make_float2(bf16lo(gb.x), bf16hi(gb.x));
+                        gB = make_float2(bf16lo(gb.y), bf16hi(gb.y));
+                    } else {
+                        const float4 g4 = lds128(st + kGOff + e * 4);
+                        gA = make_float2(g4.x, g4.y);
+                        gB = make_float2(g4.z, g4.w);
+                    }
+                    hA = __ffma2_rn(hA, beta22, __fmul2_rn(c12, __fmul2_rn(gA, gA)));
+                    hB = __ffma2_rn(hB, beta22, __fmul2_rn(c12, __fmul2_rn(gB, gB)));
+                    stg_cs(reinterpret_cast<float4*>(T.v + gofs + i * gstep), make_float4(hA.x, hA.y, hB.x, hB.y));
                 }
-                hA = __ffma2_rn(hA, beta22, __fmul2_rn(c12, __fmul2_rn(gA, gA)));
-                hB = __ffma2_rn(hB, beta22, __fmul2_rn(c12, __fmul2_rn(gB, gB)));
-                stg_cs(reinterpret_cast<float4*>(T.v + gofs + i * gstep), make_float4(hA.x, hA.y, hB.x, hB.y));
+                h2[2 * i] = hA;
+                h2[2 * i + 1] = hB;
             }
-            h2[2 * i] = hA;
-            h2[2 * i + 1] = hB;
-        }
-        // the block is in registers: release the stage
-        __syncwarp();
-        {
-            const int64_t un = u + (int64_t)S * stride;
-            if (un < n_units) issue(un, s_cur);
-        }
-        if (++s_cur == S) {
-            s_cur = 0;
-            parity ^= 1u;
-        }
+        };
+        if (p.g_kind == 2) pass_a(std::integral_constant<int, 2>{});
+        else if (p.g_kind == 1) pass_a(std::integral_constant<int, 1>{});
+        else pass_a(std::integral_constant<int, 0>{});
+        __syncwarp();  // the tile becomes the lists
         if (p.h_mode != kSalEma)
 #pragma unroll
             for (int t = 0; t < 8; ++t)
@@ -335,7 +351,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         }
         mn = lanes_min(mn, 0xffffffffu);
         mx = lanes_max(mx, 0xffffffffu);
-        if (!__any_sync(0xffffffffu, any_h))  // all saliencies zero: h = 1
+        const bool h_one = !__any_sync(0xffffffffu, any_h);
+        if (h_one)  // all saliencies zero: h = 1
 #pragma unroll
             for (int t = 0; t < 8; ++t) h2[t] = make_float2(1.0f, 1.0f);
         const float range = mx - mn;
@@ -360,17 +377,13 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 negm |= (sx & (1u << (2 * t))) | (sy & (2u << (2 * t)));
                 ad2[t] = make_float2(fabsf(d.x), fabsf(d.y));
                 const float2 hd = __fmul2_rn(h2[t], ad2[t]);
-                // the negative side's part; the difference is exact (h or 0)
-                const float2 hn = make_float2(__uint_as_float(__float_as_uint(h2[t].x) & sx),
-                                              __uint_as_float(__float_as_uint(h2[t].y) & sy));
-                const float2 un = make_float2(__uint_as_float(__float_as_uint(hd.x) & sx),
-                                              __uint_as_float(__float_as_uint(hd.y) & sy));
-                Tn = __fadd2_rn(Tn, hn);
-                Un = __fadd2_rn(Un, un);
-                Tp = __fadd2_rn(Tp, make_float2(__uint_as_float(__float_as_uint(h2[t].x) & ~sx),
-                                                __uint_as_float(__float_as_uint(h2[t].y) & ~sy)));
-                Up = __fadd2_rn(Up, make_float2(__uint_as_float(__float_as_uint(hd.x) & ~sx),
-                                                __uint_as_float(__float_as_uint(hd.y) & ~sy)));
+                // masks 0 or 1 by sign: the products are exact
+                const float2 mn2 = make_float2(__uint_as_float(sx & 0x3F800000u), __uint_as_float(sy & 0x3F800000u));
+                const float2 mp2 = make_float2(__uint_as_float(~sx & 0x3F800000u), __uint_as_float(~sy & 0x3F800000u));
+                Tn = __ffma2_rn(h2[t], mn2, Tn);
+                Un = __ffma2_rn(hd, mn2, Un);
+                Tp = __ffma2_rn(h2[t], mp2, Tp);
+                Up = __ffma2_rn(hd, mp2, Up);
                 Sd = __ffma2_rn(hd, ad2[t], Sd);
             }
             // the four per-sign sums are scattered while they are summed: lane
@@ -398,9 +411,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             // with |d| P < 1 for every factor adds to no threshold sum.  The
             // others (about a quarter of a heavy-tailed block, a half of a
             // normal one) are compacted into two lists by sign, |d| and h, in
-            // the scratch.  (The bound is 1 less a few ulps: an element too
-            // many only adds zeros.)  More than kLutListCap of them are taken
-            // in two rounds of 8 elements a lane.
+            // the tile.  (The bound is 1 less a few ulps: an element too many
+            // only adds zeros.)
             const float thr = __fdividef(0.999999f, R * p.invf_max);
             uint32_t act = 0;
 #pragma unroll
@@ -408,7 +420,43 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 if (ad2[t].x >= thr) act |= 1u << (2 * t);
                 if (ad2[t].y >= thr) act |= 2u << (2 * t);
             }
-            const int rounds = __reduce_add_sync(0xffffffffu, __popc(act)) <= kLutListCap ? 1 : 2;
+            const uint32_t ap = act & ~negm, an = act & negm;
+            // list positions: an inclusive scan of both counts
+            uint32_t at = __popc(ap) | (__popc(an) << 16);
+            const uint32_t own = at;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t up = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += up;
+            }
+            const uint32_t tot = __shfl_sync(0xffffffffu, at, 31);
+            at -= own;
+            const int np = (int)(tot & 0xFFFFu), nn = (int)(tot >> 16);
+            const int np8 = (np + 7) & ~7, nn8 = (nn + 7) & ~7;
+            {
+                float* fp = lst + (at & 0xFFFFu);
+                float* fn = lst + np8 + (at >> 16);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float a = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
+                    const float h = (i & 1) ? h2[i >> 1].y : h2[i >> 1].x;
+                    if ((ap >> i) & 1u) {
+                        fp[0] = a;
+                        fp[kLutListLen] = h;
+                        ++fp;
+                    }
+                    if ((an >> i) & 1u) {
+                        fn[0] = a;
+                        fn[kLutListLen] = h;
+                        ++fn;
+                    }
+                }
+                // zeros up to a multiple of 8 entries
+                if (lane < np8 - np) lst[np + lane] = lst[kLutListLen + np + lane] = 0.0f;
+                if (lane < nn8 - nn) lst[np8 + nn + lane] = lst[kLutListLen + np8 + nn + lane] = 0.0f;
+            }
+            __syncwarp();
+            const int steps = max(np8, nn8) >> 3;  // the longest chain of additions of a lane's sum
             const int q = lane & 3;  // the lane's share of the lists, and of the entries
 #pragma unroll 1
             for (int k0 = 0; k0 < K; k0 += 8) {
@@ -439,46 +487,11 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                         }
                     }
                 };
-                int steps = 0;  // the longest chain of additions of a lane's sum
-#pragma unroll 1
-                for (int rd = 0; rd < rounds; ++rd) {
-                    const uint32_t sel = rounds == 1 ? 0xFFFFu : (rd ? 0xFF00u : 0x00FFu);
-                    const uint32_t ap = act & sel & ~negm, an = act & sel & negm;
-                    // list positions: an inclusive scan of both counts
-                    uint32_t pos = __popc(ap) | (__popc(an) << 16);
-                    const uint32_t own = pos;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t up = __shfl_up_sync(0xffffffffu, pos, o);
-                        if (lane >= o) pos += up;
-                    }
-                    const uint32_t tot = __shfl_sync(0xffffffffu, pos, 31);
-                    pos -= own;
-                    const int np = (int)(tot & 0xFFFFu), nn = (int)(tot >> 16);
-                    const int np8 = (np + 7) & ~7, nn8 = (nn + 7) & ~7;
-                    if (rounds > 1 || k0 == 0) {
-                        float* fp = lst + (pos & 0xFFFFu);
-                        float* fn = lst + np8 + (pos >> 16);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const bool in = ((ap | an) >> i) & 1u, ng = (an >> i) & 1u;
-                            float* f = ng ? fn : fp;
-                            if (in) {
-                                f[0] = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
-                                f[kLutListLen] = (i & 1) ? h2[i >> 1].y : h2[i >> 1].x;
-                            }
-                            fp += in && !ng ? 1 : 0;
-                            fn += ng ? 1 : 0;
-                        }
-                        // zeros up to a multiple of 8 entries
-                        if (lane < np8 - np) lst[np + lane] = lst[kLutListLen + np + lane] = 0.0f;
-                        if (lane < nn8 - nn) lst[np8 + nn + lane] = lst[kLutListLen + np8 + nn + lane] = 0.0f;
-                        __syncwarp();
-                    }
-                    walk(lst, np8, Ap, Xp);
-                    walk(lst + np8, nn8, An, Xn);
-                    steps += max(np8, nn8) >> 3;
-                    if (rounds > 1) __syncwarp();  // the lists are rewritten by the next round
+                walk(lst, np8, Ap, Xp);
+                walk(lst + np8, nn8, An, Xn);
+                if (k0 + 8 >= K) {  // the lists are done with: the next block
+                    __syncwarp();
+                    if (u + stride < n_units) issue(u + stride);
                 }
                 // entries: lane q of a candidate has indices 2 q and 2 q + 1, i.e.
                 // the sign s (q >= 2: d >= 0) and levels 2, 3 (far: q = 0, 3) or 0, 1
@@ -505,7 +518,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 // exact (h) or rounded once (h |d|), over at most `depth` levels
                 const float gam = kU * p.tie_kappa * (float)(max(steps, 11) + 8);
                 float E = 0.0f, dE = 0.0f, aE = 0.0f;
-                uint32_t wb = 0, ambm = 0;
+                uint32_t ambm = 0;
+                float mean[2], dm[2], Hs[2], Xs[2], qs[2], dqs[2], dAs[2];
 #pragma unroll
                 for (int e2 = 0; e2 < 2; ++e2) {
                     // the lower level is the even index for d >= 0, the odd one below
@@ -515,41 +529,61 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                     const float gj = fmaf((float)j - 3.5f, sg, c);  // the grid point
                     const float dA = gam * (Am + Am1) + kU * H;
                     const float dX = (gam + kU) * (Xm + Xm1) + kU * X;
-                    float mean = gj, qu = 0.0f, dq = 0.0f, dm = 4.0f * kU * fabsf(gj);
+                    mean[e2] = gj;
+                    dm[e2] = 4.0f * kU * fabsf(gj);
+                    float qu = 0.0f, dq = 0.0f;
                     if (H > 0.0f) {
-                        qu = __fdividef(X, H);
-                        mean = fmaf(sgn, qu, c);
-                        dq = __fdividef(dX + qu * dA, H) + 2.0f * kU * qu;
+                        const float rh = __fdividef(1.0f, H);
+                        qu = X * rh;
+                        mean[e2] = fmaf(sgn, qu, c);
+                        dq = (dX + qu * dA) * rh + 3.0f * kU * qu;
                         // plus the roundings of w - c (relative u each), of the
                         // quotient's use and of the mean's sum
-                        dm = dq + 3.0f * kU * qu + 2.0f * kU * fabsf(mean);
+                        dm[e2] = dq + 3.0f * kU * qu + 2.0f * kU * fabsf(mean[e2]);
                     }
-                    const uint32_t cb = e4m3_encode(mean);
+                    Hs[e2] = H;
+                    Xs[e2] = X;
+                    qs[e2] = qu;
+                    dqs[e2] = dq;
+                    dAs[e2] = dA;
+                }
+                // the two entries at once, and what the bound on each mean
+                // leaves open (equal where the rounding is decided)
+                const uint32_t cb = e4m3_encode2(mean[0], mean[1]);
+                const float2 cv = e4m3_decode2(cb);
+#pragma unroll
+                for (int e2 = 0; e2 < 2; ++e2) {
+                    const int j = 2 * q + (pos ? e2 : 1 - e2);
+                    const float Am = Ac[e2], Am1 = Ac[e2 + 1], Xm = Xc[e2], Xm1 = Xc[e2 + 1];
+                    const float H = Hs[e2], X = Xs[e2], qu = qs[e2], dq = dqs[e2], dA = dAs[e2];
+                    const float dX = (gam + kU) * (Xm + Xm1) + kU * X;
+                    const float2 lh = e4m3_decode2(e4m3_encode2(mean[e2] - dm[e2], mean[e2] + dm[e2]));
                     // an index whose H is not clearly above its error bound may be
                     // empty or may hold weights of tiny saliency lost to the
                     // differences: its entry is undecided unless nothing on its
                     // side reaches its level, and its whole term is bounded below
                     const bool thin = !(H > dA) && Am + Am1 > 0.0f;
-                    const uint32_t c1b = e4m3_encode(mean - dm), c2b = e4m3_encode(mean + dm);
-                    const bool amb = thin || c1b != c2b;
-                    const float dc = e4m3_decode(cb) - mean;
+                    const bool amb = thin || lh.x != lh.y;
+                    const float dc = (e2 ? cv.y : cv.x) - mean[e2];
                     // the index's error: H (C - mean)^2 - X^2 / H (the scatter
                     // term sum h d^2 is added once below)
                     const float Sj = H > 0.0f && !thin ? fmaf(H * dc, dc, -X * qu) : 0.0f;
-                    float bj = dA * dc * dc + 2.0f * H * fabsf(dc) * dm + 3.0f * kU * H * dc * dc + dX * qu +
+                    float bj = dA * dc * dc + 2.0f * H * fabsf(dc) * dm[e2] + 3.0f * kU * H * dc * dc + dX * qu +
                                X * dq + 2.0f * kU * X * qu;
                     if (amb) {  // the other rounding moves the entry by at most this much
-                        const float c1 = e4m3_decode(c1b) - mean;
-                        const float c2 = e4m3_decode(c2b) - mean;
-                        bj += H * fabsf(c2 - c1) * (fabsf(c1) + fabsf(c2) + 2.0f * dm);
+                        const float c1 = lh.x - mean[e2];
+                        const float c2 = lh.y - mean[e2];
+                        bj += H * fabsf(c2 - c1) * (fabsf(c1) + fabsf(c2) + 2.0f * dm[e2]);
                     }
                     bj = thin ? 2.0f * (dA + fabsf(H)) * range * range : bj;
                     E += Sj;
                     dE += bj;
                     aE += fabsf(Sj);
-                    wb |= cb << (8 * (j & 1));
                     ambm |= amb ? 1u << j : 0u;
                 }
+                // stored in index order, a magnitude 0 as +0
+                const uint32_t b0 = cv.x == 0.0f ? 0u : cb & 0xFFu, b1 = cv.y == 0.0f ? 0u : cb >> 8;
+                const uint32_t wb = pos ? b0 | (b1 << 8) : b1 | (b0 << 8);
 #pragma unroll
                 for (int o = 2; o; o >>= 1) {
                     E += __shfl_xor_sync(0xffffffffu, E, o);
@@ -573,20 +607,15 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             __syncwarp();
 
             // ---- argmin (ties: lowest index); candidates that need an exact look
-            float Ek = lane < K ? cerr[lane] : INFINITY;
+            const float Ek = lane < K ? cerr[lane] : INFINITY;
             const float dEk = lane < K ? cbnd[lane] : 0.0f;
-            float Eb = Ek;
-            int kk = lane;
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                const float Eo = __shfl_xor_sync(0xffffffffu, Eb, o);
-                const int ko = __shfl_xor_sync(0xffffffffu, kk, o);
-                if (Eo < Eb || (Eo == Eb && ko < kk)) {
-                    Eb = Eo;
-                    kk = ko;
-                }
-            }
-            kb = kk;
+            // the first lane with the smallest error (lane 0 if none compares)
+            auto argmin = [&](float x, float& xb) {
+                xb = lanes_min(x, 0xffffffffu);
+                return max(__ffs(__ballot_sync(0xffffffffu, x == xb)) - 1, 0);
+            };
+            float Eb;
+            kb = argmin(Ek, Eb);
             const float dEb = __shfl_sync(0xffffffffu, dEk, kb);
             unsigned set = __ballot_sync(0xffffffffu, lane < K && lane != kb && Ek - Eb <= dEk + dEb);
             if (p.stats && lane == 0 && camb[kb]) atomicAdd(&p.stats[2], 1u);
@@ -603,6 +632,23 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 set = (K >= 32) ? 0xFFFFFFFFu : ((1u << K) - 1u);
                 if (lane < K) camb[lane] = 0xFFu;
                 __syncwarp();
+            }
+
+            // the lane's h again, for the settling steps (from the tensor: they
+            // are rare, and h would take 16 registers through the common path)
+            float2 xh[8];
+            if (set != 0u || camb[kb] != 0u) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v4 = *reinterpret_cast<const float4*>(T.v + gofs + i * gstep);
+                    float2 hh[2] = {make_float2(v4.x, v4.y), make_float2(v4.z, v4.w)};
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        if (p.h_mode == kSalEmaSquared) hh[t] = __fmul2_rn(hh[t], hh[t]);
+                        if (p.h_mode == kSalUniform || h_one) hh[t] = make_float2(1.0f, 1.0f);
+                        xh[2 * i + t] = __fmul2_rn(__fmul2_rn(hh[t], make_float2(ts1, ts1)), make_float2(ts2, ts2));
+                    }
+                }
             }
 
             // index (0..7) of element i for the grid of P
@@ -627,7 +673,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         if (index_of(i, P) == j) {
-                            const float hv = ((i & 1) ? h2[i >> 1].y : h2[i >> 1].x) * ts1 * ts2;
+                            const float hv = (i & 1) ? xh[i >> 1].y : xh[i >> 1].x;
                             const float av = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
                             Hs += hv;
                             Xs = fmaf(hv, av, Xs);
@@ -698,7 +744,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                         float acc = 0.0f;
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
-                            const float hv = ((i & 1) ? h2[i >> 1].y : h2[i >> 1].x) * ts1 * ts2;
+                            const float hv = (i & 1) ? xh[i >> 1].y : xh[i >> 1].x;
                             const float df = table[index_of(i, P)] - xwv[i];
                             acc = fmaf(hv * df, df, acc);
                         }
@@ -716,18 +762,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                     const bool in = lane < K && ((set >> lane) & 1u);
                     float Ed = in ? cerr[lane] : INFINITY;
                     const float dEd = in ? cbnd[lane] : 0.0f;
-                    float Edb = Ed;
-                    int kd = lane;
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) {
-                        const float Eo = __shfl_xor_sync(0xffffffffu, Edb, o);
-                        const int ko = __shfl_xor_sync(0xffffffffu, kd, o);
-                        if (Eo < Edb || (Eo == Edb && ko < kd)) {
-                            Edb = Eo;
-                            kd = ko;
-                        }
-                    }
-                    kb = kd;
+                    float Edb;
+                    kb = argmin(Ed, Edb);
                     const float dEdb = __shfl_sync(0xffffffffu, dEd, kb);
                     set = __ballot_sync(0xffffffffu, in && lane != kb && Ed - Edb <= dEd + dEdb);
                     if (set) set |= 1u << kb;
@@ -738,17 +774,14 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             // ---- exact look: float-float sums, exact roundings, direct error
             if (set) {
                 if (p.stats && lane == 0) atomicAdd(&p.stats[0], 1u);
-                // the lane's w again (from memory: this path is rare) and h
-                float2 xw[8], xh[8];
+                // the lane's w again (from memory: this path is rare)
+                float2 xw[8];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float4 w4 = __ldg(reinterpret_cast<const float4*>(T.w + gofs + i * gstep));
                     xw[2 * i] = make_float2(w4.x, w4.y);
                     xw[2 * i + 1] = make_float2(w4.z, w4.w);
                 }
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    xh[t] = __fmul2_rn(__fmul2_rn(h2[t], make_float2(ts1, ts1)), make_float2(ts2, ts2));
                 float best_h = 0.0f, best_l = 0.0f;
                 int best_k = -1;
                 uint32_t best_w0 = 0, best_w1 = 0;
@@ -840,6 +873,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             }
         }
 
+        if (flat && u + stride < n_units) issue(u + stride);
+
         // ---- outputs of the kept candidate: table, indices, r
         uint32_t bw0, bw1;
         if (flat) {
@@ -854,11 +889,13 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         // permute picks four entries by their indices (a nibble each)
         uint32_t tl0, tl1, th0, th1;
         {
-            // lane j holds entry j's bf16 bits in the upper half
-            const uint32_t tv = __float_as_uint(e4m3_decode(((lane & 4 ? bw1 : bw0) >> (8 * (lane & 3))) & 0xFFu)) >> 16;
             uint32_t t[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) t[j] = __shfl_sync(0xffffffffu, tv, j);
+            for (int j = 0; j < 8; j += 2) {
+                const float2 v = e4m3_decode2((j < 4 ? bw0 : bw1) >> (8 * (j & 3)) & 0xFFFFu);
+                t[j] = __float_as_uint(v.x) >> 16;
+                t[j + 1] = __float_as_uint(v.y) >> 16;
+            }
             const uint32_t a01 = __byte_perm(t[0], t[1], 0x5140), a23 = __byte_perm(t[2], t[3], 0x5140);
             const uint32_t a45 = __byte_perm(t[4], t[5], 0x5140), a67 = __byte_perm(t[6], t[7], 0x5140);
             tl0 = __byte_perm(a01, a23, 0x5410);
@@ -868,49 +905,59 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         }
         const float P = flat ? 0.0f : R * p.invf[kb];
         const float2 P2 = make_float2(P, P);
+        const uint32_t smask = flat ? 0u : 0x7777u;
+        auto outputs = [&](auto bf16, auto with_codes) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            // indices of the chunk's 4 elements, a nibble each: level m =
-            // min(floor(|d| P), 3) from the low bits of the floor on the 2^23
-            // grid; 4 + m (d >= 0) is m ^ 4 and 3 - m (d < 0) is m ^ 3
-            const float2 ya = __ffma2_rd(ad2[2 * i], P2, M2), yb = __ffma2_rd(ad2[2 * i + 1], P2, M2);
-            const uint32_t m0 = __float_as_uint(fminf(ya.x, kMagic + 3.0f)), m1 = __float_as_uint(fminf(ya.y, kMagic + 3.0f));
-            const uint32_t m2 = __float_as_uint(fminf(yb.x, kMagic + 3.0f)), m3 = __float_as_uint(fminf(yb.y, kMagic + 3.0f));
-            const uint32_t ng = negm >> (4 * i);
-            const uint32_t sx = (ng & 1u) | ((ng & 2u) << 3) | ((ng & 4u) << 6) | ((ng & 8u) << 9);
-            uint32_t sel = (m0 + (m1 << 4) + (m2 << 8) + (m3 << 12)) ^ 0x4444u ^ (sx * 7u);
-            sel = flat ? 0u : sel & 0x7777u;
-            const uint32_t lo = __byte_perm(tl0, tl1, sel), hi = __byte_perm(th0, th1, sel);
-            const uint32_t r01 = __byte_perm(lo, hi, 0x5140), r23 = __byte_perm(lo, hi, 0x7362);
-            const int64_t ge = gofs + i * gstep;
-            if (p.r_bf16)
-                stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + ge), make_uint2(r01, r23));
-            else
-                stg_cs(reinterpret_cast<float4*>(static_cast<float*>(T.r) + ge),
-                       make_float4(bf16lo(r01), bf16hi(r01), bf16lo(r23), bf16hi(r23)));
-            if (T.codes) {
-                if (!p.codes_packed) {
-                    // nibbles to bytes
-                    const uint32_t t8 = (sel | (sel << 8)) & 0x00FF00FFu;
-                    stg_cs(reinterpret_cast<uint32_t*>(T.codes + ge), (t8 | (t8 << 4)) & 0x0F0F0F0Fu);
-                } else {
-                    // 3 bits an index in block order: the lane's 12 bits at bit
-                    // 12 (32 i + lane); 8 lanes make 3 words
-                    const uint32_t s6 = (sel & 0x0707u) | ((sel & 0x7070u) >> 1);
-                    uint32_t x = (s6 & 0x3Fu) | ((s6 & 0x3F00u) >> 2);
-                    const uint32_t o1 = __shfl_xor_sync(0xffffffffu, x, 1);
-                    x = lane & 1 ? o1 | (x << 12) : x | (o1 << 12);  // 24 bits of 2 lanes
-                    const uint32_t o2 = __shfl_xor_sync(0xffffffffu, x, 2);
-                    const uint32_t xa = lane & 2 ? o2 : x, xb = lane & 2 ? x : o2;
-                    const uint32_t x0 = xa | (xb << 24), x1 = xb >> 8;  // 48 bits of 4 lanes
-                    const uint32_t o0 = __shfl_xor_sync(0xffffffffu, x0, 4), oh = __shfl_xor_sync(0xffffffffu, x1, 4);
-                    // lanes 0, 1, 2 of the 8 (the first half) write a word each
-                    const int l8 = lane & 7;
-                    if (l8 < 3)
-                        stg_cs(reinterpret_cast<uint32_t*>(T.codes) + (size_t)b * 48 + i * 12 + (lane >> 3) * 3 + l8,
-                               l8 == 0 ? x0 : (l8 == 1 ? x1 | (o0 << 16) : (o0 >> 16) | (oh << 16)));
+            for (int i = 0; i < 4; ++i) {
+                // indices of the chunk's 4 elements, a nibble each: level m =
+                // min(floor(|d| P), 3) from the low bits of the floor on the 2^23
+                // grid; 4 + m (d >= 0) is m ^ 4 and 3 - m (d < 0) is m ^ 3
+                const float2 ya = __ffma2_rd(ad2[2 * i], P2, M2), yb = __ffma2_rd(ad2[2 * i + 1], P2, M2);
+                const uint32_t m0 = __float_as_uint(fminf(ya.x, kMagic + 3.0f)), m1 = __float_as_uint(fminf(ya.y, kMagic + 3.0f));
+                const uint32_t m2 = __float_as_uint(fminf(yb.x, kMagic + 3.0f)), m3 = __float_as_uint(fminf(yb.y, kMagic + 3.0f));
+                const uint32_t ng = negm >> (4 * i);
+                const uint32_t sx = (ng & 1u) | ((ng & 2u) << 3) | ((ng & 4u) << 6) | ((ng & 8u) << 9);
+                uint32_t sel = (m0 + (m1 << 4) + (m2 << 8) + (m3 << 12)) ^ 0x4444u ^ (sx * 7u);
+                sel &= smask;
+                const uint32_t lo = __byte_perm(tl0, tl1, sel), hi = __byte_perm(th0, th1, sel);
+                const uint32_t r01 = __byte_perm(lo, hi, 0x5140), r23 = __byte_perm(lo, hi, 0x7362);
+                const int64_t ge = gofs + i * gstep;
+                if constexpr (decltype(bf16)::value)
+                    stg_cs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(T.r) + ge), make_uint2(r01, r23));
+                else
+                    stg_cs(reinterpret_cast<float4*>(static_cast<float*>(T.r) + ge),
+                           make_float4(bf16lo(r01), bf16hi(r01), bf16lo(r23), bf16hi(r23)));
+                if constexpr (decltype(with_codes)::value) {
+                    if (!p.codes_packed) {
+                        // nibbles to bytes
+                        const uint32_t t8 = (sel | (sel << 8)) & 0x00FF00FFu;
+                        stg_cs(reinterpret_cast<uint32_t*>(T.codes + ge), (t8 | (t8 << 4)) & 0x0F0F0F0Fu);
+                    } else {
+                        // 3 bits an index in block order: the lane's 12 bits at bit
+                        // 12 (32 i + lane); 8 lanes make 3 words
+                        const uint32_t s6 = (sel & 0x0707u) | ((sel & 0x7070u) >> 1);
+                        uint32_t x = (s6 & 0x3Fu) | ((s6 & 0x3F00u) >> 2);
+                        const uint32_t o1 = __shfl_xor_sync(0xffffffffu, x, 1);
+                        x = lane & 1 ? o1 | (x << 12) : x | (o1 << 12);  // 24 bits of 2 lanes
+                        const uint32_t o2 = __shfl_xor_sync(0xffffffffu, x, 2);
+                        const uint32_t xa = lane & 2 ? o2 : x, xb = lane & 2 ? x : o2;
+                        const uint32_t x0 = xa | (xb << 24), x1 = xb >> 8;  // 48 bits of 4 lanes
+                        const uint32_t o0 = __shfl_xor_sync(0xffffffffu, x0, 4), oh = __shfl_xor_sync(0xffffffffu, x1, 4);
+                        // lanes 0, 1, 2 of the 8 (the first half) write a word each
+                        const int l8 = lane & 7;
+                        if (l8 < 3)
+                            stg_cs(reinterpret_cast<uint32_t*>(T.codes) + (size_t)b * 48 + i * 12 + (lane >> 3) * 3 + l8,
+                                   l8 == 0 ? x0 : (l8 == 1 ? x1 | (o0 << 16) : (o0 >> 16) | (oh << 16)));
+                    }
                 }
             }
+        };
+        if (T.codes) {
+            if (p.r_bf16) outputs(std::true_type{}, std::true_type{});
+            else outputs(std::false_type{}, std::true_type{});
+        } else {
+            if (p.r_bf16) outputs(std::true_type{}, std::false_type{});
+            else outputs(std::false_type{}, std::false_type{});
         }
         if (lane == 0) {
             stg_cs(reinterpret_cast<uint2*>(T.book + (size_t)b * 8), make_uint2(bw0, bw1));
