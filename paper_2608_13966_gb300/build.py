@@ -33,7 +33,11 @@ UNITS = [
     ("kernels_int.cu", ["-DQUASAR_NCH=2", "-DQUASAR_SS=1"], "kernels_int_nch2_ss1.o"),
     ("kernels_nvfp4.cu", [], "kernels_nvfp4.o"),
     ("kernels_lut.cu", [], "kernels_lut.o"),
-    ("kernels_sym.cu", [], "kernels_sym.o"),
+    ("kernels_sym.cu", ["-DQUASAR_SS=8"], "kernels_sym_ss8.o"),
+    ("kernels_sym.cu", ["-DQUASAR_SS=4"], "kernels_sym_ss4.o"),
+    ("kernels_sym.cu", ["-DQUASAR_SS=3"], "kernels_sym_ss3.o"),
+    ("kernels_sym.cu", ["-DQUASAR_SS=2"], "kernels_sym_ss2.o"),
+    ("kernels_sym.cu", ["-DQUASAR_SS=1"], "kernels_sym_ss1.o"),
 ]
 
 

@@ -87,6 +87,24 @@ __device__ __forceinline__ bool warp_wait_bounded(uint64_t* bar, uint32_t parity
     return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, limit_ns));
 }
 
+// Wait until the tile of sequence number t is the one in flight into a slot
+// (its sequence word, written before the copy is issued), or until limit_ns
+// has passed; the same outcome for every lane of the warp.
+__device__ __forceinline__ bool warp_wait_seq(const volatile int* seq, int t, uint64_t limit_ns)
+{
+    bool ok = *seq == t;
+    if (!__all_sync(0xffffffffu, ok)) {
+        const uint64_t t0 = global_timer_ns();
+        for (;;) {
+#pragma unroll 1
+            for (int i = 0; i < 32 && !ok; ++i) ok = *seq == t;
+            if (ok || global_timer_ns() - t0 > limit_ns) break;
+        }
+        ok = __all_sync(0xffffffffu, ok);
+    }
+    return ok;
+}
+
 // 1-D bulk copy global -> shared, completion counted in bytes on `bar`.
 // dst, src and bytes must be multiples of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)

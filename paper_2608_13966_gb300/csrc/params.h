@@ -8,15 +8,9 @@ namespace quasar {
 // Bit set in the per-device status word when a kernel gives up on a wait.
 constexpr unsigned kStatusTimeout = 1u;
 
-constexpr int kLanesPerGroup = 8;
-// Per-warp shared scratch of the integer kernel: 32 rows of 32 floats used to
-// transpose the per-candidate sums across the lanes of a group (16-byte
-// columns XOR-swizzled by row, so neither side has bank conflicts).
-constexpr uint32_t kIntScratchBytes = 32 * 32 * 4;
-constexpr int kGroupsPerUnit = 4;
 constexpr int kMaxClip = 32;
 
-// The asymmetric integer kernel: 4 lanes a group, 8 groups a unit, and a
+// The integer kernels: 4 lanes a group, 8 groups a unit, and a
 // ring of unit tiles shared by the warps of a CTA.  Once the gradient is
 // consumed, the tile's gradient region holds the candidates' table: 16 bytes
 // for each of a chunk's 8 candidates and the unit's 8 groups.
@@ -71,11 +65,10 @@ struct IntParams {
                           // [5] one-pass error sums, [6] twin code checks
     float f[kMaxClip];     // padded with the last factor
     float invf[kMaxClip];  // fl32(1/f)
-    // code clamps: every candidate slot holds tau / qmax of its clamp set,
-    // so that the set's cap on |w - centre| is cap * range (sets of
-    // set_size consecutive slots (8 and 3 with a single chunk only), or with
-    // set_size 3 the runs of 3, 3 and 2 slots of each 8; see the integer
-    // kernel)
+    // code clamps: every candidate slot holds tau / qmax of its clamp set, so
+    // that the set's cap on |w - centre| is cap * range (symmetric codes: tau /
+    // Q, and cap * amax on |w|); sets of set_size consecutive slots, or with
+    // set_size 3 the runs of 3, 3 and 2 slots of each 8
     float cap[kMaxClip];
     int set_size;
     // the factors come in order, decreasing or increasing (as the paper's

@@ -28,7 +28,11 @@ const void* amax_init_kernel(bool batch);
 const void* amax_to_scale_kernel(bool batch);
 const void* lut_kernel();
 const void* adamw_amax_kernel();
-const void* sym_kernel(int epl);
+const void* sym_kernel_ss8(int epl);
+const void* sym_kernel_ss4(int epl);
+const void* sym_kernel_ss3(int epl);
+const void* sym_kernel_ss2(int epl);
+const void* sym_kernel_ss1(int epl);
 }  // namespace quasar
 
 // Per-device status word (bit 0: a kernel timed out on a wait).
@@ -38,9 +42,9 @@ namespace {
 
 using namespace quasar;
 
-// 8 warps per CTA: with two 5 KB tiles and the 4 KB transpose scratch per
-// warp, two CTAs fit in an SM's shared memory (16 resident warps, at 128
-// registers a thread the whole register file).
+// 8 warps per CTA: two CTAs of the integer and lookup-table kernels fill the
+// register file (16 resident warps at 128 registers a thread) and fit in an
+// SM's shared memory.
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 // The AdamW-fused integer kernel also stages m (14 instead of 10 bytes a
@@ -63,8 +67,7 @@ constexpr float kTieScaleMin = 1.0f;
 constexpr float kFitUlpsMin = 8.0f;
 
 struct Tuning {
-    int stages = 0;            // 0: chosen from the shared-memory budget
-    int smem_budget = 100 * 1024;
+    int stages = 0;            // 0: each kernel's choice
     float tie_kappa = kTieKappaMin;  // NVFP4 tie bound, in ulps
     float tie_scale = kTieScaleMin;  // multiplier of the integer kernel's summation-depth bound
     float fit_ulps = kFitUlpsMin;
@@ -83,7 +86,6 @@ const Tuning& tuning()
     static const Tuning t = [] {
         Tuning x;
         if (const char* s = std::getenv("QUASAR_STAGES")) x.stages = std::min(std::max(std::atoi(s), 0), 8);
-        if (const char* s = std::getenv("QUASAR_SMEM_BUDGET")) x.smem_budget = std::atoi(s);
         if (const char* s = std::getenv("QUASAR_TIE_KAPPA")) x.tie_kappa = env_float(s, kTieKappaMin, 1e4f);
         if (const char* s = std::getenv("QUASAR_TIE_SCALE")) x.tie_scale = env_float(s, kTieScaleMin, 1e3f);
         if (const char* s = std::getenv("QUASAR_FIT_ULPS")) x.fit_ulps = env_float(s, kFitUlpsMin, 1e4f);
@@ -148,20 +150,26 @@ void fill_clip(const float* clip, int n_clip, float* f, float* invf)
     }
 }
 
-// Code clamps of the integer kernel.  A set of consecutive candidate slots
-// shares one clamp when some tau has J f_max (1 + 1e-3) <= tau <= (J + 1)
-// f_min (1 - 1e-3), J = (qmax - 1) / 2: then min(|d|, tau range / qmax) P_k
-// has the code min(floor(|d| P_k), J) for every slot k of the set (a capped
-// |d| gives cap P_k ~ tau / f_k in [J, J + 1), and below the cap
-// |d| P_k < J + 1).  The margin covers the fp32 roundings of the cap, of R
-// and of P.  The largest set size of 4, 2, 1 whose sets all qualify is taken
-// (a set of one always does), and no larger than max_size; every slot holds
-// its set's tau / qmax.  Also the centre factor of each 8-candidate chunk.
-void fill_caps(IntParams* p, int max_size, bool single_chunk = false)
+// Code clamps of the integer kernels.  A set of consecutive candidate slots
+// shares one clamp of |w - centre| (asymmetric) or |w| (symmetric codes) when
+// the capped value has the largest code for every factor of the set and no
+// value below the cap exceeds it.  Asymmetric, J = (qmax - 1) / 2: some tau
+// with J f_max (1 + 1e-3) <= tau <= (J + 1) f_min (1 - 1e-3); then
+// min(|d|, tau range / qmax) P_k has the code min(floor(|d| P_k), J) for every
+// slot k of the set (a capped |d| gives cap P_k ~ tau / f_k in [J, J + 1), and
+// below the cap |d| P_k < J + 1).  Symmetric, codes rounded to at most Q: the
+// same with Q - 1/2 and Q + 1/2 for J and J + 1, and the cap tau amax / Q.  The
+// margin covers the fp32 roundings of the cap, of R and of P.  The largest set
+// size of 8, 4, 3, 2, 1 whose sets all qualify is taken (a set of one always
+// does), and no larger than max_size; every slot holds its set's tau / qmax (or
+// tau / Q).  Also the centre factor of each 8-candidate chunk.
+void fill_caps(IntParams* p, int max_size, bool sets_8_3 = false, bool symmetric = false)
 {
     const int J = p->qmax >> 1;
+    const int Q = (p->qmax - 1) >> 1;
+    const double below = symmetric ? Q - 0.5 : J, above = symmetric ? Q + 0.5 : J + 1;
     // the sets of a size: consecutive runs of `size` slots; 3: the runs 3, 3,
-    // 2 of every 8 slots (3 and 8: with a single chunk only)
+    // 2 of every 8 slots (3 and 8: only where the kernel is built for them)
     auto first_of = [](int size, int k) { return size == 3 ? 8 * (k / 8) + 3 * ((k % 8) / 3) : k - k % size; };
     auto len_of = [](int size, int k0) { return size == 3 ? (k0 % 8 == 6 ? 2 : 3) : size; };
     auto cap_of = [&](int k0, int n, double* tau) {
@@ -170,13 +178,13 @@ void fill_caps(IntParams* p, int max_size, bool single_chunk = false)
             fmax = std::max(fmax, (double)p->f[k]);
             fmin = std::min(fmin, (double)p->f[k]);
         }
-        const double lo = J * fmax * (1.0 + 1e-3), hi = (J + 1) * fmin * (1.0 - 1e-3);
+        const double lo = below * fmax * (1.0 + 1e-3), hi = above * fmin * (1.0 - 1e-3);
         *tau = 0.5 * (lo + hi);
         return lo < hi;
     };
     int size = 1;
     for (int cand : {8, 4, 3, 2}) {
-        if ((cand == 3 || cand == 8) ? (!single_chunk || max_size < 4) : cand > max_size) continue;
+        if ((cand == 3 || cand == 8) ? (!sets_8_3 || max_size < 4) : cand > max_size) continue;
         bool ok = true;
         double tau;
         for (int k0 = 0; k0 < kMaxClip && ok; k0 += len_of(cand, k0)) ok = cap_of(k0, len_of(cand, k0), &tau);
@@ -190,7 +198,7 @@ void fill_caps(IntParams* p, int max_size, bool single_chunk = false)
         const int k0 = first_of(size, k);
         double tau = 0.0;
         cap_of(k0, len_of(size, k0), &tau);
-        p->cap[k] = (float)(tau / p->qmax);
+        p->cap[k] = (float)(tau / (symmetric ? Q : p->qmax));
     }
     for (int c = 0; c < kMaxClip / 8; ++c) {
         double lo = 1e300, hi = 0.0;
@@ -208,26 +216,15 @@ struct Launch {
     size_t smem;
 };
 
-// Shared memory per CTA: for each of its warps, `stages` tiles of
-// unit_bytes, a scratch area, and stages + 1 mbarriers.  stages: the
-// kernel's choice, or 0 for as many of 2 to 4 as the budget holds
-// (QUASAR_STAGES overrides both).
-Launch plan(uint32_t unit_bytes, uint32_t scratch_bytes, int stages = 0, int warps = kWarps)
+// Shared memory per CTA of the kernels with per-warp rings: for each warp,
+// `stages` tiles of unit_bytes (QUASAR_STAGES overrides) and stages + 1
+// mbarriers.
+Launch plan(uint32_t unit_bytes, int stages)
 {
-    const Tuning& t = tuning();
     Launch L;
+    L.stages = tuning().stages > 0 ? tuning().stages : stages;
     L.stage_bytes = (unit_bytes + 127u) & ~127u;
-    auto total = [&](int s) {
-        return (size_t)warps * s * L.stage_bytes + (size_t)warps * scratch_bytes +
-               (size_t)warps * (s + 1) * 8;
-    };
-    int s = t.stages > 0 ? t.stages : stages;
-    if (s <= 0) {
-        s = 2;
-        while (s < 4 && total(s + 1) <= (size_t)t.smem_budget) ++s;
-    }
-    L.stages = s;
-    L.smem = total(s);
+    L.smem = (size_t)kWarps * ((size_t)L.stages * L.stage_bytes + (size_t)(L.stages + 1) * 8);
     return L;
 }
 
@@ -416,14 +413,7 @@ struct AdamHp {
     int64_t step;
 };
 
-// Stage bytes of one unit of the symmetric-code kernel: w, v, g.
-uint32_t int_unit_bytes(int group_size, int g_kind, bool adam)
-{
-    const int gbytes = g_kind == 2 ? 2 : (g_kind == 1 ? 4 : 0);
-    return (uint32_t)(kGroupsPerUnit * group_size * ((adam ? 12 : 8) + gbytes));
-}
-
-// Shared memory of the asymmetric integer kernel's CTA ring: S slots of one
+// Shared memory of an integer kernel's CTA ring: S slots of one
 // unit tile each (w, v, m for the fused AdamW step, then the gradient
 // region, which is also the candidate table and so at least kIntTableBytes
 // for each 8 candidates), S + 1 mbarriers and S sequence words.  S is one slot a
@@ -471,17 +461,15 @@ quasar_status int_params(quasar_dtype g_dtype, bool has_g, float beta2, int bits
     p->n_clip = n_clip;
     p->beta2 = beta2;
     p->c1 = 1.0f - beta2;
-    // each candidate sum is accumulated over at most G/8 (asymmetric kernel:
-    // 4 lanes a group) or G/16 (symmetric: 8 lanes) terms a packed half, plus
-    // the halves' sum and the lane tree (2 or 3 levels); the terms' own
-    // roundings and those that form N, D and E make up the rest
-    p->tie_kappa = tuning().tie_scale * (float)(group_size / (opt.symmetric ? 16 : 8) + 8);
+    // each candidate sum is accumulated over at most G/8 terms a packed half
+    // (4 lanes a group), plus the halves' sum and the lane tree (2 levels); the
+    // terms' own roundings and those that form N, D and E make up the rest
+    p->tie_kappa = tuning().tie_scale * (float)(group_size / 8 + 8);
     p->fit_ulps = tuning().fit_ulps;
     p->timeout_ns = kDefaultTimeoutNs;
     p->force_timeout_ns = (uint64_t)std::max<int64_t>(0, g_force_timeout_ns.load());
     p->stats = g_stats.load();
     fill_clip(clip, n_clip, p->f, p->invf);
-    fill_caps(p, 4);
     bool up = true, down = true;
     for (int k = 1; k < n_clip; ++k) {
         up &= p->invf[k] >= p->invf[k - 1];
@@ -510,28 +498,37 @@ template <int MAXT>
 quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaStream_t stream,
                          bool adam = false, bool symmetric = false)
 {
-    // units: 8 groups for the asymmetric kernel, 4 for the symmetric one
-    const int per_unit = symmetric ? kGroupsPerUnit : kIntGroups;
     int64_t units = 0;
     for (int i = 0; i < Lp.n_t; ++i) {
         Lp.t[i].unit0 = units;
-        units += (Lp.t[i].n_groups + per_unit - 1) / per_unit;
+        units += (Lp.t[i].n_groups + kIntGroups - 1) / kIntGroups;
     }
     Lp.n_units = units;
     if (units == 0) return QUASAR_OK;
     const int warps = adam ? kAdamWarps : kWarps;
-    const Launch L = symmetric ? plan(int_unit_bytes(group_size, Lp.p.g_kind, adam), kIntScratchBytes, 0, warps)
-                               : plan_ring(group_size, Lp.p.g_kind, adam, warps, n_clip);
+    const Launch L = plan_ring(group_size, Lp.p.g_kind, adam, warps, n_clip);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
-    const int epl = group_size / (symmetric ? kLanesPerGroup : kIntLanes);
+    const int epl = group_size / kIntLanes;
     const bool one_chunk = n_clip <= 8;
     const bool batch = MAXT > 1;
     const bool var = Lp.p.h_mode != kSalEma || Lp.p.codes_packed;
     // clamp sets: as large as the factors allow, unless switched off (sets of
-    // one); the option variants are built with sets of one, the fused AdamW
-    // step with sets of four or one
+    // one); the option variants of the asymmetric kernel are built with sets of
+    // one, the fused AdamW step with sets of four or one
     const int hoist_on = g_hoist.load() < 0 ? tuning().hoist : g_hoist.load();
+    if (symmetric) {
+        if (MAXT == 1) return QUASAR_ERR_UNSUPPORTED;
+        fill_caps(&Lp.p, hoist_on ? 4 : 1, true, true);
+        const int ss = Lp.p.set_size;
+        const void* fn = (ss == 8   ? sym_kernel_ss8
+                          : ss == 4 ? sym_kernel_ss4
+                          : ss == 3 ? sym_kernel_ss3
+                          : ss == 2 ? sym_kernel_ss2
+                                    : sym_kernel_ss1)(epl);
+        if (!fn) return QUASAR_ERR_UNSUPPORTED;
+        return launch_persistent(fn, &Lp, L.smem, units, stream, warps);
+    }
     // (sets of 8 or 3-3-2 with a single chunk, not for the fused AdamW step)
     fill_caps(&Lp.p, (!hoist_on || var) ? 1 : 4, one_chunk && !adam);
     if (adam && Lp.p.set_size == 2) fill_caps(&Lp.p, 1);
@@ -543,8 +540,7 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
     const int ss = Lp.p.set_size;
     const int si = ss == 8 ? 0 : (ss == 4 ? 1 : (ss == 3 ? 2 : (ss == 2 ? 3 : 4)));
     if (!table[ci][si]) return QUASAR_ERR_UNSUPPORTED;
-    const void* fn = symmetric ? (MAXT > 1 ? sym_kernel(epl) : nullptr)
-                               : table[ci][si](epl, batch, adam, var);
+    const void* fn = table[ci][si](epl, batch, adam, var);
     if (!fn) return QUASAR_ERR_UNSUPPORTED;
     return launch_persistent(fn, &Lp, L.smem, units, stream, warps);
 }
@@ -666,7 +662,7 @@ quasar_status nvfp4_run(Nvfp4Launch<MAXT>& Lp, AmaxBatch<MAXT>& B, int n_clip, c
     const int gbytes = Lp.p.g_kind == 2 ? 2 : (Lp.p.g_kind == 1 ? 4 : 0);
     // one tile a warp: it is in registers, and the next copy under way, before
     // the search begins
-    const Launch L = plan((uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes)), 0, 1);
+    const Launch L = plan((uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes)), 1);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
     return launch_persistent(nvfp4_kernel(MAXT > 1), &Lp, L.smem, units, s);

@@ -394,24 +394,6 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
 
 // ------------------------------------------------------------------ kernel
 
-// Wait until the tile of sequence number t is the one in flight into a slot
-// (its sequence word, written before the copy is issued), or until limit_ns
-// has passed; the same outcome for every lane of the warp.
-__device__ __forceinline__ bool warp_wait_seq(const volatile int* seq, int t, uint64_t limit_ns)
-{
-    bool ok = *seq == t;
-    if (!__all_sync(0xffffffffu, ok)) {
-        const uint64_t t0 = global_timer_ns();
-        for (;;) {
-#pragma unroll 1
-            for (int i = 0; i < 32 && !ok; ++i) ok = *seq == t;
-            if (ok || global_timer_ns() - t0 > limit_ns) break;
-        }
-        ok = __all_sync(0xffffffffu, ok);
-    }
-    return ok;
-}
-
 // Two CTAs per SM: 8-warp CTAs, 6-warp ones for the AdamW-fused variant.
 // VAR: the variants of the options (a saliency other than v', packed codes);
 // without it they compile out of the common kernel.
