@@ -323,8 +323,11 @@ quasar_status occupancy(const void* fn, size_t smem, int threads, int dev, int* 
     return QUASAR_OK;
 }
 
-// Persistent launch: at most (#SMs x resident CTAs) CTAs of `warps` warps,
-// no more than there are units of work for the warps.
+// Persistent launch: at most (#SMs x resident CTAs) CTAs of `warps` warps, and
+// no more than there are units of work: a launch with fewer units than warps
+// spreads them over the SMs (the kernels give a CTA's first warp the first of
+// its units) instead of filling a few CTAs, whose warps would share a
+// scheduler.
 quasar_status launch_persistent(const void* fn, void* params, size_t smem, int64_t n_units,
                                 cudaStream_t stream, int warps = kWarps)
 {
@@ -334,8 +337,7 @@ quasar_status launch_persistent(const void* fn, void* params, size_t smem, int64
     if (st != QUASAR_OK) return st;
     if ((st = occupancy(fn, smem, warps * 32, dev, &occ)) != QUASAR_OK) return st;
     if (occ < 1) return QUASAR_ERR_UNSUPPORTED;
-    const int64_t want = (n_units + warps - 1) / warps;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)info->nsm * occ, want));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)info->nsm * occ, n_units));
     void* args[] = {params};
     if (cudaLaunchKernel(fn, dim3(grid), dim3(warps * 32), args, smem, stream) != cudaSuccess)
         return QUASAR_ERR_CUDA;

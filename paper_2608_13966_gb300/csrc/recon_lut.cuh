@@ -225,7 +225,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         while (ti + 1 < Lp.n_t && u >= Lp.t[ti + 1].unit0) ++ti;
     };
     int ti = 0;
-    const int64_t first = (int64_t)blockIdx.x * nwarps + warp;
+    // (the units of a launch smaller than the grid's warps go to different CTAs)
+    const int64_t first = (int64_t)warp * gridDim.x + blockIdx.x;
     const int64_t stride = (int64_t)gridDim.x * nwarps;
 
     // the lane's 16 elements, in four chunks of 4: chunk i is block elements

@@ -126,7 +126,8 @@ __global__ void __launch_bounds__(256, 3) k_recon_nvfp4(const __grid_constant__ 
     };
     int ti = 0, ti_s = -1;
     float sT = 1.0f, inv_sT = 1.0f;
-    const int64_t first = (int64_t)blockIdx.x * nwarps + warp;
+    // (the units of a launch smaller than the grid's warps go to different CTAs)
+    const int64_t first = (int64_t)warp * gridDim.x + blockIdx.x;
     const int64_t stride = (int64_t)gridDim.x * nwarps;
 
 
