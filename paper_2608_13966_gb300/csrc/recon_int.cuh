@@ -127,7 +127,9 @@ __device__ __forceinline__ void ff_norm(float& hi, float& lo)
 // enters them, and what counts is how much of the instruction cache they
 // take: rolled, one Qwen3 layer at INT2, 16 factors took 1,907 us, unrolled
 // 1,953.  With up to 8 it is a tenth, and latency counts: 806 against 822 us
-// on a Llama layer at INT3.
+// on a Llama layer at INT3.  (Smaller still -- passes A and C not unrolled, one
+// reduction loop in the compensated fit, counters in registers, fast roots
+// where they only feed a bound -- the Qwen3 layer takes 1,660 us.)
 template <bool ROLL>
 __device__ __forceinline__ void ff_reduce32(float& hi, float& lo)
 {
@@ -348,10 +350,24 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
         A = __fadd_rn(A, xh);
         B = fmaf(h, wh, B);
     }
-    ff_reduce32<ROLL>(Dh, Dl);
-    ff_reduce32<ROLL>(Nh, Nl);
-    A = wsum32(A);
-    B = wsum32(B);
+    // both pairs and both sums over the warp in one loop (as ff_reduce32 and
+    // wsum32 would)
+    ff_norm(Dh, Dl);
+    ff_norm(Nh, Nl);
+#pragma unroll (ROLL ? 1 : 5)
+    for (int o = 16; o; o >>= 1) {
+        const float dh = shx(Dh, o), dl = shx(Dl, o), nh = shx(Nh, o), nl = shx(Nl, o);
+        ff_acc(Dh, Dl, dh, dl);
+        ff_norm(Dh, Dl);
+        ff_acc(Nh, Nl, nh, nl);
+        ff_norm(Nh, Nl);
+        A += shx(A, o);
+        B += shx(B, o);
+    }
+    Dh = __shfl_sync(0xffffffffu, Dh, 0);
+    Dl = __shfl_sync(0xffffffffu, Dl, 0);
+    Nh = __shfl_sync(0xffffffffu, Nh, 0);
+    Nl = __shfl_sync(0xffffffffu, Nl, 0);
     {
         float sum, err;
         two_sum(Dh, -(A * A / Ss), sum, err);
@@ -562,8 +578,9 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             auto pass_a = [&](auto gk) {
                 constexpr int GK = decltype(gk)::value;
                 float2 SS2 = make_float2(0.0f, 0.0f), SW = SS2;
-// two chunks an iteration: the loop stays small in the instruction cache
-#pragma unroll 2
+// two chunks an iteration (one with more than 8 candidates): the loop stays
+// small in the instruction cache
+#pragma unroll (NCH == 1 ? 2 : 1)
                 for (int i = 0; i < NCHK; ++i) {
                     const int eo = eoff(i);
                     const int e = gs * G + eo;
@@ -976,8 +993,10 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                     }
 #pragma unroll
                     for (int o = 2; o; o >>= 1) hmn = fminf(hmn, shx(hmn, o));
-                    const float t2s = fmaxf(tb.y * see, 0.0f), t2w = fmaxf(ss * tb.y, 0.0f);
-                    twin_q = 2.0f * ulp * (sqrtf(t2s) + fabsf(cref - mu) * sqrtf(t2w)) * qmaxf;
+                    // (the roots as x rsqrt(x), 2 ulps: inside the factor 1.0001)
+                    const float t2s = fmaxf(tb.y * see, 1e-37f), t2w = fmaxf(ss * tb.y, 1e-37f);
+                    twin_q = 2.0f * 1.0001f * ulp *
+                             (t2s * rsqrtf(t2s) + fabsf(cref - mu) * (t2w * rsqrtf(t2w))) * qmaxf;
                     twin_h = hmn * range;
                     twin_e = hmn * qmaxf * (8.0f * 5.9604645e-8f) * (range + fabsf(cref));
                 }
@@ -1010,6 +1029,13 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
         float Bz_lo = 0.0f, a_lo = 0.0f;
         bool deg_sel = false;
 
+        // the tuning counters' events of the unit (see IntParams::stats), 8 or 10
+        // bits each: [0], [1], [2] and [4], [5], [6].  (Counted here and added to
+        // the counters once: the atomics spelled out at each event cost code that
+        // the careful paths' share of the instruction cache pays for -- on the
+        // Qwen3 layer at INT2, 16 factors, 1,754 against 1,699 us.)
+        uint32_t ev1 = 0, ev2 = 0;
+
         // ---- deferred exact comparisons: the whole warp takes one group at a time
         unsigned todo = __ballot_sync(0xffffffffu, valid && !flat && set != 0 && sl == 0);
         while (todo) {
@@ -1038,7 +1064,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             auto gy0 = [&](int ch) {
                 return fminf(fmaxf(__fmaf_rd(gdmu, gR * p.invfc[ch], kGridMagic), ylo), yhi);
             };
-            if (p.stats && lane == 0) atomicAdd(&p.stats[2], 1u);
+            ev1 += 1u << 16;
             // Codes move monotonically with 1/f, element by element, so (with the
             // factors in order) two candidates with equal codes share them with
             // every candidate between them: the highest twin settles all twins
@@ -1074,7 +1100,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 const bool high = phase == kTwins ? top : phase == kAbove;
                 const int k = high ? 31 - __clz(todo_k) : __ffs(todo_k) - 1;
                 todo_k &= ~(1u << k);
-                if (p.stats && lane == 0) atomicAdd(&p.stats[6], 1u);
+                ev2 += 1u << 20;
                 const bool same = coop_same_codes<G>(tws, ggq, gR * p.invf[k], gR * p.invf[gw]);
                 if (same && phase == kBelow) {
                     gset &= ~(mono ? (2u << gw) - (2u << k) : 1u << gw);  // (k, gw]
@@ -1091,7 +1117,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 if (gs == g) kb = gw;
                 continue;
             }
-            if (p.stats && lane == 0) atomicAdd(&p.stats[0], 1u);
+            ev1 += 1u;
             float best_h = 0.0f, best_l = 0.0f, ga = 0.0f, gB = 0.0f, gkap = 0.0f;
             int best_k = -1;
             bool gdeg = false;
@@ -1116,13 +1142,14 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 const float k1 = tk.x, k2 = tk.y, k3 = tk.z, y0k = gy0(NCH == 1 ? 0 : k >> 3);
                 const float Dk = k2 - k1 * (k1 / gss), Nk = k3 - k1 * gebar;
                 const float ak = Nk / Dk, Exk = Nk * ak;
-                const float kapk = sqrtf(k2 * gsee) / fabsf(Nk) + k2 / Dk;
+                const float k2e = fmaxf(k2 * gsee, 1e-37f);
+                const float kapk = __fdividef(k2e * rsqrtf(k2e), fabsf(Nk)) + __fdividef(k2, Dk);
                 const float rel = p.fit_ulps * 5.9604645e-8f * kapk;
                 const bool quick =
                     one_chunk && Dk > 1e-3f * k2 && rel * rel * Exk < 1e-9f * (gsee - Exk);
                 float eh, el, a_k = 0.0f, B_k = 0.0f, kap_k = 0.0f;
                 bool deg_k = false;
-                if (p.stats && lane == 0) atomicAdd(&p.stats[quick ? 5 : 4], 1u);
+                ev2 += quick ? 1u << 10 : 1u;
                 // (offset at q = 0 of w - cref: mean(w - cref) - a (mean zeta + J + 1))
                 float aq = ak, bq = gdbar - ak * ((y0k - kGridMagic) + k1 / gss + Jp1);
                 if (!quick) {
@@ -1240,7 +1267,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             const float gss = __shfl_sync(0xffffffffu, ss, src);
             const float gmu = __shfl_sync(0xffffffffu, mu + ebar, src);
             const int gkb = __shfl_sync(0xffffffffu, kb, src);
-            if (p.stats && lane == 0) atomicAdd(&p.stats[1], 1u);
+            ev1 += 1u << 8;
             float ga, ga_lo, gB, gB_lo;
             coop_precise<G, NCH != 1>(ws + g * G, hs + g * G, ggq, gR * p.invf[gkb], Jp1, gss, gmu, &ga,
                             &ga_lo, &gB, &gB_lo);
@@ -1269,7 +1296,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             // fast: none of these (and the folded offset)
             auto pass_c = [&](auto general) {
                 constexpr bool GEN = decltype(general)::value;
-#pragma unroll 2
+#pragma unroll (NCH == 1 ? 2 : 1)
                 for (int i = 0; i < NCHK; ++i) {
                     const int eo = eoff(i);
                     const float4 w4 = lds128(gws + eo);
@@ -1371,6 +1398,14 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 T.a[grp] = flat ? 0.0f : a_sel;
                 T.b[grp] = flat ? mn : __fadd_rn(bh, bl);
                 if (T.idx) T.idx[grp] = flat ? 0 : (uint8_t)kb;
+            }
+        }
+
+        if (p.stats && lane == 0 && (ev1 | ev2) != 0u) {
+#pragma unroll 1
+            for (int i = 0; i < 3; ++i) {
+                atomicAdd(&p.stats[i], (ev1 >> (8 * i)) & 0xFFu);
+                atomicAdd(&p.stats[4 + i], (ev2 >> (10 * i)) & 0x3FFu);
             }
         }
 
