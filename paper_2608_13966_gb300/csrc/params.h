@@ -97,8 +97,9 @@ struct IntLaunch {
 
 constexpr int kBlocksPerUnit = 32;
 
-// One tensor of an NVFP4 launch.  tensor_scale holds s_T (written before
-// the reconstruction kernel runs); unit0 as for IntTensor.
+// One tensor of an NVFP4 launch.  amax holds the tensor's absmax (supplied by
+// the caller, or its scale slot, which becomes s_T once every kernel has read
+// it); unit0 as for IntTensor.
 struct Nvfp4Tensor {
     const float* w;
     const void* g;
@@ -107,7 +108,7 @@ struct Nvfp4Tensor {
     uint8_t* codes;
     uint8_t* scale;
     uint8_t* idx;
-    const float* tensor_scale;
+    const float* amax;
     int64_t n_blocks;
     int64_t unit0;
 };
@@ -123,6 +124,7 @@ struct Nvfp4Params {
     float tie_kappa;
     int stages;
     uint32_t stage_bytes;
+    uint32_t ahead_smem;  // shared memory offset of the pass beside it
     uint64_t timeout_ns;
     uint64_t force_timeout_ns;
     unsigned int* status;  // per-device status word
@@ -197,7 +199,7 @@ struct Nvfp4Launch {
 
 // Per-tensor absmax and scale passes of a batched NVFP4 call (kernel
 // parameters): amax of w (n elements) into *slot unless amax_in is given;
-// then *slot := s_T of amax_in (or of the slot).
+// at the end *slot := s_T of amax_in (or of the slot).
 struct AmaxItem {
     const float* w;
     int64_t n;
@@ -220,7 +222,14 @@ struct AdamwItem {
     float* v;
     int64_t n;
     float* slot;
+    int64_t unit0;  // as for IntTensor, in units of kAheadUnit weights
 };
+
+// A pass beside a reconstruction: the warps a CTA has for it; for AdamW, the
+// weights a tile holds, and the tiles a warp has in its ring.
+constexpr int kAheadWarps = 4;
+constexpr int kAheadUnit = 512;
+constexpr int kAheadTiles = 2;
 
 struct AdamwHp {
     int g_kind;            // 1 fp32, 2 bf16
@@ -232,10 +241,18 @@ struct AdamwHp {
     float eps;
 };
 
+// Second parameter of an NVFP4 launch that carries nothing for a next stage.
+struct NoAheadArg {};
+
+// Tensors a stage of an NVFP4 call takes where the launch also carries the
+// next stage's tensors (both lists within the 32 KB parameter limit).
+constexpr int kMaxStage = 128;
+
 template <int MAXT>
 struct AdamwBatch {
     AdamwHp hp;
     int n_t;
+    int64_t n_units;
     AdamwItem t[MAXT];
 };
 

@@ -23,6 +23,8 @@ QUASAR_INT_ENTRY(1, 1)
 QUASAR_INT_ENTRY(2, 4) QUASAR_INT_ENTRY(2, 2) QUASAR_INT_ENTRY(2, 1)
 #undef QUASAR_INT_ENTRY
 const void* nvfp4_kernel(bool batch);
+const void* nvfp4_amax_ahead_kernel();
+const void* nvfp4_adamw_ahead_kernel();
 const void* amax_kernel(bool batch);
 const void* amax_init_kernel(bool batch);
 const void* amax_to_scale_kernel(bool batch);
@@ -328,18 +330,23 @@ quasar_status occupancy(const void* fn, size_t smem, int threads, int dev, int* 
 // spreads them over the SMs (the kernels give a CTA's first warp the first of
 // its units) instead of filling a few CTAs, whose warps would share a
 // scheduler.
+// extra_warps: warps a CTA has beside those (a fused pass of its own, which takes
+// every resident CTA); extra: that pass's parameters, the kernel's second.
 quasar_status launch_persistent(const void* fn, void* params, size_t smem, int64_t n_units,
-                                cudaStream_t stream, int warps = kWarps)
+                                cudaStream_t stream, int warps = kWarps, void* extra = nullptr,
+                                int extra_warps = 0)
 {
     int dev = 0, occ = 0;
     const DeviceInfo* info = nullptr;
     quasar_status st = device_info(&dev, &info);
     if (st != QUASAR_OK) return st;
-    if ((st = occupancy(fn, smem, warps * 32, dev, &occ)) != QUASAR_OK) return st;
+    const int threads = (warps + extra_warps) * 32;
+    if ((st = occupancy(fn, smem, threads, dev, &occ)) != QUASAR_OK) return st;
     if (occ < 1) return QUASAR_ERR_UNSUPPORTED;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)info->nsm * occ, n_units));
-    void* args[] = {params};
-    if (cudaLaunchKernel(fn, dim3(grid), dim3(warps * 32), args, smem, stream) != cudaSuccess)
+    const int64_t all = (int64_t)info->nsm * occ;
+    const int grid = (int)std::max<int64_t>(1, extra_warps ? all : std::min<int64_t>(all, n_units));
+    void* args[] = {params, extra};
+    if (cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, stream) != cudaSuccess)
         return QUASAR_ERR_CUDA;
     return QUASAR_OK;
 }
@@ -574,7 +581,8 @@ quasar_status nvfp4_tensor(const float* w, const void* g, quasar_dtype g_dtype, 
         if (outputs_alias_inputs(w, g, g_dtype, v, n, outs, bytes, 5)) return QUASAR_ERR_INVALID_ARG;
         if (tensor_amax && overlaps(tensor_amax, 4, tensor_scale, 4)) return QUASAR_ERR_INVALID_ARG;
     }
-    *T = Nvfp4Tensor{w, g, v, r, codes, block_scale, cand_idx, tensor_scale, n_blocks, 0};
+    *T = Nvfp4Tensor{w, g, v, r, codes, block_scale, cand_idx, tensor_amax ? tensor_amax : tensor_scale,
+                     n_blocks, 0};
     *A = AmaxItem{w, n, tensor_scale, tensor_amax};
     return QUASAR_OK;
 }
@@ -604,6 +612,7 @@ quasar_status nvfp4_params(bool has_g, quasar_dtype g_dtype, float beta2, const 
 template <int MAXT>
 quasar_status zero_amax_slots(const AmaxBatch<MAXT>& B, bool all, cudaStream_t s)
 {
+    static_assert(MAXT == 1 || MAXT == kMaxBatch, "the sizes the kernel is built for");
     int flag = all ? 1 : 0;
     void* args[] = {(void*)&B, (void*)&flag};
     if (cudaLaunchKernel(amax_init_kernel(MAXT > 1), dim3(1), dim3(256), args, 0, s) != cudaSuccess)
@@ -612,10 +621,11 @@ quasar_status zero_amax_slots(const AmaxBatch<MAXT>& B, bool all, cudaStream_t s
 }
 
 // Absmax of the tensors whose amax is not supplied, into their scale slots
-// (zeroed first by the caller of each slot), then every slot := s_T.
+// (zeroed first by the caller of each slot), beside nothing.
 template <int MAXT>
 quasar_status launch_amax(const AmaxBatch<MAXT>& B, cudaStream_t s)
 {
+    static_assert(MAXT == 1 || MAXT == kMaxStage, "the sizes k_amax is built for");
     int dev = 0;
     const DeviceInfo* info = nullptr;
     const quasar_status st = device_info(&dev, &info);
@@ -634,40 +644,171 @@ quasar_status launch_amax(const AmaxBatch<MAXT>& B, cudaStream_t s)
     return QUASAR_OK;
 }
 
-// amax_done: the slots already hold each tensor's absmax (the fused AdamW
-// step took it), so only the scale pass and the reconstruction remain.
+// Every slot := s_T.
 template <int MAXT>
-quasar_status nvfp4_run(Nvfp4Launch<MAXT>& Lp, AmaxBatch<MAXT>& B, int n_clip, cudaStream_t s,
-                        bool amax_done = false)
+quasar_status launch_to_scale(const AmaxBatch<MAXT>& B, cudaStream_t s)
 {
-    quasar_status st;
-    if (!amax_done) {
-        // scale slots of tensors whose amax is computed start at 0
-        bool any = false;
-        for (int i = 0; i < B.n_t; ++i) any |= !B.t[i].amax_in;
-        if (any && (st = zero_amax_slots(B, false, s)) != QUASAR_OK) return st;
-        if ((st = launch_amax(B, s)) != QUASAR_OK) return st;
-    }
-    {
-        void* args[] = {(void*)&B};
-        if (cudaLaunchKernel(amax_to_scale_kernel(MAXT > 1), dim3(1), dim3(256), args, 0, s) !=
-            cudaSuccess)
-            return QUASAR_ERR_CUDA;
-    }
+    static_assert(MAXT == 1 || MAXT == kMaxBatch, "the sizes the kernel is built for");
+    void* args[] = {(void*)&B};
+    if (cudaLaunchKernel(amax_to_scale_kernel(MAXT > 1), dim3(1), dim3(256), args, 0, s) != cudaSuccess)
+        return QUASAR_ERR_CUDA;
+    return QUASAR_OK;
+}
+
+// Number the units of a launch's tensors and plan its tiles; returns them.
+template <int MAXT>
+int64_t nvfp4_number_units(Nvfp4Launch<MAXT>& Lp, size_t* smem)
+{
     int64_t units = 0;
     for (int i = 0; i < Lp.n_t; ++i) {
         Lp.t[i].unit0 = units;
         units += (Lp.t[i].n_blocks + kBlocksPerUnit - 1) / kBlocksPerUnit;
     }
     Lp.n_units = units;
-    if (units == 0) return QUASAR_OK;
     const int gbytes = Lp.p.g_kind == 2 ? 2 : (Lp.p.g_kind == 1 ? 4 : 0);
     // one tile a warp: it is in registers, and the next copy under way, before
     // the search begins
     const Launch L = plan((uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes)), 1);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
-    return launch_persistent(nvfp4_kernel(MAXT > 1), &Lp, L.smem, units, s);
+    *smem = L.smem;
+    return units;
+}
+
+// The reconstruction of a launch's tensors, beside nothing.
+template <int MAXT>
+quasar_status nvfp4_recon(Nvfp4Launch<MAXT>& Lp, cudaStream_t s)
+{
+    size_t smem = 0;
+    const int64_t units = nvfp4_number_units(Lp, &smem);
+    if (units == 0) return QUASAR_OK;
+    NoAheadArg none;
+    return launch_persistent(nvfp4_kernel(MAXT > 1), &Lp, smem, units, s, kWarps, &none);
+}
+
+// The AdamW steps of a launch's tensors, beside nothing.
+quasar_status launch_adamw(const AdamwBatch<kMaxStage>& B, cudaStream_t s)
+{
+    int dev = 0;
+    const DeviceInfo* info = nullptr;
+    const quasar_status st = device_info(&dev, &info);
+    if (st != QUASAR_OK) return st;
+    int64_t nmax = 0;
+    for (int i = 0; i < B.n_t; ++i) nmax = std::max(nmax, B.t[i].n);
+    if (nmax == 0) return QUASAR_OK;
+    const int64_t want = (nmax / 4 + kThreads - 1) / kThreads;
+    const int64_t per = std::max<int64_t>(1, (int64_t)info->nsm * 8 / B.n_t);
+    const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(per, want));
+    void* args[] = {(void*)&B};
+    if (cudaLaunchKernel(adamw_amax_kernel(), dim3(gx, B.n_t), dim3(kThreads), args, 0, s) != cudaSuccess)
+        return QUASAR_ERR_CUDA;
+    return QUASAR_OK;
+}
+
+// A batch is cut into stages of whole tensors whose absmax (or AdamW) pass
+// runs beside the reconstruction of the stage before: about kStages of them, so
+// that little of either pass runs alone, but none smaller than kStageMin
+// weights, about 40 us of reconstruction, below which the launches' own ends
+// cost more than the overlap gives.
+constexpr int kStages = 8;
+constexpr int64_t kStageMin = int64_t(1) << 23;
+
+// The NVFP4 call over n tensors.  fill(i, T, A, W) describes tensor i (validated
+// before); hp: the AdamW step, or nullptr for none.
+template <class Fill>
+quasar_status nvfp4_batch(int n, const Fill& fill, const Nvfp4Params& p, const AdamwHp* hp, cudaStream_t s)
+{
+    // kept off the stack
+    static thread_local Nvfp4Launch<kMaxBatch> alone;
+    static thread_local Nvfp4Launch<kMaxStage> staged;
+    static thread_local AmaxBatch<kMaxBatch> slots;
+    static thread_local AmaxBatch<kMaxStage> amax;
+    static thread_local AdamwBatch<kMaxStage> adamw;
+    quasar_status st;
+    Nvfp4Tensor T;
+    AmaxItem A;
+    AdamwItem W;
+    int64_t total = 0;
+    bool ahead = false;  // some tensor needs a pass before its reconstruction
+    for (int i = 0; i < n; ++i) {
+        fill(i, &T, &A, &W);
+        total += A.n;
+        ahead |= hp != nullptr || (!A.amax_in && A.n > 0);
+    }
+    auto all_slots = [&](auto&& launch) {
+        for (int i0 = 0; i0 < n; i0 += kMaxBatch) {
+            slots.n_t = std::min(kMaxBatch, n - i0);
+            for (int i = 0; i < slots.n_t; ++i) fill(i0 + i, &T, &slots.t[i], &W);
+            if ((st = launch()) != QUASAR_OK) return st;
+        }
+        return QUASAR_OK;
+    };
+    // scale slots of tensors whose amax is computed start at 0
+    if (all_slots([&] {
+            bool any = hp != nullptr;
+            for (int i = 0; i < slots.n_t; ++i) any |= !slots.t[i].amax_in;
+            return any ? zero_amax_slots(slots, hp != nullptr, s) : QUASAR_OK;
+        }) != QUASAR_OK)
+        return st;
+    const int64_t target = std::max<int64_t>(kStageMin, total / kStages);
+    auto stage_end = [&](int i) {
+        int64_t sum = 0;
+        const int most = ahead ? kMaxStage : kMaxBatch;
+        int j = i;
+        while (j < n && j - i < most && (!ahead || sum < target)) {
+            fill(j++, &T, &A, &W);
+            sum += A.n;
+        }
+        return j;
+    };
+    // the pass of the tensors [i0, i1): described, and launched alone
+    auto describe_ahead = [&](int i0, int i1) {
+        amax.n_t = adamw.n_t = i1 - i0;
+        if (hp) adamw.hp = *hp;
+        adamw.n_units = 0;
+        for (int i = i0; i < i1; ++i) {
+            AdamwItem& w = adamw.t[i - i0];
+            fill(i, &T, &amax.t[i - i0], &w);
+            if (!hp) continue;
+            w.unit0 = adamw.n_units;
+            adamw.n_units += (w.n + kAheadUnit - 1) / kAheadUnit;
+        }
+    };
+    auto ahead_alone = [&] { return hp ? launch_adamw(adamw, s) : launch_amax(amax, s); };
+    int a0 = 0, a1 = stage_end(0);
+    if (ahead) {
+        describe_ahead(a0, a1);
+        if ((st = ahead_alone()) != QUASAR_OK) return st;
+    }
+    while (a0 < n) {
+        const int b1 = a1 < n ? stage_end(a1) : a1;
+        size_t smem = 0;
+        bool fused = false;
+        if (ahead && b1 > a1) {
+            describe_ahead(a1, b1);
+            staged.p = p;
+            staged.n_t = a1 - a0;
+            for (int i = a0; i < a1; ++i) fill(i, &staged.t[i - a0], &A, &W);
+            const int64_t units = nvfp4_number_units(staged, &smem);
+            smem = (smem + 127) & ~size_t(127);
+            staged.p.ahead_smem = (uint32_t)smem;
+            if (hp) smem += kAheadWarps * kAheadTiles * (kAheadUnit * (hp->g_kind == 2 ? 14 : 16) + 8);
+            fused = units > 0;
+            st = fused ? launch_persistent(hp ? nvfp4_adamw_ahead_kernel() : nvfp4_amax_ahead_kernel(), &staged,
+                                           smem, units, s, kWarps, hp ? (void*)&adamw : (void*)&amax, kAheadWarps)
+                       : ahead_alone();
+            if (st != QUASAR_OK) return st;
+        }
+        if (!fused) {
+            alone.p = p;
+            alone.n_t = a1 - a0;
+            for (int i = a0; i < a1; ++i) fill(i, &alone.t[i - a0], &A, &W);
+            if ((st = nvfp4_recon(alone, s)) != QUASAR_OK) return st;
+        }
+        a0 = a1;
+        a1 = b1;
+    }
+    return all_slots([&] { return launch_to_scale(slots, s); });
 }
 
 }  // namespace
@@ -845,7 +986,12 @@ quasar_status quasar_recon_nvfp4(const float* w, const void* g, quasar_dtype g_d
     Lp.n_t = B.n_t = 1;
     if ((st = nvfp4_params(g != nullptr, g_dtype, beta2, clip, n_clip, r_dtype, &Lp.p)) != QUASAR_OK)
         return st;
-    return nvfp4_run(Lp, B, n_clip, reinterpret_cast<cudaStream_t>(stream));
+    const cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
+    if (!tensor_amax &&
+        ((st = zero_amax_slots(B, false, cs)) != QUASAR_OK || (st = launch_amax(B, cs)) != QUASAR_OK))
+        return st;
+    if ((st = nvfp4_recon(Lp, cs)) != QUASAR_OK) return st;
+    return launch_to_scale(B, cs);
 }
 
 quasar_status quasar_recon_nvfp4_batch(const quasar_nvfp4_tensor* tensors, int n_tensors,
@@ -874,32 +1020,22 @@ quasar_status quasar_recon_nvfp4_batch_ex(const quasar_nvfp4_tensor* tensors, in
         }
     if (with_g != 0 && with_g != non_empty) return QUASAR_ERR_INVALID_ARG;
     const bool has_g = with_g != 0;
-    static thread_local Nvfp4Launch<kMaxBatch> Lp;  // kept off the stack
-    static thread_local AmaxBatch<kMaxBatch> B;
+    // one tensor's checks; fills its descriptors
+    auto describe = [&](int i, Nvfp4Tensor* T, AmaxItem* A) {
+        const quasar_nvfp4_tensor& x = tensors[i];
+        return nvfp4_tensor(x.w, x.g, g_dtype, x.v, beta2, clip, n_clip, x.rows, x.cols, x.tensor_amax, x.r,
+                            r_dtype, x.codes, x.block_scale, x.tensor_scale, x.cand_idx, T, A, opt.packed);
+    };
     quasar_status st;
     for (int i = 0; i < n_tensors; ++i) {  // validate everything first
-        const quasar_nvfp4_tensor& x = tensors[i];
         Nvfp4Tensor T;
         AmaxItem A;
-        if ((st = nvfp4_tensor(x.w, x.g, g_dtype, x.v, beta2, clip, n_clip, x.rows, x.cols,
-                               x.tensor_amax, x.r, r_dtype, x.codes, x.block_scale, x.tensor_scale,
-                               x.cand_idx, &T, &A, opt.packed)) != QUASAR_OK)
-            return st;
+        if ((st = describe(i, &T, &A)) != QUASAR_OK) return st;
     }
-    if ((st = nvfp4_params(has_g, g_dtype, beta2, clip, n_clip, r_dtype, &Lp.p, opt)) != QUASAR_OK)
-        return st;
-    const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    for (int i0 = 0; i0 < n_tensors; i0 += kMaxBatch) {
-        Lp.n_t = B.n_t = std::min(kMaxBatch, n_tensors - i0);
-        for (int i = 0; i < Lp.n_t; ++i) {
-            const quasar_nvfp4_tensor& x = tensors[i0 + i];
-            nvfp4_tensor(x.w, x.g, g_dtype, x.v, beta2, clip, n_clip, x.rows, x.cols, x.tensor_amax,
-                         x.r, r_dtype, x.codes, x.block_scale, x.tensor_scale, x.cand_idx, &Lp.t[i],
-                         &B.t[i], opt.packed);
-        }
-        if ((st = nvfp4_run(Lp, B, n_clip, s)) != QUASAR_OK) return st;
-    }
-    return QUASAR_OK;
+    Nvfp4Params p;
+    if ((st = nvfp4_params(has_g, g_dtype, beta2, clip, n_clip, r_dtype, &p, opt)) != QUASAR_OK) return st;
+    return nvfp4_batch(n_tensors, [&](int i, Nvfp4Tensor* T, AmaxItem* A, AdamwItem*) { describe(i, T, A); }, p,
+                       nullptr, reinterpret_cast<cudaStream_t>(stream));
 }
 
 quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_tensors,
@@ -1011,7 +1147,7 @@ quasar_status quasar_adamw_recon_nvfp4_batch(const quasar_adamw_nvfp4_tensor* te
                                         x.tensor_scale, x.cand_idx, T, A, opt.packed);
         if (s1 != QUASAR_OK) return s1;
         const int64_t n = x.rows * x.cols;
-        *W = AdamwItem{x.w, x.g, x.m, x.v, n, x.tensor_scale};
+        *W = AdamwItem{x.w, x.g, x.m, x.v, n, x.tensor_scale, 0};
         if (n == 0) return QUASAR_OK;
         if (!x.g || !x.m || !aligned16(x.g) || !aligned16(x.m)) return QUASAR_ERR_INVALID_ARG;
         const size_t nb = (size_t)n;
@@ -1029,9 +1165,6 @@ quasar_status quasar_adamw_recon_nvfp4_batch(const quasar_adamw_nvfp4_tensor* te
                 if (overlaps(state[i], sbytes[i], state[j], sbytes[j])) return QUASAR_ERR_INVALID_ARG;
         return QUASAR_OK;
     };
-    static thread_local Nvfp4Launch<kMaxBatch> Lp;
-    static thread_local AmaxBatch<kMaxBatch> B;
-    static thread_local AdamwBatch<kMaxBatch> Ad;
     quasar_status st;
     for (int i = 0; i < n_tensors; ++i) {
         Nvfp4Tensor T;
@@ -1039,45 +1172,22 @@ quasar_status quasar_adamw_recon_nvfp4_batch(const quasar_adamw_nvfp4_tensor* te
         AdamwItem W;
         if ((st = describe(tensors[i], &T, &A, &W)) != QUASAR_OK) return st;
     }
-    if ((st = nvfp4_params(false, g_dtype, beta2, clip, n_clip, r_dtype, &Lp.p, opt)) != QUASAR_OK)
-        return st;
-    {
-        const double t = (double)step;
-        AdamwHp& hp = Ad.hp;
-        hp.g_kind = g_dtype == QUASAR_BF16 ? 2 : 1;
-        hp.beta1 = beta1;
-        hp.c1b = 1.0f - beta1;
-        hp.beta2 = beta2;
-        hp.c1 = 1.0f - beta2;
-        hp.lr_wd = (float)((double)lr * (double)weight_decay);
-        hp.step_size = (float)((double)lr / (1.0 - std::pow((double)beta1, t)));
-        hp.isbc2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)beta2, t)));
-        hp.eps = eps;
-    }
-    int dev = 0;
-    const DeviceInfo* info = nullptr;
-    if ((st = device_info(&dev, &info)) != QUASAR_OK) return st;
-    const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    for (int i0 = 0; i0 < n_tensors; i0 += kMaxBatch) {
-        Lp.n_t = B.n_t = Ad.n_t = std::min(kMaxBatch, n_tensors - i0);
-        int64_t nmax = 0;
-        for (int i = 0; i < Lp.n_t; ++i) {
-            describe(tensors[i0 + i], &Lp.t[i], &B.t[i], &Ad.t[i]);
-            nmax = std::max(nmax, Ad.t[i].n);
-        }
-        if ((st = zero_amax_slots(B, true, s)) != QUASAR_OK) return st;
-        if (nmax > 0) {
-            const int64_t want = (nmax / 4 + kThreads - 1) / kThreads;
-            const int64_t per = std::max<int64_t>(1, (int64_t)info->nsm * 8 / Ad.n_t);
-            const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(per, want));
-            void* args[] = {(void*)&Ad};
-            if (cudaLaunchKernel(adamw_amax_kernel(), dim3(gx, Ad.n_t), dim3(kThreads), args, 0, s) !=
-                cudaSuccess)
-                return QUASAR_ERR_CUDA;
-        }
-        if ((st = nvfp4_run(Lp, B, n_clip, s, true)) != QUASAR_OK) return st;
-    }
-    return QUASAR_OK;
+    Nvfp4Params p;
+    if ((st = nvfp4_params(false, g_dtype, beta2, clip, n_clip, r_dtype, &p, opt)) != QUASAR_OK) return st;
+    const double t = (double)step;
+    AdamwHp hp;
+    hp.g_kind = g_dtype == QUASAR_BF16 ? 2 : 1;
+    hp.beta1 = beta1;
+    hp.c1b = 1.0f - beta1;
+    hp.beta2 = beta2;
+    hp.c1 = 1.0f - beta2;
+    hp.lr_wd = (float)((double)lr * (double)weight_decay);
+    hp.step_size = (float)((double)lr / (1.0 - std::pow((double)beta1, t)));
+    hp.isbc2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)beta2, t)));
+    hp.eps = eps;
+    return nvfp4_batch(
+        n_tensors, [&](int i, Nvfp4Tensor* T, AmaxItem* A, AdamwItem* W) { describe(tensors[i], T, A, W); }, p, &hp,
+        reinterpret_cast<cudaStream_t>(stream));
 }
 
 quasar_status quasar_get_device_status(quasar_stream_t stream)

@@ -225,8 +225,10 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         while (ti + 1 < Lp.n_t && u >= Lp.t[ti + 1].unit0) ++ti;
     };
     int ti = 0;
-    // (the units of a launch smaller than the grid's warps go to different CTAs)
-    const int64_t first = (int64_t)warp * gridDim.x + blockIdx.x;
+    // a CTA's warps take neighbouring units (their tiles share DRAM pages); in a
+    // launch with fewer units than warps, units go to different CTAs first
+    const int64_t first = n_units < (int64_t)gridDim.x * nwarps ? (int64_t)warp * gridDim.x + blockIdx.x
+                                                                : (int64_t)blockIdx.x * nwarps + warp;
     const int64_t stride = (int64_t)gridDim.x * nwarps;
 
     // the lane's 16 elements, in four chunks of 4: chunk i is block elements

@@ -37,6 +37,7 @@
 
 #include "device_common.cuh"
 #include "params.h"
+#include "recon_adamw.cuh"
 
 namespace quasar {
 
@@ -98,18 +99,56 @@ __device__ __forceinline__ void two_prod_f(float a, float b, float& p, float& e)
     e = fmaf(a, b, -p);
 }
 
-// Three CTAs an SM (80 registers) and the loop over candidates unrolled by 2:
-// 1,021 us a layer; two CTAs 1,041, no unrolling at two CTAs 1,052.
+// What the extra warps of a launch do for the next stage's tensors: nothing,
+// their absmax, or their AdamW step.
+using NoAhead = NoAheadArg;
+
+// (warp: the extra warp's number in its CTA)
+__device__ __forceinline__ void run_ahead(const NoAhead&, const Nvfp4Params&, unsigned char*, int) {}
+
 template <int MAXT>
-__global__ void __launch_bounds__(256, 3) k_recon_nvfp4(const __grid_constant__ Nvfp4Launch<MAXT> Lp)
+__device__ __forceinline__ void run_ahead(const AmaxBatch<MAXT>& B, const Nvfp4Params&, unsigned char*, int warp)
+{
+    const int64_t i = ((int64_t)blockIdx.x * kAheadWarps + warp) * 32 + (threadIdx.x & 31);
+    const int64_t stride = (int64_t)gridDim.x * kAheadWarps * 32;
+    for (int t = 0; t < B.n_t; ++t)
+        if (!B.t[t].amax_in && B.t[t].n) amax_to_slot(amax_span<4>(B.t[t].w, B.t[t].n, i, stride), B.t[t].slot);
+}
+
+template <int MAXT>
+__device__ __forceinline__ void run_ahead(const AdamwBatch<MAXT>& B, const Nvfp4Params& p, unsigned char* smem, int warp)
+{
+    const uint32_t bytes = kAheadTiles * (kAheadUnit * (B.hp.g_kind == 2 ? 14u : 16u) + 8u);
+    adamw_ring(B, smem + p.ahead_smem + warp * bytes, (int64_t)warp * gridDim.x + blockIdx.x,
+               (int64_t)gridDim.x * kAheadWarps, p.timeout_ns, p.status);
+}
+
+// The reconstruction is bound by instruction issue, and the pass that must
+// precede it (absmax, or the AdamW step) by memory, but within a tensor the one
+// needs all of the other.  So a batch is cut into stages of whole tensors, and
+// the launch of a stage carries four more warps a CTA that run the pass of the
+// next stage's tensors beside it.  58.7 M weights of AdamW beside as many of
+// reconstruction take 346 us, 6.1 TB/s (236 + 217 one after the other); one
+// layer of AdamW + NVFP4 1,394 us (1,663), absmax and NVFP4 994 (1,015).
+// Alone: three CTAs an SM (80 registers) and the loop over candidates unrolled
+// by 2: 1,021 us a layer with its absmax pass before it; two CTAs 1,041, no
+// unrolling at two CTAs 1,052.
+template <int MAXT, class AHEAD>
+__global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 384,
+                                  std::is_same<AHEAD, NoAhead>::value ? 3 : 2)
+    k_recon_nvfp4(const __grid_constant__ Nvfp4Launch<MAXT> Lp, const __grid_constant__ AHEAD ahead)
 {
     const Nvfp4Params& p = Lp.p;
     constexpr int UNIT = kBlocksPerUnit * 16;
+    constexpr int nwarps = 8;  // those that reconstruct
     extern __shared__ __align__(128) unsigned char smem[];
+    if (!std::is_same<AHEAD, NoAhead>::value && threadIdx.x >= nwarps * 32) {
+        run_ahead(ahead, p, smem, (int)(threadIdx.x >> 5) - nwarps);
+        return;
+    }
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int nwarps = blockDim.x >> 5;
     const int S = p.stages;
     unsigned char* ring = smem + (size_t)warp * S * p.stage_bytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nwarps * S * p.stage_bytes) + warp * (S + 1);
@@ -126,8 +165,12 @@ __global__ void __launch_bounds__(256, 3) k_recon_nvfp4(const __grid_constant__ 
     };
     int ti = 0, ti_s = -1;
     float sT = 1.0f, inv_sT = 1.0f;
-    // (the units of a launch smaller than the grid's warps go to different CTAs)
-    const int64_t first = (int64_t)warp * gridDim.x + blockIdx.x;
+    // a CTA's warps take neighbouring units (their tiles share DRAM pages: an
+    // attention block without gradient takes 174 us, 178 otherwise); units go to
+    // different CTAs first in a launch with fewer units than warps, and beside
+    // another pass (AdamW + NVFP4 on one layer: 1,394 us, 1,457 otherwise)
+    const bool spread = !std::is_same<AHEAD, NoAhead>::value || n_units < (int64_t)gridDim.x * nwarps;
+    const int64_t first = spread ? (int64_t)warp * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * nwarps + warp;
     const int64_t stride = (int64_t)gridDim.x * nwarps;
 
 
@@ -252,7 +295,7 @@ __global__ void __launch_bounds__(256, 3) k_recon_nvfp4(const __grid_constant__ 
         const Nvfp4Tensor& T = Lp.t[ti];
         if (ti != ti_s) {  // a new tensor: its scale s_T
             ti_s = ti;
-            sT = *T.tensor_scale;
+            sT = tensor_scale_of(*T.amax);
             inv_sT = 1.0f / sT;
         }
         const int64_t blk = (u - T.unit0) * kBlocksPerUnit + lane;
@@ -453,42 +496,6 @@ __global__ void __launch_bounds__(256, 3) k_recon_nvfp4(const __grid_constant__ 
                                              make_uint2((uint32_t)pk, (uint32_t)(pk >> 32)));
         T.scale[blk] = (uint8_t)e_sel;
         if (T.idx) T.idx[blk] = (uint8_t)kb;
-    }
-}
-
-// Tensor absmax of a batch: blockIdx.y picks the tensor; max |w| over its n
-// elements is accumulated into *slot (which must start at 0) as the bit
-// pattern of a non-negative float (such patterns order like uints).
-// Tensors whose amax is supplied are skipped.
-template <int MAXT>
-__global__ void __launch_bounds__(256) k_amax(const __grid_constant__ AmaxBatch<MAXT> B)
-{
-    const AmaxItem& it = B.t[blockIdx.y];
-    if (it.amax_in || it.n == 0) return;
-    const float* w = it.w;
-    const int64_t n = it.n;
-    float m = 0.0f;
-    const int64_t n4 = n / 4;
-    const float4* w4 = reinterpret_cast<const float4*>(w);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 x = __ldcs(w4 + i);
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
-    }
-    for (int64_t i = n4 * 4 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        m = fmaxf(m, fabsf(w[i]));
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __shared__ float red[32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0 && m > 0.0f)
-            atomicMax(reinterpret_cast<unsigned int*>(it.slot), __float_as_uint(m));
     }
 }
 

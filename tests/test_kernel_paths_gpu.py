@@ -1,0 +1,161 @@
+"""The kernels' internal paths at the sizes where they can go wrong: chunks of
+candidates, near ties of equal codes, the lookup table's element lists, signed
+NVFP4 codes, the symmetric codes' clamp sets, and launches around the number
+of CTAs that fit the device."""
+import json
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_13966_gb300 import api, quasar, workloads as wl
+from tests import checker
+from tests import gpu_harness as H
+from tests.test_parity_gpu import CLIP8, NARROW8, _assert, _edge_inputs, _inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("clip", [wl.CLIP_16[:9], wl.CLIP_PAPER, wl.CLIP_16,
+                                  tuple(1.0 - 0.02 * i for i in range(17)),
+                                  tuple(0.3 + 0.02 * i for i in range(32)),
+                                  (0.9, 0.3, 0.6, 1.0, 0.5, 0.8, 0.4, 0.7, 0.95, 0.35)],
+                         ids=["9", "paper", "16", "17", "32_up", "10_unordered"])
+@pytest.mark.parametrize("bits,G", [(2, 64), (3, 128), (4, 32), (2, 256)])
+def test_int_chunks_of_candidates(oracle, clip, bits, G):
+    """More than 8 candidates: a partial last chunk, factors in decreasing,
+    increasing and no order, degenerate groups, a ragged last unit."""
+    w, g, v = _inputs(7, 21 * G, seed=4000 + bits)
+    w[0] = 0.25                                            # zero range
+    v[1] = 0.0; g[1] = 0.0                                 # all saliency zero
+    w[3, ::2] = 0.0                                        # many exact zeros
+    w[4, 5] = 3.0                                          # one outlier
+    w[5] = torch.linspace(-1, 1, 21 * G, device="cuda")    # codes on grid boundaries
+    w[6] += 5.0                                            # far from zero
+    _assert(*H.run_int(oracle, w, g, v, bits=bits, group_size=G, clip=list(clip),
+                       r_dtype=torch.float32))
+
+
+@pytest.mark.parametrize("bits,K", [(2, 8), (2, 16), (1, 8), (3, 8)])
+def test_int_ties_between_runs_of_equal_codes(oracle, bits, K):
+    """Groups of two tight clusters and one weight between them, of a saliency
+    from far below to near the others': the candidates fall into runs of equal
+    codes, and the runs' errors differ by little beside the explained part (the
+    case where the kept candidate is picked among twins)."""
+    gen = torch.Generator(device="cuda").manual_seed(7 + bits)
+    n, G = 4096, 128
+    u = lambda *s: torch.rand(*s, generator=gen, device="cuda")
+    w = torch.where(u(n, G) < 0.5, -1.0, 1.0) * (1.0 + 1e-3 * (u(n, G) - 0.5))
+    w[:, 17] = u(n) * 1.8 - 0.9
+    v = 1e-6 * (0.5 + u(n, G))
+    v[:, 17] = 1e-6 * 10.0 ** (-9.0 * u(n))
+    _assert(*H.run_int(oracle, w, None, v, bits=bits, group_size=G, clip=list(wl.CLIP_16[:K]),
+                       r_dtype=torch.float32))
+
+
+def _lut_case(oracle, w, v, clip):
+    w_h, v_h = H._host(w), H._host(v)
+    o = api.recon_lut_batch([(w, None, v)], clip=clip, codes=True)[0]
+    torch.cuda.synchronize()
+    w2, h2 = w_h.reshape(w.shape), v_h.reshape(w.shape)
+    O = oracle.recon_lut(w2, h2, clip)
+    gpu = {"r": H._host(o["r"]), "book": o["book"].cpu().numpy(),
+           "codes": o["codes"].cpu().numpy(), "idx": o["cand_idx"].cpu().numpy()}
+    rep = checker.check_lut(oracle, w2, h2, clip, O, gpu)
+    assert rep["ok"], json.dumps(rep)
+
+
+@pytest.mark.parametrize("K", [1, 8, 9, 32])
+@pytest.mark.parametrize("kind", ["all", "one_side", "counts"])
+def test_lut_element_lists(oracle, kind, K):
+    """Blocks whose lists of elements that reach level 1 hold all 512 weights
+    (both signs, or 511 of one), or from 2 to 65 of them."""
+    clip = [round(1.0 - 0.7 * i / max(K - 1, 1), 4) for i in range(K)]
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    n = 64
+    u = lambda *s: torch.rand(*s, generator=gen, device="cuda")
+    if kind == "all":
+        x = torch.where(u(n, 512) < 0.5, -1.0, 1.0) * (0.5 + 0.5 * u(n, 512))
+    elif kind == "one_side":
+        x = 0.6 + 0.4 * u(n, 512)
+        x[:, 100] = -1.0
+    else:  # block i: i + 2 weights far out, the rest close to the centre
+        x = 0.02 * (u(n, 512) - 0.5)
+        x[:, 0], x[:, 511] = -1.0, 1.0
+        for i in range(n):
+            k = 1 + torch.randperm(510, generator=gen, device="cuda")[:i]
+            x[i, k] = torch.where(u(i) < 0.3, -1.0, 1.0) * (0.3 + 0.7 * u(i))
+    w = (0.05 * x).reshape(n, 8, 64).permute(1, 0, 2).reshape(8, n * 64).contiguous()
+    v = torch.exp(-14.0 + 2.0 * torch.randn(w.shape, generator=gen, device="cuda"))
+    _lut_case(oracle, w, v, clip)
+
+
+@pytest.mark.parametrize("K", [1, 3, 7, 9, 15])
+def test_nvfp4_signs_zeros_and_candidate_counts(oracle, K):
+    """Negative weights that round to a code of magnitude 0, zeros of either
+    sign and zero blocks: code 0 and r = +0, in every output format."""
+    clip = [round(1.0 - 0.6 * i / max(K - 1, 1), 4) for i in range(K)]
+    w, g, v = _inputs(24, 512, seed=4200 + K)
+    w[0, ::2] = -1e-9
+    w[1] = -0.0
+    w[2, ::3] = 0.0
+    _assert(*H.run_nvfp4(oracle, w.clone(), g, v.clone(), clip=clip))
+    one = api.recon_nvfp4_batch([(w, g, v.clone())], clip=clip, codes=True, r_dtype=torch.float32)[0]
+    two = api.recon_nvfp4_batch([(w, g, v.clone())], clip=clip, codes=True, packed_codes=True)[0]
+    torch.cuda.synchronize()
+    codes = one["codes"].cpu().numpy().ravel()
+    assert np.array_equal(oracle.unpack_nvfp4_codes(two["codes"].cpu().numpy()), codes)
+    assert not (codes == 8).any()
+    r = one["r"].cpu().numpy()
+    assert not np.signbit(r[r == 0]).any()
+
+
+@pytest.mark.parametrize("bits,clip", [(2, CLIP8), (3, CLIP8), (4, CLIP8), (4, NARROW8),
+                                       (3, wl.CLIP_16), (3, wl.CLIP_PAPER), (8, CLIP8)],
+                         ids=["sets8", "sets4", "sets332", "sets8_int4", "k16", "paper", "sets1"])
+@pytest.mark.parametrize("G", [32, 64, 128, 256])
+def test_sym_clamp_sets_equal_per_candidate_clamp(bits, clip, G):
+    """|w| capped once per set of candidates gives bit for bit the outputs of
+    the cap of every candidate on its own (checked against the oracle in the
+    parity tests), on ragged shapes with degenerate groups."""
+    outs = {}
+    try:
+        for hoist in (True, False):
+            quasar.quasar_debug_set_hoist(hoist)
+            items = [_edge_inputs(r, c, seed=4300 + i) for i, (r, c) in
+                     enumerate([(37, 3 * G), (8, 2 * G), (1, G)])]
+            outs[hoist] = api.recon_int_batch(items, bits=bits, group_size=G, clip=list(clip),
+                                              codes=True, symmetric=True)
+            torch.cuda.synchronize()
+    finally:
+        quasar.quasar_debug_set_hoist(True)
+    for a, b in zip(outs[True], outs[False]):
+        for key in ("r", "a", "b", "codes", "cand_idx"):
+            assert torch.equal(a[key], b[key]), key
+
+
+@pytest.mark.parametrize("units", [1, 7, 151, 153, 303, 305, 2431, 2433])
+@pytest.mark.parametrize("kind", ["int", "sym", "nvfp4", "lut"])
+def test_launches_around_the_number_of_ctas(kind, units):
+    """As many units of work as SMs, resident CTAs or warps, more or less one:
+    the outputs equal those of the same weights passed as two tensors."""
+    rows, cols = {"int": (8 * units, 32), "sym": (8 * units, 32), "nvfp4": (units, 512),
+                  "lut": (8 * units, 64)}[kind]
+    w, g, v = _inputs(rows, cols, seed=4400 + units)
+    cut = rows // 8 // 2 * 8 if kind != "nvfp4" else rows // 2
+
+    def run(items):
+        if kind == "nvfp4":
+            amax = w.abs().max().reshape(1)
+            return api.recon_nvfp4_batch([(*it, amax) for it in items], clip=CLIP8, codes=True)
+        if kind == "lut":
+            return api.recon_lut_batch(items, clip=CLIP8, codes=True)
+        return api.recon_int_batch(items, bits=3, group_size=32, clip=CLIP8, codes=True,
+                                   symmetric=kind == "sym")
+
+    whole = run([(w, g, v.clone())])[0]
+    parts = run([(w[:cut], g[:cut], v[:cut].clone()), (w[cut:], g[cut:], v[cut:].clone())])
+    torch.cuda.synchronize()
+    for key in whole:
+        if key != "tensor_scale":
+            assert torch.equal(whole[key], torch.cat([p[key] for p in parts])), key
