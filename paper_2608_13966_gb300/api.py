@@ -47,12 +47,12 @@ def recon_int(w, g, v, *, bits, group_size, clip, beta2=0.999, r_dtype=torch.bfl
     dev = w.device
     n_groups = rows * cols // group_size
     o = out if out is not None else {}
-    r = o.get("r") if o.get("r") is not None else torch.empty((rows, cols), dtype=r_dtype, device=dev)
+    r = o.get("r") if o.get("r") is not None else torch.empty_like(w, dtype=r_dtype)
     a = o.get("a") if o.get("a") is not None else torch.empty(n_groups, dtype=torch.float32, device=dev)
     b = o.get("b") if o.get("b") is not None else torch.empty(n_groups, dtype=torch.float32, device=dev)
     c = None
     if codes:
-        c = o.get("codes") if o.get("codes") is not None else torch.empty((rows, cols), dtype=torch.uint8, device=dev)
+        c = o.get("codes") if o.get("codes") is not None else torch.empty_like(w, dtype=torch.uint8)
     k = None
     if cand_idx:
         k = o.get("cand_idx") if o.get("cand_idx") is not None else torch.empty(n_groups, dtype=torch.uint8, device=dev)
@@ -66,10 +66,10 @@ def recon_int(w, g, v, *, bits, group_size, clip, beta2=0.999, r_dtype=torch.bfl
     return res
 
 
-def _int_codes(rows, cols, bits, packed, dev):
+def _int_codes(w, bits, packed):
     if packed:  # the group bitstreams: rows*cols*bits/8 bytes
-        return torch.empty(rows * cols * bits // 8, dtype=torch.uint8, device=dev)
-    return torch.empty((rows, cols), dtype=torch.uint8, device=dev)
+        return torch.empty(w.numel() * bits // 8, dtype=torch.uint8, device=w.device)
+    return torch.empty_like(w, dtype=torch.uint8)
 
 
 def recon_int_batch(items, *, bits, group_size, clip, beta2=0.999, r_dtype=torch.bfloat16,
@@ -90,11 +90,11 @@ def recon_int_batch(items, *, bits, group_size, clip, beta2=0.999, r_dtype=torch
         rows, cols = w.shape
         dev = w.device
         n_groups = rows * cols // group_size
-        res = {"r": torch.empty((rows, cols), dtype=r_dtype, device=dev),
+        res = {"r": torch.empty_like(w, dtype=r_dtype),
                "a": torch.empty(n_groups, dtype=torch.float32, device=dev),
                "b": torch.empty(n_groups, dtype=torch.float32, device=dev)}
         if codes:
-            res["codes"] = _int_codes(rows, cols, bits, packed_codes, dev)
+            res["codes"] = _int_codes(w, bits, packed_codes)
         if cand_idx:
             res["cand_idx"] = torch.empty(n_groups, dtype=torch.uint8, device=dev)
         if g is not None and g.dtype == torch.bfloat16:
@@ -126,11 +126,11 @@ def adamw_recon_int_batch(items, *, lr, step, bits, group_size, clip, beta1=0.9,
         rows, cols = w.shape
         dev = w.device
         n_groups = rows * cols // group_size
-        res = {"r": torch.empty((rows, cols), dtype=r_dtype, device=dev),
+        res = {"r": torch.empty_like(w, dtype=r_dtype),
                "a": torch.empty(n_groups, dtype=torch.float32, device=dev),
                "b": torch.empty(n_groups, dtype=torch.float32, device=dev)}
         if codes:
-            res["codes"] = _int_codes(rows, cols, bits, packed_codes, dev)
+            res["codes"] = _int_codes(w, bits, packed_codes)
         if cand_idx:
             res["cand_idx"] = torch.empty(n_groups, dtype=torch.uint8, device=dev)
         if g is not None and g.dtype == torch.bfloat16:
@@ -155,12 +155,12 @@ def recon_nvfp4(w, g, v, *, clip, beta2=0.999, tensor_amax=None, r_dtype=torch.b
     dev = w.device
     n_blocks = rows * cols // 16
     o = out if out is not None else {}
-    r = o.get("r") if o.get("r") is not None else torch.empty((rows, cols), dtype=r_dtype, device=dev)
+    r = o.get("r") if o.get("r") is not None else torch.empty_like(w, dtype=r_dtype)
     sc = o.get("block_scale") if o.get("block_scale") is not None else torch.empty(n_blocks, dtype=torch.uint8, device=dev)
     ts = o.get("tensor_scale") if o.get("tensor_scale") is not None else torch.empty(1, dtype=torch.float32, device=dev)
     c = None
     if codes:
-        c = o.get("codes") if o.get("codes") is not None else torch.empty((rows, cols), dtype=torch.uint8, device=dev)
+        c = o.get("codes") if o.get("codes") is not None else torch.empty_like(w, dtype=torch.uint8)
     k = None
     if cand_idx:
         k = o.get("cand_idx") if o.get("cand_idx") is not None else torch.empty(n_blocks, dtype=torch.uint8, device=dev)
@@ -190,12 +190,12 @@ def recon_nvfp4_batch(items, *, clip, beta2=0.999, r_dtype=torch.bfloat16, codes
         rows, cols = w.shape
         dev = w.device
         n_blocks = rows * cols // 16
-        res = {"r": torch.empty((rows, cols), dtype=r_dtype, device=dev),
+        res = {"r": torch.empty_like(w, dtype=r_dtype),
                "block_scale": torch.empty(n_blocks, dtype=torch.uint8, device=dev),
                "tensor_scale": torch.empty(1, dtype=torch.float32, device=dev)}
         if codes:
             res["codes"] = (torch.empty(rows * cols // 2, dtype=torch.uint8, device=dev) if packed_codes
-                            else torch.empty((rows, cols), dtype=torch.uint8, device=dev))
+                            else torch.empty_like(w, dtype=torch.uint8))
         if cand_idx:
             res["cand_idx"] = torch.empty(n_blocks, dtype=torch.uint8, device=dev)
         if g is not None and g.dtype == torch.bfloat16:
@@ -226,12 +226,12 @@ def adamw_recon_nvfp4_batch(items, *, lr, step, clip, beta1=0.9, beta2=0.999, ep
         rows, cols = w.shape
         dev = w.device
         n_blocks = rows * cols // 16
-        res = {"r": torch.empty((rows, cols), dtype=r_dtype, device=dev),
+        res = {"r": torch.empty_like(w, dtype=r_dtype),
                "block_scale": torch.empty(n_blocks, dtype=torch.uint8, device=dev),
                "tensor_scale": torch.empty(1, dtype=torch.float32, device=dev)}
         if codes:
             res["codes"] = (torch.empty(rows * cols // 2, dtype=torch.uint8, device=dev) if packed_codes
-                            else torch.empty((rows, cols), dtype=torch.uint8, device=dev))
+                            else torch.empty_like(w, dtype=torch.uint8))
         if cand_idx:
             res["cand_idx"] = torch.empty(n_blocks, dtype=torch.uint8, device=dev)
         if g is not None and g.dtype == torch.bfloat16:
@@ -261,11 +261,11 @@ def recon_lut_batch(items, *, clip, beta2=0.999, r_dtype=torch.bfloat16, codes=F
         rows, cols = w.shape
         dev = w.device
         n_blocks = rows * cols // 512
-        res = {"r": torch.empty((rows, cols), dtype=r_dtype, device=dev),
+        res = {"r": torch.empty_like(w, dtype=r_dtype),
                "book": torch.empty((n_blocks, 8), dtype=torch.uint8, device=dev)}
         if codes:
             res["codes"] = (torch.empty(n_blocks * 192, dtype=torch.uint8, device=dev) if packed_codes
-                            else torch.empty((rows, cols), dtype=torch.uint8, device=dev))
+                            else torch.empty_like(w, dtype=torch.uint8))
         if cand_idx:
             res["cand_idx"] = torch.empty(n_blocks, dtype=torch.uint8, device=dev)
         if g is not None and g.dtype == torch.bfloat16:

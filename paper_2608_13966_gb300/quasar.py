@@ -10,7 +10,9 @@ from __future__ import annotations
 
 import ctypes
 import enum
+import functools
 import os
+import struct
 import threading
 
 from . import build as _build
@@ -25,6 +27,9 @@ class QuasarStatus(enum.IntEnum):
     ERR_UNSUPPORTED = 2
     ERR_CUDA = 3
     ERR_TIMEOUT = 4
+
+
+_STATUS = tuple(QuasarStatus)  # by value: indexing is cheaper than the enum call
 
 
 class QuasarError(RuntimeError):
@@ -120,9 +125,15 @@ def _stream(stream):
     return stream.cuda_stream
 
 
+@functools.lru_cache(maxsize=64)
+def _clip_floats(values):
+    """The C array of a tuple of floats (the library only reads it)."""
+    return (ctypes.c_float * len(values))(*values)
+
+
 def _clip_array(clip):
-    arr = (ctypes.c_float * len(clip))(*[float(c) for c in clip])
-    return arr, len(clip)
+    values = tuple(map(float, clip))
+    return _clip_floats(values), len(values)
 
 
 def quasar_recon_int(w, g, v, beta2, bits, group_size, clip, rows, cols, r, codes, a, b,
@@ -134,7 +145,19 @@ def quasar_recon_int(w, g, v, beta2, bits, group_size, clip, rows, cols, r, code
     st = lib.quasar_recon_int(_ptr(w), _ptr(g), gd, _ptr(v), beta2, bits, group_size, carr, nclip,
                               rows, cols, _ptr(r), rd, _ptr(codes), _ptr(a), _ptr(b),
                               _ptr(cand_idx), _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
+
+
+def _pack(cls, items, keys):
+    """A ctypes array of the descriptor cls from dicts: the pointers named by
+    keys (missing or None: NULL), then rows and cols, packed straight into the
+    array's memory (every field is 8 bytes)."""
+    arr = (cls * len(items))()
+    row = struct.Struct(f"={len(keys)}Q2q")
+    for i, d in enumerate(items):
+        row.pack_into(arr, i * row.size, *[_ptr(d.get(k)) or 0 for k in keys], int(d["rows"]),
+                      int(d["cols"]))
+    return arr
 
 
 class QuasarIntTensor(ctypes.Structure):
@@ -148,12 +171,7 @@ class QuasarIntTensor(ctypes.Structure):
 def int_tensor_array(items):
     """A ctypes array of QuasarIntTensor from dicts with keys w, g, v, r,
     codes, a, b, cand_idx (tensors, pointers or None), rows, cols."""
-    arr = (QuasarIntTensor * len(items))()
-    for i, d in enumerate(items):
-        arr[i] = QuasarIntTensor(_ptr(d["w"]), _ptr(d.get("g")), _ptr(d["v"]), _ptr(d["r"]),
-                                 _ptr(d.get("codes")), _ptr(d["a"]), _ptr(d["b"]),
-                                 _ptr(d.get("cand_idx")), int(d["rows"]), int(d["cols"]))
-    return arr
+    return _pack(QuasarIntTensor, items, ("w", "g", "v", "r", "codes", "a", "b", "cand_idx"))
 
 
 def quasar_recon_int_batch(tensors, beta2, bits, group_size, clip, g_dtype=BF16, r_dtype=BF16,
@@ -163,9 +181,9 @@ def quasar_recon_int_batch(tensors, beta2, bits, group_size, clip, g_dtype=BF16,
     if not isinstance(tensors, ctypes.Array):
         tensors = int_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_recon_int_batch(ctypes.cast(tensors, ctypes.c_void_p), len(tensors), g_dtype,
+    st = lib.quasar_recon_int_batch(tensors, len(tensors), g_dtype,
                                     beta2, bits, group_size, carr, nclip, r_dtype, _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 # quasar_saliency / quasar_codes_layout
@@ -191,7 +209,7 @@ def options(saliency="ema", packed_codes=False, symmetric=False):
 
 
 def _opt_ptr(opt):
-    return None if opt is None else ctypes.cast(ctypes.pointer(opt), ctypes.c_void_p)
+    return None if opt is None else ctypes.byref(opt)
 
 
 def quasar_recon_int_batch_ex(tensors, beta2, bits, group_size, clip, options=None, g_dtype=BF16,
@@ -201,10 +219,10 @@ def quasar_recon_int_batch_ex(tensors, beta2, bits, group_size, clip, options=No
     if not isinstance(tensors, ctypes.Array):
         tensors = int_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_recon_int_batch_ex(ctypes.cast(tensors, ctypes.c_void_p), len(tensors), g_dtype,
+    st = lib.quasar_recon_int_batch_ex(tensors, len(tensors), g_dtype,
                                        beta2, bits, group_size, carr, nclip, r_dtype,
                                        _opt_ptr(options), _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 class QuasarAdamwTensor(ctypes.Structure):
@@ -218,12 +236,7 @@ class QuasarAdamwTensor(ctypes.Structure):
 def adamw_tensor_array(items):
     """A ctypes array of QuasarAdamwTensor from dicts with keys w, g, m, v,
     r, codes, a, b, cand_idx (tensors, pointers or None), rows, cols."""
-    arr = (QuasarAdamwTensor * len(items))()
-    for i, d in enumerate(items):
-        arr[i] = QuasarAdamwTensor(_ptr(d["w"]), _ptr(d.get("g")), _ptr(d.get("m")), _ptr(d["v"]),
-                                   _ptr(d["r"]), _ptr(d.get("codes")), _ptr(d["a"]), _ptr(d["b"]),
-                                   _ptr(d.get("cand_idx")), int(d["rows"]), int(d["cols"]))
-    return arr
+    return _pack(QuasarAdamwTensor, items, ("w", "g", "m", "v", "r", "codes", "a", "b", "cand_idx"))
 
 
 def quasar_adamw_recon_int_batch(tensors, lr, beta1, beta2, eps, weight_decay, step, bits,
@@ -234,11 +247,11 @@ def quasar_adamw_recon_int_batch(tensors, lr, beta1, beta2, eps, weight_decay, s
     if not isinstance(tensors, ctypes.Array):
         tensors = adamw_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_adamw_recon_int_batch(ctypes.cast(tensors, ctypes.c_void_p), len(tensors),
+    st = lib.quasar_adamw_recon_int_batch(tensors, len(tensors),
                                           g_dtype, lr, beta1, beta2, eps, weight_decay, step,
                                           bits, group_size, carr, nclip, r_dtype,
                                           _opt_ptr(options), _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 class QuasarNvfp4Tensor(ctypes.Structure):
@@ -253,13 +266,7 @@ class QuasarNvfp4Tensor(ctypes.Structure):
 def nvfp4_tensor_array(items):
     """A ctypes array of QuasarNvfp4Tensor from dicts with keys w, g, v,
     tensor_amax, r, codes, block_scale, tensor_scale, cand_idx, rows, cols."""
-    arr = (QuasarNvfp4Tensor * len(items))()
-    for i, d in enumerate(items):
-        arr[i] = QuasarNvfp4Tensor(_ptr(d["w"]), _ptr(d.get("g")), _ptr(d["v"]),
-                                   _ptr(d.get("tensor_amax")), _ptr(d["r"]), _ptr(d.get("codes")),
-                                   _ptr(d["block_scale"]), _ptr(d["tensor_scale"]),
-                                   _ptr(d.get("cand_idx")), int(d["rows"]), int(d["cols"]))
-    return arr
+    return _pack(QuasarNvfp4Tensor, items, ("w", "g", "v", "tensor_amax", "r", "codes", "block_scale", "tensor_scale", "cand_idx"))
 
 
 def quasar_recon_nvfp4_batch(tensors, beta2, clip, g_dtype=BF16, r_dtype=BF16,
@@ -269,9 +276,9 @@ def quasar_recon_nvfp4_batch(tensors, beta2, clip, g_dtype=BF16, r_dtype=BF16,
     if not isinstance(tensors, ctypes.Array):
         tensors = nvfp4_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_recon_nvfp4_batch(ctypes.cast(tensors, ctypes.c_void_p), len(tensors), g_dtype,
+    st = lib.quasar_recon_nvfp4_batch(tensors, len(tensors), g_dtype,
                                       beta2, carr, nclip, r_dtype, _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 def quasar_recon_nvfp4_batch_ex(tensors, beta2, clip, options=None, g_dtype=BF16, r_dtype=BF16,
@@ -281,10 +288,10 @@ def quasar_recon_nvfp4_batch_ex(tensors, beta2, clip, options=None, g_dtype=BF16
     if not isinstance(tensors, ctypes.Array):
         tensors = nvfp4_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_recon_nvfp4_batch_ex(ctypes.cast(tensors, ctypes.c_void_p), len(tensors),
+    st = lib.quasar_recon_nvfp4_batch_ex(tensors, len(tensors),
                                          g_dtype, beta2, carr, nclip, r_dtype, _opt_ptr(options),
                                          _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 class QuasarAdamwNvfp4Tensor(ctypes.Structure):
@@ -298,13 +305,7 @@ class QuasarAdamwNvfp4Tensor(ctypes.Structure):
 def adamw_nvfp4_tensor_array(items):
     """A ctypes array of QuasarAdamwNvfp4Tensor from dicts with keys w, g, m,
     v, r, codes, block_scale, tensor_scale, cand_idx, rows, cols."""
-    arr = (QuasarAdamwNvfp4Tensor * len(items))()
-    for i, d in enumerate(items):
-        arr[i] = QuasarAdamwNvfp4Tensor(
-            _ptr(d["w"]), _ptr(d.get("g")), _ptr(d.get("m")), _ptr(d["v"]), _ptr(d["r"]),
-            _ptr(d.get("codes")), _ptr(d["block_scale"]), _ptr(d["tensor_scale"]),
-            _ptr(d.get("cand_idx")), int(d["rows"]), int(d["cols"]))
-    return arr
+    return _pack(QuasarAdamwNvfp4Tensor, items, ("w", "g", "m", "v", "r", "codes", "block_scale", "tensor_scale", "cand_idx"))
 
 
 def quasar_adamw_recon_nvfp4_batch(tensors, lr, beta1, beta2, eps, weight_decay, step, clip,
@@ -315,11 +316,11 @@ def quasar_adamw_recon_nvfp4_batch(tensors, lr, beta1, beta2, eps, weight_decay,
     if not isinstance(tensors, ctypes.Array):
         tensors = adamw_nvfp4_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_adamw_recon_nvfp4_batch(ctypes.cast(tensors, ctypes.c_void_p), len(tensors),
+    st = lib.quasar_adamw_recon_nvfp4_batch(tensors, len(tensors),
                                             g_dtype, lr, beta1, beta2, eps, weight_decay, step,
                                             carr, nclip, r_dtype, _opt_ptr(options),
                                             _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 class QuasarLutTensor(ctypes.Structure):
@@ -332,12 +333,7 @@ class QuasarLutTensor(ctypes.Structure):
 def lut_tensor_array(items):
     """A ctypes array of QuasarLutTensor from dicts with keys w, g, v, r,
     codes, book, cand_idx (tensors, pointers or None), rows, cols."""
-    arr = (QuasarLutTensor * len(items))()
-    for i, d in enumerate(items):
-        arr[i] = QuasarLutTensor(_ptr(d["w"]), _ptr(d.get("g")), _ptr(d["v"]), _ptr(d["r"]),
-                                 _ptr(d.get("codes")), _ptr(d["book"]), _ptr(d.get("cand_idx")),
-                                 int(d["rows"]), int(d["cols"]))
-    return arr
+    return _pack(QuasarLutTensor, items, ("w", "g", "v", "r", "codes", "book", "cand_idx"))
 
 
 def quasar_recon_lut_batch(tensors, beta2, clip, options=None, g_dtype=BF16, r_dtype=BF16,
@@ -347,9 +343,9 @@ def quasar_recon_lut_batch(tensors, beta2, clip, options=None, g_dtype=BF16, r_d
     if not isinstance(tensors, ctypes.Array):
         tensors = lut_tensor_array(tensors)
     carr, nclip = _clip_array(clip)
-    st = lib.quasar_recon_lut_batch(ctypes.cast(tensors, ctypes.c_void_p), len(tensors), g_dtype,
+    st = lib.quasar_recon_lut_batch(tensors, len(tensors), g_dtype,
                                     beta2, carr, nclip, r_dtype, _opt_ptr(options), _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 def quasar_recon_nvfp4(w, g, v, beta2, clip, rows, cols, tensor_amax, r, codes, block_scale,
@@ -362,15 +358,15 @@ def quasar_recon_nvfp4(w, g, v, beta2, clip, rows, cols, tensor_amax, r, codes, 
     st = lib.quasar_recon_nvfp4(_ptr(w), _ptr(g), gd, _ptr(v), beta2, carr, nclip, rows, cols,
                                 _ptr(tensor_amax), _ptr(r), rd, _ptr(codes), _ptr(block_scale),
                                 _ptr(tensor_scale), _ptr(cand_idx), _stream(stream))
-    return QuasarStatus(st)
+    return _STATUS[st]
 
 
 def quasar_tensor_amax(w, n, amax_out, stream=None) -> QuasarStatus:
-    return QuasarStatus(load().quasar_tensor_amax(_ptr(w), n, _ptr(amax_out), _stream(stream)))
+    return _STATUS[load().quasar_tensor_amax(_ptr(w), n, _ptr(amax_out), _stream(stream))]
 
 
 def quasar_get_device_status(stream=None) -> QuasarStatus:
-    return QuasarStatus(load().quasar_get_device_status(_stream(stream)))
+    return _STATUS[load().quasar_get_device_status(_stream(stream))]
 
 
 def quasar_debug_force_timeout(nanoseconds: int) -> None:
