@@ -159,6 +159,7 @@ struct LutTensor {
     int64_t cols;
     int64_t n_blocks;
     int64_t unit0;
+    uint32_t nbc, nbc_inv;  // blocks a row of blocks, and floor(2^32 / nbc)
 };
 
 struct LutParams {

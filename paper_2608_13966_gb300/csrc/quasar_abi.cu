@@ -1075,7 +1075,9 @@ quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_ten
             if (outputs_alias_inputs(x.w, x.g, g_dtype, x.v, n, outs, bytes, 4))
                 return QUASAR_ERR_INVALID_ARG;
         }
-        *T = LutTensor{x.w, x.g, x.v, x.r, x.codes, x.book, x.cand_idx, x.cols, n_blocks, 0};
+        const uint64_t nbc = (uint64_t)std::max<int64_t>(1, x.cols / kLutCols);
+        *T = LutTensor{x.w, x.g, x.v, x.r, x.codes, x.book, x.cand_idx, x.cols, n_blocks, 0, (uint32_t)nbc,
+                       (uint32_t)std::min<uint64_t>(UINT32_MAX, (uint64_t(1) << 32) / nbc)};
         return QUASAR_OK;
     };
     static thread_local LutLaunch<kMaxBatch> Lp;

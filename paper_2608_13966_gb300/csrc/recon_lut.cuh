@@ -224,7 +224,6 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     auto tensor_of = [&](int64_t u, int& ti) {
         while (ti + 1 < Lp.n_t && u >= Lp.t[ti + 1].unit0) ++ti;
     };
-    int ti = 0;
     // a CTA's warps take neighbouring units (their tiles share DRAM pages); in a
     // launch with fewer units than warps, units go to different CTAs first
     const int64_t first = n_units < (int64_t)gridDim.x * nwarps ? (int64_t)warp * gridDim.x + blockIdx.x
@@ -236,20 +235,25 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     // (consecutive lanes on consecutive 16-byte pieces, in the tile and in
     // memory); the offset of chunk 0 in the tensor
     auto lane_offset = [&](const LutTensor& T, uint32_t b) {
-        // block row and column (a tensor holds fewer than 2^32 blocks)
-        const uint32_t nbc = (uint32_t)(T.cols / kLutCols);
-        const uint32_t brow = b / nbc;
-        return ((int64_t)brow * kLutRows + (lane >> 4)) * T.cols + (int64_t)(b - brow * nbc) * kLutCols +
-               (lane & 15) * 4;
+        // block row and column (a tensor holds fewer than 2^32 blocks): the
+        // quotient by the divisor's reciprocal is at most one too small
+        uint32_t brow = __umulhi(b, T.nbc_inv), bcol = b - brow * T.nbc;
+        if (bcol >= T.nbc) {
+            ++brow;
+            bcol -= T.nbc;
+        }
+        return ((int64_t)brow * kLutRows + (lane >> 4)) * T.cols + (int64_t)bcol * kLutCols + (lane & 15) * 4;
     };
     // Copy a block into the tile: every lane copies the pieces that it will
     // read itself, so its own wait is all that orders them.  (24 row segments
     // a block as bulk copies took an eighth of the kernel to issue.)
+    int ti_next = 0;       // the tensor of the block in flight, and the lane's
+    int64_t off_next = 0;  // offset in it
     auto issue = [&](int64_t u) {
-        int tj = ti;
-        tensor_of(u, tj);
-        const LutTensor& T = Lp.t[tj];
+        tensor_of(u, ti_next);
+        const LutTensor& T = Lp.t[ti_next];
         const int64_t off = lane_offset(T, (uint32_t)(u - T.unit0)), step = 2 * T.cols;
+        off_next = off;
         const uint32_t d = smem_u32(st) + lane * 16;
         const float* w = T.w + off;
         const float* v = T.v + off;
@@ -298,10 +302,9 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
 
     for (int64_t u = first; u < n_units; u += stride) {
         cp_async_wait_all();
-        tensor_of(u, ti);
-        const LutTensor& T = Lp.t[ti];
+        const LutTensor& T = Lp.t[ti_next];
         const uint32_t b = (uint32_t)(u - T.unit0);
-        const int64_t gofs = lane_offset(T, b);
+        const int64_t gofs = off_next;
         const int64_t gstep = 2 * T.cols;  // from one chunk of the lane to the next
 
         // ---- pass A: w, the saliency EMA (v' out), the fit's saliency h
@@ -408,8 +411,21 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         }
         __syncwarp();
 
+        // indices of chunk i's 4 elements on the grid of P, a nibble each: level m =
+        // min(floor(|d| P), 3) from the low bits of the floor on the 2^23 grid;
+        // 4 + m (d >= 0) is m ^ 4 and 3 - m (d < 0) is m ^ 3
+        auto indices = [&](int i, float P) {
+            const float2 P2 = make_float2(P, P);
+            const float2 ya = __ffma2_rd(ad2[2 * i], P2, M2), yb = __ffma2_rd(ad2[2 * i + 1], P2, M2);
+            const uint32_t m0 = __float_as_uint(fminf(ya.x, kMagic + 3.0f)), m1 = __float_as_uint(fminf(ya.y, kMagic + 3.0f));
+            const uint32_t m2 = __float_as_uint(fminf(yb.x, kMagic + 3.0f)), m3 = __float_as_uint(fminf(yb.y, kMagic + 3.0f));
+            const uint32_t ng = negm >> (4 * i);
+            const uint32_t sx = (ng & 1u) | ((ng & 2u) << 3) | ((ng & 4u) << 6) | ((ng & 8u) << 9);
+            return ((m0 + (m1 << 4) + (m2 << 8) + (m3 << 12)) ^ 0x4444u ^ (sx * 7u)) & 0x7777u;
+        };
         int kb = 0;
         if (!flat) {
+            float2 xh[8];  // the lane's h, loaded again where an exact look needs it
             // ---- the elements that reach level 1 for some factor: an element
             // with |d| P < 1 for every factor adds to no threshold sum.  The
             // others (about a quarter of a heavy-tailed block, a half of a
@@ -637,94 +653,96 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 __syncwarp();
             }
 
-            // the lane's h again, for the settling steps (from the tensor: they
-            // are rare, and h would take 16 registers through the common path)
-            float2 xh[8];
-            if (set != 0u || camb[kb] != 0u) {
+            // candidates to settle: those within the bound of the winner, or the
+            // winner alone where its table is undecided
+            unsigned todo = set ? set | (1u << kb) : (camb[kb] ? 1u << kb : 0u);
+            if (todo) {
+                // the lane's h again (from the tensor: it would take 16 registers
+                // through the common path)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float4 v4 = *reinterpret_cast<const float4*>(T.v + gofs + i * gstep);
-                    float2 hh[2] = {make_float2(v4.x, v4.y), make_float2(v4.z, v4.w)};
+                    xh[2 * i] = make_float2(v4.x, v4.y);
+                    xh[2 * i + 1] = make_float2(v4.z, v4.w);
+                }
+                if (p.h_mode != kSalEma || h_one || ts1 != 1.0f || ts2 != 1.0f) {
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        if (p.h_mode == kSalEmaSquared) hh[t] = __fmul2_rn(hh[t], hh[t]);
-                        if (p.h_mode == kSalUniform || h_one) hh[t] = make_float2(1.0f, 1.0f);
-                        xh[2 * i + t] = __fmul2_rn(__fmul2_rn(hh[t], make_float2(ts1, ts1)), make_float2(ts2, ts2));
+                    for (int t = 0; t < 8; ++t) {
+                        if (p.h_mode == kSalEmaSquared) xh[t] = __fmul2_rn(xh[t], xh[t]);
+                        if (p.h_mode == kSalUniform || h_one) xh[t] = make_float2(1.0f, 1.0f);
+                        xh[t] = __fmul2_rn(__fmul2_rn(xh[t], make_float2(ts1, ts1)), make_float2(ts2, ts2));
                     }
                 }
             }
-
-            // index (0..7) of element i for the grid of P
-            auto index_of = [&](int i, float P) {
-                const float a = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
-                const float mf = fminf(__fmaf_rd(a, P, kMagic) - kMagic, 3.0f);
-                const int mi = (int)mf;
-                return ((negm >> i) & 1u) ? 3 - mi : 4 + mi;
-            };
-            // Undecided entries of candidate k from direct per-index sums
-            // (fp32, nonnegative exact terms, 16 + 5 levels: relative error
-            // within 24 ulps): settled (table updated) unless a rounding is
-            // still undecided.
-            auto refine = [&](int k) -> bool {
-                const float P = R * p.invf[k];
+            // Undecided entries from direct per-index sums (fp32, nonnegative
+            // exact terms, 16 + 5 levels: relative error within 24 ulps): settled
+            // (table updated) unless a rounding is still undecided.
+            bool decided = true;
+#pragma unroll 1
+            for (unsigned s2 = todo; s2; s2 &= s2 - 1) {
+                const int k = __ffs(s2) - 1;
                 uint32_t und = camb[k];
+                if (und == 0u) continue;
+                const float P = R * p.invf[k];
+                uint32_t qs[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) qs[i] = indices(i, P);
+                bool ok = true;
                 uint32_t w0 = cbook[2 * k], w1 = cbook[2 * k + 1];
+#pragma unroll 1
                 while (und) {
                     const int j = __ffs(und) - 1;
                     und &= und - 1;
                     float Hs = 0.0f, Xs = 0.0f;
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        if (index_of(i, P) == j) {
+                        if (((qs[i >> 2] >> (4 * (i & 3))) & 0xFu) == (uint32_t)j) {
                             const float hv = (i & 1) ? xh[i >> 1].y : xh[i >> 1].x;
                             const float av = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
                             Hs += hv;
                             Xs = fmaf(hv, av, Xs);
                         }
                     }
-#pragma unroll
+#pragma unroll 1
                     for (int o = 16; o; o >>= 1) {
                         Hs += __shfl_xor_sync(0xffffffffu, Hs, o);
                         Xs += __shfl_xor_sync(0xffffffffu, Xs, o);
                     }
                     Hs = __shfl_sync(0xffffffffu, Hs, 0);
                     Xs = __shfl_sync(0xffffffffu, Xs, 0);
-                    uint32_t cbj;
-                    if (!(Hs > 0.0f)) {
-                        // no weight of nonzero saliency: the grid point
-                        cbj = e4m3_encode(fmaf((float)j - 3.5f, __fdividef(1.0f, P), c));
-                    } else {
+                    // no weight of nonzero saliency: the grid point
+                    float mean = fmaf((float)j - 3.5f, __fdividef(1.0f, P), c), dm = 0.0f;
+                    if (Hs > 0.0f) {
                         const float q = Xs / Hs;
-                        const float mean = fmaf(j >= 4 ? 1.0f : -1.0f, q, c);
+                        mean = fmaf(j >= 4 ? 1.0f : -1.0f, q, c);
                         // two sums (24 ulps each), the quotient, w - c (an ulp
                         // a term), the mean's sum
-                        const float dm = 52.0f * kU * q + 2.0f * kU * fabsf(mean);
-                        if (e4m3_encode(mean - dm) != e4m3_encode(mean + dm)) return false;
-                        cbj = e4m3_encode(mean);
+                        dm = 52.0f * kU * q + 2.0f * kU * fabsf(mean);
                     }
-                    if (j < 4) w0 = (w0 & ~(0xFFu << (8 * j))) | (cbj << (8 * j));
-                    else w1 = (w1 & ~(0xFFu << (8 * (j - 4)))) | (cbj << (8 * (j - 4)));
+                    const float2 lh = e4m3_decode2(e4m3_encode2(mean - dm, mean + dm));
+                    if (lh.x != lh.y) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t cbj = e4m3_encode(mean), sh = 8 * (j & 3);
+                    if (j < 4) w0 = (w0 & ~(0xFFu << sh)) | (cbj << sh);
+                    else w1 = (w1 & ~(0xFFu << sh)) | (cbj << sh);
                 }
                 __syncwarp();
-                if (lane == 0) {
+                if (!ok) {
+                    decided = false;
+                } else if (lane == 0) {
                     cbook[2 * k] = w0;
                     cbook[2 * k + 1] = w1;
                     camb[k] = 0u;
                 }
                 __syncwarp();
-                return true;
-            };
+            }
 
             if (set == 0u) {
-                // the winner alone: its table must be decided
-                if (camb[kb] && !refine(kb)) set = 1u << kb;
+                if (!decided) set = todo;
             } else {
-                set |= 1u << kb;
-                bool decided = true;
-                for (unsigned s2 = set; s2; s2 &= s2 - 1) {
-                    const int k = __ffs(s2) - 1;
-                    if (camb[k] && !refine(k)) decided = false;
-                }
+                set = todo;
                 if (decided) {
                     // direct fp32 errors sum h (C_q - w)^2 of the candidates
                     // left (terms within 3 ulps, 21 levels: 32 ulps in all)
@@ -738,6 +756,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                         xwv[4 * i + 2] = w4.z;
                         xwv[4 * i + 3] = w4.w;
                     }
+#pragma unroll 1
                     for (unsigned s2 = set; s2; s2 &= s2 - 1) {
                         const int k = __ffs(s2) - 1;
                         const float P = R * p.invf[k];
@@ -746,12 +765,16 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                         __syncwarp();
                         float acc = 0.0f;
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const float hv = (i & 1) ? xh[i >> 1].y : xh[i >> 1].x;
-                            const float df = table[index_of(i, P)] - xwv[i];
-                            acc = fmaf(hv * df, df, acc);
-                        }
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t qi = indices(i, P);
 #pragma unroll
+                            for (int jj = 0; jj < 4; ++jj) {
+                                const float2 hh = xh[2 * i + (jj >> 1)];
+                                const float df = table[(qi >> (4 * jj)) & 0xFu] - xwv[4 * i + jj];
+                                acc = fmaf((jj & 1 ? hh.y : hh.x) * df, df, acc);
+                            }
+                        }
+#pragma unroll 1
                         for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
                         acc = __shfl_sync(0xffffffffu, acc, 0);
                         __syncwarp();
@@ -772,7 +795,6 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                     if (set) set |= 1u << kb;
                 }
             }
-
 
             // ---- exact look: float-float sums, exact roundings, direct error
             if (set) {
@@ -907,21 +929,11 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             th1 = __byte_perm(a45, a67, 0x7632);
         }
         const float P = flat ? 0.0f : R * p.invf[kb];
-        const float2 P2 = make_float2(P, P);
         const uint32_t smask = flat ? 0u : 0x7777u;
         auto outputs = [&](auto bf16, auto with_codes) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                // indices of the chunk's 4 elements, a nibble each: level m =
-                // min(floor(|d| P), 3) from the low bits of the floor on the 2^23
-                // grid; 4 + m (d >= 0) is m ^ 4 and 3 - m (d < 0) is m ^ 3
-                const float2 ya = __ffma2_rd(ad2[2 * i], P2, M2), yb = __ffma2_rd(ad2[2 * i + 1], P2, M2);
-                const uint32_t m0 = __float_as_uint(fminf(ya.x, kMagic + 3.0f)), m1 = __float_as_uint(fminf(ya.y, kMagic + 3.0f));
-                const uint32_t m2 = __float_as_uint(fminf(yb.x, kMagic + 3.0f)), m3 = __float_as_uint(fminf(yb.y, kMagic + 3.0f));
-                const uint32_t ng = negm >> (4 * i);
-                const uint32_t sx = (ng & 1u) | ((ng & 2u) << 3) | ((ng & 4u) << 6) | ((ng & 8u) << 9);
-                uint32_t sel = (m0 + (m1 << 4) + (m2 << 8) + (m3 << 12)) ^ 0x4444u ^ (sx * 7u);
-                sel &= smask;
+                const uint32_t sel = indices(i, P) & smask;
                 const uint32_t lo = __byte_perm(tl0, tl1, sel), hi = __byte_perm(th0, th1, sel);
                 const uint32_t r01 = __byte_perm(lo, hi, 0x5140), r23 = __byte_perm(lo, hi, 0x7362);
                 const int64_t ge = gofs + i * gstep;
