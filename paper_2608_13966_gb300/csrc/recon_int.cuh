@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
         gq.yhi = yhi;
         const float cref = mn + rho;  // the centre, rounded (an anchor only)
         if (h_one) ss = (float)G;
-        const float inv_ss = __fdividef(1.0f, ss);
+        const float inv_ss = rcp_ftz(ss);  // (at least 2^-40 by now)
         // mu: approximate weighted mean of w (only a centre for the sums)
         const float mu = h_one ? cref : sw * inv_ss;
         // approximate divisions (<= 2 ulp) are enough here: R scales the code
@@ -877,13 +877,14 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 const float zbar = T1 * inv_ss;
                 const float D = T2 - T1 * zbar;
                 const float N = T3 - T1 * ebar;
-                const float a = __fdividef(N, D);
+                const float a = N * rcp_ftz(D);
                 // a near-degenerate code variance, or a non-finite E (sums
-                // near the denormal range): left to the exact comparison
+                // near the denormal range, D among them): left to the exact
+                // comparison
                 const bool susp = !(D > 1e-3f * T2) || !(N * a < INFINITY);
                 const float E = N * a;
                 const float s2e = fmaxf(T2 * see, 1e-37f);
-                const float dN = ulp * (s2e * rsqrtf(s2e) * 1.001f + fabsf(T1 * ebar));
+                const float dN = ulp * (s2e * rsqrt_ftz(s2e) * 1.001f + fabsf(T1 * ebar));
                 const float dD = ulp * (T2 + fabsf(T1 * zbar));
                 const float dE = 2.0f * fabsf(a) * dN + a * a * dD;
                 const bool real = k < p.n_clip;
@@ -996,7 +997,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                     // (the roots as x rsqrt(x), 2 ulps: inside the factor 1.0001)
                     const float t2s = fmaxf(tb.y * see, 1e-37f), t2w = fmaxf(ss * tb.y, 1e-37f);
                     twin_q = 2.0f * 1.0001f * ulp *
-                             (t2s * rsqrtf(t2s) + fabsf(cref - mu) * (t2w * rsqrtf(t2w))) * qmaxf;
+                             (t2s * rsqrt_ftz(t2s) + fabsf(cref - mu) * (t2w * rsqrt_ftz(t2w))) * qmaxf;
                     twin_h = hmn * range;
                     twin_e = hmn * qmaxf * (8.0f * 5.9604645e-8f) * (range + fabsf(cref));
                 }
@@ -1143,7 +1144,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                 const float Dk = k2 - k1 * (k1 / gss), Nk = k3 - k1 * gebar;
                 const float ak = Nk / Dk, Exk = Nk * ak;
                 const float k2e = fmaxf(k2 * gsee, 1e-37f);
-                const float kapk = __fdividef(k2e * rsqrtf(k2e), fabsf(Nk)) + __fdividef(k2, Dk);
+                const float kapk = k2e * rsqrt_ftz(k2e) * rcp_ftz(fabsf(Nk)) + k2 * rcp_ftz(Dk);
                 const float rel = p.fit_ulps * 5.9604645e-8f * kapk;
                 const bool quick =
                     one_chunk && Dk > 1e-3f * k2 && rel * rel * Exk < 1e-9f * (gsee - Exk);
@@ -1189,8 +1190,10 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             const float Nc = T3b - T1b * ebar, Dc = T2b - T1b * Aq;
             // the quotient from the fast reciprocal and one correction
             // (the remainder Nc - q Dc is exact by FMA): within an ulp
-            const float q0 = __fdividef(Nc, Dc);
-            const float an = fmaf(fmaf(-q0, Dc, Nc), __fdividef(1.0f, Dc), q0);
+            // (a denormal Dc gives a NaN, which the accuracy check sends to the
+            // compensated fit)
+            const float rD = rcp_ftz(Dc), q0 = Nc * rD;
+            const float an = fmaf(fmaf(-q0, Dc, Nc), rD, q0);
             // Bz = (mu + ebar) - a (zeta0 + Aq), as a float pair
             const float z0 = y0b - kGridMagic;  // exact
             float p_h, p_l, bh, bl;
@@ -1202,7 +1205,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             Bz = bh;
             Bz_lo = bl;
             const float dse = fmaxf(T2b * see, 1e-37f);
-            kap_sel = __fdividef(dse * rsqrtf(dse), fabsf(Nc)) + __fdividef(T2b, Dc);
+            kap_sel = dse * rsqrt_ftz(dse) * rcp_ftz(fabsf(Nc)) + T2b * rD;
         }
 
         // ---- output accuracy check.  The fp32 fit's error at level q is at
@@ -1226,7 +1229,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             // the square root as x rsqrt(x), within 2 ulps: immaterial beside
             // the margin in fit_ulps)
             const float sv = fmaxf(see * inv_ss, 1e-37f);
-            const float ec = uf * (fabsf(cref) + fabsf(mu) + sv * rsqrtf(sv)) +
+            const float ec = uf * (fabsf(cref) + fabsf(mu) + sv * rsqrt_ftz(sv)) +
                              0.5f * 5.9604645e-8f * fabsf(Bz);
             // the weighted mean code (q = zeta + J + 1)
             const float qbar = (y0b - kGridMagic) + T1b * inv_ss + Jp1;

@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             // normal one) are compacted into two lists by sign, |d| and h, in
             // the tile.  (The bound is 1 less a few ulps: an element too many
             // only adds zeros.)
-            const float thr = __fdividef(0.999999f, R * p.invf_max);
+            const float thr = 0.999999f * rcp_ftz(R * p.invf_max);
             uint32_t act = 0;
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 // the sign's totals; beyond level 3: nothing)
                 const float Ac[3] = {far ? A2 : bconst[pos ? 0 : 1], far ? A3 : A1, far ? 0.0f : A2};
                 const float Xc[3] = {far ? X2 : bconst[pos ? 2 : 3], far ? X3 : X1, far ? 0.0f : X2};
-                const float sg = __fdividef(1.0f, P);
+                const float sg = rcp_ftz(P);
                 const float sgn = pos ? 1.0f : -1.0f;
                 // errors: the cumulative sums are sums of nonnegative terms,
                 // exact (h) or rounded once (h |d|), over at most `depth` levels
@@ -552,7 +552,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                     dm[e2] = 4.0f * kU * fabsf(gj);
                     float qu = 0.0f, dq = 0.0f;
                     if (H > 0.0f) {
-                        const float rh = __fdividef(1.0f, H);
+                        float rh = rcp_ftz(H);
+                        if (H < kMinNormal) rh = __fdividef(1.0f, H);
                         qu = X * rh;
                         mean[e2] = fmaf(sgn, qu, c);
                         dq = (dX + qu * dA) * rh + 3.0f * kU * qu;

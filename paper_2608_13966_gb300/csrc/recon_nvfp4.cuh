@@ -65,14 +65,6 @@ __device__ __forceinline__ float e4m3_value(uint32_t bits)
     return v;
 }
 
-// Fast reciprocal (2 ulps), denormals flushed.
-__device__ __forceinline__ float rcp_ftz(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // E2M1 codes of two values (nearest, ties to the even code, saturating at 6):
 // y.x in the low nibble, y.y in the high one, each sign << 3 | magnitude.
 __device__ __forceinline__ uint32_t e2m1_nibbles(float2 y)
@@ -362,7 +354,7 @@ __global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 38
             // degenerate, every weighted element coded 0: the search scale --
             // go the long way.)
             float x = s3 * rcp_ftz(s2) * inv_sT;
-            if (!(s2 >= 1.17549435e-38f))
+            if (!(s2 >= kMinNormal))
                 x = s2 > 0.0f ? __fdividef(s3, s2) * inv_sT : amax_b * p.f[k] * (1.0f / 6.0f) * inv_sT;
             Fit r;
             r.e = e4m3_rn_satfinite(x);

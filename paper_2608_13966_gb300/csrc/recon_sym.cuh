@@ -379,7 +379,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_sym(const __grid_constant__ In
             for (int qd = 0; qd < 2; ++qd) {
                 const int k = kq + qd * 4 + sl;
                 const float S2 = S[qd][0], S3 = S[qd][1];
-                const float E = S2 > 0.0f ? __fdividef(S3 * S3, S2) : 0.0f;
+                float E = S3 * S3 * rcp_ftz(S2);
+                if (!(S2 >= kMinNormal)) E = S2 > 0.0f ? __fdividef(S3 * S3, S2) : 0.0f;
                 const bool real = k < p.n_clip;
                 if (real && E > Eb) {  // strict: keeps the lower k of this lane
                     Eb = E;
