@@ -30,11 +30,15 @@
 // (float-float sums over the codes, whole warp), so indices, tables and the
 // kept candidate equal the exact computation's.
 //
-// What bounds it: instruction issue, 136 a weight and lane (263 with the sums
-// in registers).  One Llama layer (218 M weights, packed codes): 2,300 us with
-// the sums in registers, 2,070 with the lists, 1,576 with the pieces copied
-// and waited for by the lane that reads them, two-at-a-time E4M3 conversions,
-// redux for the minima and h re-read by the settling steps.
+// What bounds it: instruction issue, about 140 a weight and lane (263 with the
+// sums in registers), and fetching them: the common path and the settling steps
+// that a fifth of the blocks take just fill the instruction cache, and whatever
+// makes them smaller makes the kernel faster.  One Llama layer (218 M weights,
+// packed codes): 2,300 us with the sums in registers; 2,070 with the lists; 1,576
+// with the pieces copied and waited for by the lane that reads them, two-at-a-time
+// E4M3 conversions, redux for the minima and h re-read by the settling steps;
+// 1,520 with one settling loop on nibble indices; 1,407 with one rolled walk for
+// both signs' lists (walks unrolled by 2: 1,449; two walks: 1,451).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -385,7 +389,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 const float2 hd = __fmul2_rn(h2[t], ad2[t]);
                 // masks 0 or 1 by sign: the products are exact
                 const float2 mn2 = make_float2(__uint_as_float(sx & 0x3F800000u), __uint_as_float(sy & 0x3F800000u));
-                const float2 mp2 = make_float2(__uint_as_float(~sx & 0x3F800000u), __uint_as_float(~sy & 0x3F800000u));
+                const float2 mp2 = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(-mn2.x, -mn2.y));
                 Tn = __ffma2_rn(h2[t], mn2, Tn);
                 Un = __ffma2_rn(hd, mn2, Un);
                 Tp = __ffma2_rn(h2[t], mp2, Tp);
@@ -491,7 +495,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
 #pragma unroll
                 for (int l = 0; l < 3; ++l) Ap[l] = An[l] = Xp[l] = Xn[l] = make_float2(0.0f, 0.0f);
                 auto walk = [&](const float* la, int n, float2 (&A)[3], float2 (&X)[3]) {
-#pragma unroll 2
+#pragma unroll 1
                     for (int e = 2 * q; e < n; e += 8) {
                         const float2 a2 = *reinterpret_cast<const float2*>(la + e);
                         const float2 hh = *reinterpret_cast<const float2*>(la + kLutListLen + e);
@@ -506,8 +510,17 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                         }
                     }
                 };
-                walk(lst, np8, Ap, Xp);
-                walk(lst + np8, nn8, An, Xn);
+#pragma unroll 1
+                for (int sd = 0; sd < 2; ++sd) {
+                    // (one copy of the loop: the first list's sums move aside)
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) {
+                        Ap[l] = An[l];
+                        Xp[l] = Xn[l];
+                        An[l] = Xn[l] = make_float2(0.0f, 0.0f);
+                    }
+                    walk(sd ? lst + np8 : lst, sd ? nn8 : np8, An, Xn);
+                }
                 if (k0 + 8 >= K) {  // the lists are done with: the next block
                     __syncwarp();
                     if (u + stride < n_units) issue(u + stride);
@@ -694,10 +707,11 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 while (und) {
                     const int j = __ffs(und) - 1;
                     und &= und - 1;
+                    const uint32_t jj4 = (uint32_t)j * 0x1111u;
                     float Hs = 0.0f, Xs = 0.0f;
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        if (((qs[i >> 2] >> (4 * (i & 3))) & 0xFu) == (uint32_t)j) {
+                        if (((qs[i >> 2] ^ jj4) & (0xFu << (4 * (i & 3)))) == 0u) {
                             const float hv = (i & 1) ? xh[i >> 1].y : xh[i >> 1].x;
                             const float av = (i & 1) ? ad2[i >> 1].y : ad2[i >> 1].x;
                             Hs += hv;
@@ -915,19 +929,17 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
         // permute picks four entries by their indices (a nibble each)
         uint32_t tl0, tl1, th0, th1;
         {
-            uint32_t t[8];
-#pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                const float2 v = e4m3_decode2((j < 4 ? bw0 : bw1) >> (8 * (j & 3)) & 0xFFFFu);
-                t[j] = __float_as_uint(v.x) >> 16;
-                t[j + 1] = __float_as_uint(v.y) >> 16;
-            }
-            const uint32_t a01 = __byte_perm(t[0], t[1], 0x5140), a23 = __byte_perm(t[2], t[3], 0x5140);
-            const uint32_t a45 = __byte_perm(t[4], t[5], 0x5140), a67 = __byte_perm(t[6], t[7], 0x5140);
-            tl0 = __byte_perm(a01, a23, 0x5410);
-            th0 = __byte_perm(a01, a23, 0x7632);
-            tl1 = __byte_perm(a45, a67, 0x5410);
-            th1 = __byte_perm(a45, a67, 0x7632);
+            // (the upper halves of four f32 values in two registers, then their low
+            // and their high bytes)
+            auto bytes = [](uint32_t codes, uint32_t& lo, uint32_t& hi) {
+                const float2 a = e4m3_decode2(codes & 0xFFFFu), b = e4m3_decode2(codes >> 16);
+                const uint32_t x = __byte_perm(__float_as_uint(a.x), __float_as_uint(a.y), 0x7632);
+                const uint32_t y = __byte_perm(__float_as_uint(b.x), __float_as_uint(b.y), 0x7632);
+                lo = __byte_perm(x, y, 0x6420);
+                hi = __byte_perm(x, y, 0x7531);
+            };
+            bytes(bw0, tl0, th0);
+            bytes(bw1, tl1, th1);
         }
         const float P = flat ? 0.0f : R * p.invf[kb];
         const uint32_t smask = flat ? 0u : 0x7777u;
