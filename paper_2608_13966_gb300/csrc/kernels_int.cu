@@ -13,37 +13,21 @@
 
 namespace quasar {
 
-// Kernel entry for group size 4*epl: one tensor or a batch of up to
-// kMaxBatch tensors per launch.  The AdamW-fused variant is built for batches
-// with sets of 4 or 1 candidates, the option variants (var) for batches with
-// sets of 1; nullptr where not built.
+// Kernel entry for group size 4*epl: one tensor or a batch of up to kMaxBatch
+// tensors per launch; the AdamW-fused variant and the option variants (var) are
+// built for batches.  nullptr where not built.
 const void* QUASAR_NAME(QUASAR_NCH, QUASAR_SS)(int epl, bool batch, bool adam, bool var)
 {
     constexpr int C = QUASAR_NCH;
     constexpr int S = QUASAR_SS;
     constexpr int B = kMaxBatch;
     if ((adam || var) && !batch) return nullptr;
-    if (adam && (S == 2 || S == 3 || S == 8)) return nullptr;
-    if (var && S != 1) return nullptr;
     switch (epl) {
-#if QUASAR_SS == 1
-#define QUASAR_VAR(E)                                                                         \
-    if (var)                                                                                  \
-        return adam ? reinterpret_cast<const void*>(&k_recon_int<E, C, B, true, true, S>)     \
-                    : reinterpret_cast<const void*>(&k_recon_int<E, C, B, false, true, S>);
-#else
-#define QUASAR_VAR(E)
-#endif
-#if QUASAR_SS == 4 || QUASAR_SS == 1
-#define QUASAR_ADAM(E) \
-    if (adam) return reinterpret_cast<const void*>(&k_recon_int<E, C, B, true, false, S>);
-#else
-#define QUASAR_ADAM(E)
-#endif
-#define QUASAR_EPL(E)                                                                         \
-    case E:                                                                                   \
-        QUASAR_VAR(E)                                                                         \
-        QUASAR_ADAM(E)                                                                        \
+#define QUASAR_EPL(E)                                                                             \
+    case E:                                                                                       \
+        if (adam && var) return reinterpret_cast<const void*>(&k_recon_int<E, C, B, true, true, S>); \
+        if (adam) return reinterpret_cast<const void*>(&k_recon_int<E, C, B, true, false, S>);    \
+        if (var) return reinterpret_cast<const void*>(&k_recon_int<E, C, B, false, true, S>);     \
         if (!batch) return reinterpret_cast<const void*>(&k_recon_int<E, C, 1, false, false, S>); \
         return reinterpret_cast<const void*>(&k_recon_int<E, C, B, false, false, S>);
     QUASAR_EPL(8)
@@ -51,8 +35,6 @@ const void* QUASAR_NAME(QUASAR_NCH, QUASAR_SS)(int epl, bool batch, bool adam, b
     QUASAR_EPL(32)
     QUASAR_EPL(64)
 #undef QUASAR_EPL
-#undef QUASAR_ADAM
-#undef QUASAR_VAR
     default: return nullptr;
     }
 }

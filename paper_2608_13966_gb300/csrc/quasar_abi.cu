@@ -522,9 +522,7 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
     const bool one_chunk = n_clip <= 8;
     const bool batch = MAXT > 1;
     const bool var = Lp.p.h_mode != kSalEma || Lp.p.codes_packed;
-    // clamp sets: as large as the factors allow, unless switched off (sets of
-    // one); the option variants of the asymmetric kernel are built with sets of
-    // one, the fused AdamW step with sets of four or one
+    // clamp sets: as large as the factors allow, unless switched off (sets of one)
     const int hoist_on = g_hoist.load() < 0 ? tuning().hoist : g_hoist.load();
     if (symmetric) {
         if (MAXT == 1) return QUASAR_ERR_UNSUPPORTED;
@@ -538,9 +536,8 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
         if (!fn) return QUASAR_ERR_UNSUPPORTED;
         return launch_persistent(fn, &Lp, L.smem, units, stream, warps);
     }
-    // (sets of 8 or 3-3-2 with a single chunk, not for the fused AdamW step)
-    fill_caps(&Lp.p, (!hoist_on || var) ? 1 : 4, one_chunk && !adam);
-    if (adam && Lp.p.set_size == 2) fill_caps(&Lp.p, 1);
+    // (sets of 8 or 3-3-2 with a single chunk)
+    fill_caps(&Lp.p, hoist_on ? 4 : 1, one_chunk);
     using Entry = const void* (*)(int, bool, bool, bool);
     static const Entry table[2][5] = {
         {int_kernel_nch1_ss8, int_kernel_nch1_ss4, int_kernel_nch1_ss3, int_kernel_nch1_ss2, int_kernel_nch1_ss1},
