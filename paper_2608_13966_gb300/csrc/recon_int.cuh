@@ -809,7 +809,11 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
                         const float2 h = pr ? make_float2(h4.z, h4.w) : make_float2(h4.x, h4.y);
                         const float2 d = __fadd2_rn(__fadd2_rn(wv, nmn2), nrho2);
                         const float2 ev = __fadd2_rn(wv, nmu2);
-                        if (NCH == 1 || ch == 0) {
+                        // sum h e and sum h e^2, once; in groups of 64 and less with every
+                        // chunk, where three more operations a pair cost less than the
+                        // branch's code (the Qwen3 layer at INT2, 16 factors: 1,551 against
+                        // 1,592 us; INT3 g128, 15 factors: 1,259 against 1,237)
+                        if (NCH == 1 || EPL <= 16 || ch == 0) {
                             const float2 he = __fmul2_rn(h, ev);
                             SE = __fadd2_rn(SE, he);
                             SEE = __ffma2_rn(he, ev, SEE);
