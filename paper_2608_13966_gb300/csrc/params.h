@@ -17,6 +17,10 @@ constexpr int kMaxClip = 32;
 constexpr int kIntLanes = 4;
 constexpr int kIntGroups = 8;
 constexpr uint32_t kIntTableBytes = 8 * kIntGroups * 16;
+// Most warps of an integer kernel's CTA, one CTA an SM (epl = group size / 4):
+// 16 warps at up to 128 registers a thread, or, where the tiles that fit allow
+// fewer warps anyway (groups of 256), 12 at up to 168.
+constexpr int int_max_warps(int epl) { return epl == 64 ? 12 : 16; }
 
 // One tensor of an integer-code launch: its buffers, group count, and the
 // index of its first unit in the launch's sequence of units.

@@ -44,14 +44,11 @@ namespace {
 
 using namespace quasar;
 
-// 8 warps per CTA: two CTAs of the integer and lookup-table kernels fill the
-// register file (16 resident warps at 128 registers a thread) and fit in an
-// SM's shared memory.
+// 8 warps per CTA of the kernels with per-warp tiles: two CTAs of the
+// lookup-table kernel fill the register file (16 resident warps at 128 registers
+// a thread) and fit in an SM's shared memory.
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-// The AdamW-fused integer kernel also stages m (14 instead of 10 bytes a
-// weight): 6 warps per CTA keep two CTAs in an SM's shared memory.
-constexpr int kAdamWarps = 6;
 constexpr uint64_t kDefaultTimeoutNs = 1000000000ull;  // 1 s per wait
 
 std::atomic<int64_t> g_force_timeout_ns{0};
@@ -240,10 +237,11 @@ struct DeviceInfo {
 DeviceInfo g_dev[kMaxDevices];
 std::mutex g_mu;
 
-// Launch configuration of one kernel at one shared-memory size, per device.
+// Launch configuration of one kernel at one shared-memory size and block size, per device.
 struct KernelConfig {
     const void* fn = nullptr;
     size_t smem = 0;
+    int threads = 0;
     int dev = -1;
     int occupancy = 0;
 };
@@ -302,7 +300,7 @@ quasar_status occupancy(const void* fn, size_t smem, int threads, int dev, int* 
 {
     std::lock_guard<std::mutex> lock(g_mu);
     for (int i = 0; i < g_ncfg; ++i)
-        if (g_cfg[i].fn == fn && g_cfg[i].dev == dev && g_cfg[i].smem == smem) {
+        if (g_cfg[i].fn == fn && g_cfg[i].dev == dev && g_cfg[i].smem == smem && g_cfg[i].threads == threads) {
             *occ = g_cfg[i].occupancy;
             return QUASAR_OK;
         }
@@ -320,7 +318,7 @@ quasar_status occupancy(const void* fn, size_t smem, int threads, int dev, int* 
     int o = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, threads, smem) != cudaSuccess)
         return QUASAR_ERR_CUDA;
-    if (g_ncfg < kMaxConfigs) g_cfg[g_ncfg++] = KernelConfig{fn, smem, dev, o};
+    if (g_ncfg < kMaxConfigs) g_cfg[g_ncfg++] = KernelConfig{fn, smem, threads, dev, o};
     *occ = o;
     return QUASAR_OK;
 }
@@ -422,33 +420,32 @@ struct AdamHp {
     int64_t step;
 };
 
-// Shared memory of an integer kernel's CTA ring: S slots of one
-// unit tile each (w, v, m for the fused AdamW step, then the gradient
-// region, which is also the candidate table and so at least kIntTableBytes
-// for each 8 candidates), S + 1 mbarriers and S sequence words.  S is one slot a
-// warp plus `extra` slots in flight (QUASAR_STAGES, default 2).
-Launch plan_ring(int group_size, int g_kind, bool adam, int warps, int n_clip)
+// The CTA of an integer kernel: one per SM, with a ring of S slots of one unit
+// tile each (w, v, m for the fused AdamW step, then the gradient region, which
+// is also the candidate table and so at least kIntTableBytes for each 8
+// candidates), S + 1 mbarriers, S sequence words and the next tile's number.
+// As many warps as the registers allow, but one fewer than the slots that fit
+// (a copy in flight), and up to kRingAhead slots in flight (QUASAR_STAGES
+// overrides).  One slot in flight beyond the warps is enough: AdamW + INT4 g128
+// with fp32 gradients, 14 slots, 949 us with 13 warps and 974 with 12; group
+// 256, 7 slots, 518 with 6 and 556 with 5.  Of slots that are left, 8 in flight
+// are a little better than 4 or 6 in small groups (INT2 g64, 16 factors: 1,408,
+// 1,424 and 1,413 us).
+constexpr int kRingAhead = 8;
+constexpr size_t kCtaSmem = 227 * 1024;  // what a CTA may have
+
+Launch plan_ring(int group_size, int g_kind, bool adam, int n_clip, int* warps)
 {
     const uint32_t gbytes = g_kind == 2 ? 2u : (g_kind == 1 ? 4u : 0u);
     const uint32_t unit = (uint32_t)(kIntGroups * group_size);
     const uint32_t tile = unit * (adam ? 12u : 8u) + std::max(unit * gbytes, (uint32_t)((n_clip + 7) / 8) * kIntTableBytes);
     Launch L;
     L.stage_bytes = (tile + 127u) & ~127u;
-    auto total = [&](int s) {
-        return (size_t)s * L.stage_bytes + (size_t)(s + 1) * 8 + (size_t)s * 4;
-    };
-    int extra = tuning().stages;
-    if (extra <= 0) {
-        // two slots in flight, one if that keeps two CTAs on an SM (each
-        // CTA's share of the SM's 228 KB, less the 1 KB the system keeps);
-        // one if two would exceed the 227 KB a CTA may have
-        constexpr size_t kTwoCtas = 113 * 1024, kOneCta = 227 * 1024;
-        extra = 2;
-        if ((total(warps + 2) > kTwoCtas && total(warps + 1) <= kTwoCtas) || total(warps + 2) > kOneCta)
-            extra = 1;
-    }
-    L.stages = warps + extra;
-    L.smem = total(L.stages);
+    constexpr size_t kPerSlot = 8 + 4, kPerCta = 8 + 4;
+    const int fit = (int)((kCtaSmem - kPerCta) / (L.stage_bytes + kPerSlot));
+    *warps = std::min(int_max_warps(group_size / kIntLanes), fit - 1);
+    L.stages = std::min(*warps + (tuning().stages > 0 ? tuning().stages : kRingAhead), fit);
+    L.smem = (size_t)L.stages * (L.stage_bytes + kPerSlot) + kPerCta;
     return L;
 }
 
@@ -514,8 +511,8 @@ quasar_status int_launch(IntLaunch<MAXT>& Lp, int group_size, int n_clip, cudaSt
     }
     Lp.n_units = units;
     if (units == 0) return QUASAR_OK;
-    const int warps = adam ? kAdamWarps : kWarps;
-    const Launch L = plan_ring(group_size, Lp.p.g_kind, adam, warps, n_clip);
+    int warps = 0;
+    const Launch L = plan_ring(group_size, Lp.p.g_kind, adam, n_clip, &warps);
     Lp.p.stages = L.stages;
     Lp.p.stage_bytes = L.stage_bytes;
     const int epl = group_size / kIntLanes;

@@ -9,8 +9,8 @@
 // groups one shared-memory access phase covers hit different banks).  The
 // CTA runs one ring of tile slots (one unit each) filled by 1-D TMA bulk
 // copies (cp.async.bulk + mbarrier); each slot carries the sequence number of
-// the unit loading into it, warp j takes the CTA's units j, j + warps, ...
-// and, done with a tile, issues the copy of the unit that many slots ahead
+// the unit loading into it; a free warp takes the CTA's next unit that none has
+// taken and, done with its tile, issues the copy of the unit that many slots ahead
 // into the same slot.  w, g and v are read from HBM exactly once, and the
 // loads of later units overlap the arithmetic of the current ones.  After
 // pass A the tile's gradient region holds the candidates' table.  The grid
@@ -129,7 +129,8 @@ __device__ __forceinline__ void ff_norm(float& hi, float& lo)
 // 1,953.  With up to 8 it is a tenth, and latency counts: 806 against 822 us
 // on a Llama layer at INT3.  (Smaller still -- passes A and C not unrolled, one
 // reduction loop in the compensated fit, counters in registers, fast roots
-// where they only feed a bound -- the Qwen3 layer takes 1,660 us.)
+// where they only feed a bound -- the Qwen3 layer took 1,660 us.  All with two
+// CTAs an SM; it takes 1,408 now.)
 template <bool ROLL>
 __device__ __forceinline__ void ff_reduce32(float& hi, float& lo)
 {
@@ -410,7 +411,15 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
 
 // ------------------------------------------------------------------ kernel
 
-// Two CTAs per SM: 8-warp CTAs, 6-warp ones for the AdamW-fused variant.
+// One CTA per SM, its warps taking tiles from one ring as they get free.  Two
+// CTAs of 8 warps (6 with AdamW), a ring each and a fixed share of the tiles a
+// warp, had the same registers and shared memory: one Llama layer INT3 786 us
+// (one CTA with fixed shares 747, as built 740), INT3 15 factors 1,234 (now
+// 1,154), the Qwen3 layer INT2 g64 16 factors 1,551 (fixed shares 1,448, now
+// 1,408), AdamW + INT3 988 (now 916, 14 warps and 2 slots in flight, 0.985 of
+// the measured copy rate).  With fixed shares a warp count that is no multiple
+// of the SM's 4 schedulers was worse than the next lower multiple.  20 warps at
+// 96 registers spill: INT3 885 us.
 // VAR: the variants of the options (a saliency other than v', packed codes);
 // without it they compile out of the common kernel.
 // SS: candidates per clamp set (4, 2 or 1; with a single chunk also 8, or 3:
@@ -419,7 +428,7 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
 // NCH: 1 for up to 8 candidates (one chunk), 2 for up to 32 (p.n_clip / 8
 // chunks, rounded up).
 template <int EPL, int NCH, int MAXT, bool ADAM, bool VAR, int SS>
-__global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
+__global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
     k_recon_int(const __grid_constant__ IntLaunch<MAXT> Lp)
 {
     static_assert(SS == 1 || SS == 2 || SS == 4 || ((SS == 3 || SS == 8) && NCH == 1),
@@ -453,6 +462,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
     unsigned char* ring = smem;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * p.stage_bytes);
     volatile int* seq = reinterpret_cast<volatile int*>(bars + S + 1);
+    int* next = const_cast<int*>(seq) + S;  // the first tile no warp has taken
 
     const int nch = (p.n_clip + 7) >> 3;  // chunks of 8 candidates
     const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
@@ -461,8 +471,8 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
     constexpr uint32_t kMOff = UNIT * 8;
     constexpr uint32_t kGOff = UNIT * (ADAM ? 12 : 8);
 
-    // tiles: the CTA takes units blockIdx.x + t * gridDim.x, t = 0 .. nt-1,
-    // and warp w the tiles t = w, w + nwarps, ...; tile t goes to slot t % S
+    // tiles: the CTA takes units blockIdx.x + t * gridDim.x, t = 0 .. nt-1, its
+    // warps the next tile that none has taken; tile t goes to slot t % S
     const int64_t n_units = Lp.n_units;
     const int nt = n_units > (int64_t)blockIdx.x
                        ? (int)((n_units - 1 - (int64_t)blockIdx.x) / gridDim.x + 1)
@@ -499,6 +509,7 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
     if (threadIdx.x == 0) {
         for (int s = 0; s <= S; ++s) mbar_init(&bars[s], 1);
         for (int s = 0; s < S; ++s) seq[s] = -1;
+        *next = nwarps;
         mbar_init_fence();
         for (int s = 0; s < S && s < nt; ++s) issue(s, s);
     }
@@ -541,9 +552,9 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
     const float2 isbc22 = make_float2(p.isbc2, p.isbc2), eps2 = make_float2(p.eps, p.eps);
     const unsigned gmask = 0xFu << (gs * kIntLanes);  // this group's lanes
 
-    int slot = warp;  // t % S (nwarps < S)
+    int slot = warp;  // t % S (warps < S)
     uint32_t parity = 0;  // (t / S) & 1
-    for (int t = warp; t < nt; t += nwarps) {
+    for (int t = warp; t < nt;) {
         if (!warp_wait_seq(seq + slot, t, p.timeout_ns) ||
             !warp_wait_bounded(&bars[slot], parity, p.timeout_ns)) {
             fail();
@@ -1442,11 +1453,11 @@ __global__ void __launch_bounds__(ADAM ? 192 : 256, 2)
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             issue(t + S, slot);
         }
-        slot += nwarps;
-        if (slot >= S) {
-            slot -= S;
-            parity ^= 1u;
-        }
+        int tn = 0;
+        if (lane == 0) tn = atomicAdd(next, 1);
+        tn = __shfl_sync(0xffffffffu, tn, 0);
+        for (slot += tn - t; slot >= S; slot -= S) parity ^= 1u;
+        t = tn;
     }
 }
 

@@ -23,7 +23,8 @@
 //
 // What bounds it: instruction issue and the FP32 pipe (5 packed operations a
 // pair and candidate).  One Llama layer at INT4, group 128, 8 factors (clamp
-// sets 3-3-2): 791 -> 629 us, 5.57 TB/s of algorithmic traffic.
+// sets 3-3-2): 791 -> 568 us, 6.17 TB/s of algorithmic traffic (626 with two
+// CTAs an SM and a fixed share of the tiles a warp; 20 warps at 96 registers 576).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -95,7 +96,7 @@ __device__ __forceinline__ float code_n(float aw, float P, float Q)
 
 
 template <int EPL, int MAXT, int SS>
-__global__ void __launch_bounds__(256, 2) k_recon_sym(const __grid_constant__ IntLaunch<MAXT> Lp)
+__global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1) k_recon_sym(const __grid_constant__ IntLaunch<MAXT> Lp)
 {
     using namespace sym;
     static_assert(SS == 1 || SS == 2 || SS == 3 || SS == 4 || SS == 8, "clamp sets of 1, 2, 4 or 8, or 3-3-2");
@@ -127,14 +128,15 @@ __global__ void __launch_bounds__(256, 2) k_recon_sym(const __grid_constant__ In
     unsigned char* ring = smem;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * p.stage_bytes);
     volatile int* seq = reinterpret_cast<volatile int*>(bars + S + 1);
+    int* next = const_cast<int*>(seq) + S;  // the first tile no warp has taken
 
     const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
     // stage: w | v | g, then the candidates' table
     constexpr uint32_t kVOff = UNIT * 4;
     constexpr uint32_t kGOff = UNIT * 8;
 
-    // tiles: the CTA takes units blockIdx.x + t * gridDim.x, t = 0 .. nt-1,
-    // and warp w the tiles t = w, w + nwarps, ...; tile t goes to slot t % S
+    // tiles: the CTA takes units blockIdx.x + t * gridDim.x, t = 0 .. nt-1, its
+    // warps the next tile that none has taken; tile t goes to slot t % S
     const int64_t n_units = Lp.n_units;
     const int nt = n_units > (int64_t)blockIdx.x
                        ? (int)((n_units - 1 - (int64_t)blockIdx.x) / gridDim.x + 1)
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_sym(const __grid_constant__ In
     if (threadIdx.x == 0) {
         for (int s = 0; s <= S; ++s) mbar_init(&bars[s], 1);
         for (int s = 0; s < S; ++s) seq[s] = -1;
+        *next = nwarps;
         mbar_init_fence();
         for (int s = 0; s < S && s < nt; ++s) issue(s, s);
     }
@@ -202,9 +205,9 @@ __global__ void __launch_bounds__(256, 2) k_recon_sym(const __grid_constant__ In
     const float2 M2 = make_float2(kMagic, kMagic), nM2 = make_float2(-kMagic, -kMagic);
     const float gam = kU * p.tie_kappa;
 
-    int slot = warp;  // t % S (nwarps < S)
+    int slot = warp;  // t % S (warps < S)
     uint32_t parity = 0;  // (t / S) & 1
-    for (int t = warp; t < nt; t += nwarps) {
+    for (int t = warp; t < nt;) {
         if (!warp_wait_seq(seq + slot, t, p.timeout_ns) ||
             !warp_wait_bounded(&bars[slot], parity, p.timeout_ns)) {
             fail();
@@ -593,11 +596,11 @@ __global__ void __launch_bounds__(256, 2) k_recon_sym(const __grid_constant__ In
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             issue(t + S, slot);
         }
-        slot += nwarps;
-        if (slot >= S) {
-            slot -= S;
-            parity ^= 1u;
-        }
+        int tn = 0;
+        if (lane == 0) tn = atomicAdd(next, 1);
+        tn = __shfl_sync(0xffffffffu, tn, 0);
+        for (slot += tn - t; slot >= S; slot -= S) parity ^= 1u;
+        t = tn;
     }
 }
 

@@ -159,3 +159,36 @@ def test_launches_around_the_number_of_ctas(kind, units):
     for key in whole:
         if key != "tensor_scale":
             assert torch.equal(whole[key], torch.cat([p[key] for p in parts])), key
+
+
+@pytest.mark.parametrize("G,g_dtype,adam,symmetric", [
+    (32, torch.bfloat16, False, False), (128, torch.float32, False, False),
+    (256, torch.bfloat16, False, False), (256, None, False, False), (64, torch.bfloat16, True, False),
+    (128, torch.bfloat16, True, False), (256, torch.bfloat16, True, False), (256, torch.float32, True, False),
+    (32, None, False, True), (128, torch.bfloat16, False, True), (256, torch.float32, False, True)])
+def test_tiles_shared_by_the_warps_of_a_cta(G, g_dtype, adam, symmetric):
+    """Every slot of a CTA's ring is filled several times, for each number of
+    slots and warps: the outputs equal those of calls small enough that each
+    slot is filled once at most."""
+    rows, piece = 8 * (152 * 40 + 5), 8 * 152 * 4          # one group a row, 8 a tile
+    w, g, v = _inputs(rows, G, seed=4500 + G)
+    m = 1e-4 * torch.randn(rows, G, device="cuda", generator=torch.Generator("cuda").manual_seed(G))
+    g = None if g_dtype is None else g.to(g_dtype)
+
+    def run(lo, hi):
+        cut = lambda x: None if x is None else x[lo:hi].clone()
+        wc, gc, mc, vc = cut(w), cut(g), cut(m), cut(v)
+        if adam:
+            out = api.adamw_recon_int_batch([(wc, gc, mc, vc)], bits=3, group_size=G, clip=CLIP8, lr=1e-5,
+                                             step=3)[0]
+        else:
+            out = api.recon_int_batch([(wc, gc, vc)], bits=3, group_size=G, clip=CLIP8, codes=True,
+                                      symmetric=symmetric)[0]
+        return dict(out, w=wc, m=mc, v=vc)
+
+    whole = run(0, rows)
+    parts = [run(lo, min(lo + piece, rows)) for lo in range(0, rows, piece)]
+    torch.cuda.synchronize()
+    for key in whole:
+        if whole[key] is not None:
+            assert torch.equal(whole[key], torch.cat([p[key] for p in parts])), key
