@@ -151,6 +151,7 @@ constexpr int kLutListLen = kLutBlock + 16;
 constexpr uint32_t kLutListBytes = 2 * kLutListLen * 4;
 constexpr uint32_t kLutCandBytes = kMaxClip * 20;
 constexpr uint32_t kLutScratchBytes = kLutCandBytes + 64;
+constexpr int kLutWarps = 16;  // of its CTA, one CTA an SM
 
 struct LutTensor {
     const float* w;

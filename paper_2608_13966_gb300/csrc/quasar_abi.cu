@@ -1100,7 +1100,8 @@ quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_ten
     if ((st = status_ptr(&p.status)) != QUASAR_OK) return st;
     const uint32_t gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
     p.stage_bytes = (std::max(kLutBlock * (8 + gbytes), kLutListBytes) + 127u) & ~127u;
-    const size_t smem = (size_t)kWarps * (p.stage_bytes + kLutScratchBytes);
+    // (and the next unit's number)
+    const size_t smem = (size_t)kLutWarps * (p.stage_bytes + kLutScratchBytes) + sizeof(int);
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     for (int i0 = 0; i0 < n_tensors; i0 += kMaxBatch) {
         Lp.n_t = std::min(kMaxBatch, n_tensors - i0);
@@ -1112,7 +1113,7 @@ quasar_status quasar_recon_lut_batch(const quasar_lut_tensor* tensors, int n_ten
         }
         Lp.n_units = units;
         if (units == 0) continue;
-        if ((st = launch_persistent(lut_kernel(), &Lp, smem, units, s)) != QUASAR_OK) return st;
+        if ((st = launch_persistent(lut_kernel(), &Lp, smem, units, s, kLutWarps)) != QUASAR_OK) return st;
     }
     return QUASAR_OK;
 }

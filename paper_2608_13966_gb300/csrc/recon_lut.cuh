@@ -38,7 +38,8 @@
 // with the pieces copied and waited for by the lane that reads them, two-at-a-time
 // E4M3 conversions, redux for the minima and h re-read by the settling steps;
 // 1,520 with one settling loop on nibble indices; 1,407 with one rolled walk for
-// both signs' lists (walks unrolled by 2: 1,449; two walks: 1,451).
+// both signs' lists (walks unrolled by 2: 1,449; two walks: 1,451); 1,302 with the
+// SM's warps sharing its blocks.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -193,11 +194,13 @@ __device__ __forceinline__ uint32_t e4m3_round_ff(float xh, float xl)
 
 }  // namespace lut
 
-// Two CTAs an SM (128 registers): 1,639 us a layer where three (80 registers,
-// spilling) took 1,757; CTAs of 4 warps were slower at 96 registers (1,672
-// against 1,576) and at 128 (1,616).
+// One CTA of 16 warps an SM (128 registers; 24 warps at 80 spilled: 1,757 against
+// 1,639 us a layer), its warps taking blocks as they get free: the settling steps
+// make blocks unequal.  Two CTAs of 8 warps with a fixed share of the blocks a
+// warp: 1,402 against 1,302 us (one CTA with fixed shares 1,367); 16 factors, 39 M
+// weights, 770 against 561.
 template <int MAXT>
-__global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ LutLaunch<MAXT> Lp)
+__global__ void __launch_bounds__(kLutWarps * 32, 1) k_recon_lut(const __grid_constant__ LutLaunch<MAXT> Lp)
 {
     using namespace lut;
     const LutParams& p = Lp.p;
@@ -205,7 +208,6 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int nwarps = blockDim.x >> 5;
     // a warp's part: the tile, then the candidates' results.  Once the block is
     // in registers, the tile holds the lists; once they are walked, the next
     // block is copied into it.
@@ -228,11 +230,24 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     auto tensor_of = [&](int64_t u, int& ti) {
         while (ti + 1 < Lp.n_t && u >= Lp.t[ti + 1].unit0) ++ti;
     };
-    // a CTA's warps take neighbouring units (their tiles share DRAM pages); in a
+    // the CTA's units t = 0, 1, ...: warps start with theirs, then take the next
+    // that none has taken.  Neighbouring units (their tiles share DRAM pages); in a
     // launch with fewer units than warps, units go to different CTAs first
-    const int64_t first = n_units < (int64_t)gridDim.x * nwarps ? (int64_t)warp * gridDim.x + blockIdx.x
-                                                                : (int64_t)blockIdx.x * nwarps + warp;
-    const int64_t stride = (int64_t)gridDim.x * nwarps;
+    const bool spread = n_units < (int64_t)gridDim.x * kLutWarps;
+    auto unit_of = [&](int t) {
+        return spread ? (int64_t)t * gridDim.x + blockIdx.x
+                      : ((int64_t)(t / kLutWarps) * gridDim.x + blockIdx.x) * kLutWarps + t % kLutWarps;
+    };
+    int* next = reinterpret_cast<int*>(smem + (size_t)kLutWarps * (p.stage_bytes + kLutScratchBytes));
+    if (threadIdx.x == 0) *next = kLutWarps;
+    __syncthreads();
+    auto take = [&]() {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(next, 1);
+        return unit_of(__shfl_sync(0xffffffffu, t, 0));
+    };
+    const int64_t first = unit_of(warp);
+    int64_t un = 0;  // the unit after u
 
     // the lane's 16 elements, in four chunks of 4: chunk i is block elements
     // 128 i + 4 lane .. + 3, i.e. row 2 i + lane/16, columns 4 (lane % 16) ..
@@ -304,7 +319,7 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
     // quad evaluates)
     const float invf0 = p.invf[min(lane >> 2, K - 1)];
 
-    for (int64_t u = first; u < n_units; u += stride) {
+    for (int64_t u = first; u < n_units; u = un) {
         cp_async_wait_all();
         const LutTensor& T = Lp.t[ti_next];
         const uint32_t b = (uint32_t)(u - T.unit0);
@@ -523,7 +538,8 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
                 }
                 if (k0 + 8 >= K) {  // the lists are done with: the next block
                     __syncwarp();
-                    if (u + stride < n_units) issue(u + stride);
+                    un = take();
+                    if (un < n_units) issue(un);
                 }
                 // entries: lane q of a candidate has indices 2 q and 2 q + 1, i.e.
                 // the sign s (q >= 2: d >= 0) and levels 2, 3 (far: q = 0, 3) or 0, 1
@@ -913,7 +929,10 @@ __global__ void __launch_bounds__(256, 2) k_recon_lut(const __grid_constant__ Lu
             }
         }
 
-        if (flat && u + stride < n_units) issue(u + stride);
+        if (flat) {
+            un = take();
+            if (un < n_units) issue(un);
+        }
 
         // ---- outputs of the kept candidate: table, indices, r
         uint32_t bw0, bw1;
