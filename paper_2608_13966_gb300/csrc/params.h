@@ -126,9 +126,10 @@ struct Nvfp4Params {
     float beta2;
     float c1;
     float tie_kappa;
-    int stages;
     uint32_t stage_bytes;
-    uint32_t ahead_smem;  // shared memory offset of the pass beside it
+    // shared memory of the warps with a pass beside it: the first's, and each one's size
+    uint32_t ahead_smem;
+    uint32_t ahead_bytes;
     uint64_t timeout_ns;
     uint64_t force_timeout_ns;
     unsigned int* status;  // per-device status word
@@ -231,11 +232,20 @@ struct AdamwItem {
     int64_t unit0;  // as for IntTensor, in units of kAheadUnit weights
 };
 
-// A pass beside a reconstruction: the warps a CTA has for it; for AdamW, the
-// weights a tile holds, and the tiles a warp has in its ring.
-constexpr int kAheadWarps = 4;
+// Warps of an NVFP4 launch's CTA, one CTA an SM (80 registers a thread), and
+// those of them that begin with a pass for the next stage's tensors.  One layer:
+// AdamW beside the reconstruction 1,322 us with 4 warps, 1,368 with 6, 1,415
+// with 8; absmax 932, 912, 919.
+constexpr int kNvfp4Warps = 24;
+constexpr int kAdamwWarps = 4;
+constexpr int kAmaxWarps = 6;
+// AdamW beside it: the weights a tile holds, and the tiles a warp has in its
+// ring (4 warps of 4 tiles: 1,369 us, 3 of 4: 1,416).
 constexpr int kAheadUnit = 512;
 constexpr int kAheadTiles = 2;
+// Shared memory of such a warp: what its pass and then its tile take, a barrier
+// of its own at the end, rounded so that every warp's tiles are aligned.
+constexpr uint32_t ahead_region(uint32_t used) { return (used + 16 + 127) & ~127u; }
 
 struct AdamwHp {
     int g_kind;            // 1 fp32, 2 bf16

@@ -44,11 +44,8 @@ namespace {
 
 using namespace quasar;
 
-// 8 warps per CTA of the kernels with per-warp tiles: two CTAs of the
-// lookup-table kernel fill the register file (16 resident warps at 128 registers
-// a thread) and fit in an SM's shared memory.
+// Threads of the CTAs of the absmax and AdamW passes alone.
 constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 constexpr uint64_t kDefaultTimeoutNs = 1000000000ull;  // 1 s per wait
 
 std::atomic<int64_t> g_force_timeout_ns{0};
@@ -215,18 +212,6 @@ struct Launch {
     size_t smem;
 };
 
-// Shared memory per CTA of the kernels with per-warp rings: for each warp,
-// `stages` tiles of unit_bytes (QUASAR_STAGES overrides) and stages + 1
-// mbarriers.
-Launch plan(uint32_t unit_bytes, int stages)
-{
-    Launch L;
-    L.stages = tuning().stages > 0 ? tuning().stages : stages;
-    L.stage_bytes = (unit_bytes + 127u) & ~127u;
-    L.smem = (size_t)kWarps * ((size_t)L.stages * L.stage_bytes + (size_t)(L.stages + 1) * 8);
-    return L;
-}
-
 // Per-device facts looked up once: SM count and the status word's address.
 constexpr int kMaxDevices = 64;
 struct DeviceInfo {
@@ -331,7 +316,7 @@ quasar_status occupancy(const void* fn, size_t smem, int threads, int dev, int* 
 // extra_warps: warps a CTA has beside those (a fused pass of its own, which takes
 // every resident CTA); extra: that pass's parameters, the kernel's second.
 quasar_status launch_persistent(const void* fn, void* params, size_t smem, int64_t n_units,
-                                cudaStream_t stream, int warps = kWarps, void* extra = nullptr,
+                                cudaStream_t stream, int warps, void* extra = nullptr,
                                 int extra_warps = 0)
 {
     int dev = 0, occ = 0;
@@ -649,9 +634,10 @@ quasar_status launch_to_scale(const AmaxBatch<MAXT>& B, cudaStream_t s)
     return QUASAR_OK;
 }
 
-// Number the units of a launch's tensors and plan its tiles; returns them.
+// Number the units of a launch's tensors and plan the tiles of its warps that
+// reconstruct from the start; returns the units.
 template <int MAXT>
-int64_t nvfp4_number_units(Nvfp4Launch<MAXT>& Lp, size_t* smem)
+int64_t nvfp4_number_units(Nvfp4Launch<MAXT>& Lp, int warps, size_t* smem)
 {
     int64_t units = 0;
     for (int i = 0; i < Lp.n_t; ++i) {
@@ -660,12 +646,10 @@ int64_t nvfp4_number_units(Nvfp4Launch<MAXT>& Lp, size_t* smem)
     }
     Lp.n_units = units;
     const int gbytes = Lp.p.g_kind == 2 ? 2 : (Lp.p.g_kind == 1 ? 4 : 0);
-    // one tile a warp: it is in registers, and the next copy under way, before
-    // the search begins
-    const Launch L = plan((uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes)), 1);
-    Lp.p.stages = L.stages;
-    Lp.p.stage_bytes = L.stage_bytes;
-    *smem = L.smem;
+    // one tile a warp and its barrier (the tile is in registers, and the next copy
+    // under way, before the search begins), the failure hook's, the next unit's number
+    Lp.p.stage_bytes = (uint32_t)(kBlocksPerUnit * 16 * (8 + gbytes));
+    *smem = (size_t)warps * (Lp.p.stage_bytes + 8) + 16;
     return units;
 }
 
@@ -674,10 +658,10 @@ template <int MAXT>
 quasar_status nvfp4_recon(Nvfp4Launch<MAXT>& Lp, cudaStream_t s)
 {
     size_t smem = 0;
-    const int64_t units = nvfp4_number_units(Lp, &smem);
+    const int64_t units = nvfp4_number_units(Lp, kNvfp4Warps, &smem);
     if (units == 0) return QUASAR_OK;
     NoAheadArg none;
-    return launch_persistent(nvfp4_kernel(MAXT > 1), &Lp, smem, units, s, kWarps, &none);
+    return launch_persistent(nvfp4_kernel(MAXT > 1), &Lp, smem, units, s, kNvfp4Warps, &none);
 }
 
 // The AdamW steps of a launch's tensors, beside nothing.
@@ -783,13 +767,17 @@ quasar_status nvfp4_batch(int n, const Fill& fill, const Nvfp4Params& p, const A
             staged.p = p;
             staged.n_t = a1 - a0;
             for (int i = a0; i < a1; ++i) fill(i, &staged.t[i - a0], &A, &W);
-            const int64_t units = nvfp4_number_units(staged, &smem);
+            const int extra = hp ? kAdamwWarps : kAmaxWarps;
+            const int64_t units = nvfp4_number_units(staged, kNvfp4Warps - extra, &smem);
             smem = (smem + 127) & ~size_t(127);
             staged.p.ahead_smem = (uint32_t)smem;
-            if (hp) smem += kAheadWarps * kAheadTiles * (kAheadUnit * (hp->g_kind == 2 ? 14 : 16) + 8);
+            staged.p.ahead_bytes = ahead_region(
+                hp ? std::max(staged.p.stage_bytes, kAheadTiles * (kAheadUnit * (hp->g_kind == 2 ? 14u : 16u) + 8u))
+                   : staged.p.stage_bytes);
+            smem += extra * staged.p.ahead_bytes;
             fused = units > 0;
             st = fused ? launch_persistent(hp ? nvfp4_adamw_ahead_kernel() : nvfp4_amax_ahead_kernel(), &staged,
-                                           smem, units, s, kWarps, hp ? (void*)&adamw : (void*)&amax, kAheadWarps)
+                                           smem, units, s, kNvfp4Warps - extra, hp ? (void*)&adamw : (void*)&amax, extra)
                        : ahead_alone();
             if (st != QUASAR_OK) return st;
         }

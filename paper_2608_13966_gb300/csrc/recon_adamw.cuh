@@ -126,9 +126,10 @@ __global__ void __launch_bounds__(256) k_adamw_amax(const __grid_constant__ Adam
 // The step beside another kernel's work, by few warps: warp `first` of `stride`
 // takes units first, first + stride, ... (kAheadUnit weights of one tensor)
 // through a ring of tiles filled by bulk copies.  (With plain loads, two float4
-// groups a thread in flight, the eight warps an SM has for it reached 3.7 TB/s.)
+// groups a thread in flight, eight warps an SM reached 3.7 TB/s.)  False: a copy
+// did not land in time.
 template <int MAXT>
-__device__ __forceinline__ void adamw_ring(const AdamwBatch<MAXT>& B, unsigned char* ring, int64_t first,
+__device__ __forceinline__ bool adamw_ring(const AdamwBatch<MAXT>& B, unsigned char* ring, int64_t first,
                                            int64_t stride, uint64_t timeout_ns, unsigned int* status)
 {
     constexpr int S = kAheadTiles;
@@ -173,7 +174,7 @@ __device__ __forceinline__ void adamw_ring(const AdamwBatch<MAXT>& B, unsigned c
             for (int j = 0; j < S; ++j)
                 if (u + j * stride < n_units)
                     mbar_wait_bounded(&bars[(s_cur + j) % S], parity ^ (s_cur + j >= S ? 1u : 0u), timeout_ns);
-            return;
+            return false;
         }
         tensor_of(u, ti);
         const AdamwItem& T = B.t[ti];
@@ -207,6 +208,7 @@ __device__ __forceinline__ void adamw_ring(const AdamwBatch<MAXT>& B, unsigned c
         }
     }
     amax_to_slot(amax, B.t[ti_max].slot);
+    return true;
 }
 
 // Tensor absmax of a batch: blockIdx.y picks the tensor; max |w| over its n

@@ -91,59 +91,72 @@ __device__ __forceinline__ void two_prod_f(float a, float b, float& p, float& e)
     e = fmaf(a, b, -p);
 }
 
-// What the extra warps of a launch do for the next stage's tensors: nothing,
-// their absmax, or their AdamW step.
+// What some warps of a launch do first, for the next stage's tensors: nothing,
+// their absmax, or their AdamW step; and how many of a CTA's warps.
 using NoAhead = NoAheadArg;
 
-// (warp: the extra warp's number in its CTA)
-__device__ __forceinline__ void run_ahead(const NoAhead&, const Nvfp4Params&, unsigned char*, int) {}
+template <class AHEAD> struct AheadWarps { static constexpr int value = 0; };
+template <int MAXT> struct AheadWarps<AmaxBatch<MAXT>> { static constexpr int value = kAmaxWarps; };
+template <int MAXT> struct AheadWarps<AdamwBatch<MAXT>> { static constexpr int value = kAdamwWarps; };
+
+// (warp: the number among those warps; false: its copies may still land)
+__device__ __forceinline__ bool run_ahead(const NoAhead&, const Nvfp4Params&, unsigned char*, int) { return true; }
 
 template <int MAXT>
-__device__ __forceinline__ void run_ahead(const AmaxBatch<MAXT>& B, const Nvfp4Params&, unsigned char*, int warp)
+__device__ __forceinline__ bool run_ahead(const AmaxBatch<MAXT>& B, const Nvfp4Params&, unsigned char*, int warp)
 {
-    const int64_t i = ((int64_t)blockIdx.x * kAheadWarps + warp) * 32 + (threadIdx.x & 31);
-    const int64_t stride = (int64_t)gridDim.x * kAheadWarps * 32;
+    const int64_t i = ((int64_t)blockIdx.x * kAmaxWarps + warp) * 32 + (threadIdx.x & 31);
+    const int64_t stride = (int64_t)gridDim.x * kAmaxWarps * 32;
     for (int t = 0; t < B.n_t; ++t)
         if (!B.t[t].amax_in && B.t[t].n) amax_to_slot(amax_span<4>(B.t[t].w, B.t[t].n, i, stride), B.t[t].slot);
+    return true;
 }
 
 template <int MAXT>
-__device__ __forceinline__ void run_ahead(const AdamwBatch<MAXT>& B, const Nvfp4Params& p, unsigned char* smem, int warp)
+__device__ __forceinline__ bool run_ahead(const AdamwBatch<MAXT>& B, const Nvfp4Params& p, unsigned char* region, int warp)
 {
-    const uint32_t bytes = kAheadTiles * (kAheadUnit * (B.hp.g_kind == 2 ? 14u : 16u) + 8u);
-    adamw_ring(B, smem + p.ahead_smem + warp * bytes, (int64_t)warp * gridDim.x + blockIdx.x,
-               (int64_t)gridDim.x * kAheadWarps, p.timeout_ns, p.status);
+    return adamw_ring(B, region, (int64_t)warp * gridDim.x + blockIdx.x, (int64_t)gridDim.x * kAdamwWarps,
+                      p.timeout_ns, p.status);
 }
 
 // The reconstruction is bound by instruction issue, and the pass that must
-// precede it (absmax, or the AdamW step) by memory, but within a tensor the one
+// precede it (the tensor's absmax, or the AdamW step, whose w' it is of) by
+// memory, so the two belong side by side; but one tensor's reconstruction
 // needs all of the other.  So a batch is cut into stages of whole tensors, and
-// the launch of a stage carries four more warps a CTA that run the pass of the
-// next stage's tensors beside it.  58.7 M weights of AdamW beside as many of
-// reconstruction take 346 us, 6.1 TB/s (236 + 217 one after the other); one
-// layer of AdamW + NVFP4 1,394 us (1,663), absmax and NVFP4 994 (1,015).
-// Alone: three CTAs an SM (80 registers) and the loop over candidates unrolled
-// by 2: 1,021 us a layer with its absmax pass before it; two CTAs 1,041, no
-// unrolling at two CTAs 1,052.
+// some warps of a stage's launch begin with the pass of the next stage's tensors,
+// and then join those that reconstruct.  One CTA of 24 warps an SM (80
+// registers; the loop over candidates unrolled by 2), its warps taking units as
+// they get free.  One layer (218 M weights): with its absmax 994 -> 912 us, with
+// AdamW 1,405 -> 1,322, an attention block without gradient 174 -> 160.  Before:
+// a fixed share of the units a warp in three CTAs of 8 warps, or two and four
+// more each for the pass, idle after it; and with the passes one after the other,
+// 1,015 and 1,663 us.
 template <int MAXT, class AHEAD>
-__global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 384,
-                                  std::is_same<AHEAD, NoAhead>::value ? 3 : 2)
+__global__ void __launch_bounds__(kNvfp4Warps * 32, 1)
     k_recon_nvfp4(const __grid_constant__ Nvfp4Launch<MAXT> Lp, const __grid_constant__ AHEAD ahead)
 {
     const Nvfp4Params& p = Lp.p;
     constexpr int UNIT = kBlocksPerUnit * 16;
-    constexpr int nwarps = 8;  // those that reconstruct
+    constexpr bool kAlone = std::is_same<AHEAD, NoAhead>::value;
+    // those that reconstruct from the start; the others join them after the pass
+    constexpr int nwarps = kNvfp4Warps - AheadWarps<AHEAD>::value;
     extern __shared__ __align__(128) unsigned char smem[];
-    if (!std::is_same<AHEAD, NoAhead>::value && threadIdx.x >= nwarps * 32) {
-        run_ahead(ahead, p, smem, (int)(threadIdx.x >> 5) - nwarps);
-        return;
-    }
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int S = p.stages;
-    unsigned char* ring = smem + (size_t)warp * S * p.stage_bytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nwarps * S * p.stage_bytes) + warp * (S + 1);
+    // a tile a warp, their barriers, one for the failure hook, the next unit's
+    // number; then the regions of the warps with a pass of their own
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)nwarps * p.stage_bytes) + warp;
+    uint64_t* hook = bar - warp + nwarps;
+    int* next = reinterpret_cast<int*>(hook + 1);
+    unsigned char* st = smem + (size_t)warp * p.stage_bytes;
+    if (threadIdx.x == 0) *next = nwarps;
+    __syncthreads();
+    if (!kAlone && warp >= nwarps) {
+        st = smem + p.ahead_smem + (warp - nwarps) * p.ahead_bytes;
+        if (!run_ahead(ahead, p, st, warp - nwarps)) return;
+        bar = reinterpret_cast<uint64_t*>(st + p.ahead_bytes - 16);
+    }
 
     const int gbytes = p.g_kind == 2 ? 2 : (p.g_kind == 1 ? 4 : 0);
     constexpr uint32_t kVOff = UNIT * 4;
@@ -157,53 +170,55 @@ __global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 38
     };
     int ti = 0, ti_s = -1;
     float sT = 1.0f, inv_sT = 1.0f;
-    // a CTA's warps take neighbouring units (their tiles share DRAM pages: an
-    // attention block without gradient takes 174 us, 178 otherwise); units go to
-    // different CTAs first in a launch with fewer units than warps, and beside
-    // another pass (AdamW + NVFP4 on one layer: 1,394 us, 1,457 otherwise)
-    const bool spread = !std::is_same<AHEAD, NoAhead>::value || n_units < (int64_t)gridDim.x * nwarps;
-    const int64_t first = spread ? (int64_t)warp * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * nwarps + warp;
-    const int64_t stride = (int64_t)gridDim.x * nwarps;
-
+    // the CTA's units t = 0, 1, ...: warps start with theirs, then take the next
+    // that none has taken.  Neighbouring units (their tiles share DRAM pages: an
+    // attention block without gradient, fixed shares, 174 us, 178 otherwise); units
+    // go to different CTAs first in a launch with fewer units than warps, and
+    // beside another pass (NVFP4 with 109 M weights' absmax 731 us, 739 otherwise)
+    const bool spread = !kAlone || n_units < (int64_t)gridDim.x * nwarps;
+    auto unit_of = [&](int t) {
+        return spread ? (int64_t)t * gridDim.x + blockIdx.x
+                      : ((int64_t)(t >> 3) * gridDim.x + blockIdx.x) * 8 + (t & 7);
+    };
+    auto take = [&]() {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(next, 1);
+        return unit_of(__shfl_sync(0xffffffffu, t, 0));
+    };
 
     if (lane == 0) {
-        for (int s = 0; s <= S; ++s) mbar_init(&bars[s], 1);
+        mbar_init(bar, 1);
+        if (warp == 0) mbar_init(hook, 1);
         mbar_init_fence();
     }
     __syncwarp();
 
-    auto issue = [&](int64_t u, int s) {
+    auto issue = [&](int64_t u) {
         int tj = ti;
         tensor_of(u, tj);
         const Nvfp4Tensor& T = Lp.t[tj];
         const int64_t b0 = (u - T.unit0) * kBlocksPerUnit;
         const int64_t nb = min((int64_t)kBlocksPerUnit, T.n_blocks - b0);
         const uint32_t elems = (uint32_t)(nb * 16);
-        unsigned char* st = ring + (size_t)s * p.stage_bytes;
-        mbar_arrive_expect_tx(&bars[s], elems * (8u + (uint32_t)gbytes));
-        bulk_g2s(st, T.w + b0 * 16, elems * 4u, &bars[s]);
-        bulk_g2s(st + kVOff, T.v + b0 * 16, elems * 4u, &bars[s]);
+        mbar_arrive_expect_tx(bar, elems * (8u + (uint32_t)gbytes));
+        bulk_g2s(st, T.w + b0 * 16, elems * 4u, bar);
+        bulk_g2s(st + kVOff, T.v + b0 * 16, elems * 4u, bar);
         if (gbytes)
             bulk_g2s(st + kGOff, static_cast<const unsigned char*>(T.g) + b0 * 16 * gbytes,
-                     elems * (uint32_t)gbytes, &bars[s]);
+                     elems * (uint32_t)gbytes, bar);
     };
-    auto fail = [&](int64_t it) {
+    // Record the failure and wait (bounded) for the copy in flight
+    auto fail = [&](uint32_t parity) {
         if (lane == 0) record_timeout(p.status);
-        for (int j = 0; j < S; ++j) {
-            const int64_t u = first + (it + j) * stride;
-            if (u >= n_units) break;
-            mbar_wait_bounded(&bars[(it + j) % S], (uint32_t)(((it + j) / S) & 1), p.timeout_ns);
-        }
+        mbar_wait_bounded(bar, parity, p.timeout_ns);
     };
 
-    if (lane == 0)
-        for (int s = 0; s < S; ++s) {
-            const int64_t u = first + s * stride;
-            if (u < n_units) issue(u, s);
-        }
+    int64_t u = kAlone || warp < nwarps ? unit_of(warp) : take();
+    if (lane == 0 && u < n_units) issue(u);
     if (p.force_timeout_ns && blockIdx.x == 0 && warp == 0) {
-        if (!warp_wait_bounded(&bars[S], 0, p.force_timeout_ns)) {
-            fail(0);
+        if (!warp_wait_bounded(hook, 0, p.force_timeout_ns)) {
+            if (u < n_units) fail(0);
+            else if (lane == 0) record_timeout(p.status);
             return;
         }
     }
@@ -212,8 +227,8 @@ __global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 38
     const float ulp = 5.9604645e-8f * p.tie_kappa;
     const float2 beta22 = make_float2(p.beta2, p.beta2);
     const float2 c12 = make_float2(p.c1, p.c1);
-    int s_cur = 0;
     uint32_t parity = 0;
+    int64_t un = 0;  // the unit after u
 
     // E2M1 values of two values y: the hardware conversion rounds
     // to nearest, ties to the even code, and saturates at 6; converting the
@@ -227,14 +242,11 @@ __global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 38
         return __half22float2(*reinterpret_cast<__half2*>(&hh));
     };
 
-    for (int64_t it = 0;; ++it) {
-        const int64_t u = first + it * stride;
-        if (u >= n_units) break;
-        if (!warp_wait_bounded(&bars[s_cur], parity, p.timeout_ns)) {
-            fail(it);
+    for (; u < n_units; u = un, parity ^= 1u) {
+        if (!warp_wait_bounded(bar, parity, p.timeout_ns)) {
+            fail(parity);
             return;
         }
-        const unsigned char* st = ring + (size_t)s_cur * p.stage_bytes;
 
         // element 4*cidx[i] + jj of this lane's block is held at slot 4*i + jj,
         // pairs (slot 2t, 2t+1) in w2[t], h2[t].  The search keeps the signs: codes,
@@ -274,14 +286,8 @@ __global__ void __launch_bounds__(std::is_same<AHEAD, NoAhead>::value ? 256 : 38
         else if (p.g_kind == 1) load(std::integral_constant<int, 1>{});
         else load(std::integral_constant<int, 0>{});
         __syncwarp();
-        if (lane == 0) {
-            const int64_t un = u + (int64_t)S * stride;
-            if (un < n_units) issue(un, s_cur);
-        }
-        if (++s_cur == S) {
-            s_cur = 0;
-            parity ^= 1u;
-        }
+        un = take();
+        if (lane == 0 && un < n_units) issue(un);
 
         tensor_of(u, ti);
         const Nvfp4Tensor& T = Lp.t[ti];

@@ -192,3 +192,33 @@ def test_tiles_shared_by_the_warps_of_a_cta(G, g_dtype, adam, symmetric):
     for key in whole:
         if whole[key] is not None:
             assert torch.equal(whole[key], torch.cat([p[key] for p in parts])), key
+
+
+@pytest.mark.parametrize("g_dtype,adam", [(torch.bfloat16, False), (torch.float32, False), (None, False),
+                                          (torch.bfloat16, True), (torch.float32, True)])
+def test_nvfp4_warps_that_begin_with_the_next_stage(g_dtype, adam):
+    """A batch in several stages (some warps of a launch take the absmax or the
+    AdamW step of the next stage's tensors first, then reconstruct): the outputs
+    equal those of one call a tensor.  A small last tensor, a ragged row."""
+    shapes = [(4099, 2048), (4096, 2064), (8200, 1024), (3, 16)]
+    items = []
+    for i, (r, c) in enumerate(shapes):
+        w, g, v = _inputs(r, c, seed=4600 + i)
+        m = 1e-4 * torch.randn(r, c, device="cuda", generator=torch.Generator("cuda").manual_seed(i))
+        items.append((w, None if g_dtype is None else g.to(g_dtype), m, v))
+
+    def run(items):
+        items = [tuple(None if x is None else x.clone() for x in it) for it in items]
+        if adam:
+            out = api.adamw_recon_nvfp4_batch(items, clip=CLIP8, codes=True, lr=1e-5, step=3)
+        else:
+            out = api.recon_nvfp4_batch([(w, g, v) for w, g, _, v in items], clip=CLIP8, codes=True)
+        return [dict(o, w=it[0], m=it[2], v=it[3]) for o, it in zip(out, items)]
+
+    whole = run(items)
+    single = [run([it])[0] for it in items]
+    torch.cuda.synchronize()
+    for a, b in zip(whole, single):
+        for key in a:
+            if a[key] is not None:
+                assert torch.equal(a[key], b[key]), key
