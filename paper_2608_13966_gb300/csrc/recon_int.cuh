@@ -589,9 +589,11 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
             auto pass_a = [&](auto gk) {
                 constexpr int GK = decltype(gk)::value;
                 float2 SS2 = make_float2(0.0f, 0.0f), SW = SS2;
-// two chunks an iteration (one with more than 8 candidates): the loop stays
-// small in the instruction cache
-#pragma unroll (NCH == 1 ? 2 : 1)
+// two chunks an iteration; one with more than 8 candidates or groups of 64 and
+// less, whose careful paths run often and need the instruction cache (AdamW +
+// INT3 g64, 113 M weights, 598 -> 543 us; INT4 g64, 119 M, packed, 674 -> 620;
+// groups of 128 got slower, one layer INT3 by 1.5%)
+#pragma unroll (NCH == 1 && EPL > 16 ? 2 : 1)
                 for (int i = 0; i < NCHK; ++i) {
                     const int eo = eoff(i);
                     const int e = gs * G + eo;
@@ -1332,7 +1334,7 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
             // fast: none of these (and the folded offset)
             auto pass_c = [&](auto general) {
                 constexpr bool GEN = decltype(general)::value;
-#pragma unroll (NCH == 1 ? 2 : 1)
+#pragma unroll (NCH == 1 && EPL > 16 ? 2 : 1)
                 for (int i = 0; i < NCHK; ++i) {
                     const int eo = eoff(i);
                     const float4 w4 = lds128(gws + eo);
