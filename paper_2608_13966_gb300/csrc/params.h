@@ -232,15 +232,18 @@ struct AdamwItem {
     int64_t unit0;  // as for IntTensor, in units of kAheadUnit weights
 };
 
-// Warps of an NVFP4 launch's CTA, one CTA an SM (80 registers a thread), and
-// those of them that begin with a pass for the next stage's tensors.  One layer:
-// AdamW beside the reconstruction 1,322 us with 4 warps, 1,368 with 6, 1,415
-// with 8; absmax 932, 912, 919.
+// Warps of an NVFP4 launch's CTA, one CTA an SM: 24 of 80 registers a thread, or
+// 20 of 96 beside AdamW, which then need not spill; and those of them that begin
+// with a pass for the next stage's tensors.  One layer, AdamW beside the
+// reconstruction: 1,291 us with 4 of 20 warps (5: 1,330, 3: 1,425), 1,322 with 4
+// of 24 (6: 1,368, 8: 1,415), 1,304 with 4 of 16; absmax beside it 912 with 6 of
+// 24 (8: 919, 4: 932), 937 with 6 of 20.
 constexpr int kNvfp4Warps = 24;
+constexpr int kNvfp4AdamwWarps = 20;
 constexpr int kAdamwWarps = 4;
 constexpr int kAmaxWarps = 6;
 // AdamW beside it: the weights a tile holds, and the tiles a warp has in its
-// ring (4 warps of 4 tiles: 1,369 us, 3 of 4: 1,416).
+// ring (with 24 warps, 4 of 4 tiles 1,369 us, 3 of 4 tiles 1,416).
 constexpr int kAheadUnit = 512;
 constexpr int kAheadTiles = 2;
 // Shared memory of such a warp: what its pass and then its tile take, a barrier

@@ -767,8 +767,8 @@ quasar_status nvfp4_batch(int n, const Fill& fill, const Nvfp4Params& p, const A
             staged.p = p;
             staged.n_t = a1 - a0;
             for (int i = a0; i < a1; ++i) fill(i, &staged.t[i - a0], &A, &W);
-            const int extra = hp ? kAdamwWarps : kAmaxWarps;
-            const int64_t units = nvfp4_number_units(staged, kNvfp4Warps - extra, &smem);
+            const int extra = hp ? kAdamwWarps : kAmaxWarps, warps = (hp ? kNvfp4AdamwWarps : kNvfp4Warps) - extra;
+            const int64_t units = nvfp4_number_units(staged, warps, &smem);
             smem = (smem + 127) & ~size_t(127);
             staged.p.ahead_smem = (uint32_t)smem;
             staged.p.ahead_bytes = ahead_region(
@@ -777,7 +777,7 @@ quasar_status nvfp4_batch(int n, const Fill& fill, const Nvfp4Params& p, const A
             smem += extra * staged.p.ahead_bytes;
             fused = units > 0;
             st = fused ? launch_persistent(hp ? nvfp4_adamw_ahead_kernel() : nvfp4_amax_ahead_kernel(), &staged,
-                                           smem, units, s, kNvfp4Warps - extra, hp ? (void*)&adamw : (void*)&amax, extra)
+                                           smem, units, s, warps, hp ? (void*)&adamw : (void*)&amax, extra)
                        : ahead_alone();
             if (st != QUASAR_OK) return st;
         }

@@ -95,9 +95,9 @@ __device__ __forceinline__ void two_prod_f(float a, float b, float& p, float& e)
 // their absmax, or their AdamW step; and how many of a CTA's warps.
 using NoAhead = NoAheadArg;
 
-template <class AHEAD> struct AheadWarps { static constexpr int value = 0; };
-template <int MAXT> struct AheadWarps<AmaxBatch<MAXT>> { static constexpr int value = kAmaxWarps; };
-template <int MAXT> struct AheadWarps<AdamwBatch<MAXT>> { static constexpr int value = kAdamwWarps; };
+template <class AHEAD> struct AheadWarps { static constexpr int all = kNvfp4Warps, value = 0; };
+template <int MAXT> struct AheadWarps<AmaxBatch<MAXT>> { static constexpr int all = kNvfp4Warps, value = kAmaxWarps; };
+template <int MAXT> struct AheadWarps<AdamwBatch<MAXT>> { static constexpr int all = kNvfp4AdamwWarps, value = kAdamwWarps; };
 
 // (warp: the number among those warps; false: its copies may still land)
 __device__ __forceinline__ bool run_ahead(const NoAhead&, const Nvfp4Params&, unsigned char*, int) { return true; }
@@ -125,21 +125,21 @@ __device__ __forceinline__ bool run_ahead(const AdamwBatch<MAXT>& B, const Nvfp4
 // needs all of the other.  So a batch is cut into stages of whole tensors, and
 // some warps of a stage's launch begin with the pass of the next stage's tensors,
 // and then join those that reconstruct.  One CTA of 24 warps an SM (80
-// registers; the loop over candidates unrolled by 2), its warps taking units as
-// they get free.  One layer (218 M weights): with its absmax 994 -> 912 us, with
-// AdamW 1,405 -> 1,322, an attention block without gradient 174 -> 160.  Before:
+// registers, 20 of 96 beside AdamW; the loop over candidates unrolled by 2), its
+// warps taking units as they get free.  One layer (218 M weights): with its absmax 994 -> 912 us, with
+// AdamW 1,405 -> 1,291, an attention block without gradient 174 -> 160.  Before:
 // a fixed share of the units a warp in three CTAs of 8 warps, or two and four
 // more each for the pass, idle after it; and with the passes one after the other,
 // 1,015 and 1,663 us.
 template <int MAXT, class AHEAD>
-__global__ void __launch_bounds__(kNvfp4Warps * 32, 1)
+__global__ void __launch_bounds__(AheadWarps<AHEAD>::all * 32, 1)
     k_recon_nvfp4(const __grid_constant__ Nvfp4Launch<MAXT> Lp, const __grid_constant__ AHEAD ahead)
 {
     const Nvfp4Params& p = Lp.p;
     constexpr int UNIT = kBlocksPerUnit * 16;
     constexpr bool kAlone = std::is_same<AHEAD, NoAhead>::value;
     // those that reconstruct from the start; the others join them after the pass
-    constexpr int nwarps = kNvfp4Warps - AheadWarps<AHEAD>::value;
+    constexpr int nwarps = AheadWarps<AHEAD>::all - AheadWarps<AHEAD>::value;
     extern __shared__ __align__(128) unsigned char smem[];
 
     const int lane = threadIdx.x & 31;
