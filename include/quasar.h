@@ -283,9 +283,13 @@ quasar_status quasar_recon_nvfp4(const float* w, const void* g, quasar_dtype g_d
 
 /*
  * quasar_nvfp4_tensor / quasar_recon_nvfp4_batch -- quasar_recon_nvfp4 over
- * many tensors with the same settings: one absmax pass over the tensors
- * whose amax is not supplied, one scale pass, and one persistent
- * reconstruction launch whose units are numbered across the tensors.
+ * many tensors with the same settings.  With every amax supplied it is one
+ * persistent reconstruction launch whose units are numbered across the
+ * tensors.  Otherwise the tensors are processed in up to about 8 groups of
+ * consecutive tensors, each of at least 2^23 weights: one launch a group, which
+ * also takes the absmax of the next group's tensors (the first group's is a
+ * launch of its own).  The scale slots become s_T at the end, in one launch:
+ * until the call's work is complete they hold an intermediate value.
  * Each descriptor holds one tensor's arguments as quasar_recon_nvfp4 takes
  * them (same meaning and rules; each tensor has its own tensor_scale slot and
  * optional tensor_amax); either every non-empty tensor has a gradient or none
@@ -325,10 +329,12 @@ quasar_status quasar_recon_nvfp4_batch_ex(const quasar_nvfp4_tensor* tensors, in
  * step (as quasar_adamw_recon_int_batch) followed by the NVFP4
  * reconstruction (as quasar_recon_nvfp4_batch) of the updated weights with
  * saliency h = v'.  The NVFP4 tensor scale needs the absmax of w' before any
- * block is reconstructed, so the step is two passes: one over w, g, m, v
- * that writes w', m', v' and takes max |w'| per tensor (no separate absmax
- * pass), and the reconstruction pass over w', v' (no gradient: v is not
- * updated twice).  Reads 14 + 8 and writes 12 + 2 bytes a weight.
+ * block is reconstructed, so each tensor has two passes: one over w, g, m, v
+ * that writes w', m', v' and takes max |w'| (no separate absmax pass), and the
+ * reconstruction pass over w', v' (no gradient: v is not updated twice).  As in
+ * quasar_recon_nvfp4_batch, the first pass of a group of tensors runs in the
+ * reconstruction launch of the group before it.  Reads 14 + 8 and writes 12 + 2
+ * bytes a weight.
  *
  * Descriptor fields as in quasar_nvfp4_tensor without tensor_amax, plus m
  * (fp32 first moment, read and overwritten); w is overwritten with w'.  g

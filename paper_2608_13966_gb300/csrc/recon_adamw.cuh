@@ -1,9 +1,9 @@
 // The passes that come before an NVFP4 reconstruction of a tensor (which needs
 // the tensor's absmax before any block is processed): the absmax of w, or one
-// AdamW step that also takes the absmax of the updated weights.  The arithmetic is the integer kernel's fused
-// step, element for element: packed fp32, the root as v' rsqrt(v'), the
-// quotient by the fast reciprocal, and w' = w + (-(w lr wd) - step m'/den)
-// rounded once.
+// AdamW step that also takes the absmax of the updated weights.  The arithmetic
+// is the integer kernel's fused step, element for element: packed fp32, the root
+// as v' rsqrt(v'), the quotient by the fast reciprocal, and w' = w + (-(w lr wd)
+// - step m'/den) rounded once.
 #pragma once
 
 #include <cuda_bf16.h>

@@ -416,8 +416,8 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
 // warp, had the same registers and shared memory: one Llama layer INT3 786 us
 // (one CTA with fixed shares 747, as built 740), INT3 15 factors 1,234 (now
 // 1,154), the Qwen3 layer INT2 g64 16 factors 1,551 (fixed shares 1,448, now
-// 1,408), AdamW + INT3 988 (now 916, 14 warps and 2 slots in flight, 0.985 of
-// the measured copy rate).  With fixed shares a warp count that is no multiple
+// 1,408), AdamW + INT3 988 (now 916, 15 warps and one slot in flight, 0.985
+// of the measured copy rate).  With fixed shares a warp count that is no multiple
 // of the SM's 4 schedulers was worse than the next lower multiple.  20 warps at
 // 96 registers spill: INT3 885 us.
 // VAR: the variants of the options (a saliency other than v', packed codes);

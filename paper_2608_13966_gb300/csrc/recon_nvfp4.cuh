@@ -27,7 +27,7 @@
 // 95 a weight and lane at 8 candidates, 112 before (with absolute values, a
 // hash and an error kept for every candidate, and divisions, E4M3 decoding and
 // sign handling spelled out).  One Llama layer (218 M weights), absmax pass and
-// codes included: 1,152 -> 1,021 us.  Candidate lists that are not a multiple
+// codes included: 1,152 -> 1,021 us (912 as launched now).  Candidate lists that are not a multiple
 // of 8 used to send every block to the exact comparison.
 #pragma once
 
@@ -126,8 +126,9 @@ __device__ __forceinline__ bool run_ahead(const AdamwBatch<MAXT>& B, const Nvfp4
 // some warps of a stage's launch begin with the pass of the next stage's tensors,
 // and then join those that reconstruct.  One CTA of 24 warps an SM (80
 // registers, 20 of 96 beside AdamW; the loop over candidates unrolled by 2), its
-// warps taking units as they get free.  One layer (218 M weights): with its absmax 994 -> 912 us, with
-// AdamW 1,405 -> 1,291, an attention block without gradient 174 -> 160.  Before:
+// warps taking units as they get free.  One layer (218 M weights): with its
+// absmax 994 -> 912 us, with AdamW 1,405 -> 1,291, an attention block without
+// gradient 174 -> 160.  Before:
 // a fixed share of the units a warp in three CTAs of 8 warps, or two and four
 // more each for the pass, idle after it; and with the passes one after the other,
 // 1,015 and 1,663 us.
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(AheadWarps<AHEAD>::all * 32, 1)
         };
         // the best candidate, and the lowest error of the others whose key is
         // not the best's: two numbers a block instead of an error and a key a
-        // candidate, so that three CTAs fit an SM and any number of factors
+        // candidate, so that 24 warps fit an SM and any number of factors
         // takes one loop
         Fit best = evaluate(0);
         int kb = 0;
