@@ -234,4 +234,11 @@ __device__ __forceinline__ void tiny_scale(float x, float& s1, float& s2)
     s2 = __uint_as_float((uint32_t)(127 - e) << 23);
 }
 
+// Groups of integer codes whose weights' own range (symmetric codes: largest
+// magnitude) is below 2^-20 are reconstructed with their weights scaled the
+// same way, exactly, and their fit scaled back.  Down there the scale of the
+// codes, q_max / (f range), leaves fp32's range (below about 2^-120), and before
+// that the products of the error sums do.
+constexpr float kTinyWeights = 9.536743e-7f;  // 2^-20
+
 }  // namespace quasar

@@ -460,7 +460,11 @@ quasar_status int_params(quasar_dtype g_dtype, bool has_g, float beta2, int bits
     p->timeout_ns = kDefaultTimeoutNs;
     p->force_timeout_ns = (uint64_t)std::max<int64_t>(0, g_force_timeout_ns.load());
     p->stats = g_stats.load();
-    fill_clip(clip, n_clip, p->f, p->invf);
+    // a factor below 2^-90 acts as 2^-90, which keeps q_max / (f range) finite
+    // (only weights below that part of their group's range could tell)
+    float f[kMaxClip];
+    for (int k = 0; k < n_clip; ++k) f[k] = std::max(clip[k], std::ldexp(1.0f, -90));
+    fill_clip(f, n_clip, p->f, p->invf);
     bool up = true, down = true;
     for (int k = 1; k < n_clip; ++k) {
         up &= p->invf[k] >= p->invf[k - 1];

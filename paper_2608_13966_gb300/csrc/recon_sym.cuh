@@ -293,19 +293,26 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1) k_recon_sym(const 
             amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
             ss += __shfl_xor_sync(0xffffffffu, ss, o);
         }
-        // all saliencies zero: h = 1; a sum of saliencies near the bottom of
-        // the fp32 range: h scaled by a power of two
-        if (__any_sync(0xffffffffu, ss < kTinySaliency)) {
-            if (ss < kTinySaliency) {
-                float s1 = 1.0f, s2 = 1.0f;
-                if (ss > 0.0f) tiny_scale(ss, s1, s2);
+        // all saliencies zero: h = 1; a sum of saliencies, or weights, near the
+        // bottom of the fp32 range: scaled by a power of two in the tile
+        float unscale = 1.0f;  // of the fit
+        const bool h_tiny = ss < kTinySaliency, w_tiny = amax < kTinyWeights;  // (zeros stay zeros)
+        if (__any_sync(0xffffffffu, h_tiny || w_tiny)) {
+            if (h_tiny || w_tiny) {
+                float s1 = 1.0f, s2 = 1.0f, t1 = 1.0f, t2 = 1.0f;
+                if (h_tiny && ss > 0.0f) tiny_scale(ss, s1, s2);
+                if (w_tiny) tiny_scale(amax, t1, t2);
 #pragma unroll 1
                 for (int i = 0; i < NCHK; ++i) {
                     float4* hp = reinterpret_cast<float4*>(hs + gs * G + eoff(i));
-                    const float4 h4 = *hp;
+                    float4* wp = reinterpret_cast<float4*>(ws + gs * G + eoff(i));
+                    const float4 h4 = *hp, w4 = *wp;
                     *hp = ss > 0.0f ? make_float4(h4.x * s1 * s2, h4.y * s1 * s2, h4.z * s1 * s2, h4.w * s1 * s2)
                                     : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+                    *wp = make_float4(w4.x * t1 * t2, w4.y * t1 * t2, w4.z * t1 * t2, w4.w * t1 * t2);
                 }
+                amax = amax * t1 * t2;
+                unscale = (1.0f / t2) * (1.0f / t1);  // a power of two from 2^-149 on: exact
             }
         }
         // the gradient region becomes the candidates' table: every lane is past
@@ -508,6 +515,7 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1) k_recon_sym(const 
         }
 
         // ---- outputs: r = a q, codes q + Q, a, b = -a Q, index
+        a_sel *= unscale;
         const float Pk = R * p.invf[kb];
         const float capk = p.cap[kb] * amax;
         {

@@ -222,3 +222,50 @@ def test_nvfp4_warps_that_begin_with_the_next_stage(g_dtype, adam):
         for key in a:
             if a[key] is not None:
                 assert torch.equal(a[key], b[key]), key
+
+
+def _small_weights(rows, G, seed):
+    """Groups (one a row) of multiples of 2^-12, zeros among them, which a power
+    of two scales without rounding down to 2^-137."""
+    w, _, v = _inputs(rows, G, seed=seed)
+    w = torch.round(w * 4096.0) / 4096.0
+    w[0], w[1, ::2] = 0.0, 0.0
+    w[2] = (torch.arange(G, device="cuda") * 5 % 7 - 3) / 4096.0
+    w[3] += 0.125                                          # one sign, a small range
+    return w, v
+
+
+@pytest.mark.parametrize("e", [-22, -100, -122, -135])
+@pytest.mark.parametrize("bits,G,clip", [(2, 64, CLIP8), (4, 128, CLIP8), (8, 32, wl.CLIP_16),
+                                         (4, 256, (1.0, 0.25)), (3, 128, (1.0, 0.5, 1e-30, 1e-37))],
+                         ids=["int2", "int4", "int8_k16", "int4_two", "tiny_factors"])
+@pytest.mark.parametrize("symmetric", [True])
+def test_weights_scaled_by_a_power_of_two(oracle, symmetric, bits, G, clip, e):
+    """Groups of weights down to the smallest denormals keep the factor and the
+    codes that the same weights have at their usual size, and a fit and an r
+    smaller by the power of two (both code layouts)."""
+    w, v = _small_weights(40, G, seed=4700 + bits)
+    s = 2.0 ** e
+
+    def run(w, packed):
+        o = api.recon_int_batch([(w, None, v.clone())], bits=bits, group_size=G, clip=list(clip), codes=True,
+                                symmetric=symmetric, packed_codes=packed, r_dtype=torch.float32)[0]
+        torch.cuda.synchronize()
+        return o
+
+    ref, small, packed = run(w, False), run(w * s, False), run(w * s, True)
+    for key in ("codes", "cand_idx"):
+        assert torch.equal(small[key], ref[key]), key
+    assert np.array_equal(oracle.unpack_int_codes(packed["codes"].cpu().numpy(), bits, w.numel()),
+                          small["codes"].cpu().numpy().ravel())
+    for key in ("r", "a", "b"):
+        want, got = ref[key].double() * s, small[key].double()
+        # both sides within 1e-7 + 1e-5 |x| at a size about 1 (ref's own: 0.1),
+        # and the spacing of the denormals, of which r sums up to 256
+        lim = 2e-5 * want.abs() + s * 2e-7 + 256 * 2.0 ** -149
+        assert bool(((got - want).abs() <= lim).all()), key  # (a NaN fails)
+        assert torch.equal(packed[key], small[key]), key
+    w_h, h = H._host(w * s), H._host(v)
+    O = (oracle.recon_sym if symmetric else oracle.recon_int)(w_h, h, G, bits, list(clip))
+    same = (O["m_round"] >= checker.MARGIN) & (O["m_tie"] >= checker.MARGIN)
+    assert np.array_equal(small["cand_idx"].cpu().numpy()[same], O["idx"][same])
