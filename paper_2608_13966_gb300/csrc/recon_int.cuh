@@ -706,33 +706,36 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
             sw += shx(sw, o);
         }
         // all saliencies zero: the group is fitted with h = 1 (the tile's h
-        // is overwritten; v' has been written out already)
+        // is overwritten; v' has been written out already).  A sum of saliencies,
+        // or a range, near the bottom of the fp32 range: h or w scaled by a power
+        // of two in the tile, and the sums taken again
+        float unscale = 1.0f;  // of the fit
         const bool h_one = ss == 0.0f;
-        if (__any_sync(0xffffffffu, h_one)) {
-            if (h_one)
-#pragma unroll
-                for (int i = 0; i < NCHK; ++i)
-                    *reinterpret_cast<float4*>(ghs + eoff(i)) = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
-        }
-        // a sum of saliencies near the bottom of the fp32 range: h scaled by
-        // a power of two in the tile, and its sums taken again
-        const bool h_tiny = !h_one && ss < kTinySaliency;
-        if (__any_sync(0xffffffffu, h_tiny)) {
-            float s1 = 1.0f, s2 = 1.0f;
-            tiny_scale(ss, s1, s2);
+        const bool h_tiny = ss < kTinySaliency, w_tiny = mx - mn < kTinyWeights && mx > mn;
+        if (__any_sync(0xffffffffu, h_tiny || w_tiny)) {
             float2 SS2 = make_float2(0.0f, 0.0f), SW = SS2;
-            if (h_tiny) {
+            if (h_tiny || w_tiny) {
+                float s1 = 1.0f, s2 = 1.0f, t1 = 1.0f, t2 = 1.0f;
+                if (h_tiny && !h_one) tiny_scale(ss, s1, s2);
+                if (w_tiny) tiny_scale(mx - mn, t1, t2);
 #pragma unroll 1
                 for (int i = 0; i < NCHK; ++i) {
-                    const float4 w4 = lds128(gws + eoff(i));
-                    float4 h4 = lds128(ghs + eoff(i));
-                    h4 = make_float4(h4.x * s1 * s2, h4.y * s1 * s2, h4.z * s1 * s2, h4.w * s1 * s2);
-                    *reinterpret_cast<float4*>(ghs + eoff(i)) = h4;
+                    float4* wp = reinterpret_cast<float4*>(ws + gs * G + eoff(i));
+                    float4* hp = reinterpret_cast<float4*>(ghs + eoff(i));
+                    float4 w4 = *wp, h4 = *hp;
+                    w4 = make_float4(w4.x * t1 * t2, w4.y * t1 * t2, w4.z * t1 * t2, w4.w * t1 * t2);
+                    h4 = h_one ? make_float4(1.0f, 1.0f, 1.0f, 1.0f)
+                               : make_float4(h4.x * s1 * s2, h4.y * s1 * s2, h4.z * s1 * s2, h4.w * s1 * s2);
+                    *wp = w4;
+                    *hp = h4;
                     const float2 hA = make_float2(h4.x, h4.y), hB = make_float2(h4.z, h4.w);
                     SS2 = __fadd2_rn(SS2, __fadd2_rn(hA, hB));
                     SW = __ffma2_rn(hA, make_float2(w4.x, w4.y), SW);
                     SW = __ffma2_rn(hB, make_float2(w4.z, w4.w), SW);
                 }
+                mn = mn * t1 * t2;
+                mx = mx * t1 * t2;
+                unscale = (1.0f / t2) * (1.0f / t1);  // a power of two from 2^-149 on: exact
             }
             float ss2 = SS2.x + SS2.y, sw2 = SW.x + SW.y;
 #pragma unroll
@@ -740,7 +743,7 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
                 ss2 += shx(ss2, o);
                 sw2 += shx(sw2, o);
             }
-            if (h_tiny) {
+            if (h_tiny || w_tiny) {
                 ss = ss2;
                 sw = sw2;
             }
@@ -757,7 +760,6 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
         gq.ylo = ylo;
         gq.yhi = yhi;
         const float cref = mn + rho;  // the centre, rounded (an anchor only)
-        if (h_one) ss = (float)G;
         const float inv_ss = rcp_ftz(ss);  // (at least 2^-40 by now)
         // mu: approximate weighted mean of w (only a centre for the sums)
         const float mu = h_one ? cref : sw * inv_ss;
@@ -1321,6 +1323,10 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1)
         // with the clamp of its set, as pass B formed them)
         const float Pk = R * p.invf[kb];
         const float capk = p.cap[kb] * range;
+        a_sel *= unscale;
+        a_lo *= unscale;
+        Bz *= unscale;
+        Bz_lo *= unscale;
         {
             const float2 a2 = make_float2(a_sel, a_sel), B2 = make_float2(Bz, Bz);
             const float2 alo2 = make_float2(a_lo, a_lo), Blo2 = make_float2(Bz_lo, Bz_lo);

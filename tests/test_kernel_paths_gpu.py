@@ -239,7 +239,7 @@ def _small_weights(rows, G, seed):
 @pytest.mark.parametrize("bits,G,clip", [(2, 64, CLIP8), (4, 128, CLIP8), (8, 32, wl.CLIP_16),
                                          (4, 256, (1.0, 0.25)), (3, 128, (1.0, 0.5, 1e-30, 1e-37))],
                          ids=["int2", "int4", "int8_k16", "int4_two", "tiny_factors"])
-@pytest.mark.parametrize("symmetric", [True])
+@pytest.mark.parametrize("symmetric", [True, False])
 def test_weights_scaled_by_a_power_of_two(oracle, symmetric, bits, G, clip, e):
     """Groups of weights down to the smallest denormals keep the factor and the
     codes that the same weights have at their usual size, and a fit and an r
