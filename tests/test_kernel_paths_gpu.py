@@ -269,3 +269,31 @@ def test_weights_scaled_by_a_power_of_two(oracle, symmetric, bits, G, clip, e):
     O = (oracle.recon_sym if symmetric else oracle.recon_int)(w_h, h, G, bits, list(clip))
     same = (O["m_round"] >= checker.MARGIN) & (O["m_tie"] >= checker.MARGIN)
     assert np.array_equal(small["cand_idx"].cpu().numpy()[same], O["idx"][same])
+
+
+@pytest.mark.parametrize("bits,K", [(2, 8), (2, 16), (3, 8), (4, 16), (8, 8)])
+@pytest.mark.parametrize("descending", [True, False])
+def test_sym_ties_between_runs_of_equal_codes(oracle, bits, K, descending):
+    """Groups of two tight clusters and one weight between them, of a saliency
+    so far below the others' that its codes do not move the fp32 sums: factors
+    of equal sums have different codes and errors."""
+    gen = torch.Generator(device="cuda").manual_seed(17 + bits)
+    n, G = 2048, 128
+    u = lambda *s: torch.rand(*s, generator=gen, device="cuda")
+    w = torch.where(u(n, G) < 0.5, -1.0, 1.0)
+    w[n // 2:] *= 1.0 + 1e-4 * (u(n - n // 2, G) - 0.5)
+    w[:, 17] = u(n) * 1.8 - 0.9
+    v = 1e-6 * (0.5 + u(n, G))
+    v[:, 17] = 1e-6 * 10.0 ** (-10.0 * u(n))
+    clip = list(wl.CLIP_16[:K]) if descending else list(wl.CLIP_16[:K])[::-1]
+    if descending and K == 16:
+        clip = clip[1::2] + clip[::2]                      # in no order
+    w_h, h = H._host(w), H._host(v)
+    o = api.recon_int_batch([(w, None, v)], bits=bits, group_size=G, clip=clip, codes=True, symmetric=True,
+                            r_dtype=torch.float32)[0]
+    torch.cuda.synchronize()
+    O = oracle.recon_sym(w_h, h, G, bits, clip)
+    gpu = {"r": H._host(o["r"]), "a": o["a"].cpu().numpy(), "b": o["b"].cpu().numpy(),
+           "codes": o["codes"].cpu().numpy().ravel(), "idx": o["cand_idx"].cpu().numpy()}
+    rep = checker.check_sym(oracle, w_h, h, bits, clip, O, gpu, G, False)
+    assert rep["ok"], json.dumps(rep)
