@@ -40,6 +40,8 @@ namespace sym {
 
 constexpr float kMagic = 8388608.0f;  // 2^23: adding it rounds to an integer (nearest even)
 constexpr float kU = 5.9604645e-8f;
+// Sums of saliencies beyond this are scaled by 2^-64: S2 and S3^2 stay finite.
+constexpr float kLargeSaliency = 1073741824.0f;  // 2^30
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
 {
@@ -294,14 +296,16 @@ __global__ void __launch_bounds__(int_max_warps(EPL) * 32, 1) k_recon_sym(const 
             ss += __shfl_xor_sync(0xffffffffu, ss, o);
         }
         // all saliencies zero: h = 1; a sum of saliencies, or weights, near the
-        // bottom of the fp32 range: scaled by a power of two in the tile
+        // bottom of the fp32 range, or saliencies whose sums' square could leave
+        // it at the top: scaled by a power of two in the tile
         float unscale = 1.0f;  // of the fit
-        const bool h_tiny = ss < kTinySaliency, w_tiny = amax < kTinyWeights;  // (zeros stay zeros)
-        if (__any_sync(0xffffffffu, h_tiny || w_tiny)) {
-            if (h_tiny || w_tiny) {
+        const bool h_out = ss < kTinySaliency || ss > kLargeSaliency, w_out = amax < kTinyWeights;  // (zeros stay zeros)
+        if (__any_sync(0xffffffffu, h_out || w_out)) {
+            if (h_out || w_out) {
                 float s1 = 1.0f, s2 = 1.0f, t1 = 1.0f, t2 = 1.0f;
-                if (h_tiny && ss > 0.0f) tiny_scale(ss, s1, s2);
-                if (w_tiny) tiny_scale(amax, t1, t2);
+                if (ss > kLargeSaliency) s1 = 5.421011e-20f;  // 2^-64
+                else if (h_out && ss > 0.0f) tiny_scale(ss, s1, s2);
+                if (w_out) tiny_scale(amax, t1, t2);
 #pragma unroll 1
                 for (int i = 0; i < NCHK; ++i) {
                     float4* hp = reinterpret_cast<float4*>(hs + gs * G + eoff(i));

@@ -297,3 +297,19 @@ def test_sym_ties_between_runs_of_equal_codes(oracle, bits, K, descending):
            "codes": o["codes"].cpu().numpy().ravel(), "idx": o["cand_idx"].cpu().numpy()}
     rep = checker.check_sym(oracle, w_h, h, bits, clip, O, gpu, G, False)
     assert rep["ok"], json.dumps(rep)
+
+
+@pytest.mark.parametrize("bits,G", [(3, 128), (8, 32)])
+def test_sym_saliencies_scaled_by_a_power_of_two(bits, G):
+    """Saliencies as large as their type holds give the outputs of the same ones
+    at their usual size: a common scale of h changes nothing."""
+    w, _, v = _inputs(40, G, seed=4800 + bits)
+    v = v.clamp(max=0.5)
+    outs = []
+    for e in (0, 64, 126):
+        outs.append(api.recon_int_batch([(w, None, v * 2.0 ** e)], bits=bits, group_size=G, clip=CLIP8,
+                                        codes=True, symmetric=True)[0])
+        torch.cuda.synchronize()
+    for o in outs[1:]:
+        for key in ("r", "a", "b", "codes", "cand_idx"):
+            assert torch.equal(o[key], outs[0][key]), key
