@@ -385,6 +385,12 @@ __global__ void __launch_bounds__(AheadWarps<AHEAD>::all * 32, 1)
         // takes one loop
         Fit best = evaluate(0);
         int kb = 0;
+        if (!(best.err < INFINITY)) {
+            // moments that overflow: the first candidate of a finite error, or,
+            // where there is none, a scale of 0
+            best.e = 0u;
+            best.err = INFINITY;
+        }
         float En = INFINITY;
 #pragma unroll 2
         for (int k = 1; k < p.n_clip; ++k) {

@@ -313,3 +313,16 @@ def test_sym_saliencies_scaled_by_a_power_of_two(bits, G):
     for o in outs[1:]:
         for key in ("r", "a", "b", "codes", "cand_idx"):
             assert torch.equal(o[key], outs[0][key]), key
+
+
+def test_nvfp4_first_factor_of_overflowing_moments(oracle):
+    """Saliencies so large that the moments of the smaller factors, which come
+    first, overflow (their codes are larger), and those of the last do not: a
+    factor whose error is finite is kept, as the oracle keeps it."""
+    clip = [0.3, 0.35, 1.0]
+    w = torch.zeros(8, 16, device="cuda")
+    v = torch.full((8, 16), 1e-6, device="cuda")
+    w[:, 0] = 400.0                                        # code 6 for every factor
+    w[:, 3], v[:, 3] = 132.0, 2e37                         # code 6 at 0.3 and 0.35, else 2
+    rep, ema = H.run_nvfp4(oracle, w, None, v, clip=clip, r_dtype=torch.float32)
+    _assert(rep, ema)
