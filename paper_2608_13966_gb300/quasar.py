@@ -148,15 +148,19 @@ def quasar_recon_int(w, g, v, beta2, bits, group_size, clip, rows, cols, r, code
     return _STATUS[st]
 
 
+_OPTIONAL = frozenset(("g", "m", "codes", "cand_idx", "tensor_amax"))  # a descriptor may lack
+
+
 def _pack(cls, items, keys):
     """A ctypes array of the descriptor cls from dicts: the pointers named by
-    keys (missing or None: NULL), then rows and cols, packed straight into the
-    array's memory (every field is 8 bytes)."""
+    keys (None, or an optional one that is missing: NULL), then rows and cols,
+    packed straight into the array's memory (every field is 8 bytes)."""
     arr = (cls * len(items))()
     row = struct.Struct(f"={len(keys)}Q2q")
     for i, d in enumerate(items):
-        row.pack_into(arr, i * row.size, *[_ptr(d.get(k)) or 0 for k in keys], int(d["rows"]),
-                      int(d["cols"]))
+        row.pack_into(arr, i * row.size,
+                      *[_ptr(d.get(k) if k in _OPTIONAL else d[k]) or 0 for k in keys],
+                      int(d["rows"]), int(d["cols"]))
     return arr
 
 

@@ -288,3 +288,25 @@ def test_symmetric_option_validation(lib):
                                           options=sym, stream=0) == st.ERR_UNSUPPORTED
     assert Q.quasar_recon_nvfp4_batch_ex([_ndesc()], 0.999, CLIP, sym, stream=0) == st.ERR_INVALID_ARG
     assert Q.quasar_recon_lut_batch([_ldesc()], 0.999, CLIP, sym, stream=0) == st.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("array,required,optional", [
+    (Q.int_tensor_array, "w v r a b", "g codes cand_idx"),
+    (Q.adamw_tensor_array, "w v r a b", "g m codes cand_idx"),
+    (Q.nvfp4_tensor_array, "w v r block_scale tensor_scale", "g tensor_amax codes cand_idx"),
+    (Q.adamw_nvfp4_tensor_array, "w v r block_scale tensor_scale", "g m codes cand_idx"),
+    (Q.lut_tensor_array, "w v r book", "g codes cand_idx"),
+], ids=["int", "adamw", "nvfp4", "adamw_nvfp4", "lut"])
+def test_descriptor_keys(array, required, optional):
+    """A descriptor's optional keys may be missing (NULL); one without a
+    required key is refused, also where its tensor is empty."""
+    full = {k: 16 * (i + 1) for i, k in enumerate(required.split() + optional.split())}
+    full.update(rows=0, cols=0)
+    arr = array([full, full])
+    for k, x in full.items():
+        assert (getattr(arr[1], k) or 0) == x, k
+    for k in optional.split():
+        assert not getattr(array([{n: x for n, x in full.items() if n != k}])[0], k)
+    for k in required.split() + ["rows", "cols"]:
+        with pytest.raises(KeyError):
+            array([{n: x for n, x in full.items() if n != k}])
