@@ -1,7 +1,8 @@
 """The kernels' internal paths at the sizes where they can go wrong: chunks of
 candidates, near ties of equal codes, the lookup table's element lists, signed
-NVFP4 codes, the symmetric codes' clamp sets, and launches around the number
-of CTAs that fit the device."""
+NVFP4 codes, the symmetric codes' clamp sets and candidates of equal sums,
+weights and saliencies at the ends of fp32's range, and launches around the
+number of CTAs or warps that the device holds."""
 import json
 
 import numpy as np
@@ -134,11 +135,12 @@ def test_sym_clamp_sets_equal_per_candidate_clamp(bits, clip, G):
             assert torch.equal(a[key], b[key]), key
 
 
-@pytest.mark.parametrize("units", [1, 7, 151, 153, 303, 305, 2431, 2433])
+@pytest.mark.parametrize("units", [1, 7, 151, 153, 303, 305, 2431, 2433, 3647, 3649])
 @pytest.mark.parametrize("kind", ["int", "sym", "nvfp4", "lut"])
 def test_launches_around_the_number_of_ctas(kind, units):
-    """As many units of work as SMs, resident CTAs or warps, more or less one:
-    the outputs equal those of the same weights passed as two tensors."""
+    """As many units of work as the 152 SMs, twice as many, or as warps (16 an SM,
+    NVFP4 24), more or less one: the outputs equal those of the same weights
+    passed as two tensors."""
     rows, cols = {"int": (8 * units, 32), "sym": (8 * units, 32), "nvfp4": (units, 512),
                   "lut": (8 * units, 64)}[kind]
     w, g, v = _inputs(rows, cols, seed=4400 + units)
