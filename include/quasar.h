@@ -140,7 +140,8 @@ typedef struct {
  *   bits       1..8.
  *   group_size 32, 64, 128 or 256; cols % group_size == 0.
  *   clip       HOST array of n_clip factors, each in (0, 1], in search order;
- *              copied before the call returns.  1 <= n_clip <= 32.
+ *              copied before the call returns.  1 <= n_clip <= 32.  (A factor
+ *              below 2^-90 acts as 2^-90.)
  *   r          [rows, cols] reconstruction, dtype r_dtype (written).
  *   codes      [rows, cols] uint8 codes of the kept candidate, or NULL.
  *   a, b       [rows*cols/group_size] fp32 scale and offset (written).

@@ -194,7 +194,8 @@ __device__ __forceinline__ void stg_cs(uint32_t* p, uint32_t v)
 // Fast reciprocal and reciprocal square root (2 ulps), denormals flushed: one
 // instruction each, where __fdividef and rsqrtf spend five to eight on arguments
 // near the ends of the range.  On normal arguments x * rcp_ftz(y) has
-// __fdividef's bits; callers take care of denormal ones.
+// __fdividef's bits (from 2^126 on both give 0); callers take care of denormal
+// ones, whose reciprocal here is an infinity.
 __device__ __forceinline__ float rcp_ftz(float x)
 {
     float r;

@@ -232,8 +232,9 @@ struct AdamwItem {
     int64_t unit0;  // as for IntTensor, in units of kAheadUnit weights
 };
 
-// Warps of an NVFP4 launch's CTA, one CTA an SM: 24 of 80 registers a thread, or
-// 20 of 96 beside AdamW, which then need not spill; and those of them that begin
+// Warps of an NVFP4 launch's CTA, one CTA an SM: 24 of 80 registers a thread
+// (beside the absmax pass 24 bytes of a thread are spilled: 20 warps of 96 are
+// slower there), or 20 of 96 beside AdamW, which then need not spill; and those of them that begin
 // with a pass for the next stage's tensors.  One layer, AdamW beside the
 // reconstruction: 1,291 us with 4 of 20 warps (5: 1,330, 3: 1,425), 1,322 with 4
 // of 24 (6: 1,368, 8: 1,415), 1,304 with 4 of 16; absmax beside it 912 with 6 of

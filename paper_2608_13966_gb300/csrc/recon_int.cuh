@@ -130,7 +130,7 @@ __device__ __forceinline__ void ff_norm(float& hi, float& lo)
 // on a Llama layer at INT3.  (Smaller still -- passes A and C not unrolled, one
 // reduction loop in the compensated fit, counters in registers, fast roots
 // where they only feed a bound -- the Qwen3 layer took 1,660 us.  All with two
-// CTAs an SM; it takes 1,408 now.)
+// CTAs an SM; it takes 1,385 now.)
 template <bool ROLL>
 __device__ __forceinline__ void ff_reduce32(float& hi, float& lo)
 {
@@ -414,9 +414,9 @@ __device__ void coop_precise(const float* ws, const float* hs, const GroupGeom& 
 // One CTA per SM, its warps taking tiles from one ring as they get free.  Two
 // CTAs of 8 warps (6 with AdamW), a ring each and a fixed share of the tiles a
 // warp, had the same registers and shared memory: one Llama layer INT3 786 us
-// (one CTA with fixed shares 747, as built 740), INT3 15 factors 1,234 (now
-// 1,154), the Qwen3 layer INT2 g64 16 factors 1,551 (fixed shares 1,448, now
-// 1,408), AdamW + INT3 988 (now 916, 15 warps and one slot in flight, 0.985
+// (one CTA with fixed shares 747, now 737), INT3 15 factors 1,234 (now
+// 1,150), the Qwen3 layer INT2 g64 16 factors 1,551 (fixed shares 1,448, now
+// 1,385), AdamW + INT3 988 (now 929, 15 warps and one slot in flight, 0.97
 // of the measured copy rate).  With fixed shares a warp count that is no multiple
 // of the SM's 4 schedulers was worse than the next lower multiple.  20 warps at
 // 96 registers spill: INT3 885 us.

@@ -1,7 +1,7 @@
 // QUASAR for NVFP4 (Sec. 4.2): E2M1 codes, one E4M3 scale per 16-element
 // block, one fp32 scale per tensor s_T = amax/(6*448).  For each block and
 // each search factor f: sigma = f*amax_b/6, codes on the E2M1 grid of
-// |w|/sigma (saturating at 6, ties to even), least-squares slope
+// w/sigma (saturating at 6, ties to even), least-squares slope
 // a* = sum h q w / sum h q^2, E4M3 scale e = rne_satfinite(a* / s_T) (the
 // nearest E4M3 value is exactly optimal because the error is a symmetric
 // quadratic in the scale), error sum h (s_T*e*q - w)^2; keep the lowest.
@@ -18,17 +18,20 @@
 // Per candidate the codes stay in registers: moments -> a* -> E4M3 scale,
 // then the error summed directly, sum h (w - alpha*q)^2 (no cancellation,
 // so its fp32 error is a few ulps of itself).  A candidate within that bound
-// of the best, unless its codes and scale equal the best's (the sum of codes
-// never decreases with the scale factor, so equal sums mean equal codes),
-// sends its block to an exact, float-float comparison.
+// of the best sends its block to an exact, float-float comparison, unless it
+// has the best's key, a 32-bit hash of the moments and the scale: equal codes
+// give equal keys and errors, and the lower index is kept.  (Keys can be equal
+// with other codes, by an element of tiny saliency that moves neither moment,
+// or by chance, about 2^-32: such a candidate is judged by its direct error
+// alone, so the kept one's is within the bound of the least.)
 //
 // What bounds it: instruction issue.  A candidate costs 11 instructions a pair
 // of elements (7 of them packed, two issue cycles each) and about 35 a block;
 // 95 a weight and lane at 8 candidates, 112 before (with absolute values, a
 // hash and an error kept for every candidate, and divisions, E4M3 decoding and
 // sign handling spelled out).  One Llama layer (218 M weights), absmax pass and
-// codes included: 1,152 -> 1,021 us (912 as launched now).  Candidate lists that are not a multiple
-// of 8 used to send every block to the exact comparison.
+// codes included: 1,152 -> 1,021 us (909 as launched now).  Candidate lists that
+// are not a multiple of 8 used to send every block to the exact comparison.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -374,8 +377,7 @@ __global__ void __launch_bounds__(AheadWarps<AHEAD>::all * 32, 1)
                 E2 = __ffma2_rn(__fmul2_rn(h2[t], ev), ev, E2);
             }
             r.err = E2.x + E2.y;
-            // candidates with equal moments and scale have, to within rounding
-            // below the tie margin, equal codes and errors: a key of the three
+            // the key: equal for equal codes
             r.key = (__float_as_uint(s2) * 0x9E3779B1u + __float_as_uint(s3)) ^ r.e;
             return r;
         };

@@ -19,11 +19,12 @@
 // Both sums are over non-negative terms (h |q|^2 and h |q| |w|), so each
 // carries a small relative error and S3^2 / S2 a bound of a few ulps:
 // candidates within the bound of the best are compared exactly (float-float
-// direct errors, whole warp), and the kept fit needs no refinement.
+// direct errors, whole warp), and the kept fit needs no refinement.  Candidates
+// of the best's very sums are settled by their codes.
 //
 // What bounds it: instruction issue and the FP32 pipe (5 packed operations a
 // pair and candidate).  One Llama layer at INT4, group 128, 8 factors (clamp
-// sets 3-3-2): 791 -> 568 us, 6.17 TB/s of algorithmic traffic (626 with two
+// sets 3-3-2): 785 -> 566 us, 6.19 TB/s of algorithmic traffic (626 with two
 // CTAs an SM and a fixed share of the tiles a warp; 20 warps at 96 registers 576).
 #pragma once
 

@@ -241,19 +241,26 @@ def _small_weights(rows, G, seed):
 @pytest.mark.parametrize("bits,G,clip", [(2, 64, CLIP8), (4, 128, CLIP8), (8, 32, wl.CLIP_16),
                                          (4, 256, (1.0, 0.25)), (3, 128, (1.0, 0.5, 1e-30, 1e-37))],
                          ids=["int2", "int4", "int8_k16", "int4_two", "tiny_factors"])
-@pytest.mark.parametrize("symmetric", [True, False])
-def test_weights_scaled_by_a_power_of_two(oracle, symmetric, bits, G, clip, e):
+@pytest.mark.parametrize("kind", ["sym", "int", "adamw"])
+def test_weights_scaled_by_a_power_of_two(oracle, kind, bits, G, clip, e):
     """Groups of weights down to the smallest denormals keep the factor and the
     codes that the same weights have at their usual size, and a fit and an r
-    smaller by the power of two (both code layouts)."""
+    smaller by the power of two (both code layouts; an AdamW step of rate 0)."""
     w, v = _small_weights(40, G, seed=4700 + bits)
     s = 2.0 ** e
 
     def run(w, packed):
-        o = api.recon_int_batch([(w, None, v.clone())], bits=bits, group_size=G, clip=list(clip), codes=True,
-                                symmetric=symmetric, packed_codes=packed, r_dtype=torch.float32)[0]
+        kw = dict(bits=bits, group_size=G, clip=list(clip), codes=True, packed_codes=packed,
+                  r_dtype=torch.float32)
+        v1, z = v.clone(), torch.zeros_like(w)
+        if kind == "adamw":
+            w1 = w.clone()
+            o = api.adamw_recon_int_batch([(w1, z, z.clone(), v1)], lr=0.0, step=1, **kw)[0]
+            assert torch.equal(w1, w)
+        else:
+            o = api.recon_int_batch([(w, None, v1)], symmetric=kind == "sym", **kw)[0]
         torch.cuda.synchronize()
-        return o
+        return dict(o, v=v1)
 
     ref, small, packed = run(w, False), run(w * s, False), run(w * s, True)
     for key in ("codes", "cand_idx"):
@@ -267,8 +274,8 @@ def test_weights_scaled_by_a_power_of_two(oracle, symmetric, bits, G, clip, e):
         lim = 2e-5 * want.abs() + s * 2e-7 + 256 * 2.0 ** -149
         assert bool(((got - want).abs() <= lim).all()), key  # (a NaN fails)
         assert torch.equal(packed[key], small[key]), key
-    w_h, h = H._host(w * s), H._host(v)
-    O = (oracle.recon_sym if symmetric else oracle.recon_int)(w_h, h, G, bits, list(clip))
+    w_h, h = H._host(w * s), H._host(small["v"])
+    O = (oracle.recon_sym if kind == "sym" else oracle.recon_int)(w_h, h, G, bits, list(clip))
     same = (O["m_round"] >= checker.MARGIN) & (O["m_tie"] >= checker.MARGIN)
     assert np.array_equal(small["cand_idx"].cpu().numpy()[same], O["idx"][same])
 
